@@ -1,0 +1,152 @@
+// Building blocks shared by the reduction kernels (panel QR, bulge chase):
+// arithmetic on real and complex entries behind one set of names, sums over
+// neighbouring lanes in a fixed tree, the Householder reflector's scalars,
+// and mbarrier arrivals and waits across the blocks of a cluster.
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+#include "tcgen05.cuh"
+
+namespace gb {
+
+struct Zc {
+    double re, im;
+};
+
+__device__ __forceinline__ void zero_of(double &x) { x = 0.0; }
+__device__ __forceinline__ void zero_of(Zc &x) { x.re = x.im = 0.0; }
+__device__ __forceinline__ void one_of(double &x) { x = 1.0; }
+__device__ __forceinline__ void one_of(Zc &x) { x = Zc{1.0, 0.0}; }
+__device__ __forceinline__ double conj_of(double a) { return a; }
+__device__ __forceinline__ Zc conj_of(Zc a) { return {a.re, -a.im}; }
+__device__ __forceinline__ double mul(double a, double b) { return a * b; }
+__device__ __forceinline__ Zc mul(Zc a, Zc b) { return {fma(a.re, b.re, -a.im * b.im), fma(a.re, b.im, a.im * b.re)}; }
+__device__ __forceinline__ double add(double a, double b) { return a + b; }
+__device__ __forceinline__ Zc add(Zc a, Zc b) { return {a.re + b.re, a.im + b.im}; }
+__device__ __forceinline__ double scale(double a, double f) { return a * f; }
+__device__ __forceinline__ Zc scale(Zc a, double f) { return {a.re * f, a.im * f}; }
+__device__ __forceinline__ double re_of(double a) { return a; }
+__device__ __forceinline__ double re_of(Zc a) { return a.re; }
+__device__ __forceinline__ bool is_zero(double a) { return a == 0.0; }
+__device__ __forceinline__ bool is_zero(Zc a) { return a.re == 0.0 && a.im == 0.0; }
+// a b + c
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ Zc mad(Zc a, Zc b, Zc c)
+{
+    return {fma(-a.im, b.im, fma(a.re, b.re, c.re)), fma(a.im, b.re, fma(a.re, b.im, c.im))};
+}
+// conj(a) b + c
+__device__ __forceinline__ double madc(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ Zc madc(Zc a, Zc b, Zc c)
+{
+    return {fma(a.im, b.im, fma(a.re, b.re, c.re)), fma(-a.im, b.re, fma(a.re, b.im, c.im))};
+}
+template <class T>
+__device__ __forceinline__ T one_v()
+{
+    T x;
+    one_of(x);
+    return x;
+}
+// c - a b
+__device__ __forceinline__ double nmad(double a, double b, double c) { return fma(-a, b, c); }
+__device__ __forceinline__ Zc nmad(Zc a, Zc b, Zc c) { return mad(Zc{-a.re, -a.im}, b, c); }
+
+// Sum over TP neighbouring lanes, each holding V / TP of V partial sums
+// (partial `lane + TP w` in a[w]).  The tree over the V partials is the same
+// for every TP, so that a problem's results do not depend on the cluster
+// shape its chase ran on (alone or in a batch with wider bands).
+__device__ __forceinline__ double xor_add(double x, int o) { return x + __shfl_xor_sync(0xffffffffu, x, o); }
+__device__ __forceinline__ Zc xor_add(Zc x, int o) { return {xor_add(x.re, o), xor_add(x.im, o)}; }
+template <int V, int TP, class T>
+__device__ __forceinline__ T tree_sum(T (&a)[V / TP])
+{
+#pragma unroll
+    for (int h = V / TP / 2; h >= 1; h /= 2)
+#pragma unroll
+        for (int i = 0; i < h; i++) a[i] = add(a[i], a[i + h]);
+    T x = a[0];
+#pragma unroll
+    for (int o = TP / 2; o >= 1; o /= 2) x = xor_add(x, o);
+    return x;
+}
+
+__device__ __forceinline__ double ld_cg(const double *p) { return __ldcg(p); }
+__device__ __forceinline__ Zc ld_cg(const Zc *p)
+{
+    const double2 t = __ldcg(reinterpret_cast<const double2 *>(p));
+    return {t.x, t.y};
+}
+
+// tau, scale and beta of the reflector (LAPACK form, v_0 = 1): alpha the
+// first entry, ss the sum of |x_i|^2 below it.  The two quotients are
+// computed by two lanes of the calling warp at once (all lanes call).
+struct Refl {
+    double tau, scal, beta;
+};
+struct ReflZ {
+    Zc tau, scal;
+    double beta;
+};
+__device__ __forceinline__ Refl reflector(double alpha, double ss)
+{
+    double tau = 0.0, scal = 0.0, beta = alpha;
+    if (ss != 0.0) {
+        const double nrm = sqrt(alpha * alpha + ss);
+        beta = (alpha >= 0.0) ? -nrm : nrm;
+        const bool odd = threadIdx.x & 1;
+        const double qt = (odd ? 1.0 : beta - alpha) / (odd ? alpha - beta : beta);
+        tau = __shfl_sync(0xffffffffu, qt, 0);
+        scal = __shfl_sync(0xffffffffu, qt, 1);
+    }
+    return {tau, scal, beta};
+}
+__device__ __forceinline__ ReflZ reflector(Zc alpha, double ss)
+{
+    Zc tau{0.0, 0.0}, scal{0.0, 0.0};
+    double beta = alpha.re;
+    if (!(ss == 0.0 && alpha.im == 0.0)) {
+        const double nrm = sqrt(alpha.re * alpha.re + alpha.im * alpha.im + ss);
+        beta = (alpha.re >= 0.0) ? -nrm : nrm;
+        const double dr = alpha.re - beta;                    // 1 / (alpha - beta)
+        const double dd = dr * dr + alpha.im * alpha.im;
+        const int l = threadIdx.x & 3;
+        const double num = l == 0 ? beta - alpha.re : l == 1 ? -alpha.im : l == 2 ? dr : -alpha.im;
+        const double q = num / (l < 2 ? beta : dd);
+        tau = Zc{__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1)};
+        scal = Zc{__shfl_sync(0xffffffffu, q, 2), __shfl_sync(0xffffffffu, q, 3)};
+    }
+    return {tau, scal, beta};
+}
+
+__device__ __forceinline__ unsigned long long now_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// one arrival on the barrier at `bar`'s offset in block `rank` of the cluster
+__device__ __forceinline__ void mbar_arrive_remote(void *bar, int rank)
+{
+    asm volatile(
+        "{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, %1;\n"
+        "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n}\n" ::"r"(tc5::smem_addr(bar)),
+        "r"(rank)
+        : "memory");
+}
+
+__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        "selp.b32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+}  // namespace gb
