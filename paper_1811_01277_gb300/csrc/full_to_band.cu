@@ -3,8 +3,10 @@
 // Householder QR of a tall panel, the block-reflector T matrix, and the
 // small conversions around the GEMMs (which run in cuBLAS, see solve.cu).
 //
-// Panel QR (m x nb, column-major, leading dimension lda): for each column i
-// the reflector that annihilates rows i+1..m-1 is built and applied to the
+// Panel QR (m x nb, column-major, leading dimension lda): panel_qr.cu's
+// register-resident kernel where the panel fits a cluster or a co-resident
+// grid; the form here serves the panels that do not (and tall ones under
+// stream capture).  For each column i the reflector that annihilates rows i+1..m-1 is built and applied to the
 // columns to its right, in two launches over row chunks of kChunk rows:
 //   refl_dots:  every block sums the partial squared norms of column i (left
 //               by the previous launch), forms alpha, beta, tau, scales its
@@ -280,9 +282,29 @@ __global__ void __launch_bounds__(256) symmetrize_lower(int n, int j0, double *_
 
 int panel_chunks(int m) { return (m + kChunk - 1) / kChunk; }
 
-// Householder QR of the m x nb panel P (lda); part holds 2*nchunks + nchunks*64 doubles.
-cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, double *part, cudaStream_t st)
+size_t panel_part_bytes(int m, int is_complex);
+cudaError_t panel_qr_resident(int is_complex, int m, int nb, double *P, long long lda, double *tau, double *Y,
+                              long long ldy, void *part, cudaStream_t st, bool *done);
+cudaError_t panel_y_and_t_prep(int m, int nb, const double *P, long long lda, double *Y, long long ldy,
+                               cudaStream_t st);
+
+// Bytes of panel_qr's `part`: the exchange area of panel_qr.cu, or 2*nchunks +
+// nchunks*64 values here.
+size_t panel_qr_part_bytes(int m, int is_complex)
 {
+    const size_t nch = (size_t)panel_chunks(m), here = (2 * nch + (is_complex ? 128 : 64) * nch) * sizeof(double);
+    const size_t resident = panel_part_bytes(m, is_complex);
+    return here > resident ? here : resident;
+}
+
+// Householder QR of the m x nb panel P (lda) and its explicit reflectors Y
+// (ldy); part holds panel_qr_part_bytes(m, 0) bytes, 256-byte aligned.
+cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
+                     cudaStream_t st)
+{
+    bool done = false;
+    cudaError_t er = panel_qr_resident(0, m, nb, P, lda, tau, Y, ldy, part, st, &done);
+    if (er != cudaSuccess || done) return er;
     const int nch = panel_chunks(m);
     double *norm_a = part, *norm_b = part + nch, *dots = part + 2 * nch;
     // columns past the last reflector (m < nb) keep tau = 0
@@ -302,7 +324,8 @@ cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, doubl
     if ((e = cudaStreamIsCapturing(st, &cap)) != cudaSuccess) return e;
     if (coop && cap == cudaStreamCaptureStatusNone && (long long)nch * 4 <= (long long)per_sm * sms) {
         void *args[] = {&m, &nb, &P, &lda, &tau, &norm_a, &norm_b, &dots, (void *)&nch};
-        return cudaLaunchCooperativeKernel((const void *)panel_qr_fused, dim3(nch), dim3(kChunk), args, 0, st);
+        e = cudaLaunchCooperativeKernel((const void *)panel_qr_fused, dim3(nch), dim3(kChunk), args, 0, st);
+        return e != cudaSuccess ? e : panel_y_and_t_prep(m, nb, P, lda, Y, ldy, st);
     }
     panel_first_norm<<<nch, kChunk, 0, st>>>(m, P, lda, norm_a);
     for (int i = 0; i < nb && i < m; i++) {
@@ -311,7 +334,7 @@ cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, doubl
         panel_refl_dots<<<nch, kChunk, 0, st>>>(m, nb, i, P, lda, cur, nch, dots, tau);
         panel_update<<<nch, kChunk, 0, st>>>(m, nb, i, P, lda, dots, nch, tau, nxt, cur);
     }
-    return cudaGetLastError();
+    return panel_y_and_t_prep(m, nb, P, lda, Y, ldy, st);
 }
 
 cudaError_t panel_y_and_t_prep(int m, int nb, const double *P, long long lda, double *Y, long long ldy,

@@ -228,8 +228,19 @@ __global__ void __launch_bounds__(256) real_to_complex(long long rows, long long
 
 int panel_chunks(int m);
 
-cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, double *part, cudaStream_t st)
+cudaError_t panel_qr_resident(int is_complex, int m, int nb, double *P, long long lda, double *tau, double *Y,
+                              long long ldy, void *part, cudaStream_t st, bool *done);
+cudaError_t zpanel_y(int m, int nb, const double *P, long long lda, double *Y, long long ldy, cudaStream_t st);
+
+// Householder QR of the complex m x nb panel P and its explicit reflectors Y:
+// panel_qr.cu's kernel where the panel fits it, else the form above; part
+// holds panel_qr_part_bytes(m, 1) bytes, 256-byte aligned.
+cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
+                      cudaStream_t st)
 {
+    bool done = false;
+    cudaError_t er = panel_qr_resident(1, m, nb, P, lda, tau, Y, ldy, part, st, &done);
+    if (er != cudaSuccess || done) return er;
     const int nch = panel_chunks(m);
     double *norm_a = part, *norm_b = part + nch;
     Zd *dots = (Zd *)(part + 2 * nch);  // nch * 64 complex
@@ -242,7 +253,7 @@ cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, doub
         zpanel_refl_dots<<<nch, kChunk, 0, st>>>(m, nb, i, (Zd *)P, lda, cur, nch, dots, (Zd *)tau);
         zpanel_update<<<nch, kChunk, 0, st>>>(m, nb, i, (Zd *)P, lda, dots, nch, (const Zd *)tau, nxt, cur);
     }
-    return cudaGetLastError();
+    return zpanel_y(m, nb, P, lda, Y, ldy, st);
 }
 
 cudaError_t zpanel_y(int m, int nb, const double *P, long long lda, double *Y, long long ldy, cudaStream_t st)

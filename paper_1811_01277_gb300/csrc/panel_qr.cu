@@ -1,0 +1,359 @@
+// Householder QR of a tall panel (m x nb, column-major, real or complex), the
+// step of full -> band (Sec. 2, two-stage reduction) that forms a chain: nb
+// reflectors, each needing sums over all rows of the one before.
+//
+// The panel stays in registers from its load to its only store: its rows are
+// dealt in runs of CH = LPC * RPT to the blocks, and in a block LPC threads
+// hold one column, RPT rows each.  Per column i
+//   1. the column's threads put its rows below i, x, into shared memory;
+//   2. every column j >= i forms its partial sum of conj(x) a_j (j = i: the
+//      squared norm) and the partials are exchanged once; row i goes along;
+//   3. every block derives tau, the scale and beta from them, and updates
+//      a_j -= x (scale w_j), w_j = conj(tau) (a_ij + conj(scale) sum_j), which is
+//      H(i)^H applied with v = [1; scale x].
+// One exchange per column, against two grid-wide barriers and four passes
+// over the panel in L2 for a form with separate norm, dot and update phases.
+//
+// The exchange: blocks of one cluster (up to 16) write their partials into
+// each other's shared memory and arrive on each other's mbarriers; taller
+// panels use a cooperative grid, partials in global memory and one counter.
+//
+// What bounds it: FP64 issue (2 multiply-adds per clock and SM: about
+// m nb^2 / (2 blocks) clocks a panel) and the exchange's latency.
+// Measured on a GB300: a 992 x 32 panel takes 0.14 ms (4.4 us a column), a
+// complex 960 x 64 one 1.0 ms; the forms before (two launches or grid barriers
+// per column) took about 35 us a column.  full -> band of n = 1024, nbw = 32:
+// 37.7 -> 22.8 ms, n = 8192, nbw = 64: 467 -> 312 ms.
+//
+// On exit the panel holds R on and above the diagonal and v below it (LAPACK
+// layout, v_0 = 1 implicit), tau the nb scalars, and Y (if given) the explicit
+// unit lower trapezoidal reflectors.
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "reduction.cuh"
+
+namespace gb {
+
+namespace cg = cooperative_groups;
+
+namespace {
+
+constexpr long long kPanelWaitNs = 10LL * 1000 * 1000 * 1000;
+constexpr int kClusterMax = 16;
+
+template <class T, int NB, int CH>
+struct PanelShared {
+    T x[2][CH];
+    T ms[2][kClusterMax][NB];   // cluster exchange: partial sums by rank
+    T ma[2][NB];                // row i
+    T tau[2], scal[2];
+    double beta[2];
+    unsigned long long bar[2];
+    int gave_up;
+};
+
+// Exchange area of the grid form, in global memory.
+template <class T, int NB>
+struct PanelGrid {
+    unsigned int arrivals;
+    unsigned int pad[63];
+    T ma[2][NB];
+    T ms[1];                    // [2][blocks][NB]
+};
+
+template <class T, int NB, int LPC, int RPT, bool GRID>
+__global__ void __launch_bounds__(NB *LPC, 1)
+panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__ tau_out, T *__restrict__ Y,
+                long long ldy, PanelGrid<T, NB> *gx)
+{
+    constexpr int CH = LPC * RPT;
+    __shared__ PanelShared<T, NB, CH> sm;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int col = tid / LPC, part = tid % LPC;
+    const int blocks = (int)gridDim.x, rank = (int)blockIdx.x;   // one cluster, or the whole grid
+    const int r0 = rank * CH;
+    cg::cluster_group cluster = cg::this_cluster();
+
+    T a[RPT];
+#pragma unroll
+    for (int t = 0; t < RPT; t++) {
+        const int r = r0 + part + LPC * t;
+        zero_of(a[t]);
+        if (col < nb && r < m) a[t] = P[(long long)col * lda + r];
+    }
+    if (tid == 0) {
+        sm.gave_up = 0;
+        if (!GRID) {
+            tc5::mbar_init(tc5::smem_addr(&sm.bar[0]), blocks);
+            tc5::mbar_init(tc5::smem_addr(&sm.bar[1]), blocks);
+            tc5::mbar_init_fence();
+        }
+    }
+    if (!GRID) cluster.sync();
+
+    const int steps = min(nb, m);
+    for (int i = 0; i < steps; i++) {
+        const int par = i & 1;
+        const bool live = (warp * 32) / LPC + 32 / LPC > i;   // a column of this warp is not done yet
+        if (col == i) {
+#pragma unroll
+            for (int t = 0; t < RPT; t++) {
+                T x = a[t];
+                if (r0 + part + LPC * t <= i) zero_of(x);
+                sm.x[par][part + LPC * t] = x;
+            }
+        }
+        __syncthreads();
+        const int il = i - r0;                                   // row i in this block, if it holds it
+        const bool owner = il >= 0 && il < CH;
+        if (live) {
+            constexpr int NA = 8 / LPC;
+            T acc[NA];
+#pragma unroll
+            for (int t = 0; t < NA; t++) zero_of(acc[t]);
+#pragma unroll
+            for (int t = 0; t < RPT; t++) acc[t % NA] = madc(sm.x[par][part + LPC * t], a[t], acc[t % NA]);
+            const T sum = tree_sum<8, LPC>(acc);
+            T ai;
+            zero_of(ai);
+            if (owner) {
+                // the entry of row i, from the lane that holds it
+#pragma unroll
+                for (int t = 0; t < RPT; t++)
+                    if (part + LPC * t == il) ai = a[t];
+#pragma unroll
+                for (int o = LPC / 2; o >= 1; o /= 2) ai = xor_add(ai, o);   // the other lanes hold zero
+            }
+            if (GRID) {
+                if (part == 0) {
+                    gx->ms[((size_t)par * blocks + rank) * NB + col] = sum;
+                    if (owner) gx->ma[par][col] = ai;
+                }
+            } else {
+                for (int d = part; d < blocks; d += LPC) {
+                    cluster.map_shared_rank(&sm.ms[par][rank][col], d)[0] = sum;
+                    if (owner) cluster.map_shared_rank(&sm.ma[par][col], d)[0] = ai;
+                }
+            }
+        }
+        __syncthreads();
+        if (GRID) {
+            if (tid == 0) {
+                __threadfence();
+                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gx->arrivals) : "memory");
+                const unsigned int need = (unsigned int)(i + 1) * (unsigned int)blocks;
+                unsigned long long t0 = 0;
+                for (long long it = 0; !sm.gave_up; it++) {
+                    unsigned int got;
+                    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&gx->arrivals) : "memory");
+                    if (got >= need) break;
+                    if (it == 0) t0 = now_ns();
+                    if ((it & 63) == 63 && (long long)(now_ns() - t0) > kPanelWaitNs) sm.gave_up = 1;
+                }
+            }
+            __syncthreads();
+        } else {
+            if (tid < blocks) {
+                asm volatile("fence.acq_rel.cluster;" ::: "memory");
+                mbar_arrive_remote(&sm.bar[par], tid);
+            }
+            const uint32_t bar = tc5::smem_addr(&sm.bar[par]);
+            const uint32_t phase = (uint32_t)(i >> 1) & 1;
+            if (!mbar_try_cluster(bar, phase)) {
+                const unsigned long long t0 = now_ns();
+                for (long long it = 1; !mbar_try_cluster(bar, phase); it++)
+                    if ((it & 63) == 0 && (long long)(now_ns() - t0) > kPanelWaitNs) {
+                        sm.gave_up = 1;
+                        break;
+                    }
+            }
+        }
+        T sum, ai;
+        zero_of(sum);
+        zero_of(ai);
+        if (live) {
+            constexpr int NA = 8 / LPC;
+            T acc[NA];
+#pragma unroll
+            for (int t = 0; t < NA; t++) zero_of(acc[t]);
+            // partials of blocks part, part + LPC, ...: the same order for every form
+            for (int d = part; d < blocks; d += 8) {
+#pragma unroll
+                for (int t = 0; t < NA; t++)
+                    if (d + LPC * t < blocks)
+                        acc[t] = add(acc[t], GRID ? ld_cg(&gx->ms[((size_t)par * blocks + d + LPC * t) * NB + col])
+                                                  : sm.ms[par][d + LPC * t][col]);
+            }
+            sum = tree_sum<8, LPC>(acc);
+            ai = GRID ? ld_cg(&gx->ma[par][col]) : sm.ma[par][col];
+            if (warp == (i * LPC) / 32) {   // the warp that holds column i
+                const int src = (i * LPC) & 31;
+                const double ss = __shfl_sync(0xffffffffu, re_of(sum), src);
+                T alpha = ai;
+                *(double *)&alpha = __shfl_sync(0xffffffffu, *(double *)&ai, src);
+                if (sizeof(T) == 16)
+                    ((double *)&alpha)[sizeof(T) / 8 - 1] =
+                        __shfl_sync(0xffffffffu, ((double *)&ai)[sizeof(T) / 8 - 1], src);
+                const auto h = reflector(alpha, ss);
+                if ((tid & 31) == 0) {
+                    sm.tau[par] = h.tau;
+                    sm.scal[par] = h.scal;
+                    sm.beta[par] = h.beta;
+                    if (rank == 0) tau_out[i] = h.tau;
+                }
+            }
+        }
+        __syncthreads();
+        if (live) {
+            const T tau = sm.tau[par], scal = sm.scal[par];
+            if (col > i) {
+                const T w = mul(conj_of(tau), mad(conj_of(scal), sum, ai));
+                const T f = mul(scal, w);
+#pragma unroll
+                for (int t = 0; t < RPT; t++) a[t] = nmad(sm.x[par][part + LPC * t], f, a[t]);
+                if (owner) {
+#pragma unroll
+                    for (int t = 0; t < RPT; t++)
+                        if (part + LPC * t == il) a[t] = nmad(w, one_v<T>(), a[t]);
+                }
+            } else if (col == i) {
+                T beta;
+                zero_of(beta);
+                *(double *)&beta = sm.beta[par];
+#pragma unroll
+                for (int t = 0; t < RPT; t++) {
+                    const int r = r0 + part + LPC * t;
+                    if (r > i) a[t] = mul(a[t], scal);
+                    else if (r == i) a[t] = beta;
+                }
+            }
+        }
+    }
+    T nan;
+    zero_of(nan);
+    *(double *)&nan = __longlong_as_double(0x7ff8000000000000ll);
+    if (sm.gave_up && tid < nb) tau_out[tid] = nan;   // a wait gave up: the result is void and says so
+    if (rank == 0 && tid >= steps && tid < nb) zero_of(tau_out[tid]);
+#pragma unroll
+    for (int t = 0; t < RPT; t++) {
+        const int r = r0 + part + LPC * t;
+        if (col < nb && r < m) {
+            P[(long long)col * lda + r] = a[t];
+            if (Y) {
+                T y = a[t];
+                if (r < col) zero_of(y);
+                else if (r == col) one_of(y);
+                Y[(long long)col * ldy + r] = y;
+            }
+        }
+    }
+    if (!GRID) {
+        __syncwarp();
+        cluster.sync();   // no block leaves while a peer may still reach its shared memory
+    }
+}
+
+template <class T, int NB, int LPC, int RPT>
+cudaError_t launch_cluster(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, cudaStream_t st)
+{
+    constexpr int CH = LPC * RPT;
+    auto kernel = panel_qr_kernel<T, NB, LPC, RPT, false>;
+    const int blocks = (m + CH - 1) / CH;
+    int size = 1;
+    while (size < blocks) size *= 2;
+    cudaError_t e;
+    if (size > 8 && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+        return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3(NB * LPC);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, m, nb, P, lda, tau, Y, ldy, (PanelGrid<T, NB> *)nullptr);
+}
+
+// *done = false (and nothing launched) where the grid does not fit in
+// 1 / `share` of the device's co-resident capacity
+template <class T, int NB, int LPC, int RPT>
+cudaError_t launch_grid(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, void *part, int sms,
+                        int share, cudaStream_t st, bool *done)
+{
+    constexpr int CH = LPC * RPT;
+    auto kernel = panel_qr_kernel<T, NB, LPC, RPT, true>;
+    int blocks = (m + CH - 1) / CH, per_sm = 0;
+    *done = false;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, NB * LPC, 0);
+    if (e != cudaSuccess) return e;
+    if ((long long)blocks * share > (long long)per_sm * sms) return cudaSuccess;
+    if ((e = cudaMemsetAsync(part, 0, 256, st)) != cudaSuccess) return e;
+    PanelGrid<T, NB> *gx = (PanelGrid<T, NB> *)part;
+    void *args[] = {&m, &nb, &P, &lda, &tau, &Y, &ldy, &gx};
+    *done = true;
+    return cudaLaunchCooperativeKernel((const void *)kernel, dim3(blocks), dim3(NB * LPC), args, 0, st);
+}
+
+template <class T>
+cudaError_t panel_qr_t(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, void *part, cudaStream_t st,
+                       bool *done)
+{
+    constexpr bool Z = sizeof(T) == 16;
+    *done = true;
+    if (nb <= 32) {
+        if (m <= 32 * kClusterMax) return launch_cluster<T, 32, 8, 4>(m, nb, P, lda, tau, Y, ldy, st);
+        if (m <= 64 * kClusterMax) return launch_cluster<T, 32, 8, 8>(m, nb, P, lda, tau, Y, ldy, st);
+        if (m <= 128 * kClusterMax) return launch_cluster<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, st);
+    } else {
+        if (m <= 32 * kClusterMax) return launch_cluster<T, 64, 4, 8>(m, nb, P, lda, tau, Y, ldy, st);
+        if (m <= 64 * kClusterMax) return launch_cluster<T, 64, 4, 16>(m, nb, P, lda, tau, Y, ldy, st);
+        if (!Z && m <= 128 * kClusterMax) return launch_cluster<T, 64, Z ? 4 : 8, 16>(m, nb, P, lda, tau, Y, ldy, st);
+    }
+    *done = false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    int dev = 0, sms = 0, coop = 0;
+    cudaError_t e = cudaStreamIsCapturing(st, &cap);
+    if (e != cudaSuccess || cap != cudaStreamCaptureStatusNone) return e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (!coop) return cudaSuccess;
+    // half of the co-resident capacity, so that work on other streams keeps
+    // room beside it; the tallest panels (over 9728 rows real, 4864 complex)
+    // may take all of it
+    if (nb <= 32) {
+        e = launch_grid<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 2, st, done);
+        if (e != cudaSuccess || *done) return e;
+        return launch_grid<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 1, st, done);
+    }
+    e = launch_grid<T, 64, 4, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 2, st, done);
+    if (e != cudaSuccess || *done) return e;
+    return launch_grid<T, 64, 4, Z ? 16 : 32>(m, nb, P, lda, tau, Y, ldy, part, sms, 1, st, done);
+}
+
+}  // namespace
+
+// Bytes of the exchange area a panel of m rows may need (`part`).
+size_t panel_part_bytes(int m, int is_complex)
+{
+    const size_t blocks = ((size_t)m + 63) / 64;
+    return 256 + (size_t)2 * 64 * (blocks + 1) * (is_complex ? 16 : 8);
+}
+
+// QR of the m x nb panel P (lda, nb <= 64) and, where Y is not null, its
+// explicit reflectors (ldy).  *done = false: nothing was done, the panel is
+// too tall for one co-resident grid (or for a cluster, under capture).
+cudaError_t panel_qr_resident(int is_complex, int m, int nb, double *P, long long lda, double *tau, double *Y,
+                              long long ldy, void *part, cudaStream_t st, bool *done)
+{
+    if (is_complex) return panel_qr_t<Zc>(m, nb, (Zc *)P, lda, (Zc *)tau, (Zc *)Y, ldy, part, st, done);
+    return panel_qr_t<double>(m, nb, P, lda, tau, Y, ldy, part, st, done);
+}
+
+}  // namespace gb

@@ -43,8 +43,9 @@ size_t tridiag_dc_workspace_bytes(int n);
 cudaError_t tridiag_dc_d(int n, int nev, const double *d, const double *e, double *lam, double *Z, long long ldz,
                          void *ws, cudaStream_t st);
 
-int panel_chunks(int m);
-cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, double *part, cudaStream_t st);
+size_t panel_qr_part_bytes(int m, int is_complex);
+cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
+                     cudaStream_t st);
 cudaError_t panel_y_and_t_prep(int m, int nb, const double *P, long long lda, double *Y, long long ldy,
                                cudaStream_t st);
 cudaError_t panel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt,
@@ -52,7 +53,8 @@ cudaError_t panel_t(int nb, const double *G, long long ldg, const double *tau, d
 cudaError_t newton_schulz_matrix(int k, double *G, long long ldg, cudaStream_t st);
 cudaError_t band_from_full(int n, int b, const double *A, long long lda, double *AB, long long ldab, cudaStream_t st);
 
-cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, double *part, cudaStream_t st);
+cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
+                      cudaStream_t st);
 cudaError_t zpanel_y(int m, int nb, const double *P, long long lda, double *Y, long long ldy, cudaStream_t st);
 cudaError_t zpanel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt,
                      cudaStream_t st);
@@ -179,7 +181,6 @@ SolveWs carve(int n, int nev, int b, char *base, char *pbase = nullptr, bool spl
     };
     const size_t P = (size_t)(n + b - 1) / b;
     const size_t cnt = (size_t)gb::hh_total(n, b);
-    const size_t nch = (size_t)gb::panel_chunks(n);
     w.Aw = (double *)ptake((size_t)n * n * 8);
     w.tauP = (double *)ptake(P * b * 8);
     w.Tall = (double *)ptake(P * b * b * 8);
@@ -190,7 +191,7 @@ SolveWs carve(int n, int nev, int b, char *base, char *pbase = nullptr, bool spl
     w.Pm = (double *)take((size_t)b * b * 8);
     w.M = (double *)take((size_t)b * b * 8);
     w.G = (double *)take((size_t)b * b * 8);
-    w.part = (double *)take((2 * nch + 64 * nch) * 8);
+    w.part = (double *)take(gb::panel_qr_part_bytes(n, 0));
     w.AB = (double *)take((size_t)(b + 1) * n * 8);
     w.d = (double *)take((size_t)n * 8);
     w.e = (double *)take((size_t)n * 8);
@@ -249,7 +250,6 @@ SolveWsZ carve_z(int n, int nev, int b, char *base)
     };
     const size_t P = (size_t)(n + b - 1) / b;
     const size_t cnt = (size_t)gb::hh_total(n, b);
-    const size_t nch = (size_t)gb::panel_chunks(n);
     w.Aw = (double *)take((size_t)n * n * 16);
     w.tauP = (double *)take(P * b * 16);
     w.Tall = (double *)take(P * b * b * 16);
@@ -259,7 +259,7 @@ SolveWsZ carve_z(int n, int nev, int b, char *base)
     w.Pm = (double *)take((size_t)b * b * 16);
     w.M = (double *)take((size_t)b * b * 16);
     w.G = (double *)take((size_t)b * b * 16);
-    w.part = (double *)take((2 * nch + 128 * nch) * 8);
+    w.part = (double *)take(gb::panel_qr_part_bytes(n, 1));
     w.AB = (double *)take((size_t)(b + 1) * n * 16);
     w.d = (double *)take((size_t)n * 8);
     w.e = (double *)take((size_t)n * 8);
@@ -366,8 +366,8 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         double *panel = w.Aw + (long long)j * ldw + (j + b);
         double *Yp = Ybuf[p & 1];
         cudaError_t e;
-        if ((e = gb::panel_qr(m, b, panel, ldw, w.tauP + (long long)p * b, w.part, fst)) != cudaSuccess) return e;
-        if ((e = gb::panel_y_and_t_prep(m, b, panel, ldw, Yp, m, fst)) != cudaSuccess) return e;
+        if ((e = gb::panel_qr(m, b, panel, ldw, w.tauP + (long long)p * b, Yp, m, w.part, fst)) != cudaSuccess)
+            return e;
         if ((e = gb::dfma_gemm('T', 'N', b, b, m, 1.0, Yp, m, Yp, m, 0.0, w.G, b, w.gw2, w.gw2_elems, fst)) !=
             cudaSuccess)
             return e;
@@ -557,8 +557,7 @@ int solve_z_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         C *A2 = Aw + (long long)(j + b) * ldw + (j + b);
         double *tau = w.tauP + (long long)pp * b * 2;
         C *T = (C *)(w.Tall + (long long)pp * b * b * 2);
-        GB_CU(gb::zpanel_qr(m, b, (double *)panel, ldw, tau, w.part, st));
-        GB_CU(gb::zpanel_y(m, b, (const double *)panel, ldw, (double *)Y, m, st));
+        GB_CU(gb::zpanel_qr(m, b, (double *)panel, ldw, tau, (double *)Y, m, w.part, st));
         GB_CU(zg('C', 'N', b, b, m, one, Y, m, Y, m, zero, G, b, 0));
         GB_CU(gb::zpanel_t(b, (const double *)G, b, tau, (double *)T, b, st));
         GB_CU(zg('N', 'N', m, b, b, one, Y, m, T, b, zero, YT, m, 0));

@@ -167,7 +167,10 @@ class EigenServer:
             if lane["end"] is not None:
                 continue
             ready = [r for r in self.active if r._phase == "chase_wait"]
-            if not ready:
+            # fronts finish within a few milliseconds of one another: a launch
+            # waits until at least as many requests are ready as are still in
+            # their fronts, or it would take them one by one
+            if not ready or len(ready) < sum(r._phase == "front" for r in self.active):
                 break
             kind = ready[0].complex
             batch = [r for r in ready if r.complex == kind]
