@@ -1,20 +1,17 @@
-// FP64 products on the bf16 tensor cores by exact digit slicing; the scheme
-// and its accuracy are described in dgemm_sliced.cuh.
+// FP64 and FP32 products on the tensor cores by splitting the operands into
+// 16-bit planes; the schemes and their accuracy are described in
+// dgemm_sliced.cuh.  The FP64-accurate digit products run in sliced_tc5.cu
+// (tcgen05); this file holds the FP32 split and its product,
+// the split-K reduction and the whole-product forms.
 //
-// Slicing: two passes over 32 x 32 tiles of the slice-row view, staged in
-// shared memory so that global reads follow the source's contiguous index;
-// pass 1 takes each row's largest magnitude (atomicMax on the bit pattern),
-// pass 2 cuts every entry into digits with integer arithmetic on its bit
-// pattern (no FP64 instructions) and writes the bf16 planes, k fastest.
-//
+// FP32 split: each entry's FP32 rounding becomes three bf16 planes, k fastest.
 // Product: one 256-thread block per 64 x 32 tile of C, warps 4 (rows) x 2
-// (columns), each warp 16 x 16 = two m16n8 accumulator tiles per level.
-// K advances 32 at a time through a two-stage cp.async pipeline holding the
-// D digit planes of the A and B tiles that the product forms (rows padded to
-// 80 bytes so that the ldmatrix row addresses of a phase fall in distinct
-// banks).  Per k16 step the warp loads the D A-plane fragments once and, per
-// B plane j, issues mma.sync m16n8k16 bf16 for every A plane i whose level
-// i + j is formed, into the accumulator of that level.
+// (columns), each warp 16 x 16 = two m16n8 accumulator tiles.  K advances 32
+// at a time through a two-stage cp.async pipeline holding the three planes of
+// the A and B tiles (rows padded to 80 bytes so that the ldmatrix row
+// addresses of a phase fall in distinct banks).  Per k16 step the warp loads
+// the A-plane fragments once and, per B plane j, issues mma.sync m16n8k16 bf16
+// for the A planes i <= 2 - j.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -23,6 +20,7 @@
 
 #include "dgemm_sliced.cuh"
 #include "mma_bf16.cuh"
+#include "slice_views.cuh"
 
 namespace gb {
 
@@ -32,16 +30,9 @@ constexpr int kBM = 64, kBN = 32, kBK = 32;
 constexpr int kRowPad = 40;  // bf16 per staged row (32 used)
 constexpr int kThreads = 256;
 constexpr int kStages = 2;
-// bf16 per pipeline stage and dynamic shared memory of a D-digit product
-template <int D>
-__host__ __device__ constexpr size_t stage_elems() { return (size_t)D * (kBM + kBN) * kRowPad; }
-template <int D>
-__host__ __device__ constexpr size_t product_smem() { return kStages * stage_elems<D>() * sizeof(uint16_t); }
-
-static_assert(kSlices * kDigitBits <= 56, "digits come from the 56-bit fixed-point magnitude");
-static_assert(kSlices == 8 && kLevels == 9, "the level folding below assumes at most eight digits, levels 0..8");
-static_assert(kSlices * 127 * 127 * kFlushK < (1 << 24), "every level must stay below 2^24 units per flush");
-constexpr int kMaxSplitK = 65536;  // keeps lo below 2^61: 512 flushes of at most 2^52
+// bf16 per pipeline stage and dynamic shared memory
+constexpr size_t kStageElems = (size_t)kSplitPlanes * (kBM + kBN) * kRowPad;
+constexpr size_t kProductSmem = kStages * kStageElems * sizeof(uint16_t);
 
 size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
@@ -50,97 +41,22 @@ struct SliceLayout {
     size_t planes, e, rmax, total;
 };
 
-// (the layout always has room for kSlices planes, so one buffer serves every
-// digit count)
+// (the layout has room for the digit planes, so one buffer serves both forms:
+// three planes of Rp x Kp take less)
 SliceLayout slice_layout(int R, int K)
 {
-    const size_t Rp = (size_t)round_up(R > 0 ? R : 1, kBM), Kp = (size_t)round_up(K > 0 ? K : 1, kBK);
+    const size_t Rp = (size_t)tc5_rows_padded(R);
     SliceLayout L;
     L.planes = 0;
-    L.e = a256(L.planes + (size_t)kSlices * Rp * Kp * sizeof(uint16_t));
+    L.e = a256(L.planes + tc5_planes_bytes(R, K));
     L.rmax = a256(L.e + Rp * sizeof(int));
-    L.total = a256(L.rmax + Rp * sizeof(unsigned long long));
+    L.total = a256(L.rmax + Rp * sizeof(uint32_t));
     return L;
 }
 
-// entry (a, b) of the 2 x 2 real block [x -y; y x] of x + iy
-__device__ __forceinline__ double zblock(double x, double y, int a, int b) { return a == b ? x : (a ? y : -y); }
-
-// element (r, k) of the view (r < R, k < K)
-__device__ __forceinline__ double view_at(int view, const double *__restrict__ src, long long ld, int r, int k)
-{
-    switch (view) {
-    case kViewRow: return src[r + (long long)k * ld];
-    case kViewCol: return src[k + (long long)r * ld];
-    case kViewSym: return r >= k ? src[r + (long long)k * ld] : src[k + (long long)r * ld];
-    case kViewZExpandN: {
-        const double *p = src + 2 * ((r >> 1) + (long long)(k >> 1) * ld);
-        return zblock(p[0], p[1], r & 1, k & 1);
-    }
-    case kViewZExpandC: {  // A^H(i, j) = conj(A(j, i))
-        const double *p = src + 2 * ((k >> 1) + (long long)(r >> 1) * ld);
-        return zblock(p[0], -p[1], r & 1, k & 1);
-    }
-    case kViewZHermExpand: {
-        const int i = r >> 1, j = k >> 1;
-        if (i > j) {
-            const double *p = src + 2 * (i + (long long)j * ld);
-            return zblock(p[0], p[1], r & 1, k & 1);
-        }
-        const double *p = src + 2 * (j + (long long)i * ld);
-        return zblock(p[0], i == j ? 0.0 : -p[1], r & 1, k & 1);
-    }
-    default: {  // kViewZRowConj
-        const double *p = src + 2 * (r + (long long)(k >> 1) * ld);
-        return (k & 1) ? -p[1] : p[0];
-    }
-    }
-}
-
-// Loads the 32 x 32 tile at (r0, k0) into t[r][k] (zero outside R x K), with
-// the thread index running along the source's contiguous index.
-__device__ __forceinline__ void load_tile(int view, const double *__restrict__ src, long long ld, int R, int K,
-                                          int r0, int k0, double (*t)[33])
-{
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    // which index is contiguous in memory for this tile
-    bool along_r;
-    if (view == kViewRow || view == kViewZExpandN || view == kViewZRowConj) along_r = true;
-    else if (view == kViewCol || view == kViewZExpandC) along_r = false;
-    else along_r = (r0 >= k0 + 31) || !(r0 + 31 < k0);  // lower or diagonal tiles: read src[r + k ld]
-    for (int i = ty; i < 32; i += 8) {
-        const int a = along_r ? i : tx, bb = along_r ? tx : i;  // a: k offset, bb: r offset
-        const int r = r0 + bb, k = k0 + a;
-        double v = 0.0;
-        if (r < R && k < K) v = view_at(view, src, ld, r, k);
-        t[bb][a] = v;
-    }
-}
-
-__global__ void __launch_bounds__(256) slice_rowmax(int view, const double *__restrict__ src, long long ld, int R,
-                                                     int K, unsigned long long *__restrict__ rmax)
-{
-    __shared__ double t[32][33];
-    const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
-    load_tile(view, src, ld, R, K, r0, k0, t);
-    __syncthreads();
-    for (int i = threadIdx.y; i < 32; i += 8) {
-        unsigned long long m = (unsigned long long)__double_as_longlong(t[i][threadIdx.x]) & 0x7fffffffffffffffull;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long u = __shfl_xor_sync(0xffffffffu, m, o);
-            m = u > m ? u : m;
-        }
-        if (threadIdx.x == 0 && r0 + i < R && m) atomicMax(rmax + r0 + i, m);
-    }
-}
-
-
-// Writes the eight digit planes, or the three planes of the FP32 split.
-__global__ void __launch_bounds__(256) slice_digits(int view, const double *__restrict__ src, long long ld, int R,
-                                                     int K, int Rp, int Kp, const unsigned long long *__restrict__ rmax,
-                                                     uint16_t *__restrict__ planes, int *__restrict__ e_out,
-                                                     int digits)
+// Writes the three planes of the FP32 split.
+__global__ void __launch_bounds__(256) split_planes(int view, const double *__restrict__ src, long long ld, int R,
+                                                     int K, int Rp, int Kp, uint16_t *__restrict__ planes)
 {
     __shared__ double t[32][33];
     const int r0 = blockIdx.y * 32, k0 = blockIdx.x * 32;
@@ -150,40 +66,25 @@ __global__ void __launch_bounds__(256) slice_digits(int view, const double *__re
     for (int i = threadIdx.y; i < 32; i += 8) {
         const int r = r0 + i, k = k0 + threadIdx.x;
         if (r >= Rp || k >= Kp) continue;
-        const double x = t[i][threadIdx.x];
-        if (digits == kSplitPlanes) {  // FP32 value split into three bf16 parts (exact)
-            if (blockIdx.x == 0 && threadIdx.x == 0) e_out[r] = 0;
-            const float f = __double2float_rn(x);
-            const __nv_bfloat16 h0 = __float2bfloat16_rn(f);
-            const float r1 = f - __bfloat162float(h0);
-            const __nv_bfloat16 h1 = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 h2 = __float2bfloat16_rn(r1 - __bfloat162float(h1));
-            const size_t at = (size_t)r * Kp + k;
-            planes[at] = __bfloat16_as_ushort(h0);
-            planes[plane + at] = __bfloat16_as_ushort(h1);
-            planes[2 * plane + at] = __bfloat16_as_ushort(h2);
-            continue;
-        }
-        const int er = r < R ? exponent_above(rmax[r]) : 0;
-        if (blockIdx.x == 0 && threadIdx.x == 0) e_out[r] = er;
-        const unsigned long long Y = fixed56(x, er);
-        const bool neg = x < 0.0;
-#pragma unroll
-        for (int s = 0; s < kSlices; s++) {
-            if (s >= digits) break;
-            const uint16_t h = bf16_digit((int)((Y >> (kDigitBits * (kSlices - 1 - s))) & 127u), s, neg);
-            planes[s * plane + (size_t)r * Kp + k] = h;
-        }
+        const float f = __double2float_rn(t[i][threadIdx.x]);
+        const __nv_bfloat16 h0 = __float2bfloat16_rn(f);
+        const float r1 = f - __bfloat162float(h0);
+        const __nv_bfloat16 h1 = __float2bfloat16_rn(r1);
+        const __nv_bfloat16 h2 = __float2bfloat16_rn(r1 - __bfloat162float(h1));
+        const size_t at = (size_t)r * Kp + k;
+        planes[at] = __bfloat16_as_ushort(h0);
+        planes[plane + at] = __bfloat16_as_ushort(h1);
+        planes[2 * plane + at] = __bfloat16_as_ushort(h2);
     }
 }
 
-// Stage loader: the leading D digit planes of the A rows [m0, m0+kBM) and B
-// rows [n0, n0+kBN) for k in [kt, kt+32).
-template <int D>
+// Stage loader: the planes of the A rows [m0, m0+kBM) and B rows
+// [n0, n0+kBN) for k in [kt, kt+32).
 __device__ __forceinline__ void load_stage(uint16_t *stage, const uint16_t *__restrict__ Ap, size_t a_plane,
                                            int a_kp, const uint16_t *__restrict__ Bp, size_t b_plane, int b_kp,
                                            int m0, int n0, int kt)
 {
+    constexpr int D = kSplitPlanes;
     // D planes x rows x 4 chunks of 16 bytes (32 bf16 of k)
     constexpr int kChunksA = D * kBM * 4, kChunksB = D * kBN * 4;
     constexpr int kTotal = kChunksA + kChunksB;
@@ -204,51 +105,31 @@ __device__ __forceinline__ void load_stage(uint16_t *stage, const uint16_t *__re
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// Levels a product forms: i + j <= 8 for the eight digits; the FP32 split
-// (D = kSplitPlanes) sums its pairs i + j <= 2 in one FP32 accumulator.
-template <int D>
-__host__ __device__ constexpr int product_levels() { return D == kSlices ? kLevels : 1; }
-
 // One kBM x kBN tile of C (or of split z's partial product).  Warps 4 x 2,
-// each 16 x 16 (two m16n8 tiles); level l = i + j < product_levels<D>() of
-// the digit pairs has its own FP32 accumulator, exact over kFlushK values of
-// k, folded into two 64-bit integers: hi = sum_{l<4} L_l 2^(7(3-l)),
-// lo = sum_{l>=4} L_l 2^(7(8-l)), with L_l the level's sum in units of
-// 2^(-7l).
-template <int D>
-__global__ void __launch_bounds__(kThreads, D == kSlices ? 1 : 2)
-sliced_product(const uint16_t *__restrict__ Ap, const int *__restrict__ ea, int a_rp, int a_kp,
-               const uint16_t *__restrict__ Bp, const int *__restrict__ eb, int b_rp, int b_kp, int m, int n,
-               int ksplit, int K, double alpha, double beta, double *__restrict__ C, long long ldc, int fill,
-               double *__restrict__ part)
+// each 16 x 16 (two m16n8 tiles); the six pairs i + j <= 2 share one FP32
+// accumulator, folded into FP64 every kFlushK values of k.
+__global__ void __launch_bounds__(kThreads, 2)
+split_product(const uint16_t *__restrict__ Ap, int a_rp, int a_kp, const uint16_t *__restrict__ Bp, int b_rp, int b_kp,
+              int m, int n, int ksplit, int K, double alpha, double beta, double *__restrict__ C, long long ldc,
+              int fill, double *__restrict__ part)
 {
-    constexpr int kLev = product_levels<D>();
-    constexpr bool kSplit = D == kSplitPlanes;
-    constexpr size_t kStageElems = stage_elems<D>();
+    constexpr int D = kSplitPlanes;
     extern __shared__ __align__(16) uint16_t smem[];
     const int tm = blockIdx.y, tn = blockIdx.x;
     const int m0 = tm * kBM, n0 = tn * kBN;
     if (fill == kFillLower && m0 + kBM - 1 < n0) return;          // tile wholly above the diagonal
-    if (fill == kFillZLower && ((m0 + kBM - 1) >> 1) < n0) return;
     const int kbeg = blockIdx.z * ksplit, kend = min(K, kbeg + ksplit);
     const size_t a_plane = (size_t)a_rp * a_kp, b_plane = (size_t)b_rp * b_kp;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wm = warp & 3, wn = warp >> 2;
 
-    float acc[kLev][2][4];
-    long long hi[2][4], lo[2][4];
-    double dacc[2][4];  // FP32 split: the FP32 sums folded every kFlushK
-#pragma unroll
-    for (int l = 0; l < kLev; l++)
-#pragma unroll
-        for (int t = 0; t < 2; t++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) acc[l][t][q] = 0.f;
+    float acc[2][4];
+    double dacc[2][4];
 #pragma unroll
     for (int t = 0; t < 2; t++)
 #pragma unroll
         for (int q = 0; q < 4; q++) {
-            hi[t][q] = lo[t][q] = 0;
+            acc[t][q] = 0.f;
             dacc[t][q] = 0.0;
         }
 
@@ -257,13 +138,12 @@ sliced_product(const uint16_t *__restrict__ Ap, const int *__restrict__ ea, int 
     const int b_row = wn * 16 + (lane & 7) + (lane >> 4) * 8, b_k = ((lane >> 3) & 1) * 8;
 
     int stage = 0;
-    if (kbeg < kend) load_stage<D>(smem, Ap, a_plane, a_kp, Bp, b_plane, b_kp, m0, n0, kbeg);
+    if (kbeg < kend) load_stage(smem, Ap, a_plane, a_kp, Bp, b_plane, b_kp, m0, n0, kbeg);
     int steps = 0;
     for (int kt = kbeg; kt < kend; kt += kBK, steps++) {
         const bool more = kt + kBK < kend;
         if (more)
-            load_stage<D>(smem + (size_t)(stage ^ 1) * kStageElems, Ap, a_plane, a_kp, Bp, b_plane, b_kp, m0, n0,
-                          kt + kBK);
+            load_stage(smem + (size_t)(stage ^ 1) * kStageElems, Ap, a_plane, a_kp, Bp, b_plane, b_kp, m0, n0, kt + kBK);
         if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
         else asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
@@ -283,37 +163,24 @@ sliced_product(const uint16_t *__restrict__ Ap, const int *__restrict__ ea, int 
                         Bs + ((size_t)j * kBN + b_row) * kRowPad + ks * 16 + b_k);
 #pragma unroll
                 for (int i = 0; i < D; i++)
-                    if (kSplit ? i + j <= 2 : i + j < kLev)
+                    if (i + j <= 2)
 #pragma unroll
-                        for (int t = 0; t < 2; t++) mma_bf16(acc[kSplit ? 0 : i + j][t], af[i], bf[t][0], bf[t][1]);
+                        for (int t = 0; t < 2; t++) mma_bf16(acc[t], af[i], bf[t][0], bf[t][1]);
             }
         }
         __syncthreads();  // this stage's buffer is refilled two steps later
         stage ^= 1;
-        // fold the levels into the integer accumulators every kFlushK
         if ((steps + 1) % (kFlushK / kBK) == 0 || !more) {
 #pragma unroll
-            for (int l = 0; l < kLev; l++)
+            for (int t = 0; t < 2; t++)
 #pragma unroll
-                for (int t = 0; t < 2; t++)
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        if (kSplit) {
-                            dacc[t][q] += (double)acc[l][t][q];
-                            acc[l][t][q] = 0.f;
-                            continue;
-                        }
-                        // level l holds an integer multiple of 2^(-7l) below 2^24 units
-                        const float unit = __int_as_float((127 + kDigitBits * l) << 23);  // 2^(7l)
-                        const long long iv = __float2int_rn(acc[l][t][q] * unit);
-                        if (l < 4) hi[t][q] += iv << (kDigitBits * (3 - l));
-                        else lo[t][q] += iv << (kDigitBits * (kLevels - 1 - l));
-                        acc[l][t][q] = 0.f;
-                    }
+                for (int q = 0; q < 4; q++) {
+                    dacc[t][q] += (double)acc[t][q];
+                    acc[t][q] = 0.f;
+                }
         }
     }
 
-    // epilogue: value = (hi 2^-21 + lo 2^-56) 2^(ea + eb - 14)
     const int g = lane >> 2, tig = lane & 3;
 #pragma unroll
     for (int t = 0; t < 2; t++)
@@ -321,20 +188,8 @@ sliced_product(const uint16_t *__restrict__ Ap, const int *__restrict__ ea, int 
         for (int q = 0; q < 4; q++) {
             const int r = m0 + wm * 16 + g + (q >> 1) * 8;
             const int c = n0 + wn * 16 + t * 8 + tig * 2 + (q & 1);
-            if (r >= m || c >= n || (fill == kFillLower && r < c) || (fill == kFillZLower && (r >> 1) < c))
-                continue;
-            double v;
-            if (kSplit) {
-                v = dacc[t][q];
-            } else {
-                v = (double)hi[t][q] * 0x1p-21 + (double)lo[t][q] * 0x1p-56;
-                v = scale_by_pow2(v, ea[r] + eb[c] - 2 * kDigitBits);
-            }
-            if (fill == kFillZLower && (r >> 1) == c && (r & 1)) {  // Hermitian diagonal: real
-                if (part) part[(size_t)blockIdx.z * m * n + (size_t)c * m + r] = 0.0;
-                else C[r + (long long)c * ldc] = 0.0;
-                continue;
-            }
+            if (r >= m || c >= n || (fill == kFillLower && r < c)) continue;
+            const double v = dacc[t][q];
             if (part) {
                 part[(size_t)blockIdx.z * m * n + (size_t)c * m + r] = v;
             } else {
@@ -375,7 +230,7 @@ cudaError_t slice_matrix(SliceView view, int R, int K, const double *src, long l
     char *base = (char *)buf;
     uint16_t *planes = (uint16_t *)(base + L.planes);
     int *e = (int *)(base + L.e);
-    unsigned long long *rmax = (unsigned long long *)(base + L.rmax);
+    uint32_t *rmax = (uint32_t *)(base + L.rmax);
     out->planes = planes;
     out->e = e;
     out->R = R;
@@ -383,52 +238,35 @@ cudaError_t slice_matrix(SliceView view, int R, int K, const double *src, long l
     out->Rp = Rp;
     out->Kp = Kp;
     out->digits = digits;
-    cudaError_t err = cudaMemsetAsync(rmax, 0, (size_t)Rp * sizeof(unsigned long long), st);
-    if (err != cudaSuccess) return err;
     const dim3 block(32, 8);
-    if (R > 0 && K > 0 && digits != kSplitPlanes) {  // the split needs no row maxima
-        const dim3 grid((K + 31) / 32, (R + 31) / 32);
-        slice_rowmax<<<grid, block, 0, st>>>((int)view, src, ld, R, K, rmax);
-        if ((err = cudaGetLastError()) != cudaSuccess) return err;
+    if (digits == kSplitPlanes) {   // needs no row maxima; planes over the padded extent
+        split_planes<<<dim3(Kp / 32, Rp / 32), block, 0, st>>>((int)view, src, ld, R, K, Rp, Kp, planes);
+        return cudaGetLastError();
     }
-    // digits over the padded extent (zeros outside R x K)
-    const dim3 grid2(Kp / 32, Rp / 32);
-    slice_digits<<<grid2, block, 0, st>>>((int)view, src, ld, R, K, Rp, Kp, rmax, planes, e, digits);
-    return cudaGetLastError();
+    return tc5_slice_matrix(view, R, K, src, ld, rmax, planes, e, st);
 }
 
-namespace {
-
-template <int D>
-cudaError_t launch_product(dim3 grid, cudaStream_t st, const SlicedOp &A, const SlicedOp &B, int m, int n, int ksplit,
-                           int Kp, double alpha, double beta, double *C, long long ldc, int fill, double *part)
+cudaError_t sliced_reduce_launch(int m, int n, int splits, const double *part, double alpha, double beta, double *C,
+                                 long long ldc, int fill, cudaStream_t st)
 {
-    // opt in to the large dynamic shared memory (cheap; per device, so every call)
-    cudaError_t e = cudaFuncSetAttribute(sliced_product<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)product_smem<D>());
-    if (e != cudaSuccess) return e;
-    sliced_product<D><<<grid, kThreads, product_smem<D>(), st>>>(A.planes, A.e, A.Rp, A.Kp, B.planes, B.e, B.Rp,
-                                                                B.Kp, m, n, ksplit, Kp, alpha, beta, C, ldc, fill,
-                                                                part);
+    const long long total = (long long)m * n;
+    sliced_reduce<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(m, n, splits, part, alpha, beta, C, ldc, fill);
     return cudaGetLastError();
 }
-
-}  // namespace
 
 cudaError_t sliced_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double alpha, double beta, double *C,
                         long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st)
 {
     if (m <= 0 || n <= 0) return cudaSuccess;
     if (A.K != B.K || A.Kp != B.Kp || m > A.R || n > B.R) return cudaErrorInvalidValue;
-    const int D = std::min(A.digits, B.digits);
+    if (A.digits != B.digits) return cudaErrorInvalidValue;
+    if (A.digits == kSlices) return tc5_gemm(A, B, m, n, alpha, beta, C, ldc, fill, work, work_elems, st);
+    if (A.digits != kSplitPlanes || fill == kFillZLower) return cudaErrorInvalidValue;
     const int tiles_m = (m + kBM - 1) / kBM, tiles_n = (n + kBN - 1) / kBN;
     long long tiles = (long long)tiles_m * tiles_n;
     if (fill != kFillAll) {  // tiles not wholly above the diagonal
         tiles = 0;
-        for (int tm = 0; tm < tiles_m; tm++) {
-            const int top = fill == kFillZLower ? (tm * kBM + kBM - 1) >> 1 : tm * kBM + kBM - 1;
-            tiles += std::min(tiles_n, top / kBN + 1);
-        }
+        for (int tm = 0; tm < tiles_m; tm++) tiles += std::min(tiles_n, (tm * kBM + kBM - 1) / kBN + 1);
     }
     const int Kp = A.Kp;
     // split the reduction when the tiles alone cannot fill the device
@@ -442,10 +280,6 @@ cudaError_t sliced_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, doub
         if (splits > max_by_k) splits = max_by_k > 1 ? max_by_k : 1;
         while (splits > 1 && (size_t)splits * m * n > work_elems) splits--;
     }
-    if (splits < (Kp + kMaxSplitK - 1) / kMaxSplitK) {  // very long sums: split so every part stays exact
-        splits = (Kp + kMaxSplitK - 1) / kMaxSplitK;
-        if (!work || (size_t)splits * m * n > work_elems) return cudaErrorInvalidValue;
-    }
     int ksplit = Kp;
     if (splits > 1) {
         ksplit = round_up((Kp + splits - 1) / splits, kFlushK);
@@ -453,15 +287,13 @@ cudaError_t sliced_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, doub
     }
     const dim3 grid(tiles_n, tiles_m, splits);
     double *part = splits > 1 ? work : nullptr;
-    cudaError_t e;
-    if ((A.digits == kSplitPlanes) != (B.digits == kSplitPlanes)) return cudaErrorInvalidValue;
-    if (D == kSplitPlanes) e = launch_product<kSplitPlanes>(grid, st, A, B, m, n, ksplit, Kp, alpha, beta, C, ldc, fill, part);
-    else if (D == kSlices) e = launch_product<kSlices>(grid, st, A, B, m, n, ksplit, Kp, alpha, beta, C, ldc, fill, part);
-    else return cudaErrorInvalidValue;
-    if (e != cudaSuccess || splits == 1) return e;
-    const long long total = (long long)m * n;
-    sliced_reduce<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(m, n, splits, work, alpha, beta, C, ldc, fill);
-    return cudaGetLastError();
+    // opt in to the large dynamic shared memory (cheap; per device, so every call)
+    cudaError_t e = cudaFuncSetAttribute(split_product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProductSmem);
+    if (e != cudaSuccess) return e;
+    split_product<<<grid, kThreads, kProductSmem, st>>>(A.planes, A.Rp, A.Kp, B.planes, B.Rp, B.Kp, m, n, ksplit, Kp, alpha,
+                                                       beta, C, ldc, fill, part);
+    if ((e = cudaGetLastError()) != cudaSuccess || splits == 1) return e;
+    return sliced_reduce_launch(m, n, splits, work, alpha, beta, C, ldc, fill, st);
 }
 
 }  // namespace gb

@@ -4,20 +4,14 @@
 // multiplication", Numer. Algorithms 59 (2012), in its fixed-point form).
 //
 // Every row of op(A) and every column of op(B) is scaled by a power of two
-// so that its largest entry is below one, and each entry's magnitude is cut
-// into kSlices digits of kDigitBits bits (|digit| <= 127, all digits carry
-// the entry's sign).  Digit t is stored as the bf16 value d * 2^(-7t), which
-// bf16 holds exactly.  The product of digit planes i (of A) and j (of B) is
-// an exact multiple of 2^(-7(i+j)) and lands in "level" i+j.  Pairs with
-// i+j <= 8 are formed; the rest lie 2^-62 below the scaled row/column
-// maxima, and digits are cut from the magnitude rounded to nearest, so the
-// errors stay unbiased and grow like sqrt(k) even in sums of one sign.  Every level has its own FP32 tensor-core
-// accumulator; over kFlushK consecutive k its sum is an integer multiple of
-// 2^(-7 level) below 2^24 units (kSlices * 127^2 * kFlushK < 2^24), so it is
-// exact, and it is folded into two 64-bit integers per output every kFlushK.
-// The result is rounded to FP64 once, at the end.  (A shared FP32
-// accumulator for the low levels is not enough: its truncating additions
-// reach 2^-46 of the result on sums of one sign.)
+// so that its largest entry is below one, rounded to 62 fraction bits and cut
+// into kSlices balanced base-256 digits in [-128, 127], each exact in FP16.
+// The product of digit planes i (of A) and j (of B) lands in "level" i + j.
+// Pairs with i + j <= 7 are formed; the rest lie 2^-62 sqrt(k) below the scaled
+// row / column maxima.  Every level has its own FP32 tensor-core accumulator;
+// over 128 consecutive k its sum is an integer of at most 2^24, so it is exact,
+// and it is folded into one 96-bit integer per output.  The result is rounded
+// to FP64 once, at the end (sliced_tc5.cu).
 //
 // Accuracy is that of an FP64 product measured against the scaled maxima:
 // |C - AB| <~ 2^-53 k max_j|a_ij| max_i|b_ij| per entry.  Inputs must be
@@ -42,8 +36,6 @@
 namespace gb {
 
 constexpr int kSlices = 8;
-constexpr int kLevels = 9;  // digit pairs i + j <= 8 are formed
-constexpr int kDigitBits = 7;
 constexpr int kFlushK = 128;
 constexpr int kSplitPlanes = 3;  // `digits` value of the FP32 split
 
@@ -73,8 +65,9 @@ enum SliceView {
 };
 
 struct SlicedOp {
-    const uint16_t *planes;  // digits planes of Rp x Kp bf16, row-major (k fastest)
-    const int *e;            // Rp row exponents: the row's entries are below 2^e
+    const uint16_t *planes;  // kSlices: FP16 digit planes in blocks of 128 rows x 32 k (sliced_tc5.cu);
+                             // kSplitPlanes: planes of Rp x Kp bf16, row-major (k fastest)
+    const int *e;            // row exponents: the row's entries are below 2^e (kSlices)
     int R, K, Rp, Kp;        // Rp: R rounded up to 64; Kp: K rounded up to 32
     int digits;              // kSlices digit planes, or kSplitPlanes (the FP32 split)
 };
@@ -104,6 +97,18 @@ enum SlicedFill {
 // reduction splits while splits * m * n <= work_elems.
 cudaError_t sliced_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double alpha, double beta, double *C,
                         long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st);
+
+// The digit form's parts (sliced_tc5.cu): plane bytes of an R x K operand, its
+// padded rows, cutting it (rmax: one word per row, scratch), and the product.
+size_t tc5_planes_bytes(int R, int K);
+int tc5_rows_padded(int R);
+cudaError_t tc5_slice_matrix(SliceView view, int R, int K, const double *src, long long ld, uint32_t *rmax,
+                             uint16_t *planes, int *e, cudaStream_t st);
+cudaError_t tc5_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double alpha, double beta, double *C,
+                     long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st);
+// C = alpha (sum of `splits` partials of m x n) + beta C
+cudaError_t sliced_reduce_launch(int m, int n, int splits, const double *part, double alpha, double beta, double *C,
+                                 long long ldc, int fill, cudaStream_t st);
 
 // Whole products (slice both operands into ws, multiply), with the DFMA
 // forms' conventions (dgemm_dfma.cuh); ws must hold the matching *_ws_bytes.

@@ -1,0 +1,98 @@
+"""Edges of the tcgen05 digit products: tiles of 128 x 64, stages of 32 and
+exact sums of 128 values of k, splits, the swapped orientation of short wide
+results, lower triangles and both halves of alpha / beta.
+
+Operands are integers in [-9, 9], so every result is an integer below 2^53 and
+a correct product equals the FP64 one exactly: no tolerance.
+"""
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gb():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1811_01277_gb300 as m
+    from paper_1811_01277_gb300 import build
+    build.build()
+    m.load()
+    return m
+
+
+def ints(g, *shape):
+    return torch.randint(-9, 10, shape, generator=g, device="cuda").to(torch.float64)
+
+
+SHAPES = [(1, 1, 1), (128, 64, 32), (129, 65, 33), (127, 63, 31), (64, 64, 128), (65, 129, 129), (128, 128, 160),
+          (64, 700, 161), (40, 300, 4100), (700, 40, 2049), (300, 1000, 64), (1000, 300, 513), (2500, 2500, 96)]
+
+
+@pytest.mark.parametrize("m,n,k", SHAPES)
+@pytest.mark.parametrize("ta,tb,alpha,beta", [("N", "N", 1.0, 0.0), ("T", "N", -1.0, 1.0), ("N", "T", 2.0, -3.0)])
+def test_gemm_exact(gb, m, n, k, ta, tb, alpha, beta):
+    g = torch.Generator(device="cuda").manual_seed(m + 10 * n + 100 * k)
+    A = ints(g, *((k, m + 3) if ta == "N" else (m, k + 1)))       # column-major: (columns, leading dimension)
+    B = ints(g, *((n, k + 2) if tb == "N" else (k, n + 5)))
+    C = ints(g, n, m + 1)
+    left = A[:, :m].T if ta == "N" else A[:, :k]
+    right = B[:, :k].T if tb == "N" else B[:, :n]
+    want = alpha * (left @ right) + (beta * C[:, :m].T if beta else 0.0)
+    if beta == 0.0:
+        C[:, :m] = float("nan")                                   # must not be read
+    pad = C[:, m:].clone()
+    wsb = gb.gb_dgemm_sliced_workspace_bytes(m, n, k)
+    ws = torch.full((wsb,), 255, dtype=torch.uint8, device="cuda")
+    gb.gb_dgemm_sliced(ta, tb, m, n, k, alpha, A, A.shape[1], B, B.shape[1], beta, C, m + 1, ws, wsb,
+                       torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert torch.equal(C[:, :m].T, want)
+    assert torch.equal(C[:, m:], pad)
+
+
+@pytest.mark.parametrize("n", [1, 31, 64, 65, 128, 129, 200, 513])
+@pytest.mark.parametrize("k", [1, 64, 130])
+def test_triangles_and_symmetric_exact(gb, n, k):
+    g = torch.Generator(device="cuda").manual_seed(7 * n + k)
+    X, Y, C = ints(g, k, n), ints(g, k, n), ints(g, n, n)
+    st = torch.cuda.current_stream()
+    low = torch.ones(n, n, dtype=torch.bool, device="cuda").tril()
+    # rank-2k update of the lower triangle (column-major: the transposed tensor)
+    want = torch.where(low, C.T - (X.T @ Y + Y.T @ X), C.T)
+    wsb = gb.gb_dsyr2k_sliced_workspace_bytes(n, k)
+    ws = torch.full((wsb,), 255, dtype=torch.uint8, device="cuda")
+    got = C.clone()
+    gb.gb_dsyr2k_sliced(n, k, -1.0, X, n, Y, n, 1.0, got, n, ws, wsb, st)
+    assert torch.equal(got.T, want)
+    # symmetric times tall: only the lower triangle is read
+    S = ints(g, n, n)
+    S = S.tril() + S.tril(-1).T
+    stored = torch.where(low, S, torch.full_like(S, float("nan"))).T.contiguous()
+    wsb = gb.gb_dsymm_sliced_workspace_bytes("L", n, k)
+    ws = torch.full((wsb,), 255, dtype=torch.uint8, device="cuda")
+    out = torch.zeros(k, n, dtype=torch.float64, device="cuda")
+    gb.gb_dsymm_sliced("L", n, k, 1.0, stored, n, X, n, 0.0, out, n, ws, wsb, st)
+    assert torch.equal(out.T, S @ X.T)
+
+
+@pytest.mark.parametrize("e", [-1040, -1000, 0, 970])
+def test_scales_at_the_ends_of_the_range(gb, e):
+    """One row of A times 2^e: normal, subnormal and large results, each the
+    nearest FP64 number (scaling by a power of two commutes with rounding while
+    the result is normal)."""
+    m, n, k = 130, 70, 50
+    g = torch.Generator(device="cuda").manual_seed(5)
+    A, B = ints(g, k, m), ints(g, n, k)
+    C = torch.zeros(n, m, dtype=torch.float64, device="cuda")
+    As = A.clone()
+    As[:, 7] = torch.ldexp(torch.ldexp(A[:, 7], torch.tensor(e // 2, device="cuda")), torch.tensor(e - e // 2, device="cuda"))
+    want = (A.T @ B.T)
+    want[7] = torch.ldexp(torch.ldexp(want[7], torch.tensor(e // 2, device="cuda")), torch.tensor(e - e // 2, device="cuda"))
+    if e == -1040:   # subnormal operands read as zero
+        want[7] = 0.0
+    wsb = gb.gb_dgemm_sliced_workspace_bytes(m, n, k)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    gb.gb_dgemm_sliced("N", "N", m, n, k, 1.0, As, m, B, k, 0.0, C, m, ws, wsb, torch.cuda.current_stream())
+    assert torch.equal(C.T, want)
