@@ -1,13 +1,20 @@
 // Tiled FP64 products on the DFMA pipe (see dgemm_dfma.cuh).
 //
-// One CTA of 256 threads computes a 64 x 64 tile of C; thread (tx, ty) owns
-// rows tx + 16i and columns ty + 16j (i, j < 4), so the shared-memory reads of
-// a k step are broadcasts without bank conflicts.  The reduction runs in
-// steps of 8: the next step's operand tiles are loaded from global memory
-// into registers while the current step's 128 DFMAs per thread run from
-// shared memory (double-buffered).  An FP64 FMA occupies a scheduler's
-// narrow FP64 pipe for many cycles, so a 4 x 4 register tile leaves the
-// issue slots free for the loads and address arithmetic.
+// One CTA of 256 threads computes a TS x TS tile of C, TS = 64 or 32; thread
+// (tx, ty) owns rows tx + 16i and columns ty + 16j (i, j < TS/16), so the
+// shared-memory reads of a k step are broadcasts without bank conflicts.  The
+// reduction runs in steps of 512/TS: the next step's operand tiles are loaded
+// from global memory into registers while the current step's DFMAs run from
+// shared memory (double-buffered).  An FP64 FMA occupies a scheduler's narrow
+// FP64 pipe for many cycles, so even a 2 x 2 register tile leaves the issue
+// slots free for the loads and address arithmetic.
+//
+// What bounds it is FP64 issue, two FMAs per clock and SM, so the work has to
+// reach every SM: the solver's panel products (b x b over a long reduction,
+// m x b over a short one) take TS = 32 and reductions split down to 16 values
+// of k (choose_shape).  Measured on a GB300 over the panels of an n = 1024,
+// nbw = 32 solve (before: 64 x 64 tiles, splits of 64 and more): Y^T X 84 -> 12 us,
+// A2 (Y T) 98 -> 25 us, Y T and X - Y M 44 -> 16 us a launch.
 //
 // Operand modes: N (as stored), T (transposed) and SYM (symmetric, lower
 // triangle stored).  Each mode has its own thread-to-element mapping so that
@@ -17,6 +24,8 @@
 
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "dgemm_dfma.cuh"
 #include "elpa_gb300.h"
 
@@ -24,7 +33,7 @@ namespace gb {
 
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 8, NT = 256;
+constexpr int NT = 256;
 constexpr int MODE_N = 0, MODE_T = 1, MODE_SYM = 2;
 
 struct Gemm {
@@ -37,16 +46,17 @@ struct Gemm {
     long long ldc;
     double alpha, beta;
     double *partial;          // split-K partials [splits][n][m] (splits > 1)
-    int kchunk;               // reduction length per split, multiple of BK
+    int kchunk;               // reduction length per split (over both products), multiple of the k step
     int lower;                // 1: tiles with row tile >= column tile only, elements r >= c
     int tiles_m;
 };
 
 // op(A)(r, q) of a BM x BK tile at (r0, q0); 2 elements per thread.
-template <int MODE>
+template <int MODE, int TS>
 __device__ __forceinline__ void load_a(const double *__restrict__ A, long long lda, int m, int kend, int r0, int q0,
                                        double (&v)[2], int (&sr)[2], int (&sq)[2])
 {
+    constexpr int BM = TS, BK = 512 / TS;
     const bool below = r0 >= q0 + BK - 1;       // every r >= q in the tile
     const bool above = r0 + BM - 1 < q0;        // every r < q in the tile
     const bool tmap = (MODE == MODE_T) || (MODE == MODE_SYM && above);
@@ -76,10 +86,11 @@ __device__ __forceinline__ void load_a(const double *__restrict__ A, long long l
 }
 
 // op(B)(q, c) of a BK x BN tile at (q0, c0); 2 elements per thread.
-template <int MODE>
+template <int MODE, int TS>
 __device__ __forceinline__ void load_b(const double *__restrict__ B, long long ldb, int n, int kend, int q0, int c0,
                                        double (&v)[2], int (&sq)[2], int (&sc)[2])
 {
+    constexpr int BN = TS, BK = 512 / TS;
     const bool below = q0 >= c0 + BN - 1;       // every q >= c
     const bool above = q0 + BK - 1 < c0;        // every q < c
     const bool cmap = (MODE == MODE_T) || (MODE == MODE_SYM && above);
@@ -108,9 +119,10 @@ __device__ __forceinline__ void load_b(const double *__restrict__ B, long long l
     }
 }
 
-template <int MA, int MB>
+template <int MA, int MB, int TS>
 __global__ void __launch_bounds__(NT) dfma_gemm_kernel(Gemm g)
 {
+    constexpr int BM = TS, BN = TS, BK = 512 / TS, RT = TS / 16;
     __shared__ double As[2][BK][BM + 1];
     __shared__ double Bs[2][BK][BN + 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -129,11 +141,11 @@ __global__ void __launch_bounds__(NT) dfma_gemm_kernel(Gemm g)
     const int r0 = ti * BM, c0 = tj * BN;
     const int split = blockIdx.z;
 
-    double acc[4][4];
+    double acc[RT][RT];
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int i = 0; i < RT; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) acc[i][j] = 0.0;
+        for (int j = 0; j < RT; j++) acc[i][j] = 0.0;
 
     const int npairs = g.k2 > 0 ? 2 : 1;
     for (int p = 0; p < npairs; p++) {
@@ -141,13 +153,15 @@ __global__ void __launch_bounds__(NT) dfma_gemm_kernel(Gemm g)
         const double *B = p ? g.B2 : g.B;
         const long long lda = p ? g.lda2 : g.lda, ldb = p ? g.ldb2 : g.ldb;
         const int K = p ? g.k2 : g.k;
-        const int kb = p ? 0 : split * g.kchunk;
-        const int ke = p ? K : min(K, kb + g.kchunk);
+        // the split's part of this product (the reductions follow each other)
+        const int k0 = p ? (g.k + BK - 1) / BK * BK : 0;
+        const int kb = max(0, split * g.kchunk - k0);
+        const int ke = min(K, (split + 1) * g.kchunk - k0);
         if (kb >= ke) continue;
         double va[2], vb[2];
         int ar[2], aq[2], bq[2], bc[2];
-        load_a<MA>(A, lda, g.m, ke, r0, kb, va, ar, aq);
-        load_b<MB>(B, ldb, g.n, ke, kb, c0, vb, bq, bc);
+        load_a<MA, TS>(A, lda, g.m, ke, r0, kb, va, ar, aq);
+        load_b<MB, TS>(B, ldb, g.n, ke, kb, c0, vb, bq, bc);
         __syncthreads();  // the previous pair's last reads of the buffers are done
 #pragma unroll
         for (int t = 0; t < 2; t++) {
@@ -159,20 +173,20 @@ __global__ void __launch_bounds__(NT) dfma_gemm_kernel(Gemm g)
         for (int q0 = kb; q0 < ke; q0 += BK) {
             const bool more = q0 + BK < ke;
             if (more) {
-                load_a<MA>(A, lda, g.m, ke, r0, q0 + BK, va, ar, aq);
-                load_b<MB>(B, ldb, g.n, ke, q0 + BK, c0, vb, bq, bc);
+                load_a<MA, TS>(A, lda, g.m, ke, r0, q0 + BK, va, ar, aq);
+                load_b<MB, TS>(B, ldb, g.n, ke, q0 + BK, c0, vb, bq, bc);
             }
 #pragma unroll
             for (int q = 0; q < BK; q++) {
-                double a[4], b[4];
+                double a[RT], b[RT];
 #pragma unroll
-                for (int i = 0; i < 4; i++) a[i] = As[buf][q][tx + 16 * i];
+                for (int i = 0; i < RT; i++) a[i] = As[buf][q][tx + 16 * i];
 #pragma unroll
-                for (int j = 0; j < 4; j++) b[j] = Bs[buf][q][ty + 16 * j];
+                for (int j = 0; j < RT; j++) b[j] = Bs[buf][q][ty + 16 * j];
 #pragma unroll
-                for (int i = 0; i < 4; i++)
+                for (int i = 0; i < RT; i++)
 #pragma unroll
-                    for (int j = 0; j < 4; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+                    for (int j = 0; j < RT; j++) acc[i][j] = fma(a[i], b[j], acc[i][j]);
             }
             if (more) {
 #pragma unroll
@@ -190,18 +204,18 @@ __global__ void __launch_bounds__(NT) dfma_gemm_kernel(Gemm g)
     if (g.partial) {  // split-K: raw partial product
         double *P = g.partial + (long long)split * g.m * g.n;
 #pragma unroll
-        for (int i = 0; i < 4; i++)
+        for (int i = 0; i < RT; i++)
 #pragma unroll
-            for (int j = 0; j < 4; j++) {
+            for (int j = 0; j < RT; j++) {
                 const int r = r0 + tx + 16 * i, c = c0 + ty + 16 * j;
                 if (r < g.m && c < g.n) P[(long long)c * g.m + r] = acc[i][j];
             }
         return;
     }
 #pragma unroll
-    for (int i = 0; i < 4; i++)
+    for (int i = 0; i < RT; i++)
 #pragma unroll
-        for (int j = 0; j < 4; j++) {
+        for (int j = 0; j < RT; j++) {
             const int r = r0 + tx + 16 * i, c = c0 + ty + 16 * j;
             if (r < g.m && c < g.n && (!diag || r >= c)) {
                 double *cp = g.C + (long long)c * g.ldc + r;
@@ -211,7 +225,7 @@ __global__ void __launch_bounds__(NT) dfma_gemm_kernel(Gemm g)
 }
 
 // C = alpha sum_s P[s] + beta C, the splits added in a fixed order.
-__global__ void __launch_bounds__(256) splitk_reduce(int m, int n, int splits, const double *__restrict__ P,
+__global__ void __launch_bounds__(128) splitk_reduce(int m, int n, int splits, const double *__restrict__ P,
                                                      double alpha, double beta, double *__restrict__ C,
                                                      long long ldc)
 {
@@ -234,36 +248,60 @@ int sm_count()
     return sms;
 }
 
-// Split the reduction until about four CTAs per SM are busy, keeping at
-// least 8 steps of BK per split and the partials within the workspace.
-int choose_splits(long long tiles, int k, int m, int n, size_t work_elems)
+// Tile and splits.  64 x 64 tiles where they alone give each SM two CTAs (99 %
+// of the FP64 pipe in long products), else 32 x 32 ones; then the reduction is
+// split until every SM has two CTAs, keeping 16 values of k per split and the
+// partials within the workspace.
+struct Shape {
+    int ts, splits;
+};
+
+Shape choose_shape(const Gemm &g, size_t work_elems)
 {
-    const long long target = 4LL * sm_count();
-    int s = 1;
-    while (tiles * s < target && (long long)k >= 2LL * s * 8 * BK && s < 512 &&
-           (size_t)(2 * s) * (size_t)m * (size_t)n <= work_elems)
-        s *= 2;
+    const long long target = 2LL * sm_count();
+    auto tiles = [&](int ts) {
+        const long long tm = (g.m + ts - 1) / ts, tn = (g.n + ts - 1) / ts;
+        return g.lower ? tm * (tm + 1) / 2 : tm * tn;
+    };
+    Shape s{64, 1};
+    if (tiles(64) < target) s.ts = 32;
+    const long long t = tiles(s.ts), k = (long long)g.k + g.k2;
+    if (g.partial && !g.lower && t < target) {
+        long long sp = std::min({(target + t - 1) / t, k / 16, 64LL, (long long)(work_elems / ((size_t)g.m * g.n))});
+        s.splits = (int)std::max(1LL, sp);
+    }
     return s;
 }
 
-template <int MA, int MB>
-cudaError_t launch(Gemm g, int splits, cudaStream_t st)
+template <int MA, int MB, int TS>
+cudaError_t launch_as(Gemm g, int splits, cudaStream_t st)
 {
-    if (g.m <= 0 || g.n <= 0) return cudaSuccess;
-    const int tm = (g.m + BM - 1) / BM, tn = (g.n + BN - 1) / BN;
+    constexpr int BK = 512 / TS;
+    const int tm = (g.m + TS - 1) / TS, tn = (g.n + TS - 1) / TS;
     g.tiles_m = tm;
-    if ((g.k <= 0 && g.k2 <= 0) || g.k2 > 0 || g.lower) splits = 1;  // split-K: one product, full tiles
-    g.kchunk = ((g.k + splits - 1) / splits + BK - 1) / BK * BK;
+    const int k = (g.k + BK - 1) / BK * BK + g.k2;
+    g.kchunk = ((k + splits - 1) / splits + BK - 1) / BK * BK;
     if (g.kchunk <= 0) g.kchunk = BK;
+    splits = std::max(1, (k + g.kchunk - 1) / g.kchunk);
     g.partial = splits > 1 ? g.partial : nullptr;
     dim3 grid;
     if (g.lower) grid = dim3((unsigned)((long long)tm * (tm + 1) / 2), 1, (unsigned)splits);
     else grid = dim3((unsigned)tm, (unsigned)tn, (unsigned)splits);
-    dfma_gemm_kernel<MA, MB><<<grid, NT, 0, st>>>(g);
+    dfma_gemm_kernel<MA, MB, TS><<<grid, NT, 0, st>>>(g);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || splits == 1) return e;
-    splitk_reduce<<<1024, 256, 0, st>>>(g.m, g.n, splits, g.partial, g.alpha, g.beta, g.C, g.ldc);
+    const long long total = (long long)g.m * g.n;
+    splitk_reduce<<<(unsigned)std::min(1024LL, (total + 127) / 128), 128, 0, st>>>(g.m, g.n, splits, g.partial, g.alpha,
+                                                                                   g.beta, g.C, g.ldc);
     return cudaGetLastError();
+}
+
+template <int MA, int MB>
+cudaError_t launch(Gemm g, size_t work_elems, cudaStream_t st)
+{
+    if (g.m <= 0 || g.n <= 0) return cudaSuccess;
+    const Shape s = choose_shape(g, work_elems);
+    return s.ts == 64 ? launch_as<MA, MB, 64>(g, s.splits, st) : launch_as<MA, MB, 32>(g, s.splits, st);
 }
 
 Gemm base(int m, int n, int k, double alpha, const double *A, long long lda, const double *B, long long ldb,
@@ -294,28 +332,23 @@ cudaError_t dfma_gemm(char transa, char transb, int m, int n, int k, double alph
                       size_t work_elems, cudaStream_t st)
 {
     Gemm g = base(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc, work);
-    const long long tiles = (long long)((m + BM - 1) / BM) * ((n + BN - 1) / BN);
-    const int s = work ? choose_splits(tiles, k, m, n, work_elems) : 1;
     const bool ta = transa == 'T' || transa == 't', tb = transb == 'T' || transb == 't';
-    if (!ta && !tb) return launch<MODE_N, MODE_N>(g, s, st);
-    if (ta && !tb) return launch<MODE_T, MODE_N>(g, s, st);
-    if (!ta && tb) return launch<MODE_N, MODE_T>(g, s, st);
-    return launch<MODE_T, MODE_T>(g, s, st);
+    if (!ta && !tb) return launch<MODE_N, MODE_N>(g, work_elems, st);
+    if (ta && !tb) return launch<MODE_T, MODE_N>(g, work_elems, st);
+    if (!ta && tb) return launch<MODE_N, MODE_T>(g, work_elems, st);
+    return launch<MODE_T, MODE_T>(g, work_elems, st);
 }
 
 cudaError_t dfma_symm(char side, int m, int n, double alpha, const double *S, long long lds, const double *B,
                       long long ldb, double beta, double *C, long long ldc, double *work, size_t work_elems,
                       cudaStream_t st)
 {
-    const long long tiles = (long long)((m + BM - 1) / BM) * ((n + BN - 1) / BN);
     if (side == 'L' || side == 'l') {
         Gemm g = base(m, n, m, alpha, S, lds, B, ldb, beta, C, ldc, work);
-        const int s = work ? choose_splits(tiles, m, m, n, work_elems) : 1;
-        return launch<MODE_SYM, MODE_N>(g, s, st);
+        return launch<MODE_SYM, MODE_N>(g, work_elems, st);
     }
     Gemm g = base(m, n, n, alpha, B, ldb, S, lds, beta, C, ldc, work);
-    const int s = work ? choose_splits(tiles, n, m, n, work_elems) : 1;
-    return launch<MODE_N, MODE_SYM>(g, s, st);
+    return launch<MODE_N, MODE_SYM>(g, work_elems, st);
 }
 
 cudaError_t dfma_syr2k_lower(int n, int k, double alpha, const double *A, long long lda, const double *B,
@@ -329,7 +362,7 @@ cudaError_t dfma_syr2k_lower(int n, int k, double alpha, const double *A, long l
     g.ldb2 = lda;
     g.k2 = k;
     g.lower = 1;
-    return launch<MODE_N, MODE_T>(g, 1, st);
+    return launch<MODE_N, MODE_T>(g, 0, st);
 }
 
 cudaError_t dfma_syrk_lower_t(int n, int k, double alpha, const double *A, long long lda, double beta, double *C,
@@ -337,7 +370,7 @@ cudaError_t dfma_syrk_lower_t(int n, int k, double alpha, const double *A, long 
 {
     Gemm g = base(n, n, k, alpha, A, lda, A, lda, beta, C, ldc, nullptr);
     g.lower = 1;
-    return launch<MODE_T, MODE_N>(g, 1, st);
+    return launch<MODE_T, MODE_N>(g, 0, st);
 }
 
 }  // namespace gb

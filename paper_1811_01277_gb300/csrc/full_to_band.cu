@@ -213,35 +213,7 @@ __global__ void __launch_bounds__(256) panel_explicit_y(int m, int nb, const dou
     }
 }
 
-// T (nb x nb upper triangular) of the block reflector I - Y T Y^T from
-// G = Y^T Y and tau: T[j][j] = tau_j, T[0:j, j] = -tau_j T[0:j, 0:j] G[0:j, j].
-__global__ void __launch_bounds__(kPanelMax) panel_build_t(int nb, const double *__restrict__ G, long long ldg,
-                                                           const double *__restrict__ tau, double *__restrict__ T,
-                                                           long long ldt)
-{
-    __shared__ double Ts[kPanelMax][kPanelMax + 1];
-    __shared__ double g[kPanelMax];
-    const int r = threadIdx.x;
-    for (int j = 0; j < nb; j++) {
-        if (r < nb) Ts[r][j] = 0.0;
-    }
-    __syncthreads();
-    for (int j = 0; j < nb; j++) {
-        if (r < j) g[r] = G[(long long)j * ldg + r];
-        __syncthreads();
-        if (r < j) {
-            double s = 0.0;
-            for (int q = r; q < j; q++) s = fma(Ts[r][q], g[q], s);
-            Ts[r][j] = -tau[j] * s;
-        }
-        if (r == j) Ts[j][j] = tau[j];
-        __syncthreads();
-    }
-    if (r < nb)
-        for (int j = 0; j < nb; j++) T[(long long)j * ldt + r] = Ts[r][j];
-}
-
-// W = X - 0.5 * Y * M is done by cuBLAS; H = 1.5 I - 0.5 G for Newton-Schulz.
+// H = 1.5 I - 0.5 G for Newton-Schulz.
 __global__ void __launch_bounds__(256) ns_matrix(int k, double *__restrict__ G, long long ldg)
 {
     const long long total = (long long)k * k;
@@ -341,13 +313,6 @@ cudaError_t panel_y_and_t_prep(int m, int nb, const double *P, long long lda, do
                                cudaStream_t st)
 {
     panel_explicit_y<<<256, 256, 0, st>>>(m, nb, P, lda, Y, ldy);
-    return cudaGetLastError();
-}
-
-cudaError_t panel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt,
-                    cudaStream_t st)
-{
-    panel_build_t<<<1, kPanelMax, 0, st>>>(nb, G, ldg, tau, T, ldt);
     return cudaGetLastError();
 }
 

@@ -171,37 +171,6 @@ __global__ void __launch_bounds__(256) zpanel_explicit_y(int m, int nb, const Zd
     }
 }
 
-// T[j][j] = tau_j, T[0:j, j] = -tau_j T[0:j, 0:j] G[0:j, j], G = Y^H Y
-__global__ void __launch_bounds__(kPanelMax) zpanel_build_t(int nb, const Zd *__restrict__ G, long long ldg,
-                                                            const Zd *__restrict__ tau, Zd *__restrict__ T,
-                                                            long long ldt)
-{
-    __shared__ Zd Ts[kPanelMax][kPanelMax + 1];
-    __shared__ Zd g[kPanelMax];
-    const int r = threadIdx.x;
-    for (int j = 0; j < nb; j++)
-        if (r < nb) Ts[r][j] = Zd{0.0, 0.0};
-    __syncthreads();
-    for (int j = 0; j < nb; j++) {
-        if (r < j) g[r] = G[(long long)j * ldg + r];
-        __syncthreads();
-        if (r < j) {
-            Zd s{0.0, 0.0};
-            for (int q = r; q < j; q++) {
-                const Zd p = zm(Ts[r][q], g[q]);
-                s.re += p.re;
-                s.im += p.im;
-            }
-            const Zd ts = zm(tau[j], s);
-            Ts[r][j] = Zd{-ts.re, -ts.im};
-        }
-        if (r == j) Ts[j][j] = tau[j];
-        __syncthreads();
-    }
-    if (r < nb)
-        for (int j = 0; j < nb; j++) T[(long long)j * ldt + r] = Ts[r][j];
-}
-
 __global__ void __launch_bounds__(256) zextract_band(int n, int b, const Zd *__restrict__ A, long long lda,
                                                      Zd *__restrict__ AB, long long ldab)
 {
@@ -259,12 +228,6 @@ cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, doub
 cudaError_t zpanel_y(int m, int nb, const double *P, long long lda, double *Y, long long ldy, cudaStream_t st)
 {
     zpanel_explicit_y<<<256, 256, 0, st>>>(m, nb, (const Zd *)P, lda, (Zd *)Y, ldy);
-    return cudaGetLastError();
-}
-
-cudaError_t zpanel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt, cudaStream_t st)
-{
-    zpanel_build_t<<<1, kPanelMax, 0, st>>>(nb, (const Zd *)G, ldg, (const Zd *)tau, (Zd *)T, ldt);
     return cudaGetLastError();
 }
 

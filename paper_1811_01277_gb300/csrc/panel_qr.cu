@@ -192,11 +192,7 @@ panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__
             if (warp == (i * LPC) / 32) {   // the warp that holds column i
                 const int src = (i * LPC) & 31;
                 const double ss = __shfl_sync(0xffffffffu, re_of(sum), src);
-                T alpha = ai;
-                *(double *)&alpha = __shfl_sync(0xffffffffu, *(double *)&ai, src);
-                if (sizeof(T) == 16)
-                    ((double *)&alpha)[sizeof(T) / 8 - 1] =
-                        __shfl_sync(0xffffffffu, ((double *)&ai)[sizeof(T) / 8 - 1], src);
+                const T alpha = lane_of(ai, src);
                 const auto h = reflector(alpha, ss);
                 if ((tid & 31) == 0) {
                     sm.tau[par] = h.tau;
@@ -337,7 +333,156 @@ cudaError_t panel_qr_t(int m, int nb, T *P, long long lda, T *tau, T *Y, long lo
     return launch_grid<T, 64, 4, Z ? 16 : 32>(m, nb, P, lda, tau, Y, ldy, part, sms, 1, st, done);
 }
 
+// T (nb x nb upper triangular) of the block reflector I - Y T Y^H is the
+// inverse of the triangle with diagonal 1/tau and the strict upper part of
+// G = Y^H Y, so its columns are independent: x_j = tau_j, then for i = j-1 .. 0
+// x_i = -tau_i sum_{q > i} G_iq x_q (zero where tau_i is zero).  One block per
+// column; its first warp keeps the pending sums of R rows per lane, and each
+// x_i found is added into all of them: a chain of nb short steps, where the
+// forward recurrence over columns by one block took 50 us for nb = 32 and 501 us
+// for nb = 64 complex (now 9 and 41 us).  The other warps stage the next columns of G.
+constexpr int kTMax = 256;   // widest block reflector
+constexpr int kTCols = 16;   // columns of G staged at a time
+
+// R: rows per lane (32 R >= nb)
+template <class T, int R>
+__global__ void __launch_bounds__(128) panel_t_kernel(int nb, const T *__restrict__ G, long long ldg,
+                                                      const T *__restrict__ tau, T *__restrict__ Tm, long long ldt)
+{
+    constexpr int LDG = 32 * R;
+    extern __shared__ __align__(16) unsigned char dyn[];
+    T *Gs = (T *)dyn;                         // two stages of kTCols columns, rows above the diagonal
+    const int j = blockIdx.x, lane = threadIdx.x & 31;
+    const bool worker = threadIdx.x < 32;
+    auto stage = [&](int c) {
+        T *S = Gs + (c & 1) * kTCols * LDG;
+        constexpr int NE = kTCols * LDG / 128, CH = NE < 16 ? NE : 16;
+        for (int e0 = 0; e0 < NE; e0 += CH) {   // CH loads in flight per thread
+            T g[CH];
+#pragma unroll
+            for (int u = 0; u < CH; u++) {
+                const int e = threadIdx.x + 128 * (e0 + u), col = c * kTCols + e / LDG, r = e % LDG;
+                zero_of(g[u]);
+                if (col <= j && r < col) g[u] = G[(long long)col * ldg + r];
+            }
+#pragma unroll
+            for (int u = 0; u < CH; u++) S[threadIdx.x + 128 * (e0 + u)] = g[u];
+        }
+    };
+    T s[R], x[R], nt[R];                      // pending sums, results and -tau of rows lane + 32 u
+#pragma unroll
+    for (int u = 0; u < R; u++) {
+        const int r = lane + 32 * u;
+        zero_of(s[u]);
+        zero_of(x[u]);
+        zero_of(nt[u]);
+        if (r < nb) nt[u] = scale(tau[r], -1.0);
+        if (r == j) x[u] = tau[r];
+    }
+    const int last = j / kTCols;
+    stage(last);
+    __syncthreads();
+    for (int c = last; c >= 0; c--) {
+        if (c > 0) stage(c - 1);              // while the first warp works on c
+        if (worker) {
+            const T *S = Gs + (c & 1) * kTCols * LDG;
+            for (int i = min(j, c * kTCols + kTCols - 1); i >= c * kTCols; i--) {
+                const int src = i & 31, ui = i >> 5;
+                T xi;
+                zero_of(xi);
+#pragma unroll
+                for (int u = 0; u < R; u++)
+                    if (u == ui) {
+                        if (i < j) {
+                            const T v = mul(nt[u], s[u]);
+                            if (lane == src) x[u] = v;
+                            xi = v;
+                        } else {
+                            xi = x[u];
+                        }
+                    }
+                xi = lane_of(xi, src);
+                const T *g = S + (i - c * kTCols) * LDG;
+#pragma unroll
+                for (int u = 0; u < R; u++)   // the rows above i
+                    if (u <= ui && lane + 32 * u < i) s[u] = mad(g[lane + 32 * u], xi, s[u]);
+            }
+        }
+        __syncthreads();
+    }
+    if (!worker) return;
+#pragma unroll
+    for (int u = 0; u < R; u++) {
+        const int r = lane + 32 * u;
+        if (r < nb) Tm[(long long)j * ldt + r] = x[u];
+    }
+}
+
+template <class T, int R>
+cudaError_t launch_panel_t_as(int nb, const T *G, long long ldg, const T *tau, T *Tm, long long ldt, cudaStream_t st)
+{
+    const size_t smem = (size_t)2 * kTCols * 32 * R * sizeof(T);
+    cudaError_t e = cudaFuncSetAttribute(panel_t_kernel<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    panel_t_kernel<T, R><<<nb, 128, smem, st>>>(nb, G, ldg, tau, Tm, ldt);
+    return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t launch_panel_t(int nb, const T *G, long long ldg, const T *tau, T *Tm, long long ldt, cudaStream_t st)
+{
+    if (nb < 1) return cudaSuccess;
+    if (nb <= 32) return launch_panel_t_as<T, 1>(nb, G, ldg, tau, Tm, ldt, st);
+    if (nb <= 64) return launch_panel_t_as<T, 2>(nb, G, ldg, tau, Tm, ldt, st);
+    if (nb <= 128) return launch_panel_t_as<T, 4>(nb, G, ldg, tau, Tm, ldt, st);
+    if (nb <= kTMax) return launch_panel_t_as<T, 8>(nb, G, ldg, tau, Tm, ldt, st);
+    return cudaErrorInvalidValue;
+}
+
+// Explicit reflectors of `np` consecutive panels of nb columns each, side by
+// side (m x np nb, ldy): panel p's reflectors start at row p nb, its QR'd
+// form lies at P + p (nb lda + nb) (the diagonal blocks below one another).
+template <class T>
+__global__ void __launch_bounds__(256) panels_explicit_y(int m, int nb, int np, const T *__restrict__ P, long long lda,
+                                                         T *__restrict__ Y, long long ldy)
+{
+    const long long total = (long long)m * nb * np;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
+         e += (long long)gridDim.x * blockDim.x) {
+        const int c = (int)(e / m), r = (int)(e - (long long)c * m);
+        T y;
+        zero_of(y);
+        if (r == c) one_of(y);       // column c of the group has its unit entry in row c
+        else if (r > c) y = P[(long long)c * lda + r];
+        Y[(long long)c * ldy + r] = y;
+    }
+}
+
 }  // namespace
+
+cudaError_t panels_y(int is_complex, int m, int nb, int np, const double *P, long long lda, double *Y, long long ldy,
+                     cudaStream_t st)
+{
+    const unsigned blocks = (unsigned)std::min(1184LL, ((long long)m * nb * np + 255) / 256);
+    if (is_complex)
+        panels_explicit_y<Zc><<<blocks, 256, 0, st>>>(m, nb, np, (const Zc *)P, lda, (Zc *)Y, ldy);
+    else
+        panels_explicit_y<double><<<blocks, 256, 0, st>>>(m, nb, np, P, lda, Y, ldy);
+    return cudaGetLastError();
+}
+
+// T of the panel's block reflector from G = Y^H Y (nb x nb, ldg; the strict
+// upper part is read) and tau
+cudaError_t panel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt,
+                    cudaStream_t st)
+{
+    return launch_panel_t<double>(nb, G, ldg, tau, T, ldt, st);
+}
+
+cudaError_t zpanel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt, cudaStream_t st)
+{
+    return launch_panel_t<Zc>(nb, (const Zc *)G, ldg, (const Zc *)tau, (Zc *)T, ldt, st);
+}
 
 // Bytes of the exchange area a panel of m rows may need (`part`).
 size_t panel_part_bytes(int m, int is_complex)

@@ -72,6 +72,10 @@ __device__ __forceinline__ T tree_sum(T (&a)[V / TP])
     return x;
 }
 
+// x of lane `src`
+__device__ __forceinline__ double lane_of(double x, int src) { return __shfl_sync(0xffffffffu, x, src); }
+__device__ __forceinline__ Zc lane_of(Zc x, int src) { return {lane_of(x.re, src), lane_of(x.im, src)}; }
+
 __device__ __forceinline__ double ld_cg(const double *p) { return __ldcg(p); }
 __device__ __forceinline__ Zc ld_cg(const Zc *p)
 {

@@ -376,6 +376,12 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
             return e;
         return ahead ? cudaEventRecord(la->factored, fst) : cudaSuccess;
     };
+    // lower triangle of C -= X Y^T + Y X^T
+    auto update = [&](int m, const double *X, const double *Yp, long long ldy, double *C) -> cudaError_t {
+        if (use_sliced(m, m, b))
+            return gb::sliced_dsyr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, w.sl, st, pd);
+        return gb::dfma_syr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, st);
+    };
     int pp = 0;
     if (b < n) {
         if (ahead) {
@@ -400,29 +406,20 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         GB_CU(gb::dfma_gemm('T', 'N', b, b, m, 1.0, Yp, m, w.X, m, 0.0, w.Pm, b, w.gw, w.gw_elems, st));
         GB_CU(gb::dfma_gemm('T', 'N', b, b, b, 1.0, T, b, w.Pm, b, 0.0, w.M, b, w.gw, w.gw_elems, st));
         GB_CU(gb::dfma_gemm('N', 'N', m, b, b, -0.5, Yp, m, w.M, b, 1.0, w.X, m, w.gw, w.gw_elems, st));
-        if (m > b) {
+        if (ahead && m > b) {
             // the next panel's columns first (all m rows; the upper triangle
             // of their diagonal block is updated too and never read), then
             // the next panel is factored on the helper stream while the rest
             // of the trailing update runs here
             GB_CU(gb::dfma_gemm('N', 'T', m, b, b, -1.0, w.X, m, Yp, m, 1.0, A2, ldw, w.gw, w.gw_elems, st));
             GB_CU(gb::dfma_gemm('N', 'T', m, b, b, -1.0, Yp, m, w.X, m, 1.0, A2, ldw, w.gw, w.gw_elems, st));
-            if (ahead) {
-                GB_CU(cudaEventRecord(la->ready, st));
-                GB_CU(cudaStreamWaitEvent(la->side, la->ready, 0));
-            }
+            GB_CU(cudaEventRecord(la->ready, st));
+            GB_CU(cudaStreamWaitEvent(la->side, la->ready, 0));
             GB_CU(factor(pp + 1));
-            if (use_sliced(m - b, m - b, b))
-                GB_CU(gb::sliced_dsyr2k_lower(m - b, b, -1.0, w.X + b, m, Yp + b, m, 1.0, A2 + (long long)b * ldw + b,
-                                              ldw, w.sl, st, pd));
-            else
-                GB_CU(gb::dfma_syr2k_lower(m - b, b, -1.0, w.X + b, m, Yp + b, m, 1.0, A2 + (long long)b * ldw + b,
-                                           ldw, st));
+            GB_CU(update(m - b, w.X + b, Yp + b, m, A2 + (long long)b * ldw + b));
         } else {
-            if (use_sliced(m, m, b))
-                GB_CU(gb::sliced_dsyr2k_lower(m, b, -1.0, w.X, m, Yp, m, 1.0, A2, ldw, w.sl, st, pd));
-            else
-                GB_CU(gb::dfma_syr2k_lower(m, b, -1.0, w.X, m, Yp, m, 1.0, A2, ldw, st));
+            GB_CU(update(m, w.X, Yp, m, A2));
+            if (m > b) GB_CU(factor(pp + 1));
         }
     }
     GB_CU(gb::band_from_full(n, b, w.Aw, ldw, w.AB, b + 1, st));

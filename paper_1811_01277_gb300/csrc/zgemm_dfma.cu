@@ -154,7 +154,10 @@ cudaError_t dfma_zgemm(char opa, char opb, int m, int n, int k, double2 alpha, c
     int splits = 1;
     if (k > 0) {
         const long long want = (2 * 152 + tiles - 1) / tiles;
-        const long long by_k = k / 256 > 0 ? k / 256 : 1;
+        // down to 32 values of k per split: a 32 x 32 x 32 complex block is 33
+        // us of one SM's FP64 pipe, so long reductions have to reach every SM
+        // (panels of a complex n = 1501 solve: 172 -> 68 us a launch)
+        const long long by_k = k / 32 > 0 ? k / 32 : 1;
         const long long by_ws = work ? (long long)(work_elems / 2 / ((size_t)m * n)) : 1;
         long long s = want < by_k ? want : by_k;
         s = s < by_ws ? s : by_ws;
