@@ -3,9 +3,11 @@
 //
 // 1. Multisection on the Sturm count: the number of negative pivots of the
 //    LDL^T factorisation of T - xI is the number of eigenvalues below x.
-//    Four lanes per eigenvalue evaluate the count at four interior points of
-//    the current interval (which shrinks five-fold per round), starting from
-//    the Gershgorin interval, until it stops shrinking in FP64.
+//    P = 4 to 32 lanes per eigenvalue evaluate the count at P interior points
+//    of the current interval, which shrinks P + 1-fold per round.  The first 18
+//    bits come from counts in FP32, whose interval is widened by many times
+//    their error and checked by two FP64 counts; FP64 rounds follow until the
+//    interval stops shrinking.
 // 2. Inverse iteration, one thread per eigenvalue: T - lambda I is factored
 //    by Gaussian elimination with partial pivoting (a tridiagonal LU with one
 //    extra super-diagonal from the interchanges); three solves from a
@@ -56,23 +58,29 @@ __global__ void __launch_bounds__(256) tridiag_bounds(int n, const double *__res
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        double nrm = snr[0] > 0 ? snr[0] : 1.0;
-        out[0] = slo[0] - 2.0 * 0x1p-52 * nrm;
-        out[1] = shi[0] + 2.0 * 0x1p-52 * nrm;
-        out[2] = nrm;
+        out[0] = slo[0] - 2.0 * 0x1p-52 * snr[0];   // both zero for a zero matrix
+        out[1] = shi[0] + 2.0 * 0x1p-52 * snr[0];
+        out[2] = snr[0] > 0 ? snr[0] : 1.0;
     }
 }
 
-__global__ void __launch_bounds__(256) square_offdiag(int n, const double *__restrict__ e, double *__restrict__ e2,
-                                                      double *pivmin_out)
+__global__ void __launch_bounds__(256) square_offdiag(int n, const double *__restrict__ d, const double *__restrict__ e,
+                                                      const double *__restrict__ bounds, double *__restrict__ e2,
+                                                      double *pivmin_out, float2 *__restrict__ t32)
 {
-    // e2[i] = e[i]^2 ; pivmin = (smallest normal) * max(1, max e^2)
+    // e2[i] = e[i]^2 ; pivmin = (smallest normal) * max(1, max e^2); t32[i] =
+    // (d[i], e[i-1]^2) of T / ||T|| in FP32
     __shared__ double sm[256];
+    const double inv = 1.0 / bounds[2];
     double mx = 1.0;
-    for (int i = threadIdx.x; i < n - 1; i += blockDim.x) {
-        double v = e[i] * e[i];
-        e2[i] = v;
-        mx = fmax(mx, v);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        if (i < n - 1) {
+            double v = e[i] * e[i];
+            e2[i] = v;
+            mx = fmax(mx, v);
+        }
+        const double s = i > 0 ? e[i - 1] * inv : 0.0;
+        t32[i] = make_float2((float)(d[i] * inv), (float)(s * s));
     }
     sm[threadIdx.x] = mx;
     __syncthreads();
@@ -130,42 +138,98 @@ __device__ __forceinline__ int sturm_count(int n, const double *__restrict__ d, 
     return cnt;
 }
 
-// Multisection: kMultisect lanes per eigenvalue k (0-based, ascending).  In
-// each round the lanes evaluate the Sturm count at the kMultisect points that
-// split [lo, hi] into kMultisect + 1 equal parts, exchange the counts, and the
-// group keeps the part in which the count passes k.  Rounds stop when the
-// interval is within max(u ||T||, 2 (kMultisect + 1) u |x|) or cannot shrink.
-constexpr int kMultisect = 4;
-
-__global__ void __launch_bounds__(128) tridiag_bisect(int n, int nev, const double *__restrict__ d,
-                                                       const double *__restrict__ e2, const double *bounds,
-                                                       const double *pivmin_p, double *__restrict__ lam)
+// The same in FP32 for T / ||T||: exact for a matrix within a few 2^-24 of it.
+__device__ __forceinline__ int sturm_count32(int n, const float2 *__restrict__ t, float x)
 {
-    constexpr int P = kMultisect;
+    float q = 1.0f;
+    int cnt = 0;
+#pragma unroll 8
+    for (int i = 0; i < n; i++) {
+        const float2 a = t[i];   // a.y = 0 in the first row
+        float r;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(q));
+        q = fmaf(-a.y, r, a.x - x);
+        if (fabsf(q) < 1e-20f) q = -1e-20f;
+        cnt += (int)(__float_as_uint(q) >> 31);
+    }
+    return cnt;
+}
+
+// Multisection: P lanes per eigenvalue k (0-based, ascending).  In each round
+// the lanes evaluate the Sturm count at the P points that split [lo, hi] into
+// P + 1 equal parts, exchange the counts, and the group keeps the part in
+// which the count passes k.  Rounds stop when the interval is within
+// max(u ||T||, 10 u |x|) or cannot shrink (points may coincide by then).
+//
+// What bounds it: every count is a chain of n pivots.  An FP64 instruction of
+// a warp occupies its scheduler's FP64 pipe for 64 clocks, so a pivot costs
+// about 600 clocks as long as a scheduler has one warp, whatever P is: P is the
+// largest power of two up to 32 that keeps the warps within the schedulers.
+// FP32 pivots cost about a tenth; they take the first 18 of 53 bits.
+// Measured on a GB300 (before: four lanes, FP64 throughout): 2048 eigenvalues of
+// n = 8192 59.5 -> 32.4 ms, 450 of n = 1501 10.9 -> 4.0 ms.
+constexpr float kStop32 = 0x1p-18f;      // FP32 rounds end here (relative to ||T||)
+constexpr double kMargin32 = 0x1p-18;    // and the interval is widened by this much on each side
+
+template <int P>
+__global__ void __launch_bounds__(128) tridiag_bisect(int n, int nev, const double *__restrict__ d,
+                                                       const double *__restrict__ e2, const float2 *__restrict__ t32,
+                                                       const double *bounds, const double *pivmin_p,
+                                                       double *__restrict__ lam)
+{
     const int gt = blockIdx.x * blockDim.x + threadIdx.x;
     const int k = gt / P;
     const int j = gt % P;
     const int lane0 = (threadIdx.x & 31) & ~(P - 1);  // first lane of this group in the warp
     const double pivmin = *pivmin_p;
     const unsigned long long pivkey = abs_key(pivmin);
-    const double abstol = 0x1p-53 * bounds[2];
-    double lo = bounds[0], hi = bounds[1];
+    const double nrm = bounds[2];
+    const double abstol = 0x1p-53 * nrm;
     bool done = k >= nev;
-    for (int round = 0; round < 400; round++) {
-        const double w = hi - lo;
-        if (!done) {
-            const double tol = fmax(abstol, (2.0 * (P + 1) * 0x1p-53) * fmax(fabs(lo), fabs(hi)));
-            done = !(w > tol);
-        }
-        if (__all_sync(0xffffffffu, done)) break;
-        const double h = w * (1.0 / (P + 1));
-        const int c = done ? 0 : sturm_count(n, d, e2, fma((double)(j + 1), h, lo), pivmin, pivkey);
-        int first = P;  // first point whose count exceeds k
+    // first point whose count exceeds k (P: none)
+    auto first_above = [&](int c) {
+        int first = P;
 #pragma unroll
         for (int m = P - 1; m >= 0; m--) {
             const int cm = __shfl_sync(0xffffffffu, c, lane0 + m);
             if (cm > k) first = m;
         }
+        return first;
+    };
+
+    float flo = -1.001f, fhi = 1.001f;   // the spectrum of T / ||T||
+    for (int round = 0; round < 64; round++) {
+        const float w = fhi - flo;
+        const bool narrow = done || !(w > kStop32);
+        if (__all_sync(0xffffffffu, narrow)) break;
+        const float h = w * (1.0f / (P + 1));
+        const int first = first_above(narrow ? 0 : sturm_count32(n, t32, fmaf((float)(j + 1), h, flo)));
+        if (!narrow) {
+            const float nlo = (first == 0) ? flo : fmaf((float)first, h, flo);
+            const float nhi = (first == P) ? fhi : fmaf((float)(first + 1), h, flo);
+            flo = nlo;
+            fhi = nhi;
+        }
+    }
+    double lo = fmax(bounds[0], ((double)flo - kMargin32) * nrm), hi = fmin(bounds[1], ((double)fhi + kMargin32) * nrm);
+    {
+        // the widened interval holds eigenvalue k, or the search starts anew
+        const int c = done ? 0 : sturm_count(n, d, e2, (j & 1) ? hi : lo, pivmin, pivkey);
+        const int clo = __shfl_sync(0xffffffffu, c, lane0), chi = __shfl_sync(0xffffffffu, c, lane0 + 1);
+        if (!(clo <= k && chi > k)) {
+            lo = bounds[0];
+            hi = bounds[1];
+        }
+    }
+    for (int round = 0; round < 400; round++) {
+        const double w = hi - lo;
+        if (!done) {
+            const double tol = fmax(abstol, (10.0 * 0x1p-53) * fmax(fabs(lo), fabs(hi)));
+            done = !(w > tol);
+        }
+        if (__all_sync(0xffffffffu, done)) break;
+        const double h = w * (1.0 / (P + 1));
+        const int first = first_above(done ? 0 : sturm_count(n, d, e2, fma((double)(j + 1), h, lo), pivmin, pivkey));
         if (!done) {
             const double nlo = (first == 0) ? lo : fma((double)first, h, lo);
             const double nhi = (first == P) ? hi : fma((double)(first + 1), h, lo);
@@ -175,6 +239,29 @@ __global__ void __launch_bounds__(128) tridiag_bisect(int n, int nev, const doub
         }
     }
     if (j == 0 && k < nev) lam[k] = 0.5 * (lo + hi);
+}
+
+// lam[k] = max(lam[0..k]): eigenvalues equal to working accuracy, found from
+// intervals of their own, may differ from ascending order in the last place.
+__global__ void __launch_bounds__(1024) tridiag_ascending(int nev, double *__restrict__ lam)
+{
+    __shared__ double top[1024];
+    const int per = (nev + 1023) / 1024, a = threadIdx.x * per, b = min(nev, a + per);
+    double m = -1.7976931348623157e308;
+    for (int k = a; k < b; k++) m = fmax(m, lam[k]);
+    top[threadIdx.x] = m;
+    __syncthreads();
+    for (int o = 1; o < 1024; o <<= 1) {
+        const double x = threadIdx.x >= o ? top[threadIdx.x - o] : m;
+        __syncthreads();
+        top[threadIdx.x] = m = fmax(m, x);
+        __syncthreads();
+    }
+    m = threadIdx.x > 0 ? top[threadIdx.x - 1] : -1.7976931348623157e308;
+    for (int k = a; k < b; k++) {
+        m = fmax(m, lam[k]);
+        lam[k] = m;
+    }
 }
 
 // Deterministic pseudo-random start vector entry in [-0.5, 0.5): 52 hashed
@@ -555,9 +642,22 @@ cudaError_t tridiag_bisect_d(int n, int nev, const double *d, const double *e, d
 {
     EigWork w = carve_eig(n, nev, ws);
     tridiag_bounds<<<1, 256, 0, st>>>(n, d, e, w.bounds);
-    square_offdiag<<<1, 256, 0, st>>>(n, e, w.e2, w.pivmin);
-    const long long lanes = (long long)nev * kMultisect;
-    tridiag_bisect<<<(unsigned)((lanes + 127) / 128), 128, 0, st>>>(n, nev, d, w.e2, w.bounds, w.pivmin, lam);
+    float2 *t32 = (float2 *)w.Y;   // scratch of the next phase
+    square_offdiag<<<1, 256, 0, st>>>(n, d, e, w.bounds, w.e2, w.pivmin, t32);
+    int dev = 0, sms = 0;
+    cudaError_t err;
+    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
+    if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
+    const long long warps = 4LL * sms;   // one per scheduler
+    auto run = [&](auto kernel, int p) {
+        const long long lanes = (long long)nev * p;
+        kernel<<<(unsigned)((lanes + 127) / 128), 128, 0, st>>>(n, nev, d, w.e2, t32, w.bounds, w.pivmin, lam);
+    };
+    if (nev <= warps) run(tridiag_bisect<32>, 32);
+    else if (nev <= 2 * warps) run(tridiag_bisect<16>, 16);
+    else if (nev <= 4 * warps) run(tridiag_bisect<8>, 8);
+    else run(tridiag_bisect<4>, 4);
+    tridiag_ascending<<<1, 1024, 0, st>>>(nev, lam);
     return cudaGetLastError();
 }
 
