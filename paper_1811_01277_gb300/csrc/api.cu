@@ -16,6 +16,7 @@ constexpr size_t kMaxSmem = 227 * 1024;
 
 struct Opts {
     int variant, nb, threads, hold, column_batch, lead_tiles;
+    bool lanes;   // PIPELINE with several lanes per column (its default blocking, few columns)
     long long spin;
 };
 
@@ -31,7 +32,7 @@ constexpr long long kTimeoutNs = 10LL * 1000 * 1000 * 1000;
 // variant requested for unsupported real cases runs as PIPELINE, and for
 // complex data PIPELINE_TC (real only) and an unsupported PIPELINE_TC5 run as
 // WAVEFRONT.
-int resolve(const gb_trans_ev_opts *o, int n, int nbw, int is_complex, Opts *r)
+int resolve(const gb_trans_ev_opts *o, int n, int nbw, int nev, int is_complex, Opts *r)
 {
     int variant = GB_VARIANT_AUTO, nb = 0, threads = 0;
     r->spin = kDefaultSpinPolls;
@@ -66,9 +67,11 @@ int resolve(const gb_trans_ev_opts *o, int n, int nbw, int is_complex, Opts *r)
     }
     if (variant == GB_VARIANT_PIPELINE && !pipe_ok) variant = GB_VARIANT_WAVEFRONT;
     r->variant = variant;
+    r->lanes = variant == GB_VARIANT_PIPELINE && !nb && !threads && !r->lead_tiles && n > 1 && nev > 0 &&
+               gb::pipeline_takes_lanes(n, nbw, nev);
     const bool smem = is_complex || nbw > kMaxRegNbw;
     r->nb = nb ? nb : (smem ? 8 : 16);
-    r->threads = threads ? threads : (variant == GB_VARIANT_PIPELINE || smem ? 64 : 128);
+    r->threads = r->lanes ? 32 : threads ? threads : (variant == GB_VARIANT_PIPELINE || smem ? 64 : 128);
     // the shared-memory kernels take 32 or 64 columns per block and shrink
     // them or the tile depth until the window fits
     if (smem) {
@@ -137,7 +140,7 @@ int gb_max_nbw(void) { return kMaxNbw; }
 size_t gb_trans_ev_workspace_bytes(int n, int nbw, int nev, int is_complex, const gb_trans_ev_opts *opts)
 {
     Opts o;
-    if (n < 1 || nbw < 1 || nev < 0 || resolve(opts, n, nbw, is_complex, &o) != 0) return 0;
+    if (n < 1 || nbw < 1 || nev < 0 || resolve(opts, n, nbw, nev, is_complex, &o) != 0) return 0;
     if (o.variant == GB_VARIANT_PIPELINE_TC && n > 1 && nev > 0) return gb::pipeline_tc_workspace_bytes(n, nbw, nev);
     if (o.variant == GB_VARIANT_PIPELINE_TC5 && n > 1 && nev > 0)
         return gb::pipeline_tc5_workspace_bytes(n, nbw, nev, is_complex);
@@ -153,7 +156,7 @@ int gb_trans_ev_tridi_to_band_d(int n, int nbw, int nev, const double *hh_v, con
     int rc = check_common(n, nbw, nev, hh_v, hh_tau, Z, ldz, sizeof(double));
     if (rc) return rc;
     Opts o;
-    if ((rc = resolve(opts, n, nbw, 0, &o)) != 0) return rc;
+    if ((rc = resolve(opts, n, nbw, nev, 0, &o)) != 0) return rc;
     size_t need = gb_trans_ev_workspace_bytes(n, nbw, nev, 0, opts);
     if (need > 0 && (!workspace || ((uintptr_t)workspace % 256) != 0)) return -8;
     if (ws_bytes < need) return -9;
@@ -166,6 +169,9 @@ int gb_trans_ev_tridi_to_band_d(int n, int nbw, int nev, const double *hh_v, con
     else if (o.variant == GB_VARIANT_PIPELINE_TC)
         e = gb::pipeline_tc_d(n, nbw, nev, hh_v, hh_tau, Z, ldz, o.column_batch, workspace, need, o.spin, kTimeoutNs,
                               o.hold, (cudaStream_t)stream);
+    else if (o.lanes)
+        e = gb::pipeline_lanes_d(n, nbw, nev, hh_v, hh_tau, Z, ldz, o.column_batch, workspace, need, o.spin, kTimeoutNs,
+                                 o.hold, (cudaStream_t)stream);
     else if (o.variant == GB_VARIANT_PIPELINE)
         e = gb::pipeline_d(n, nbw, nev, hh_v, hh_tau, Z, ldz, o.nb, o.threads, o.column_batch, o.lead_tiles, workspace, need,
                            o.spin, kTimeoutNs, o.hold, (cudaStream_t)stream);
@@ -183,7 +189,7 @@ int gb_trans_ev_tridi_to_band_z(int n, int nbw, int nev, const double *hh_v, con
     int rc = check_common(n, nbw, nev, hh_v, hh_tau, Z, ldz, 2 * sizeof(double));
     if (rc) return rc;
     Opts o;
-    if ((rc = resolve(opts, n, nbw, 1, &o)) != 0) return rc;
+    if ((rc = resolve(opts, n, nbw, nev, 1, &o)) != 0) return rc;
     const size_t need = gb_trans_ev_workspace_bytes(n, nbw, nev, 1, opts);
     if (need > 0 && (!workspace || ((uintptr_t)workspace % 256) != 0)) return -8;
     if (ws_bytes < need) return -9;
@@ -215,7 +221,7 @@ int gb_trans_ev_tridi_to_band_d_host(int n, int nbw, int nev, const double *hh_v
     int rc = check_common(n, nbw, nev, hh_v, hh_tau, Z, ldz, sizeof(double));
     if (rc) return rc;
     Opts o;
-    if ((rc = resolve(opts, n, nbw, 0, &o)) != 0) return rc;
+    if ((rc = resolve(opts, n, nbw, nev, 0, &o)) != 0) return rc;
     size_t need = gb_trans_ev_host_buffer_bytes(n, nbw, nev, ldz, 0, opts);
     if (!dev_buf || ((uintptr_t)dev_buf % 256) != 0) return -8;
     if (dev_bytes < need) return -9;
@@ -252,14 +258,14 @@ int gb_trans_ev_query(const void *workspace, size_t ws_bytes, void *stream)
 int gb_trans_ev_variant(int n, int nbw, int nev, int is_complex, const gb_trans_ev_opts *opts)
 {
     Opts o;
-    if (n < 1 || nbw < 1 || nbw > kMaxNbw || nev < 0 || resolve(opts, n, nbw, is_complex, &o) != 0) return -1;
+    if (n < 1 || nbw < 1 || nbw > kMaxNbw || nev < 0 || resolve(opts, n, nbw, nev, is_complex, &o) != 0) return -1;
     return o.variant;
 }
 
 long long gb_trans_ev_launch_count(int n, int nbw, int nev, int is_complex, const gb_trans_ev_opts *opts)
 {
     Opts o;
-    if (n < 1 || nbw < 1 || nbw > kMaxNbw || nev < 0 || resolve(opts, n, nbw, is_complex, &o) != 0) return -1;
+    if (n < 1 || nbw < 1 || nbw > kMaxNbw || nev < 0 || resolve(opts, n, nbw, nev, is_complex, &o) != 0) return -1;
     if (n == 1 || nev == 0) return 0;
     if (o.variant == GB_VARIANT_PIPELINE) return 1;
     if (o.variant == GB_VARIANT_PIPELINE_TC || o.variant == GB_VARIANT_PIPELINE_TC5)
