@@ -13,30 +13,38 @@
 // The working matrix is kept in lower band storage of width 2b (entries up
 // to 2b-1 below the diagonal, where the bulges live), in a workspace.
 //
-// What bounds it: the chain of sweeps.  O(s,k) needs O(s-1,k), D(s-1,k) and,
-// for its last entry only, the beta of H(s-1,k+1); D(s,k) needs D(s-1,k),
-// O(s-1,k+1) and the first entry of D(s-1,k+1).  So sweep s trails sweep s-1
-// by one O step and the generation of the next reflector, and the stage
-// takes n times that.  One SM issues two FP64 multiply-adds per clock, so a
-// step's 12 b^2 flops of arithmetic per flop pair cost several microseconds
-// on one SM; a sweep therefore runs on a cluster of C + CD blocks:
+// What bounds it: the chain of sweeps.  O(s,k) shares all but its last column
+// with O(s-1,k); the last column is the first of D(s-1,k), and its last entry
+// the beta of H(s-1,k+1).  D(s,k) shares all but its last row with D(s-1,k); that
+// row is the first of O(s-1,k+1) and, on the diagonal, the first entry of
+// D(s-1,k+1).  So sweep s trails sweep s-1 by one O step and one hop of those few
+// entries, and the stage takes n times that.  One SM issues two FP64
+// multiply-adds per clock, so a step's arithmetic (4 b^2 multiply-adds in O, 2 b^2
+// and more in D) costs several microseconds on one SM; a sweep therefore runs
+// on a cluster of C + CD blocks:
 //   * ranks 0 .. C-1 hold b/C rows of O each.  The right product is local to
 //     a row; the column sums x^T A (x the raw source column, A's own first
-//     column giving x^T x) are exchanged once per step through distributed
-//     shared memory, and every rank derives tau, the scale and v from them:
-//     v^T a_j = a_0j + scale * sum_{i>0} x_i a_ij;
+//     column giving x^T x) are exchanged once per step as asynchronous stores
+//     into the peers' shared memory that count on their mbarriers, and every
+//     rank derives tau, the scale and v from them: v^T a_j = a_0j + scale *
+//     sum_{i>0} x_i a_ij.  128 threads keep this chain; another 128 take the
+//     left product and the stores, while the chain is at the next block;
 //   * ranks C .. C+CD-1 receive x as well and update D (rows dealt round
-//     robin); with CD = 2 they exchange their parts of D v.
-// Each block has 256 computing threads, four loader warps that wait for the
-// flags of sweep s-1 and stage the next block in shared memory while the
-// current one is worked on, and one publisher warp that makes the stores
-// visible and raises this sweep's flags, so that neither the loads nor the
-// fences sit on the chain.
+//     robin), D x before the reflector's scalars are known; with CD = 2 they
+//     exchange their parts of D v.
+// Each block also has four loader warps, which wait for the flags of sweep s-1
+// and stage the next block in shared memory while the current one is worked on,
+// and one publisher warp, which raises this sweep's flags.  The few entries on
+// the chain (betas, first columns of D) skip the flags: they pass through slots
+// in global memory that say themselves whether they are full.
 //
-// Measured on a GB300 (whole stage, before: one block of 256 threads per
-// sweep with a lag of three tasks; now): real n = 512, nbw = 32: 15.1 -> 4.2 ms;
-// nbw = 64: n = 2048 82 -> 23.5, 8192 339 -> 119, 16384 684 -> 348; complex
-// n = 512, nbw = 32: 46 -> 6.9; nbw = 64: n = 2048 322 -> 50, 8192 1351 -> 325.
+// Measured on a GB300 (whole stage; before: one block of 256 threads per sweep
+// with a lag of three tasks; then: clusters with every block behind flags; now):
+// real n = 512, nbw = 32: 15.1, 4.2, 3.3 ms; nbw = 64: n = 2048 82, 23.5, 17.9;
+// 8192 339, 119, 99; 16384 684, 348, 292; complex n = 512, nbw = 32: 46, 6.9,
+// 6.9; nbw = 64: n = 2048 322, 50, 39; 8192 1351, 325, 310.  At n = 2048 an O
+// step's chain is 3.3 us (2.0 from the block's arrival to the exchanged sums, 1.2
+// for the reflector and v), a hop 3.4 us and the lag 8.6 us: jitter adds to both.
 //
 // Sweeps are taken by ticket in increasing s by a persistent grid of
 // clusters, so every wait targets a smaller ticket, which a resident cluster
@@ -61,9 +69,15 @@ namespace cg = cooperative_groups;
 namespace {
 
 constexpr int kMain = 256;       // computing threads of a block
+constexpr int kChain = 128;      // O blocks: threads 0 .. 127 keep the chain, 128 .. 255 finish the blocks
 constexpr int kLoaders = 128;    // threads 256 .. 383
 constexpr int kChaseThreads = kMain + kLoaders + 32;  // and the publisher warp
-constexpr int kFlags = 4;        // ints per sweep: reflectors generated, O parts done, D parts done, unused
+constexpr int kFlags = 8;        // ints per sweep: the steps each block of its cluster has stored (one 32-byte sector)
+// The few entries that two sweeps meet at, the betas and the first columns of
+// the D blocks, pass from a sweep to the next through slots that say themselves
+// whether they are full (this signalling NaN is no result of arithmetic), so
+// that no fence, flag or second load stands between a value and its reader.
+constexpr unsigned long long kEmpty = 0x7ff4c0de00be7a00ull;
 
 __device__ __forceinline__ int ld_acq(const int *p)
 {
@@ -72,20 +86,43 @@ __device__ __forceinline__ int ld_acq(const int *p)
     return v;
 }
 
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_relaxed(unsigned long long *p, unsigned long long v)
+{
+    asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
 __device__ __forceinline__ void st_rel(int *p, int v)
 {
     asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-__device__ __forceinline__ void red_rel(int *p, int v)
-{
-    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ void main_sync()
+__device__ __forceinline__ void main_sync()   // the computing threads of a D block
 {
     __syncwarp();
     asm volatile("bar.sync 1, 256;" ::: "memory");
+}
+__device__ __forceinline__ void chain_sync()  // the chain's threads of an O block
+{
+    __syncwarp();
+    asm volatile("bar.sync 3, 128;" ::: "memory");
+}
+// D blocks: the publisher warp hands the reflector's scalars to the others
+__device__ __forceinline__ void scalars_give()
+{
+    __syncwarp();
+    asm volatile("bar.arrive 4, 288;" ::: "memory");
+}
+__device__ __forceinline__ void scalars_take()
+{
+    __syncwarp();
+    asm volatile("bar.sync 4, 288;" ::: "memory");
 }
 __device__ __forceinline__ void loader_sync()
 {
@@ -104,14 +141,18 @@ struct ChaseState {
     int error;
 };
 
-// One problem of a batched chase: its working band and reflector arrays and
-// its progress flags (kFlags ints per sweep).
+// One problem of a batched chase: its working band and reflector arrays, its
+// progress flags (kFlags ints per sweep) and its slots, for odd and for even
+// sweeps: a beta per step, and b entries per step for the first column of D.  A
+// slot is emptied by its reader, sweep s+1, before its next writer, sweep s+2,
+// can be there.
 struct ChaseProblem {
     int n, b;
     void *W;
     long long ldw;
     void *hh_v, *hh_tau;
     int *progress;
+    unsigned long long *betas, *firsts;
 };
 
 // Lower band storage of width 2b: A(i,j), i >= j, at W[(i-j) + j*ldw];
@@ -133,28 +174,32 @@ struct ChaseGeo {
     static constexpr int LD = BM + 4;             // entries per staged row
     static constexpr int NO = 2;                  // staged O blocks
     static constexpr int ND = sizeof(T) == 16 ? 1 : 2;  // staged D blocks
-    static constexpr int TPR = kMain / RW;        // threads per O row (right product)
-    static constexpr int TPC = kMain / BM;        // threads per O column (left product)
+    static constexpr int TPR = kChain / RW;       // threads per O row (right product)
+    static constexpr int TPC = kChain / BM;       // threads per O column (column sums, left product)
     static constexpr int TPD = kMain / RD;        // threads per D row
     static constexpr int NG = BM / 16;            // 16-row groups of the column sums
     static constexpr int NGR = RW / 16;           // of a rank
     static constexpr int OBUF = RW * LD, DBUF = RD * LD;
     static constexpr size_t STAGE = sizeof(T) * (size_t)(NO * OBUF > ND * DBUF ? NO * OBUF : ND * DBUF);
-    static_assert(TPR >= 1 && TPR <= 32 && TPC >= 1 && TPC <= 8 && TPR <= 16 && TPD <= 16, "threads of a row or column share a warp");
-    static_assert(S <= 8 && RW * S <= kMain && BM <= 64, "cluster and mailbox sizes");
+    // bytes of a step's messages: column sums, row 0 and the source column to
+    // an O rank; the source column, its own sums and its first entry to a D rank
+    static constexpr uint32_t O_BYTES = (uint32_t)sizeof(T) * (NG * BM + 2 * BM);
+    static constexpr uint32_t D_BYTES = (uint32_t)sizeof(T) * (BM + NG + 1);
+    static constexpr uint32_t P_BYTES = (uint32_t)sizeof(T) * BM;
+    static_assert(TPR >= 1 && TPC >= 1 && TPC <= 8 && TPR <= 16 && TPD <= 16, "threads of a row or column share a warp");
+    static_assert(S <= kFlags && RW * S <= kChain && BM <= 64 && RW % 16 == 0, "cluster and mailbox sizes");
 };
 
 template <class T, int BM, int C>
 struct ChaseShared {
-    T mx[2][BM];        // mailbox: the source column x
+    T mx[2][BM];            // mailbox: the source column x
     T ms[2][BM / 16][BM];   // partial column sums sum_{i>0} conj(x_i) a_ij by 16-row group
-    T ma[2][BM];        // row 0 of the block
-    T mp[2][BM];        // tau D v (D ranks)
-    T v[2][BM];         // v(s,k) by step parity
-    T w[BM], sum[BM], q[BM];
-    T tau, scal, kk;
-    double beta[2];
-    unsigned long long full[2], empty[2], xo[2], xd, gen[2], st[2];
+    T ma[2][BM];            // row 0 of the block
+    T mp[2][BM];            // tau D v (D ranks)
+    T v[2][BM], w[2][BM];   // v(s,k) and conj(tau) v^H A by step parity
+    T tau[2], scal[2];
+    T sum[BM], q[BM], kk;
+    unsigned long long full[2], empty[2], xo[2], xd[2], vw[2], st[2];
     int sweep[2], abort;
 };
 
@@ -186,24 +231,85 @@ __device__ __forceinline__ void chase_wait(void *bar, uint32_t parity, long long
     chase_give_up(state, abort);
 }
 
-// one loader thread: wait until a flag of sweep s-1 reaches `need`
-__device__ __forceinline__ void chase_flag(const int *flag, int need, long long timeout_ns, ChaseState *state,
-                                           int *abort)
+// A loader warp waits until every block of sweep s-1 has stored its part (lane
+// r looks at block r's flag: need_o steps of the O blocks, need_d of the D
+// blocks).  One flag per block: blocks may be two steps apart, so a sum
+// over them would not say that each is there.
+template <int C, int CD>
+__device__ __forceinline__ void chase_flags(const int *prev, int need_o, int need_d, long long timeout_ns,
+                                            ChaseState *state, int *abort)
 {
-    if (ld_acq(flag) >= need) return;
+    const int lane = threadIdx.x & 31;
+    const int need = lane < C ? need_o : lane < C + CD ? need_d : 0;
+    auto there = [&]() { return __all_sync(0xffffffffu, need == 0 || ld_acq(prev + lane) >= need); };
+    if (there()) return;
     const unsigned long long t0 = now_ns();
     for (long long i = 1;; i++) {
-        if (ld_acq(flag) >= need) return;
+        if (there()) return;
         if ((i & 15) == 0) {
-            if (*(volatile int *)&state->abort) break;
-            if ((long long)(now_ns() - t0) > timeout_ns) {
-                chase_give_up(state, abort);
-                return;
+            const bool stop = *(volatile int *)&state->abort != 0;
+            const bool late = (long long)(now_ns() - t0) > timeout_ns;
+            if (__any_sync(0xffffffffu, late)) {
+                if (lane == 0) chase_give_up(state, abort);
+                break;
             }
-            __nanosleep(20);
+            if (__any_sync(0xffffffffu, stop)) break;
         }
     }
     *(volatile int *)abort = 1;
+}
+
+// one loader thread: the value in `slot`, which is emptied
+__device__ __forceinline__ double take(unsigned long long *slot, long long timeout_ns, ChaseState *state, int *abort)
+{
+    unsigned long long v = ld_relaxed(slot);
+    if (v == kEmpty) {
+        const unsigned long long t0 = now_ns();
+        for (long long i = 1; (v = ld_relaxed(slot)) == kEmpty; i++) {
+            if ((i & 15) == 0) {
+                if (*(volatile int *)&state->abort) break;
+                if ((long long)(now_ns() - t0) > timeout_ns) {
+                    chase_give_up(state, abort);
+                    break;
+                }
+            }
+        }
+        if (v == kEmpty) {
+            *(volatile int *)abort = 1;
+            return 0.0;
+        }
+    }
+    st_relaxed(slot, kEmpty);
+    return __longlong_as_double((long long)v);
+}
+__device__ __forceinline__ void take_entry(double &x, unsigned long long *slots, int i, long long timeout_ns,
+                                           ChaseState *state, int *abort)
+{
+    x = take(slots + i, timeout_ns, state, abort);
+}
+__device__ __forceinline__ void take_entry(Zc &x, unsigned long long *slots, int i, long long timeout_ns,
+                                           ChaseState *state, int *abort)
+{
+    x.re = take(slots + 2 * i, timeout_ns, state, abort);
+    x.im = take(slots + 2 * i + 1, timeout_ns, state, abort);
+}
+__device__ __forceinline__ void put_entry(unsigned long long *slots, int i, double x)
+{
+    st_relaxed(slots + i, (unsigned long long)__double_as_longlong(x));
+}
+__device__ __forceinline__ void put_entry(unsigned long long *slots, int i, Zc x)
+{
+    put_entry(slots, 2 * i, x.re);
+    put_entry(slots, 2 * i + 1, x.im);
+}
+
+// |x|^2 below the source column's first entry, from its sums over groups
+template <int NG, class T>
+__device__ __forceinline__ double group_sum(const T *ms, int stride)
+{
+    double t = re_of(ms[0]) + re_of(ms[stride]);
+    if (NG == 4) t += re_of(ms[2 * stride]) + re_of(ms[3 * stride]);
+    return t;
 }
 
 // ---- a cluster: sweeps by ticket --------------------------------------------
@@ -217,7 +323,7 @@ struct ChaseWork {
 };
 
 template <class T, int BM, int C, int CD>
-__global__ void __launch_bounds__(kChaseThreads, 1)
+__global__ void __launch_bounds__(kChaseThreads, sizeof(T) == 16 ? 1 : 2)
 chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
 {
     using G = ChaseGeo<T, BM, C, CD>;
@@ -237,13 +343,13 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
     if (tid == 0) {
         sm.abort = 0;
         for (int i = 0; i < 2; i++) {
-            tc5::mbar_init(tc5::smem_addr(&sm.full[i]), kLoaders);
-            tc5::mbar_init(tc5::smem_addr(&sm.empty[i]), kMain + 1);
-            tc5::mbar_init(tc5::smem_addr(&sm.xo[i]), is_o ? C + CD : C);
-            tc5::mbar_init(tc5::smem_addr(&sm.gen[i]), 1);
-            tc5::mbar_init(tc5::smem_addr(&sm.st[i]), kMain);
+            tc5::mbar_init(tc5::smem_addr(&sm.full[i]), kLoaders / 32);
+            tc5::mbar_init(tc5::smem_addr(&sm.empty[i]), (is_o ? kChain : kMain) / 32 + 1);
+            tc5::mbar_init(tc5::smem_addr(&sm.xo[i]), is_o ? 1 + CD : 1);
+            tc5::mbar_init(tc5::smem_addr(&sm.xd[i]), 1);
+            tc5::mbar_init(tc5::smem_addr(&sm.vw[i]), 1);
+            tc5::mbar_init(tc5::smem_addr(&sm.st[i]), (is_o ? kChain : kMain) / 32);
         }
-        tc5::mbar_init(tc5::smem_addr(&sm.xd), CD);
         tc5::mbar_init_fence();
     }
     cluster.sync();
@@ -273,19 +379,22 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
         const long long first = sweep_first(n, b, s);
         int *mine = pr.progress + (size_t)kFlags * (s - 1);
         const int *prev = mine - kFlags;
+        const int nk1 = sweep_count(n, b, 1);
+        unsigned long long *betas = pr.betas + (size_t)(s & 1) * nk1, *betas_prev = pr.betas + (size_t)(~s & 1) * nk1;
+        constexpr int words = sizeof(T) / 8;
+        unsigned long long *firsts = pr.firsts + (size_t)(s & 1) * nk1 * b * words;
+        unsigned long long *firsts_prev = pr.firsts + (size_t)(~s & 1) * nk1 * b * words;
 
-        if (tid < kMain && is_o) {
-            // ================= O: right product, reflector, left product
+        if (is_o && tid < kChain) {
+            // ================= O, the chain: right product, column sums, reflector
             const int i0 = rank * RW;
             bool active = false;                      // H(s,k-1) is not the identity
             T ptau;
             zero_of(ptau);
             for (int k = 0; k < nk; k++, kk++) {
-                const int r = s + k * b, len = min(b, n - r);
-                const int c = (k == 0) ? s - 1 : r - b;
-                const int ncols = (k == 0) ? 1 : b;
                 const int par = kk & 1;
                 T *B = stage + (kk % G::NO) * G::OBUF;
+                if (tid == 0) mbar_expect(&sm.xo[par], G::O_BYTES);
                 chase_wait(&sm.full[kk % G::NO], (kk / G::NO) & 1, wait_ns, state, &sm.abort);
                 if (active) {
                     const int row = tid / G::TPR, part = tid % G::TPR;
@@ -304,153 +413,174 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                     for (int u = 0; u < BM / G::TPR; u++)
                         B[row * LD + part + G::TPR * u] = nmad(y, conj_of(vp[part + G::TPR * u]), e[u]);
                 }
-                main_sync();
-                // column sums with the raw source column (the block's first)
+                chain_sync();
+                // the source column (the block's first) and row 0 as they are
+                // now, then the column sums with the raw source column
+                if (tid < RW * G::S)
+                    send(&sm.mx[par][i0 + tid % RW], B[(tid % RW) * LD], &sm.xo[par], tid / RW);
                 const int col = tid / G::TPC, cp = tid % G::TPC;
-                T e[RW / G::TPC];
-                {
-                    constexpr int NE = 16 / G::TPC, NA = 8 / G::TPC;
-#pragma unroll
-                    for (int g = 0; g < G::NGR; g++) {
-                        T acc[NA];
-#pragma unroll
-                        for (int u = 0; u < NA; u++) zero_of(acc[u]);
-#pragma unroll
-                        for (int u = 0; u < NE; u++) {
-                            const int i = 16 * g + cp + G::TPC * u;
-                            e[g * NE + u] = B[i * LD + col];
-                            if (i0 + i > 0) acc[u % NA] = madc(B[i * LD], e[g * NE + u], acc[u % NA]);
-                        }
-                        const T sum = tree_sum<8, G::TPC>(acc);
-                        T *to = &sm.ms[par][rank * G::NGR + g][col];
-                        for (int d = cp; d < C; d += G::TPC) cluster.map_shared_rank(to, d)[0] = sum;
-                        if (col == 0 && cp < CD) cluster.map_shared_rank(to, C + cp)[0] = sum;
-                    }
-                    if (rank == 0) {
-                        const T a0 = B[col];
-                        for (int d = cp; d < C; d += G::TPC) cluster.map_shared_rank(&sm.ma[par][col], d)[0] = a0;
-                        if (col == 0 && cp < CD) cluster.map_shared_rank(&sm.ma[par][0], C + cp)[0] = a0;
-                    }
-                    if (tid < RW * G::S)
-                        cluster.map_shared_rank(&sm.mx[par][i0 + tid % RW], tid / RW)[0] = B[(tid % RW) * LD];
+                if (rank == 0) {
+                    const T a0 = B[col];
+                    for (int d = cp; d < C; d += G::TPC) send(&sm.ma[par][col], a0, &sm.xo[par], d);
+                    if (col == 0)
+                        for (int d = cp; d < CD; d += G::TPC) send(&sm.ma[par][0], a0, &sm.xo[par], C + d);
                 }
-                main_sync();
-                if (tid < G::S) {
-                    asm volatile("fence.acq_rel.cluster;" ::: "memory");
-                    mbar_arrive_remote(&sm.xo[par], tid);
+                constexpr int NE = 16 / G::TPC, NB8 = 8 / G::TPC;
+#pragma unroll
+                for (int g = 0; g < G::NGR; g++) {
+                    T acc[NB8];
+#pragma unroll
+                    for (int u = 0; u < NB8; u++) zero_of(acc[u]);
+#pragma unroll
+                    for (int u = 0; u < NE; u++) {
+                        const int i = 16 * g + cp + G::TPC * u;
+                        if (i0 + i > 0) acc[u % NB8] = madc(B[i * LD], B[i * LD + col], acc[u % NB8]);
+                    }
+                    const T sum = tree_sum<8, G::TPC>(acc);
+                    T *to = &sm.ms[par][rank * G::NGR + g][col];
+                    for (int d = cp; d < C; d += G::TPC) send(to, sum, &sm.xo[par], d);
+                    if (col == 0)
+                        for (int d = cp; d < CD; d += G::TPC) send(to, sum, &sm.xo[par], C + d);
                 }
                 chase_wait(&sm.xo[par], (kk >> 1) & 1, wait_ns, state, &sm.abort);
-                // every rank: the reflector, and the sums over ranks
+                // every rank: the reflector, and the sums over groups
                 if (warp == 0) {
-                    double ss = 0.0;
-                    for (int q = 0; q < G::NG; q++) ss += re_of(sm.ms[par][q][0]);
-                    const auto h = reflector(sm.ma[par][0], ss);
+                    const auto h = reflector(sm.ma[par][0], group_sum<G::NG>(&sm.ms[par][0][0], BM));
                     if (lane == 0) {
-                        sm.tau = h.tau;
-                        sm.scal = h.scal;
-                        sm.beta[par] = h.beta;
-                        mbar_arrive(&sm.gen[par]);
+                        sm.tau[par] = h.tau;
+                        sm.scal[par] = h.scal;
+                        // beta: final where k = 0 (the subdiagonal of T), else on
+                        // to the next sweep, whose last entry of O(s+1,k-1) it is
+                        if (rank == 0) {
+                            if (k > 0) {
+                                st_relaxed(betas + k, (unsigned long long)__double_as_longlong(h.beta));
+                            } else {
+                                T z;
+                                zero_of(z);
+                                *(double *)&z = h.beta;
+                                *A.at(s, s - 1) = z;
+                            }
+                        }
                     }
-                } else if (tid >= 64 && tid < 64 + BM) {
-                    T t2;
-                    zero_of(t2);
-                    for (int q = 0; q < G::NG; q++) t2 = add(t2, sm.ms[par][q][tid - 64]);
-                    sm.sum[tid - 64] = t2;
+                } else if (tid < 32 + BM) {
+                    const int j = tid - 32;
+                    T t2 = sm.ms[par][0][j];
+                    for (int q = 1; q < G::NG; q++) t2 = add(t2, sm.ms[par][q][j]);
+                    sm.sum[j] = t2;
                 }
-                main_sync();
-                const T tau = sm.tau, scal = sm.scal;
+                chain_sync();
+                const T tau = sm.tau[par], scal = sm.scal[par];
                 if (tid < BM) {
                     T vi;
                     if (tid == 0) one_of(vi);
                     else vi = mul(sm.mx[par][tid], scal);   // scal = 0 where tau = 0; x = 0 past len
                     sm.v[par][tid] = vi;
-                } else if (tid >= 128 && tid < 128 + BM) {
+                } else if (tid >= 64 && tid < 64 + BM) {
                     // w_j = conj(tau) v^H a_j
-                    const int j = tid - 128;
-                    sm.w[j] = mul(conj_of(tau), mad(conj_of(scal), sm.sum[j], sm.ma[par][j]));
+                    const int j = tid - 64;
+                    sm.w[par][j] = mul(conj_of(tau), mad(conj_of(scal), sm.sum[j], sm.ma[par][j]));
                 }
-                main_sync();
-                const bool act = !is_zero(tau);
-                {
-                    const T wj = sm.w[col];
-                    if (col < ncols) {
+                chain_sync();
+                if (tid == 0) mbar_arrive(&sm.vw[par]);
+                active = !is_zero(tau);
+                ptau = tau;
+            }
+        } else if (is_o && tid < kMain) {
+            // ================= O, the finish: left product and stores, while
+            // the chain is at the next block
+            const int i0 = rank * RW, ft = tid - kChain;
+            const int col = ft / G::TPC, cp = ft % G::TPC;
+            for (int k = 0; k < nk; k++, kk++) {
+                const int r = s + k * b, len = min(b, n - r);
+                const int c = (k == 0) ? s - 1 : r - b;
+                const int ncols = (k == 0) ? 1 : b;
+                const int par = kk & 1;
+                const T *B = stage + (kk % G::NO) * G::OBUF;
+                chase_wait(&sm.vw[par], (kk >> 1) & 1, wait_ns, state, &sm.abort);
+                const bool act = !is_zero(sm.tau[par]);
+                if (col < ncols) {
+                    const T wj = sm.w[par][col];
 #pragma unroll
-                        for (int u = 0; u < RW / G::TPC; u++) {
-                            const int gi = i0 + cp + G::TPC * u;   // e[u]'s row: the groups follow each other
-                            if (gi < len) {
-                                if (col > 0) {
-                                    *A.at(r + gi, c + col) = act ? nmad(sm.v[par][gi], wj, e[u]) : e[u];
-                                } else if (gi > 0) {     // the annihilated column (its beta: the publisher)
-                                    T z;
-                                    zero_of(z);
-                                    *A.at(r + gi, c) = act ? z : e[u];
-                                }
+                    for (int u = 0; u < RW / G::TPC; u++) {
+                        const int i = cp + G::TPC * u, gi = i0 + i;
+                        if (gi < len) {
+                            const T e = B[i * LD + col];
+                            if (col > 0) {
+                                *A.at(r + gi, c + col) = act ? nmad(sm.v[par][gi], wj, e) : e;
+                            } else if (gi > 0) {     // the annihilated column (its beta went its own way)
+                                T z;
+                                zero_of(z);
+                                *A.at(r + gi, c) = act ? z : e;
                             }
                         }
                     }
                 }
-                mbar_arrive(&sm.st[par]);
-                mbar_arrive(&sm.empty[kk % G::NO]);
-                active = act;
-                ptau = tau;
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&sm.st[par]);
+                    mbar_arrive(&sm.empty[kk % G::NO]);
+                }
             }
         } else if (tid < kMain) {
             // ================= D: symmetric two-sided update
             const int dr = rank - C;
+            const int rr = tid / G::TPD, part = tid % G::TPD;
+            const int i = dr + CD * rr;                     // this thread's row of D
+            // entry i of the first column: row 0 is the last entry of D(s+1,k-1),
+            // the others the last column of O(s+1,k); D(s,0)'s first entry is final
+            auto to_next = [&](int row, int k, T x) {
+                if (row > 0 || k > 0) put_entry(firsts + (size_t)k * b * words, row, x);
+                else *A.at(s, s) = x;
+            };
             for (int k = 0; k < nk; k++, kk++) {
                 const int r = s + k * b, len = min(b, n - r);
                 const int par = kk & 1;
                 const long long idx = first + k;
+                const T *B = stage + (kk % G::ND) * G::DBUF;
+                if (tid == 0) mbar_expect(&sm.xo[par], G::D_BYTES);
+                chase_wait(&sm.full[kk % G::ND], (kk / G::ND) & 1, wait_ns, state, &sm.abort);
                 chase_wait(&sm.xo[par], (kk >> 1) & 1, wait_ns, state, &sm.abort);
-                if (warp == 0) {
-                    double ss = 0.0;
-                    for (int q = 0; q < G::NG; q++) ss += re_of(sm.ms[par][q][0]);
-                    const auto h = reflector(sm.ma[par][0], ss);
-                    if (lane == 0) {
-                        sm.tau = h.tau;
-                        sm.scal = h.scal;
-                    }
+                // D x over x's entries past the first, while the publisher warp
+                // has the reflector's scalars: D v = D e_0 + scale D x
+                constexpr int NA = 16 / G::TPD;
+                T e[BM / G::TPD], acc[NA];
+#pragma unroll
+                for (int u = 0; u < NA; u++) zero_of(acc[u]);
+#pragma unroll
+                for (int u = 0; u < BM / G::TPD; u++) {
+                    const int j = part + G::TPD * u;
+                    e[u] = B[rr * LD + j];
+                    if (j > 0) acc[u % NA] = mad(e[u], sm.mx[par][j], acc[u % NA]);
                 }
-                main_sync();
-                const T tau = sm.tau;
+                const T dx = tree_sum<16, G::TPD>(acc);
+                scalars_take();
+                const T tau = sm.tau[par], scal = sm.scal[par];
+                const bool act = !is_zero(tau);
                 if (tid < BM) {
                     T vi;
                     if (tid == 0) one_of(vi);
-                    else vi = mul(sm.mx[par][tid], sm.scal);
+                    else vi = mul(sm.mx[par][tid], scal);
                     sm.v[0][tid] = vi;
                     if (dr == 0 && tid < b) ((T *)pr.hh_v)[idx * b + tid] = vi;
                 }
                 if (dr == 0 && tid == 64) ((T *)pr.hh_tau)[idx] = tau;
+                const int pp = nxd & 1;
+                if (act) {
+                    if (CD > 1 && tid == 0) mbar_expect(&sm.xd[pp], G::P_BYTES);
+                    const T pi = mul(tau, mad(scal, dx, B[rr * LD]));
+                    if (CD == 1) {
+                        if (part == 0) sm.mp[pp][i] = pi;
+                    } else if (part < CD) {
+                        send(&sm.mp[pp][i], pi, &sm.xd[pp], C + part);
+                    }
+                }
                 main_sync();
                 // the mailbox is consumed: credit for the O ranks' next step
                 if (tid < C) mbar_arrive_remote(&sm.xo[par ^ 1], tid);
-                T *B = stage + (kk % G::ND) * G::DBUF;
-                chase_wait(&sm.full[kk % G::ND], (kk / G::ND) & 1, wait_ns, state, &sm.abort);
-                if (!is_zero(tau)) {
-                    const int rr = tid / G::TPD, part = tid % G::TPD;
-                    const int i = dr + CD * rr;                     // this thread's row of D
-                    const T *v = sm.v[0];
-                    const int pp = nxd & 1;
-                    constexpr int NA = 16 / G::TPD;
-                    T e[BM / G::TPD], acc[NA];
-#pragma unroll
-                    for (int u = 0; u < NA; u++) zero_of(acc[u]);
-#pragma unroll
-                    for (int u = 0; u < BM / G::TPD; u++) {
-                        e[u] = B[rr * LD + part + G::TPD * u];
-                        acc[u % NA] = mad(e[u], v[part + G::TPD * u], acc[u % NA]);
-                    }
-                    const T pi = mul(tau, tree_sum<16, G::TPD>(acc));
-                    if (part < CD) cluster.map_shared_rank(&sm.mp[pp][i], C + part)[0] = pi;
-                    main_sync();
-                    if (CD > 1) {
-                        if (tid < CD) {
-                            asm volatile("fence.acq_rel.cluster;" ::: "memory");
-                            mbar_arrive_remote(&sm.xd, C + tid);
-                        }
-                        chase_wait(&sm.xd, nxd & 1, wait_ns, state, &sm.abort);
-                    }
+                if (act) {
+                    if (CD > 1) chase_wait(&sm.xd[pp], (nxd >> 1) & 1, wait_ns, state, &sm.abort);
                     nxd++;
+                    const T *v = sm.v[0];
                     // K = conj(tau)/2 v^H p, q = p - K v
                     if (warp == 0) {
                         T a[1];
@@ -466,12 +596,23 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
 #pragma unroll
                     for (int u = 0; u < BM / G::TPD; u++) {
                         const int j = part + G::TPD * u;
-                        if (j <= i && i < len)
-                            *A.at(r + i, r + j) = nmad(vi, conj_of(sm.q[j]), nmad(qi, conj_of(v[j]), e[u]));
+                        if (j <= i) e[u] = nmad(vi, conj_of(sm.q[j]), nmad(qi, conj_of(v[j]), e[u]));
+                        if (u == 0 && part == 0 && i < len) to_next(i, k, e[0]);
                     }
+                    if (i < len)
+#pragma unroll
+                        for (int u = 0; u < BM / G::TPD; u++) {
+                            const int j = part + G::TPD * u;
+                            if (j > 0 && j <= i) *A.at(r + i, r + j) = e[u];
+                        }
+                } else if (part == 0 && i < len) {
+                    to_next(i, k, e[0]);
                 }
-                mbar_arrive(&sm.st[par]);
-                mbar_arrive(&sm.empty[kk % G::ND]);
+                __syncwarp();
+                if (lane == 0) {
+                    mbar_arrive(&sm.st[par]);
+                    mbar_arrive(&sm.empty[kk % G::ND]);
+                }
             }
         } else if (tid < kMain + kLoaders) {
             // ================= loaders: stage the next block
@@ -481,11 +622,11 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                 T *B = stage + (kk % nbuf) * bufsz;
                 if (kk >= (uint32_t)nbuf)
                     chase_wait(&sm.empty[kk % nbuf], (kk / nbuf - 1) & 1, wait_ns, state, &sm.abort);
-                const int upto = is_o ? min(k + 1, nkp) : min(k + 2, nkp);
-                if (lt == 0 && s > 1 && !*(volatile int *)&sm.abort) {
-                    chase_flag(prev + 1, C * upto, timeout_ns, state, &sm.abort);
-                    chase_flag(prev + 2, CD * upto, timeout_ns, state, &sm.abort);
-                }
+                // O(s,k): O(s-1,k), whose successor shares all but the last column
+                // and row; D(s,k): D(s-1,k), and the first row of O(s-1,k+1)
+                if (lt < 32 && s > 1 && !__any_sync(0xffffffffu, *(volatile int *)&sm.abort))
+                    chase_flags<C, CD>(prev, min(is_o ? k + 1 : k + 2, nkp), is_o ? 0 : min(k + 1, nkp), timeout_ns, state,
+                                       &sm.abort);
                 loader_sync();
                 if (is_o) {
                     const int i0 = rank * RW;
@@ -500,8 +641,8 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                         for (int u = 0; u < CH; u++) {
                             const int e = lt + kLoaders * (u0 + u), col = e / RW, i = e % RW;
                             zero_of(x[u]);
-                            const bool corner = col == ncols - 1 && i0 + i == b - 1;   // beta of H(s-1,k+1): below
-                            if (col < ncols && i0 + i < len && !corner) x[u] = ld_cg(A.at(r + i0 + i, c + col));
+                            // (the last column follows below)
+                            if (col < ncols - (s > 1 ? 1 : 0) && i0 + i < len) x[u] = ld_cg(A.at(r + i0 + i, c + col));
                         }
 #pragma unroll
                         for (int u = 0; u < CH; u++) {
@@ -509,13 +650,18 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                             B[i * LD + col] = x[u];
                         }
                     }
-                    const int ci = b - 1 - i0;
-                    if (len == b && ci >= 0 && ci < RW) {
+                    // the last column: the first column of D(s-1,k) from its
+                    // second entry on, and the beta of H(s-1,k+1)
+                    if (s > 1) {
                         loader_sync();
-                        if (lt == 0) {
-                            if (s > 1 && !*(volatile int *)&sm.abort)
-                                chase_flag(prev, min(k + 2, nkp), timeout_ns, state, &sm.abort);
-                            B[ci * LD + ncols - 1] = ld_cg(A.at(r + b - 1, c + ncols - 1));
+                        if (lt < RW && i0 + lt < len && !*(volatile int *)&sm.abort) {
+                            T x;
+                            zero_of(x);
+                            if (i0 + lt == b - 1)
+                                *(double *)&x = take(betas_prev + k + 1, timeout_ns, state, &sm.abort);
+                            else
+                                take_entry(x, firsts_prev + (size_t)k * b * words, i0 + lt + 1, timeout_ns, state, &sm.abort);
+                            B[lt * LD + ncols - 1] = x;
                         }
                     }
                 } else {
@@ -531,7 +677,8 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                             const int q = e / (BM + 1), t2 = q + e % (BM + 1);   // row of column q, or past its end
                             const int j = t2 < BM ? q : BM - 1 - q, i = t2 < BM ? t2 : t2 - BM + j;
                             zero_of(x[u]);
-                            if (e < N2 && i < len) x[u] = ld_cg(A.at(r + i, r + j));   // j <= i
+                            const bool corner = s > 1 && j == b - 1;   // D(s-1,k+1)'s first entry: below
+                            if (e < N2 && i < len && !corner) x[u] = ld_cg(A.at(r + i, r + j));   // j <= i
                         }
 #pragma unroll
                         for (int u = 0; u < CH; u++) {
@@ -544,33 +691,41 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                             }
                         }
                     }
-                }
-                mbar_arrive(&sm.full[kk % nbuf]);
-            }
-        } else if (lane == 0) {
-            // ================= publisher: beta, fences and flags
-            for (int k = 0; k < nk; k++, kk++) {
-                const int par = kk & 1;
-                if (is_o) {
-                    chase_wait(&sm.gen[par], (kk >> 1) & 1, wait_ns, state, &sm.abort);
-                    if (rank == 0 && !*(volatile int *)&sm.abort) {
-                        const int r = s + k * b, c = (k == 0) ? s - 1 : r - b;
-                        T z;
-                        zero_of(z);
-                        *(double *)&z = sm.beta[par];
-                        *A.at(r, c) = z;
-                        st_rel(mine, k + 1);
+                    if (s > 1 && len == b && (b - 1) % CD == dr) {
+                        loader_sync();
+                        if (lt == 0 && !*(volatile int *)&sm.abort) {
+                            T x;
+                            take_entry(x, firsts_prev + (size_t)(k + 1) * b * words, 0, timeout_ns, state, &sm.abort);
+                            B[((b - 1) / CD) * LD + b - 1] = x;
+                        }
                     }
                 }
-                chase_wait(&sm.st[par], (kk >> 1) & 1, wait_ns, state, &sm.abort);
-                if (!*(volatile int *)&sm.abort) {
-                    __threadfence();
-                    red_rel(mine + (is_o ? 1 : 2), 1);
-                }
-                mbar_arrive(&sm.empty[kk % nbuf]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sm.full[kk % nbuf]);
             }
         } else {
-            kk += nk;
+            // ================= publisher warp: fences and flags; in D
+            // blocks the reflector's scalars too
+            for (int k = 0; k < nk; k++, kk++) {
+                const int par = kk & 1;
+                if (!is_o) {
+                    chase_wait(&sm.xo[par], (kk >> 1) & 1, wait_ns, state, &sm.abort);
+                    const auto h = reflector(sm.ma[par][0], group_sum<G::NG>(&sm.ms[par][0][0], BM));
+                    if (lane == 0) {
+                        sm.tau[par] = h.tau;
+                        sm.scal[par] = h.scal;
+                    }
+                    scalars_give();
+                }
+                if (lane == 0) {
+                    chase_wait(&sm.st[par], (kk >> 1) & 1, wait_ns, state, &sm.abort);
+                    // (the release orders the block's stores, seen through the
+                    // barrier, before the flag)
+                    if (!*(volatile int *)&sm.abort) st_rel(mine + rank, k + 1);
+                    mbar_arrive(&sm.empty[kk % nbuf]);
+                }
+                __syncwarp();
+            }
         }
     }
     __syncwarp();
@@ -579,8 +734,11 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
 
 template <class T>
 __global__ void __launch_bounds__(256) band_init(int n, int b, const T *__restrict__ AB, long long ldab,
-                                                 T *__restrict__ W, long long ldw)
+                                                 T *__restrict__ W, long long ldw,
+                                                 unsigned long long *__restrict__ slots, size_t nslots)
 {
+    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < nslots; e += (size_t)gridDim.x * blockDim.x)
+        slots[e] = kEmpty;
     const long long total = (long long)n * ldw;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
@@ -604,29 +762,46 @@ __global__ void __launch_bounds__(256) band_extract(int n, const T *__restrict__
 }  // namespace
 
 // Workspace: [256-byte head {ticket, abort, error}][progress: kFlags ints per
-// sweep] then, 256-byte aligned, the 2b x n working band.
-static size_t flags_bytes(int n) { return (256 + (size_t)n * kFlags * sizeof(int) + 255) & ~(size_t)255; }
+// sweep][slots: 2 nk(1) betas, 2 nk(1) b entries of one or two words] then,
+// 256-byte aligned, the 2b x n working band.
+static size_t progress_bytes(int n) { return (256 + (size_t)n * kFlags * sizeof(int) + 255) & ~(size_t)255; }
+static size_t slot_words(int n, int b, int words)
+{
+    const size_t nk1 = ((size_t)n + b - 1) / b;
+    return 2 * nk1 + 2 * nk1 * b * words;
+}
+static size_t flags_bytes(int n, int b, int words)
+{
+    return progress_bytes(n) + ((slot_words(n, b, words) * 8 + 255) & ~(size_t)255);
+}
+static ChaseProblem chase_problem(int n, int b, int words, void *ws, void *hh_v, void *hh_tau)
+{
+    char *flags = (char *)ws;
+    unsigned long long *slots = (unsigned long long *)(flags + progress_bytes(n));
+    return ChaseProblem{n,      b,      flags + flags_bytes(n, b, words), 2LL * b, hh_v, hh_tau, (int *)(flags + 256), slots,
+                        slots + 2 * (((size_t)n + b - 1) / b)};
+}
 
 size_t band_to_tridi_workspace_bytes(int n, int b)
 {
     size_t band = 2 * (size_t)b * (size_t)n * sizeof(double);
-    return flags_bytes(n) + ((band + 255) & ~(size_t)255);
+    return flags_bytes(n, b, 1) + ((band + 255) & ~(size_t)255);
 }
 
 size_t band_to_tridi_workspace_bytes_z(int n, int b)
 {
     size_t band = 2 * (size_t)b * (size_t)n * 2 * sizeof(double);
-    return flags_bytes(n) + ((band + 255) & ~(size_t)255);
+    return flags_bytes(n, b, 2) + ((band + 255) & ~(size_t)255);
 }
 
-// Sweeps that can be in flight at once: sweep s trails sweep s-1 by one O
-// step and the generation of the next reflector, somewhat more than one step
-// of its nk(1); further clusters would only poll, holding SM slots that
-// concurrent work on other streams could use.
+// Sweeps that can be in flight at once: sweep s trails sweep s-1 by about two
+// of its nk(1) steps; further clusters would only poll, holding SM slots that
+// concurrent work on other streams could use (n = 2048: 17.8 ms with 16 clusters,
+// 17.6 with 19, 19.7 with 30).
 static int chase_active(int n, int b)
 {
     const int nk1 = (n - 1 + b - 1) / b;
-    return max(1, min(n - 1, (2 * nk1 + 2) / 3 + 2));
+    return max(1, min(n - 1, (nk1 + 1) / 2 + 3));
 }
 
 template <class T, int BM, int C, int CD>
@@ -656,11 +831,11 @@ static cudaError_t chase_launch_as(const ChaseWork &work, long long active, int 
 }
 
 // `active`: sweeps in flight over all problems; bmax: the widest band.
-// Real, b > 32: clusters of 6 (4 row parts of O, 2 of D: 11.5 us a sweep at
-// n = 2048) while those of the sweeps in flight fit the SMs, else clusters of
-// 3 (14.5 us a sweep at n = 8192, where clusters of 6 would leave half of the
-// sweeps without SMs).  b <= 32 has a quarter of the work a step: clusters of
-// 3 (8.1 us a sweep); complex steps have four times the work: 6 from b = 33.
+// Real, b > 32: clusters of 6 (4 row parts of O, 2 of D) up to twice the
+// sweeps that find SMs: n = 2048 17.6 ms against 22.8 with clusters of 3, 4096
+// 42.5 against 46.0, 8192 99.8 against 124; beyond that (n = 16384) clusters of 3,
+// which keep twice the sweeps in flight.  b <= 32 has a quarter of the work a
+// step: clusters of 3; complex steps have four times the work: 6 from b = 33.
 static cudaError_t chase_launch(const ChaseWork &work, long long active, int bmax, int is_complex, ChaseState *state,
                                 long long timeout_ns, cudaStream_t st)
 {
@@ -673,16 +848,16 @@ static cudaError_t chase_launch(const ChaseWork &work, long long active, int bma
         return chase_launch_as<Zc, 64, 4, 2>(work, active, sms, state, timeout_ns, st);
     }
     if (bmax <= 32) return chase_launch_as<double, 32, 2, 1>(work, active, sms, state, timeout_ns, st);
-    if (active * 6 <= sms) return chase_launch_as<double, 64, 4, 2>(work, active, sms, state, timeout_ns, st);
+    if (active * 6 <= 4LL * sms) return chase_launch_as<double, 64, 4, 2>(work, active, sms, state, timeout_ns, st);
     return chase_launch_as<double, 64, 2, 1>(work, active, sms, state, timeout_ns, st);
 }
 
-static ChaseWork chase_one(int n, int b, void *W, void *hh_v, void *hh_tau, int *progress)
+static ChaseWork chase_one(const ChaseProblem &problem)
 {
     ChaseWork w{};
     w.count = 1;
-    w.smax = n - 1;
-    w.one = ChaseProblem{n, b, W, 2LL * b, hh_v, hh_tau, progress};
+    w.smax = problem.n - 1;
+    w.one = problem;
     return w;
 }
 
@@ -690,17 +865,18 @@ cudaError_t band_to_tridi_prepare_z(int n, int b, const double *AB, int ldab, vo
 {
     const long long ldw = 2LL * b;
     char *flags = (char *)ws;
-    Zc *W = (Zc *)(flags + flags_bytes(n));
-    cudaError_t err = cudaMemsetAsync(flags, 0, flags_bytes(n), st);
+    Zc *W = (Zc *)(flags + flags_bytes(n, b, 2));
+    cudaError_t err = cudaMemsetAsync(flags, 0, progress_bytes(n), st);
     if (err != cudaSuccess) return err;
-    band_init<Zc><<<1024, 256, 0, st>>>(n, b, (const Zc *)AB, ldab, W, ldw);
+    band_init<Zc><<<1024, 256, 0, st>>>(n, b, (const Zc *)AB, ldab, W, ldw,
+                                        (unsigned long long *)(flags + progress_bytes(n)), slot_words(n, b, 2));
     return cudaGetLastError();
 }
 
 cudaError_t band_to_tridi_finish_z(int n, int b, const void *ws, double *d, double *e, cudaStream_t st)
 {
     const long long ldw = 2LL * b;
-    const Zc *W = (const Zc *)((const char *)ws + flags_bytes(n));
+    const Zc *W = (const Zc *)((const char *)ws + flags_bytes(n, b, 2));
     band_extract<Zc><<<64, 256, 0, st>>>(n, W, ldw, d, e);
     return cudaGetLastError();
 }
@@ -712,7 +888,7 @@ cudaError_t band_to_tridi_z(int n, int b, const double *AB, int ldab, double *d,
     cudaError_t err = band_to_tridi_prepare_z(n, b, AB, ldab, ws, st);
     if (err != cudaSuccess) return err;
     if (n > 1) {
-        const ChaseWork w = chase_one(n, b, flags + flags_bytes(n), hh_v, hh_tau, (int *)(flags + 256));
+        const ChaseWork w = chase_one(chase_problem(n, b, 2, ws, hh_v, hh_tau));
         if ((err = chase_launch(w, chase_active(n, b), b, 1, (ChaseState *)flags, timeout_ns, st)) != cudaSuccess)
             return err;
     }
@@ -723,17 +899,17 @@ cudaError_t band_to_tridi_prepare_d(int n, int b, const double *AB, int ldab, vo
 {
     const long long ldw = 2LL * b;
     char *flags = (char *)ws;
-    double *W = (double *)(flags + flags_bytes(n));
-    cudaError_t err = cudaMemsetAsync(flags, 0, flags_bytes(n), st);
+    double *W = (double *)(flags + flags_bytes(n, b, 1));
+    cudaError_t err = cudaMemsetAsync(flags, 0, progress_bytes(n), st);
     if (err != cudaSuccess) return err;
-    band_init<double><<<1024, 256, 0, st>>>(n, b, AB, ldab, W, ldw);
+    band_init<double><<<1024, 256, 0, st>>>(n, b, AB, ldab, W, ldw, (unsigned long long *)(flags + progress_bytes(n)), slot_words(n, b, 1));
     return cudaGetLastError();
 }
 
 cudaError_t band_to_tridi_finish_d(int n, int b, const void *ws, double *d, double *e, cudaStream_t st)
 {
     const long long ldw = 2LL * b;
-    const double *W = (const double *)((const char *)ws + flags_bytes(n));
+    const double *W = (const double *)((const char *)ws + flags_bytes(n, b, 1));
     band_extract<double><<<64, 256, 0, st>>>(n, W, ldw, d, e);
     return cudaGetLastError();
 }
@@ -746,7 +922,7 @@ cudaError_t band_to_tridi_d(int n, int b, const double *AB, int ldab, double *d,
     cudaError_t err = band_to_tridi_prepare_d(n, b, AB, ldab, ws, st);
     if (err != cudaSuccess) return err;
     if (n > 1) {
-        const ChaseWork w = chase_one(n, b, flags + flags_bytes(n), hh_v, hh_tau, (int *)(flags + 256));
+        const ChaseWork w = chase_one(chase_problem(n, b, 1, ws, hh_v, hh_tau));
         if ((err = chase_launch(w, chase_active(n, b), b, 0, (ChaseState *)flags, timeout_ns, st)) != cudaSuccess)
             return err;
     }
@@ -764,14 +940,12 @@ size_t chase_batched_table_bytes(int count) { return 256 + (((size_t)count * siz
 // band_to_tridi_prepare_d has run on every problem's workspace ws[i].
 cudaError_t band_to_tridi_chase_batched_upload_d(int count, const int *n, const int *b, void *const *ws,
                                                  double *const *hh_v, double *const *hh_tau, void *table,
-                                                 cudaStream_t st)
+                                                 int is_complex, cudaStream_t st)
 {
     if (count < 1) return cudaSuccess;
     std::vector<ChaseProblem> host((size_t)count);
     for (int i = 0; i < count; i++) {
-        char *flags = (char *)ws[i];
-        host[i] = ChaseProblem{n[i], b[i], flags + flags_bytes(n[i]), 2LL * b[i], hh_v[i], hh_tau[i],
-                               (int *)(flags + 256)};
+        host[i] = chase_problem(n[i], b[i], is_complex ? 2 : 1, ws[i], hh_v[i], hh_tau[i]);
     }
     cudaError_t err = cudaMemsetAsync(table, 0, 256, st);
     if (err != cudaSuccess) return err;

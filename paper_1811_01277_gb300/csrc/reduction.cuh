@@ -83,9 +83,45 @@ __device__ __forceinline__ Zc ld_cg(const Zc *p)
     return {t.x, t.y};
 }
 
+// 1/x from the hardware's approximate FP64 reciprocal and two Newton-Raphson
+// steps, to about one ulp, for 2^-1000 <= |x| < 2^1000.
+__device__ __forceinline__ double newton_recip(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    double t = fma(-x, r, 1.0);
+    r = fma(r, t, r);
+    t = fma(-x, r, 1.0);
+    return fma(r, t, r);
+}
+
+// s in (2^-1000, 2^1000): *nrm = sqrt(s) and *inv = 1 / sqrt(s), from the
+// approximate reciprocal square root: two Newton-Raphson steps for the
+// inverse, and one for the root itself (within an ulp each).
+__device__ __forceinline__ void newton_sqrt(double s, double *nrm, double *inv)
+{
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(s));
+    double e = fma(-s * r, r, 1.0);
+    r = fma(0.5 * r, e, r);
+    e = fma(-s * r, r, 1.0);
+    r = fma(0.5 * r, e, r);
+    const double g = s * r;
+    *nrm = fma(0.5 * r, fma(-g, g, s), g);
+    *inv = r;
+}
+
+__device__ __forceinline__ bool mid_range(double x)   // 2^-1000 <= |x| < 2^1000
+{
+    return (((unsigned)__double2hiint(x) >> 20) & 0x7FFu) - 23u < 2000u;
+}
+
 // tau, scale and beta of the reflector (LAPACK form, v_0 = 1): alpha the
-// first entry, ss the sum of |x_i|^2 below it.  The two quotients are
-// computed by two lanes of the calling warp at once (all lanes call).
+// first entry, ss the sum of |x_i|^2 below it; called by whole warps with the
+// same arguments.  It sits on the chain of both reductions, and every dependent
+// FP64 operation costs a warp about 64 clocks there: beta = -sgn(alpha) nrm
+// gives tau = 1 + |alpha| / nrm without waiting for a division, and scale =
+// sgn(alpha) / (|alpha| + nrm) takes one Newton reciprocal.
 struct Refl {
     double tau, scal, beta;
 };
@@ -97,12 +133,23 @@ __device__ __forceinline__ Refl reflector(double alpha, double ss)
 {
     double tau = 0.0, scal = 0.0, beta = alpha;
     if (ss != 0.0) {
-        const double nrm = sqrt(alpha * alpha + ss);
-        beta = (alpha >= 0.0) ? -nrm : nrm;
-        const bool odd = threadIdx.x & 1;
-        const double qt = (odd ? 1.0 : beta - alpha) / (odd ? alpha - beta : beta);
-        tau = __shfl_sync(0xffffffffu, qt, 0);
-        scal = __shfl_sync(0xffffffffu, qt, 1);
+        const double s = fma(alpha, alpha, ss), a = fabs(alpha);
+        if (mid_range(s)) {
+            double nrm, inv;
+            newton_sqrt(s, &nrm, &inv);
+            tau = fma(a, inv, 1.0);
+            scal = copysign(newton_recip(a + nrm), alpha);
+            beta = -copysign(nrm, alpha);
+        } else {
+            const double nrm = sqrt(s);
+            beta = -copysign(nrm, alpha);
+            tau = (beta - alpha) / beta;
+            scal = 1.0 / (alpha - beta);
+        }
+        if (alpha == 0.0) {   // sgn(0) = +1, also for a negative zero
+            beta = -fabs(beta);
+            scal = fabs(scal);
+        }
     }
     return {tau, scal, beta};
 }
@@ -111,15 +158,18 @@ __device__ __forceinline__ ReflZ reflector(Zc alpha, double ss)
     Zc tau{0.0, 0.0}, scal{0.0, 0.0};
     double beta = alpha.re;
     if (!(ss == 0.0 && alpha.im == 0.0)) {
-        const double nrm = sqrt(alpha.re * alpha.re + alpha.im * alpha.im + ss);
-        beta = (alpha.re >= 0.0) ? -nrm : nrm;
-        const double dr = alpha.re - beta;                    // 1 / (alpha - beta)
-        const double dd = dr * dr + alpha.im * alpha.im;
-        const int l = threadIdx.x & 3;
-        const double num = l == 0 ? beta - alpha.re : l == 1 ? -alpha.im : l == 2 ? dr : -alpha.im;
-        const double q = num / (l < 2 ? beta : dd);
-        tau = Zc{__shfl_sync(0xffffffffu, q, 0), __shfl_sync(0xffffffffu, q, 1)};
-        scal = Zc{__shfl_sync(0xffffffffu, q, 2), __shfl_sync(0xffffffffu, q, 3)};
+        const double s = fma(alpha.re, alpha.re, fma(alpha.im, alpha.im, ss));
+        const double sg = alpha.re >= 0.0 ? 1.0 : -1.0, a = fabs(alpha.re);
+        double nrm, inv;
+        if (mid_range(s)) newton_sqrt(s, &nrm, &inv);
+        else inv = 1.0 / (nrm = sqrt(s));
+        beta = -sg * nrm;
+        // tau = (beta - alpha) / beta; 1 / (alpha - beta) with alpha - beta =
+        // sg (a + nrm) + i im, |alpha - beta|^2 = (a + nrm)^2 + im^2
+        tau = Zc{fma(a, inv, 1.0), sg * alpha.im * inv};
+        const double dr = a + nrm, dd = fma(dr, dr, alpha.im * alpha.im);
+        const double f = mid_range(dd) ? newton_recip(dd) : 1.0 / dd;
+        scal = Zc{sg * dr * f, -alpha.im * f};
     }
     return {tau, scal, beta};
 }
@@ -139,6 +189,33 @@ __device__ __forceinline__ void mbar_arrive_remote(void *bar, int rank)
         "mbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n}\n" ::"r"(tc5::smem_addr(bar)),
         "r"(rank)
         : "memory");
+}
+
+// One value into block `rank`'s shared memory at `to`'s offset, counted in bytes
+// on the mbarrier at `bar`'s offset there: data and signal in one message.
+__device__ __forceinline__ void send(double *to, double x, void *bar, int rank)
+{
+    asm volatile(
+        "{\n.reg .b32 a, b;\nmapa.shared::cluster.u32 a, %0, %3;\nmapa.shared::cluster.u32 b, %1, %3;\n"
+        "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [a], %2, [b];\n}\n" ::"r"(tc5::smem_addr(to)),
+        "r"(tc5::smem_addr(bar)), "l"(__double_as_longlong(x)), "r"(rank)
+        : "memory");
+}
+__device__ __forceinline__ void send(Zc *to, Zc x, void *bar, int rank)
+{
+    asm volatile(
+        "{\n.reg .b32 a, b;\nmapa.shared::cluster.u32 a, %0, %4;\nmapa.shared::cluster.u32 b, %1, %4;\n"
+        "st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [a], {%2, %3}, [b];\n}\n" ::"r"(
+            tc5::smem_addr(to)),
+        "r"(tc5::smem_addr(bar)), "l"(__double_as_longlong(x.re)), "l"(__double_as_longlong(x.im)), "r"(rank)
+        : "memory");
+}
+
+// this block's arrival on its own barrier, which then waits for `bytes` too
+__device__ __forceinline__ void mbar_expect(void *bar, uint32_t bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc5::smem_addr(bar)), "r"(bytes)
+                 : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity)

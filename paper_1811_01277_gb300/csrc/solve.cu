@@ -727,7 +727,7 @@ int gb_solve_stage_chase_batched(int is_complex, int count, const int *n, const 
         }
     }
     const cudaStream_t st = (cudaStream_t)stream;
-    if (gb::band_to_tridi_chase_batched_upload_d(count, n, nbw, cws.data(), hv.data(), ht.data(), table, st) !=
+    if (gb::band_to_tridi_chase_batched_upload_d(count, n, nbw, cws.data(), hv.data(), ht.data(), table, is_complex, st) !=
         cudaSuccess)
         return GB_ERR_CUDA;
     return gb::band_to_tridi_chase_batched(count, n, nbw, table, 10LL * 1000 * 1000 * 1000, st, is_complex) == cudaSuccess
@@ -1137,7 +1137,7 @@ int gb_solve_batched_staged_d(int count, const int *n, const int *nev, const int
             hv[i] = ws[i].hv;
             ht[i] = ws[i].ht;
         }
-        if (gb::band_to_tridi_chase_batched_upload_d(count, n, bw.data(), cws.data(), hv.data(), ht.data(), base,
+        if (gb::band_to_tridi_chase_batched_upload_d(count, n, bw.data(), cws.data(), hv.data(), ht.data(), base, 0,
                                                      (cudaStream_t)streams[0]) != cudaSuccess)
             return GB_ERR_CUDA;
     }

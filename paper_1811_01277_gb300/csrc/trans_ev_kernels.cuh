@@ -44,7 +44,7 @@ cudaError_t band_to_tridi_finish_d(int n, int b, const void *ws, double *d, doub
 size_t chase_batched_table_bytes(int count);
 cudaError_t band_to_tridi_chase_batched_upload_d(int count, const int *n, const int *b, void *const *ws,
                                                  double *const *hh_v, double *const *hh_tau, void *table,
-                                                 cudaStream_t st);
+                                                 int is_complex, cudaStream_t st);
 cudaError_t band_to_tridi_chase_batched_d(int count, const int *n, const int *b, void *table, long long timeout_ns,
                                           cudaStream_t st);
 cudaError_t band_to_tridi_chase_batched(int count, const int *n, const int *b, void *table, long long timeout_ns,

@@ -59,3 +59,38 @@ def test_chase_edges(gb, n, b, cplx):
     Q = oracle.trans_ev(n, b, hv, ht, np.eye(n, dtype=B.dtype))
     T = np.diag(d) + np.diag(e, -1) + np.diag(e, 1)
     assert np.abs(Q.conj().T @ B @ Q - T).max() <= tol
+
+
+@pytest.mark.parametrize("cplx,n,b", [(False, 700, 64), (False, 500, 32), (True, 300, 64)])
+def test_chase_concurrent(gb, cplx, n, b):
+    """Many chases at once, so that a sweep's blocks get out of step with each
+    other: every one gives the bits of a chase that runs alone."""
+    dev = torch.device("cuda")
+    B = inputs.band_symmetric(n, b, seed=n + b, cplx=cplx)
+    AB = np.zeros((n, b + 1), dtype=B.dtype)
+    for k in range(b + 1):
+        AB[:n - k, k] = np.diag(B, -k)
+    AB = torch.from_numpy(AB).to(dev)
+    cnt = gb.gb_hh_count(n, b)
+    wsb = (gb.gb_band_to_tridi_workspace_bytes_z if cplx else gb.gb_band_to_tridi_workspace_bytes)(n, b)
+    run = gb.gb_band_to_tridi_z if cplx else gb.gb_band_to_tridi_d
+
+    def buffers():
+        return (torch.zeros(n, dtype=torch.float64, device=dev), torch.zeros(n - 1, dtype=torch.float64, device=dev),
+                torch.zeros(cnt * b, dtype=AB.dtype, device=dev), torch.zeros(cnt, dtype=AB.dtype, device=dev),
+                torch.empty(wsb, dtype=torch.uint8, device=dev))
+
+    alone = buffers()
+    run(n, b, AB, b + 1, *alone[:4], alone[4], wsb, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(24)]
+    for _ in range(6):
+        many = [buffers() for _ in streams]
+        torch.cuda.synchronize()
+        for st, w in zip(streams, many):
+            run(n, b, AB, b + 1, *w[:4], w[4], wsb, st)
+        torch.cuda.synchronize()
+        for st, w in zip(streams, many):
+            assert gb.gb_trans_ev_query(w[4], wsb, st) == 0
+            for x, y in zip(w[:4], alone[:4]):
+                assert torch.equal(x, y)
