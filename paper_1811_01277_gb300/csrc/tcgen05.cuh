@@ -62,6 +62,17 @@ __device__ __forceinline__ void mma_smem_a(uint32_t d_tmem, uint64_t a_desc, uin
         "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
 }
 
+// One lane of a converged warp, the same each time.  A branch on it, with the
+// MMAs' operands compile-time constants and warp-uniform values, issues an MMA
+// every 58 cycles at most; branches on a thread index and elections per
+// MMA take 94 to 120 (the operands' moves to uniform registers).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
+    return e != 0;
+}
+
 // the mbarrier receives one arrival when every tcgen05.mma this thread has
 // issued so far has completed
 __device__ __forceinline__ void commit(uint32_t mbar)

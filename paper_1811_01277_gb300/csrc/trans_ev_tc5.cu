@@ -42,18 +42,33 @@
 //
 // Data movement per tile (b = 64, NB = 32, LP = 96):
 //  * the tile record is a V part (V digit planes in the MMA's canonical
-//    K-major layout, 48 KB) and a U part (U^T digit planes by 32-row
-//    chunks, the row exponents of V and U; 48.5 KB), built once per tile by
-//    tc5_tile_prep; each part arrives by cp.async.bulk on its own mbarrier,
-//    requested as soon as the previous tile no longer needs the buffer;
+//    K-major layout, 48 KB) and a U part (U^T digit planes by 16-row
+//    chunks, the folds' constants of V's columns and U's rows; 50 KB), built
+//    once per tile by tc5_tile_prep; each part arrives by cp.async.bulk on its
+//    own mbarrier, requested as soon as the previous tile no longer needs the
+//    buffer;
 //  * the window (LP rows x 128 columns, int64) lives in shared memory; the
-//    64 new rows come from global memory through L2, NB-1 rows carry over;
+//    64 new rows come from global memory through L2, NB-1 rows carry over
+//    where they are (the window turns in its slots);
 //  * Z's digit planes are cut by the threads straight into TMEM (tcgen05.st)
 //    and are the A operand of the first product, W's digit planes the A
 //    operand of the second.
-// TMEM (512 columns): Z digits of up to ZR K steps [0, 64 ZR) (two rounds
-// when all K steps do not fit), W levels [64 ZR, + 9 NB); then W digits
-// [0, 64 NB/16) and the dZ levels of a 32-row chunk [64 NB/16, + 9 32).
+// TMEM (512 columns): Z digits of ZR K steps in turn [0, 64 ZR), W levels [64
+// ZR, + 9 NB); then W digits [0, 64 NB/16) and the dZ levels of two 16-row
+// chunks [64 NB/16, + 2 9 16).
+//
+// What bounds it: 16 thousand digit cuts and as many folds a tile on the
+// integer pipe, in 16 warps (one block per SM: the window and the record fill
+// shared memory), against 8 thousand clocks of MMAs.  So the 16 warps do nothing
+// else: a driver warp issues the MMAs of a K step or chunk as soon as the
+// workers have arrived there (named barriers on which only the driver waits),
+// a flags' warp publishes stored tiles and looks for the next one's rows, and
+// what a fold needs besides its sums is in the record.  A tile of n = 8192, nev =
+// 4096 takes 25.8 thousand clocks (34.3 with everything in the same 16 warps and
+// K steps and chunks in series): cuts and the first product 6.1, folding
+// and cutting W 3.2, the second product and its folds 10.1, loads and
+// stores 5.0.  Whole calls: n = 16384, nev = 4096 261 -> 193 ms; complex n = 4096,
+// nev = 1228 37.1 -> 20.5; n = nev = 1024, nbw = 32 (a chain of 64 groups) 1.24 -> 0.92.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -70,7 +85,11 @@ namespace gb {
 namespace {
 
 constexpr int kCols5 = 128;       // eigenvector columns per work item (the MMA's M)
-constexpr int kThreads5 = 512;    // 16 warps: four per TMEM lane quarter (and per SM sub-partition)
+constexpr int kWork5 = 512;       // 16 working warps: four per TMEM lane quarter (and per SM sub-partition)
+constexpr int kThreads5 = kWork5 + 128;  // and a warpgroup of which one warp is the driver (MMAs, record
+                                 // copies) and one has the flags; it gives registers to the workers: 96 at launch, then 64 and 104
+constexpr int kHandOver = kWork5 + 32;  // threads at the barriers from workers to driver
+constexpr int kInStep = kWork5 + 64;    // and at the tile's barriers: with the flags' warp too
 constexpr int kPlanes = 8;        // balanced base-256 digits of a 64-bit value
 constexpr int kLevels5 = 9;       // digit-pair levels 0..8
 constexpr int kColumnBatch5 = 8;  // 128-column blocks per ticket batch (2 and 4 re-read the records more, 16 gains nothing)
@@ -94,26 +113,29 @@ struct Geo {
     static constexpr int KSTEPS = LP / 16;              // K steps of the first product
     static constexpr int KD = NBC / 16;                 // K steps of the second
     // tile record: V part [8 planes][NBC rows q][LP] and U part [chunks of
-    // 32 rows][8 planes][rows][NBC] + eV[NBC] + eU[LP], canonical K-major
+    // NCH rows][8 planes][rows][NBC] + the folds' constants by reflector (NBC) and
+    // row (LP) + a flag, canonical K-major
     static constexpr int VPLANE = NBC * LP * 2;
     static constexpr int VBYTES = kPlanes * VPLANE;
     static constexpr int UBYTES = kPlanes * LP * NBC * 2;
     static constexpr int U_EV = UBYTES;
-    static constexpr int U_EU = UBYTES + NBC * 4;
-    static constexpr int UPART = (UBYTES + (NBC + LP) * 4 + 127) / 128 * 128;
+    static constexpr int U_EU = UBYTES + NBC * 16;
+    static constexpr int U_FAR = UBYTES + (NBC + LP) * 16;          // some row's exponent is above 13
+    static constexpr int UPART = (U_FAR + 4 + 127) / 128 * 128;
     static constexpr int REC = VBYTES + UPART;
     static constexpr int SBO_V = 16 * LP;               // bytes between 8-row groups of V (N = q)
     static constexpr int SBO_U = 16 * NBC;              // bytes between 8-row groups of U^T (N = j)
     // window: [128 columns][ZROW] int64, ZROW = 2 mod 4 so that a warp's
     // 16-byte accesses to one row pair of 32 columns are conflict-free
     static constexpr int ZROW = LP + 2;
-    // dZ row chunks of up to 32 rows (N = 32 rows x up to 8 U planes <= 256)
-    static constexpr int NCH = 32;
-    static constexpr int CHUNKS = (LP + NCH - 1) / NCH;
+    // dZ row chunks of 16 rows (N = 16 rows x up to 8 U planes), two in tensor
+    // memory at once: one is folded while the next one's products run
+    static constexpr int NCH = 16;
+    static constexpr int CHUNKS = LP / NCH;
+    static constexpr int DZBUF = kLevels5 * NCH;        // TMEM columns of a chunk's levels
     // TMEM columns
     static constexpr int WLEV = kLevels5 * NBC;                     // W level accumulators
     static constexpr int ZR = (kTmemCols - WLEV) / 64 < KSTEPS ? (kTmemCols - WLEV) / 64 : KSTEPS;
-    static constexpr int ROUNDS = (KSTEPS + ZR - 1) / ZR;
     static constexpr int T_ZD = 0;
     static constexpr int T_WACC = 64 * ZR;
     static constexpr int T_WD = 0;
@@ -122,17 +144,22 @@ struct Geo {
     static constexpr int S_V = 0;
     static constexpr int S_U = VBYTES;
     static constexpr int S_Z = REC;
-    static constexpr int S_BAR = S_Z + kCols5 * ZROW * 8;    // 3 mbarriers + TMEM base
+    static constexpr int S_BAR = S_Z + kCols5 * ZROW * 8;    // 5 + ZR mbarriers, TMEM base
     // at least 116 KB, so that shared memory alone keeps the kernel at one
     // CTA per SM: every CTA allocates all 512 TMEM columns
-    static constexpr int SMEM = (S_BAR + 64) > 116 * 1024 ? (S_BAR + 64) : 116 * 1024;
+    static constexpr int SMEM = (S_BAR + 128) > 116 * 1024 ? (S_BAR + 128) : 116 * 1024;
     static_assert(ZR >= 1 && T_WACC + WLEV <= kTmemCols, "Z digits and W levels fit in TMEM");
-    static_assert(T_DZ + kLevels5 * NCH <= kTmemCols, "W digits and dZ levels fit in TMEM");
+    static_assert(T_DZ + 2 * DZBUF <= kTmemCols, "W digits and two chunks of dZ levels fit in TMEM");
+    static_assert(ADV % 8 == 0 && CHUNKS >= 2, "window units stay whole when the window turns");
     // level bounds per K with the top digits bounded by 32 (Z, W) and 64
     // (V, U): at most 7 x 2^14 + 32 128 + 128 64 (level 7) or 7 x 2^14 (level 8)
     static_assert(LP * (7 * 128 * 128) < (1 << 24), "W level sums stay exact in FP32");
     static_assert(NBC * (7 * 128 * 128) < (1 << 22), "dZ level sums stay below 2^22");
-    static_assert(LP * (32 * 128 + 128 * 128 + 128 * 64) < (1 << 22), "W levels 0..2 stay below 2^22");
+    // levels of W that stay below 2^22: a column of V has ADV nonzero rows, and
+    // level l < 8 has l - 1 inner pairs
+    static constexpr int w_level(int l) { return ADV * (l == 8 ? 7 * 16384 : l == 0 ? 2048 : (l - 1) * 16384 + 4096 + 8192); }
+    static constexpr int WMAGIC = w_level(8) < (1 << 22) && w_level(7) < (1 << 22) ? 9 : w_level(4) < (1 << 22) ? 5 : 3;
+    static_assert(w_level(2) < (1 << 22), "W levels 0..2 stay below 2^22");
     static_assert(LP % 16 == 0 && NBC % 16 == 0 && NB <= B && CARRY <= ADV, "tile shape");
     static_assert(VBYTES % 128 == 0 && REC % 128 == 0 && S_Z % 16 == 0, "record alignment");
     static_assert(SMEM <= 227 * 1024, "shared memory");
@@ -164,40 +191,89 @@ __device__ __forceinline__ void cut_pair(long long x0, long long x1, uint32_t (&
     for (int s = 4; s < 8; s++) out[s] = digit_pair(a_lo, b_lo, 7 - s);
 }
 
-// sum_l L_l 2^(50 - 8 l + e) from nine exact level sums, rounded once:
-// hi = sum_{l<4} L_l 2^(8(3-l)), lo = sum_{l>=4} L_l 2^(8(8-l)).
-// (mod 2^64 arithmetic; the result fits since it is a fixed-point entry)
-__device__ __forceinline__ long long fold9(const int (&Lv)[kLevels5], int e)
-{
-    const long long hi = ((long long)Lv[0] << 24) + ((long long)Lv[1] << 16) + ((long long)Lv[2] << 8) + Lv[3];
-    const long long lo = ((long long)Lv[4] << 32) + ((long long)Lv[5] << 24) + ((long long)Lv[6] << 16) +
-                         ((long long)Lv[7] << 8) + Lv[8];
-    return (long long)((unsigned long long)shift_ll(hi, 26 + e) + (unsigned long long)shift_ll(lo, e - 14));
-}
-
+// Folds of nine exact level sums, sum_l L_l 2^(50 - 8 l + e) rounded once:
+// with hi = sum_{l<4} L_l 2^(8(3-l)) and lo = sum_{l>=4} L_l 2^(8(8-l)) it is
+// hi 2^(26+e) + lo 2^(e-14) (mod 2^64; the result fits since it is a
+// fixed-point entry).  These are 16 thousand folds a tile on the integer pipe,
+// so what depends on the exponent alone is in the tile's record.
+//
 // An FP32 level sum x (an integer, |x| < 2^22) plus 1.5 2^23 has the bit
-// pattern 0x4B400000 + x.  Two such patterns combine into the int32
-// L_a 2^8 + L_b with one multiply-add and one subtraction of the combined
-// offset (257 * 0x4B400000 mod 2^32), exact whenever |L_a 2^8 + L_b| < 2^31.
+// pattern 0x4B400000 + x.  Two such patterns combine with one multiply-add
+// into the unsigned 32-bit value L_a 2^8 + L_b + kPairBias (no wrap: |L_a 2^8 +
+// L_b| < 2^30 + 2^22 and kPairBias lies between that and 2^32 less that), and
+// unsigned wide multiply-adds go on from there without sign extensions; the
+// biases leave as one 64-bit constant of hi and one of lo.
 constexpr uint32_t kMagicBits = 0x4B400000u;
-constexpr uint32_t kPairBias = 0x4B400000u * 257u;
+constexpr uint32_t kPairBias = 0x4B400000u * 257u;    // mod 2^32
+constexpr unsigned long long kHiBias = (unsigned long long)kPairBias * 65537ull;
+constexpr unsigned long long kLoBias =                // nine magic patterns
+    (unsigned long long)kPairBias * ((1ull << 24) + 256ull) + (unsigned long long)kMagicBits;
+constexpr unsigned long long kLoBias4 = (unsigned long long)kMagicBits << 32;   // level 4 alone
+static_assert(kPairBias > (1u << 30) + (1u << 22) && kPairBias < 0xffffffffu - (1u << 30) - (1u << 22), "pairs do not wrap");
+
+// The constants of a row or reflector of exponent e: lo's bias and rounding,
+// and the two shifts (s = 26 + e left, t = 14 - e right).  Exponents are at
+// least -26 (below, a row would be held finer than half a unit of the result
+// by 2^-27); above 13 (reflectors far from orthogonal) t <= 0 and the fold
+// shifts lo left.
+struct alignas(16) FoldConst {
+    unsigned long long lo_add;
+    int s, t;
+};
+constexpr int kMinExp = -26;
+__device__ __forceinline__ FoldConst fold_const(int e, unsigned long long lo_bias)
+{
+    FoldConst f;
+    f.s = 26 + e;
+    f.t = 14 - e;
+    f.lo_add = (e <= 13 ? 1ull << (13 - e) : 0ull) - lo_bias;
+    return f;
+}
 
 __device__ __forceinline__ uint32_t magic_bits(uint32_t f)
 {
     return __float_as_uint(__fadd_rn(__uint_as_float(f), 12582912.0f));
 }
 
-__device__ __forceinline__ int pair_from_bits(uint32_t a, uint32_t b) { return (int)(a * 256u + b - kPairBias); }
-
-// fold9 for level sums below 2^22 given as magic bit patterns (the dZ product)
-__device__ __forceinline__ long long fold9_bits(const uint32_t (&b)[kLevels5], int e)
+__device__ __forceinline__ unsigned long long wide(uint32_t a, uint32_t b, unsigned long long c)
 {
-    const int p0 = pair_from_bits(b[0], b[1]), p1 = pair_from_bits(b[2], b[3]);
-    const int p2 = pair_from_bits(b[4], b[5]), p3 = pair_from_bits(b[6], b[7]);
-    const int l8 = (int)(b[8] - kMagicBits);
-    const long long hi = (long long)p0 * 65536 + p1;
-    const long long lo = ((long long)p2 * 65536 + p3) * 256 + l8;
-    return (long long)((unsigned long long)shift_ll(hi, 26 + e) + (unsigned long long)shift_ll(lo, e - 14));
+    return (unsigned long long)a * b + c;
+}
+
+__device__ __forceinline__ long long fold_shift(unsigned long long hi, unsigned long long lo, FoldConst f)
+{
+    return (long long)(((hi - kHiBias) << f.s) + (unsigned long long)((long long)(lo + f.lo_add) >> f.t));
+}
+
+// level sums below 2^22, as magic bit patterns; FAR: the exponent may be above 13
+template <bool FAR>
+__device__ __forceinline__ long long fold9_bits(const uint32_t (&b)[kLevels5], FoldConst f)
+{
+    const uint32_t p0 = b[0] * 256u + b[1], p1 = b[2] * 256u + b[3];
+    const uint32_t p2 = b[4] * 256u + b[5], p3 = b[6] * 256u + b[7];
+    const unsigned long long hi = wide(p0, 65536u, p1);
+    const unsigned long long lo = wide(p2, 1u << 24, wide(p3, 256u, b[8]));
+    if (FAR && f.t <= 0)
+        return (long long)((unsigned long long)shift_ll((long long)(hi - kHiBias), f.s) +
+                           (unsigned long long)shift_ll((long long)(lo + f.lo_add), -f.t));
+    return fold_shift(hi, lo, f);
+}
+
+// level sums (FP32) below 2^24 of which the first NM stay below 2^22 (a
+// conversion runs at an eighth of an addition's rate).  Reflectors have unit
+// length: no exponent is above 13.
+template <int NM>
+__device__ __forceinline__ long long fold9_big(const uint32_t (&f)[kLevels5], FoldConst c)
+{
+    uint32_t m[5];
+#pragma unroll
+    for (int l = 0; l < 5; l++)
+        m[l] = l < NM ? magic_bits(f[l]) : kMagicBits + (uint32_t)__float2int_rn(__uint_as_float(f[l]));
+    const unsigned long long hi = wide(m[0] * 256u + m[1], 65536u, m[2] * 256u + m[3]);
+    const int l5 = __float2int_rn(__uint_as_float(f[5])), l6 = __float2int_rn(__uint_as_float(f[6]));
+    const int l7 = __float2int_rn(__uint_as_float(f[7])), l8 = __float2int_rn(__uint_as_float(f[8]));
+    const long long lo = (long long)l5 * (1 << 24) + ((long long)l6 * 65536 + ((long long)l7 * 256 + l8));
+    return fold_shift(hi, (unsigned long long)lo + ((unsigned long long)m[4] << 32), c);
 }
 
 // round(x 2^(62 - e)) for |x| < 2^e, to nearest with ties to even: the row's
@@ -339,26 +415,29 @@ __global__ void __launch_bounds__(256) tc5_tile_prep(int n, const double *__rest
             const unsigned long long u = (unsigned long long)__double_as_longlong(V[j * NB1 + threadIdx.x]) & ~(1ull << 63);
             m = u > m ? u : m;
         }
-        seV[threadIdx.x] = exponent_above(m);
-        ((int *)(ru + Gm::U_EV))[threadIdx.x] = seV[threadIdx.x];
+        seV[threadIdx.x] = max(exponent_above(m), kMinExp);
+        ((FoldConst *)(ru + Gm::U_EV))[threadIdx.x] = fold_const(seV[threadIdx.x], Gm::WMAGIC == 9 ? kLoBias : kLoBias4);
     }
+    bool far = false;
     for (int j = threadIdx.x; j < LP; j += blockDim.x) {
         unsigned long long m = 0;
         for (int q = 0; q < NB; q++) {
             const unsigned long long u = (unsigned long long)__double_as_longlong(U[j * NB1 + q]) & ~(1ull << 63);
             m = u > m ? u : m;
         }
-        seU[j] = exponent_above(m);
-        ((int *)(ru + Gm::U_EU))[j] = seU[j];
+        seU[j] = max(exponent_above(m), kMinExp);
+        far |= seU[j] > 13;
+        ((FoldConst *)(ru + Gm::U_EU))[j] = fold_const(seU[j], kLoBias);
     }
-    __syncthreads();
+    const int any_far = __syncthreads_or(far);
+    if (threadIdx.x == 0) *(int *)(ru + Gm::U_FAR) = any_far;
     // digit planes in the canonical K-major layout of the B operands:
     // V (N = q, K = j), plane t: byte t VPLANE + (q/8) SBO_V + (j/8) 128 +
     // (q%8) 16 + (j%8) 2, so the planes follow each other along N at the same
     // 8-row stride (an MMA's B may span planes t0, t0+1, ...);
-    // U^T (N = j, K = q), by chunks of 32 rows: chunk c = j/32 at c 32 SBO_U,
+    // U^T (N = j, K = q), by chunks of 16 rows: chunk c = j/16 at c 16 SBO_U,
     // within it plane t at t (rows of the chunk / 8) SBO_U, then
-    // (j%32/8) SBO_U + (q/8) 128 + (j%8) 16 + (q%8) 2 (again the planes of a
+    // (j%16/8) SBO_U + (q/8) 128 + (j%8) 16 + (q%8) 2 (again the planes of a
     // chunk contiguous along N)
     for (int e = threadIdx.x; e < NB * LP; e += blockDim.x) {
         const int q = e / LP, j = e % LP;
@@ -500,10 +579,12 @@ __global__ void __launch_bounds__(256) tc5_tile_prep_z(int n, const double2 *__r
             const double2 v = V[j * NB1 + threadIdx.x];
             m = max(m, max(absbits(v.x), absbits(v.y)));
         }
-        seV[threadIdx.x] = exponent_above(m);
-        ((int *)(ru + Gm::U_EV))[2 * threadIdx.x] = seV[threadIdx.x];
-        ((int *)(ru + Gm::U_EV))[2 * threadIdx.x + 1] = seV[threadIdx.x];
+        seV[threadIdx.x] = max(exponent_above(m), kMinExp);
+        const FoldConst f = fold_const(seV[threadIdx.x], Gm::WMAGIC == 9 ? kLoBias : kLoBias4);
+        ((FoldConst *)(ru + Gm::U_EV))[2 * threadIdx.x] = f;
+        ((FoldConst *)(ru + Gm::U_EV))[2 * threadIdx.x + 1] = f;
     }
+    bool far = false;
     for (int j = threadIdx.x; j < LP / 2; j += blockDim.x) {
         unsigned long long m = 0;
         if (j < LC)
@@ -511,12 +592,15 @@ __global__ void __launch_bounds__(256) tc5_tile_prep_z(int n, const double2 *__r
                 const double2 u = U[j * NB1 + q];
                 m = max(m, max(absbits(u.x), absbits(u.y)));
             }
-        const int ev = exponent_above(m);
+        const int ev = max(exponent_above(m), kMinExp);
+        far |= ev > 13;
         if (j < LC) seU[j] = ev;
-        ((int *)(ru + Gm::U_EU))[2 * j] = ev;
-        ((int *)(ru + Gm::U_EU))[2 * j + 1] = ev;
+        const FoldConst f = fold_const(ev, kLoBias);
+        ((FoldConst *)(ru + Gm::U_EU))[2 * j] = f;
+        ((FoldConst *)(ru + Gm::U_EU))[2 * j + 1] = f;
     }
-    __syncthreads();
+    const int any_far = __syncthreads_or(far);
+    if (threadIdx.x == 0) *(int *)(ru + Gm::U_FAR) = any_far;
     // V' (N = q' = 2q+p', K = j' = 2j+p) and the second product's B
     // (N = j', K = q'), in the layouts of the real record
     for (int e = threadIdx.x; e < NBC * LP; e += blockDim.x) {
@@ -537,7 +621,7 @@ __global__ void __launch_bounds__(256) tc5_tile_prep_z(int n, const double2 *__r
         const int jj = e / NBC, qq = e % NBC;
         const int q = qq >> 1, pq = qq & 1, j = jj >> 1, pj = jj & 1;
         double x = 0.0;
-        int ev = 0;
+        int ev = kMinExp;
         if (j < LC) {
             const double2 u = U[j * NB1 + q];
             x = (pj == pq) ? u.x : (pq ? -u.y : u.y);
@@ -556,20 +640,46 @@ __global__ void __launch_bounds__(256) tc5_tile_prep_z(int n, const double2 *__r
 
 // ---- the main kernel ------------------------------------------------------
 
-struct Tc5Shared {
-    int item;
-    int abort;
-    int u_issued;   // U parts requested so far (written by the thread that requests them)
+template <bool V>
+struct Bool {
+    static constexpr bool value = V;
 };
 
-// every thread: wait for an mbarrier phase; on giving up record the timeout
-__device__ __forceinline__ bool tc5_wait(uint32_t bar, uint32_t parity, TcState *state, Tc5Shared &sh)
+struct Tc5Shared {
+    int item;
+    int ready;      // the next tile's rows are there (looked up while this tile's dZ is folded)
+};
+
+// wait for an mbarrier phase; on giving up record the timeout
+__device__ __forceinline__ bool tc5_wait(uint32_t bar, uint32_t parity, TcState *state)
 {
     if (tc5::mbar_wait(bar, parity, kMbarTimeoutNs)) return true;
     tc_set_error(state, GB_ERR_TIMEOUT);
     atomicExch(&state->abort, 1);
-    sh.abort = 1;
     return false;
+}
+
+// the workers arrive at barrier `id`, the driver waits there for them
+__device__ __forceinline__ void workers_arrive(int id)
+{
+    __syncwarp();
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kHandOver) : "memory");
+}
+__device__ __forceinline__ void driver_takes(int id)
+{
+    __syncwarp();
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kHandOver) : "memory");
+}
+// workers, driver and flags' warp together: true (in all of them) if a wait of any gave up
+__device__ __forceinline__ bool in_step(bool gave_up)
+{
+    uint32_t r;
+    __syncwarp();
+    asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred q, 15, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+                 : "=r"(r)
+                 : "r"((uint32_t)gave_up), "n"(kInStep)
+                 : "memory");
+    return r != 0;
 }
 
 // n: the data's order (complex rows for RF = 2); Zi, ldz: the real form
@@ -588,10 +698,12 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
     long long *Zs = (long long *)(smem + Gm::S_Z);
     const uint32_t bar_v = tc5::smem_addr(smem + Gm::S_BAR);
     const uint32_t bar_u = bar_v + 8;
-    const uint32_t bar_mma = bar_v + 16;
-    uint32_t *tmem_slot = (uint32_t *)(smem + Gm::S_BAR + 32);
-    const int *eV = (const int *)(smem + Gm::S_U + Gm::U_EV);
-    const int *eU = (const int *)(smem + Gm::S_U + Gm::U_EU);
+    const uint32_t bar_dz = bar_v + 16;                     // two: one per chunk buffer
+    const uint32_t bar_k = bar_v + 32;                      // one per K step of Z digits in tensor memory
+    const uint32_t bar_end = bar_k + 8 * ZR;
+    uint32_t *tmem_slot = (uint32_t *)(smem + Gm::S_BAR + 40 + 8 * ZR);
+    const FoldConst *eV = (const FoldConst *)(smem + Gm::S_U + Gm::U_EV);
+    const FoldConst *eU = (const FoldConst *)(smem + Gm::S_U + Gm::U_EU);
     __shared__ Tc5Shared sh;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -599,21 +711,24 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
     const int col = quarter * 32 + lane;                    // this thread's column of the item (its TMEM lane)
     const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
     const int b = B;
+    const bool lead = tid == kWork5;                        // the driver's thread that issues
 
-    if (tid == 0) {
+    if (lead) {
         sh.item = atomicAdd(&state->ticket, 1);
-        sh.abort = 0;
-        sh.u_issued = 1;
+        sh.ready = 0;
         tc5::mbar_init(bar_v, 1);
         tc5::mbar_init(bar_u, 1);
-        tc5::mbar_init(bar_mma, 1);
+        tc5::mbar_init(bar_dz, 1);
+        tc5::mbar_init(bar_end, 1);
+        tc5::mbar_init(bar_dz + 8, 1);
+        for (int i = 0; i < ZR; i++) tc5::mbar_init(bar_k + 8 * i, 1);
         tc5::mbar_init_fence();
     }
     if (warp == 0) tc5::tmem_alloc(tc5::smem_addr(tmem_slot), kTmemCols);
     tc5::fence_before_sync();
     __syncthreads();
     tc5::fence_after_sync();
-    const uint32_t tmem = *(volatile uint32_t *)tmem_slot;
+    constexpr uint32_t tmem = 0;   // all 512 columns are this block's, so they start at 0 (checked below)
 
     const int item = sh.item;
     const int batch = item / (G * CB);
@@ -627,353 +742,417 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
     const int col0 = c * kCols5;
     const unsigned char *rec_g = rec + (size_t)off[g] * Gm::REC;
 
-    uint32_t mma_phase = 0;
-    bool mma_pending = false;
-    int v_issued = 0;   // V parts requested so far (thread 0)
+    int v_issued = 0, u_issued = 0;   // V and U parts requested so far (lead)
+    if (tid == 0 && *(volatile uint32_t *)tmem_slot != tmem) {
+        tc_set_error(state, GB_ERR_CUDA);
+        atomicExch(&state->abort, 1);
+    }
+    bool gave_up = false;     // this thread's waits: the block leaves at the next barrier
 
-    if (tid == 0) {
+    if (lead) {
         if (g + 1 != hold_group) st_release(progress + (long long)g * C + c, 0);
         tc5::bulk_load(tc5::smem_addr(smem + Gm::S_V), rec_g, Gm::VBYTES, bar_v);
         tc5::bulk_load(tc5::smem_addr(smem + Gm::S_U), rec_g + Gm::VBYTES, Gm::UPART, bar_u);
-        v_issued = 1;
+        v_issued = u_issued = 1;
     }
-    // window padding rows stay zero for the whole item
-    for (int e = tid; e < kCols5 * (LP - L); e += kThreads5) Zs[(e / (LP - L)) * ZROW + L + e % (LP - L)] = 0;
-
-    for (int k = 0; k < K; k++) {
-        // ---- dependency wait
-        if (tid == 0) {
-            int abort = 0;
-            const int need = (g + 1 < G) ? min(k + 1, Knext) : 0;
+    bool loaded = false;      // the window already holds this tile's rows
+    if (warp >= kWork5 / 32) {
+        // ================= the driver: dependency flags, record copies, MMAs (the
+        // other three warps of its warpgroup have nothing to do)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        if (warp == kWork5 / 32 + 1) {
+            // the flags: waits for group g+1, says whether the next tile's rows are
+            // there, publishes a tile's rows as soon as they are stored (a fence
+            // and a flag; on the driver's way they would hold up the products)
             const int *flag = progress + (long long)(g + 1) * C + c;
-            unsigned long long t0 = 0;
-            long long polls = 0;
-            while (need > 0 && ld_acquire(flag) < need) {
-                if (*(volatile int *)&state->abort) { abort = 1; break; }
-                if (polls == 0) t0 = now_ns();
-                if (++polls >= spin_polls || (long long)(now_ns() - t0) > timeout_ns) {
-                    tc_set_error(state, GB_ERR_TIMEOUT);
-                    atomicExch(&state->abort, 1);
-                    abort = 1;
-                    break;
+            for (int k = 0; k < K; k++) {
+                if (!loaded) {
+                    if (lane == 0) {
+                        const int need = (g + 1 < G) ? min(k + 1, Knext) : 0;
+                        unsigned long long t0 = 0;
+                        long long polls = 0;
+                        bool abort = false;
+                        while (need > 0 && ld_acquire(flag) < need) {
+                            if (*(volatile int *)&state->abort) { abort = true; break; }
+                            if (polls == 0) t0 = now_ns();
+                            if (++polls >= spin_polls || (long long)(now_ns() - t0) > timeout_ns) {
+                                tc_set_error(state, GB_ERR_TIMEOUT);
+                                atomicExch(&state->abort, 1);
+                                abort = true;
+                                break;
+                            }
+                            __nanosleep(64);
+                        }
+                        gave_up |= abort || *(volatile int *)&state->abort;
+                    }
+                    if (in_step(gave_up)) break;
+                    in_step(false);   // the workers have loaded the window
                 }
-                __nanosleep(128);
-            }
-            if (!abort && *(volatile int *)&state->abort) abort = 1;
-            if (abort) sh.abort = 1;
-        }
-        __syncthreads();
-        if (sh.abort) break;
-        // ---- window: new rows from global memory (through L2: rows written
-        // by other SMs), the NB-1 rows shared with the previous tile carried
-        const long long row0 = (long long)RF * ((long long)s0 + (long long)k * b);
-        const int jlo = (k == 0) ? 0 : CARRY;
-        {
-            constexpr int H = (L + 31) / 32;               // passes of 32 rows per column
-            constexpr int CW = kCols5 / (kThreads5 / 32);  // columns per warp
-            long long v[CW][H];
-#pragma unroll
-            for (int i = 0; i < CW; i++) {
-                const int cc = warp * CW + i;
-                const long long *zc = Zi + (long long)(col0 + cc < nev ? col0 + cc : 0) * ldz;
-#pragma unroll
-                for (int h = 0; h < H; h++) {
-                    const int j = jlo + lane + 32 * h;
-                    v[i][h] = (col0 + cc < nev && j < L && row0 + j < nrows) ? __ldcg(zc + row0 + j) : 0ll;
+                if (in_step(gave_up)) break;   // W's digits are there
+                if (lane == 0) {
+                    const int next = (g + 1 < G) ? min(k + 2, Knext) : 0;
+                    bool there = k + 1 < K && (next == 0 || ld_acquire(flag) >= next);
+                    if (k + 1 < K && !there) {   // once more when the last chunk's products are done
+                        constexpr int q = (Gm::CHUNKS - 1) & 1, uses = (Gm::CHUNKS - q + 1) / 2;
+                        gave_up |= !tc5_wait(bar_dz + 8 * q, (uint32_t)((k + 1) * uses - 1) & 1, state);
+                        there = ld_acquire(flag) >= next;
+                    }
+                    sh.ready = there;
                 }
-            }
-            if (k > 0) {
-                for (int e = tid; e < kCols5 * CARRY; e += kThreads5) {
-                    const int cc = e / CARRY, j = e % CARRY;
-                    Zs[cc * ZROW + j] = Zs[cc * ZROW + j + ADV];
+                if (in_step(gave_up)) break;   // dZ is folded
+                loaded = sh.ready != 0;
+                in_step(false);                // the tile's final rows are stored
+                // every thread's stores happen before this thread's fence and release
+                // (barrier, then a cumulative release at GPU scope)
+                if (lane == 0 && g + 1 != hold_group) {
+                    __threadfence();
+                    st_release(progress + (long long)g * C + c, k + 1);
                 }
-                __syncthreads();  // carried rows read before the new rows overwrite them
+                if (lane == 0) gave_up |= *(volatile int *)&state->abort != 0;   // another block gave up
             }
-#pragma unroll
-            for (int i = 0; i < CW; i++) {
-                const int cc = warp * CW + i;
-#pragma unroll
-                for (int h = 0; h < H; h++) {
-                    const int j = jlo + lane + 32 * h;
-                    if (j < L) Zs[cc * ZROW + j] = v[i][h];
-                }
+        } else
+        for (int k = warp == kWork5 / 32 ? 0 : K; k < K; k++) {
+            const uint64_t vdesc = tc5::smem_desc(tc5::smem_addr(smem + Gm::S_V), 128, Gm::SBO_V);
+            const uint64_t udesc = tc5::smem_desc(tc5::smem_addr(smem + Gm::S_U), 128, Gm::SBO_U);
+            const bool more = k + 1 < K;
+            if (!loaded) {
+                if (in_step(gave_up)) break;
+                in_step(false);   // the workers have loaded the window
             }
-        }
-        __syncthreads();
-        // ---- W^T = Z^T V, in rounds of ZR K steps (Z digit planes cut into
-        // TMEM, K step kk of the round at columns (kk - r ZR) 64 + s 8 + pair;
-        // units of 8 rows go round-robin to the four warps of a lane quarter)
-        const long long *zc = Zs + col * ZROW;
-#pragma unroll 1
-        for (int r = 0; r < Gm::ROUNDS; r++) {
-            const int kk0 = r * ZR, kk1 = (kk0 + ZR < KSTEPS) ? kk0 + ZR : KSTEPS;
-            if (r > 0) {   // the previous round's MMAs read the Z-digit columns
-                mma_pending = true;
-                if (tc5_wait(bar_mma, mma_phase & 1, state, sh)) mma_pending = false;
-                mma_phase++;
+            // ---- W^T = Z^T V by K steps, each when the workers have cut its Z digits
+#pragma unroll
+            for (int kk = 0; kk < KSTEPS; kk++) {
+                if (kk == 0) gave_up |= !tc5_wait(bar_v, (uint32_t)(k & 1), state);   // this tile's V planes
+                driver_takes(1 + kk);
+                // one MMA per Z digit plane s: B spans V planes 0 .. 8-s
+                // along N, so plane t lands in level s+t (D columns T_WACC +
+                // NB (s+t)); in the first K step level 8 is first written by
+                // its own MMA (s = 1, t = 7), every other level by s = 0
                 tc5::fence_after_sync();
-            }
-            for (int u = 2 * kk0 + wq; u < 2 * kk1; u += 4) {
-                uint32_t w[kPlanes][4];
+                if (tc5::elect_one()) {
+                    const int sl = kk % ZR;
+                    const uint64_t b0 = vdesc + (uint64_t)((kk * 256) >> 4);
 #pragma unroll
-                for (int p = 0; p < 4; p++) {
-                    const longlong2 z2 = *(const longlong2 *)(zc + u * 8 + 2 * p);
+                    for (int s = 0; s < kPlanes; s++) {
+                        const uint32_t a_t = tmem + Gm::T_ZD + sl * 64 + s * 8;
+                        const int nt = s == 0 ? kPlanes : kLevels5 - s;          // planes t = 0 .. nt-1
+                        if (kk == 0 && s == 1) {
+                            tc5::mma_tmem_a(tmem + Gm::T_WACC + NBC * 8, a_t, b0 + (uint64_t)((7 * Gm::VPLANE) >> 4),
+                                                 tc5::idesc_f16_f32(128, NBC), 0u);
+                            tc5::mma_tmem_a(tmem + Gm::T_WACC + NBC, a_t, b0, tc5::idesc_f16_f32(128, NBC * 7), 1u);
+                        } else {
+                            tc5::mma_tmem_a(tmem + Gm::T_WACC + NBC * s, a_t, b0, tc5::idesc_f16_f32(128, NBC * nt),
+                                                 (kk > 0 || s > 0) ? 1u : 0u);
+                        }
+                    }
+                    tc5::commit(bar_k + 8 * sl);
+                }
+                __syncwarp();
+            }
+            {
+                constexpr int sl = (KSTEPS - 1) % ZR, turns = (KSTEPS - sl + ZR - 1) / ZR;
+                gave_up |= !tc5_wait(bar_k + 8 * sl, (uint32_t)(k * turns + (KSTEPS - 1) / ZR) & 1, state);
+            }
+            tc5::fence_after_sync();
+            // the V buffer is free: request the next tile's V planes
+            if (lead && more) {
+                tc5::bulk_load(tc5::smem_addr(smem + Gm::S_V), rec_g + (size_t)(k + 1) * Gm::REC, Gm::VBYTES, bar_v);
+                v_issued = k + 2;
+            }
+            if (in_step(gave_up)) break;   // W's digits are there
+            // ---- dZ^T = W^T U^T by chunks of 16 rows (M 128, N = rows x planes, K NB)
+#pragma unroll
+            for (int ch = 0; ch < Gm::CHUNKS; ch++) {
+                if (ch >= 2) driver_takes(1 + ch - 2);   // chunk ch - 2 is read, its buffer free
+                // per W digit plane s and K step one MMA whose B spans the chunk's
+                // U planes 0 .. 8-s along N (level l = s+t at D columns l N of the
+                // chunk's buffer); level 8 first written alone (s = 1, t = 7)
+                constexpr int N = Gm::NCH;
+                tc5::fence_after_sync();
+                constexpr uint32_t pstride = (uint32_t)(N / 8) * Gm::SBO_U;   // bytes between the chunk's planes
+                const uint32_t dz = tmem + Gm::T_DZ + (ch & 1) * Gm::DZBUF;
+                if (tc5::elect_one()) {
+#pragma unroll
+                    for (int kd = 0; kd < KD; kd++)
+#pragma unroll
+                        for (int s = 0; s < kPlanes; s++) {
+                            const uint32_t a_t = tmem + Gm::T_WD + kd * 64 + s * 8;
+                            const uint64_t b0 = udesc + (uint64_t)((ch * N * Gm::SBO_U + kd * 256) >> 4);
+                            const int nt = s == 0 ? kPlanes : kLevels5 - s;
+                            if (kd == 0 && s == 1) {
+                                tc5::mma_tmem_a(dz + 8 * N, a_t, b0 + (uint64_t)((7 * pstride) >> 4),
+                                                     tc5::idesc_f16_f32(128, N), 0u);
+                                tc5::mma_tmem_a(dz + N, a_t, b0, tc5::idesc_f16_f32(128, 7 * N), 1u);
+                            } else {
+                                tc5::mma_tmem_a(dz + s * N, a_t, b0, tc5::idesc_f16_f32(128, nt * N),
+                                                     (kd > 0 || s > 0) ? 1u : 0u);
+                            }
+                        }
+                    tc5::commit(bar_dz + 8 * (ch & 1));
+                }
+                __syncwarp();
+            }
+            if (in_step(gave_up)) break;   // dZ is folded
+            tc5::fence_after_sync();
+            // the U part is consumed (planes by the MMAs, exponents by the folds):
+            // request the next tile's
+            if (lead && more) {
+                tc5::fence_proxy_async_smem();
+                tc5::bulk_load(tc5::smem_addr(smem + Gm::S_U), rec_g + (size_t)(k + 1) * Gm::REC + Gm::VBYTES, Gm::UPART,
+                               bar_u);
+                u_issued = k + 2;
+            }
+            loaded = sh.ready != 0;
+            in_step(false);   // the tile's final rows are stored
+        }
+    } else {
+        // ================= the workers
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        // The window turns in its LP slots: logical row j of tile k is in slot
+        // (j + k ADV) mod LP, so carried rows stay where they are and new rows take
+        // the slots of the rows that left.  (Rows L .. LP-1 hold what was there:
+        // V's and U's digits are zero in them.)
+        int base = 0;
+        auto slot = [&](int j) { return j + base < LP ? j + base : j + base - LP; };
+        uint32_t dz_phase = 0;          // bit q: the phase of chunk barrier q to wait for next
+        constexpr int CW = kCols5 / (kWork5 / 32);  // columns per warp in loads and stores
+        for (int k = 0; k < K; k++) {
+            const long long row0 = (long long)RF * ((long long)s0 + (long long)k * b);
+            if (!loaded) {
+                if (in_step(gave_up)) break;   // group g+1 has stored this tile's rows
+                // ---- window: new rows from global memory (through L2: rows written
+                // by other SMs)
+                const int jlo = (k == 0) ? 0 : CARRY;
+                constexpr int H = (L + 31) / 32, CL = H > 3 ? CW / 2 : CW;   // passes of 32 rows, columns at once
+#pragma unroll 1
+                for (int i0 = 0; i0 < CW; i0 += CL) {
+                    long long v[CL][H];
+#pragma unroll
+                    for (int i = 0; i < CL; i++) {
+                        const int cc = warp * CW + i0 + i;
+                        const long long *zc = Zi + (long long)(col0 + cc < nev ? col0 + cc : 0) * ldz;
+#pragma unroll
+                        for (int h = 0; h < H; h++) {
+                            const int j = jlo + lane + 32 * h;
+                            v[i][h] = (col0 + cc < nev && j < L && row0 + j < nrows) ? __ldcg(zc + row0 + j) : 0ll;
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < CL; i++)
+#pragma unroll
+                        for (int h = 0; h < H; h++) {
+                            const int j = jlo + lane + 32 * h;
+                            if (j < L) Zs[(warp * CW + i0 + i) * ZROW + slot(j)] = v[i][h];
+                        }
+                }
+                in_step(false);
+            }
+            // ---- Z digits: four rows per warp of a lane quarter and K step, step kk
+            // at columns (kk mod ZR) 64 + plane 8 + pair
+            const long long *zc = Zs + col * ZROW;
+#pragma unroll 1
+            for (int kk = 0; kk < KSTEPS; kk++) {
+                const int sl = kk % ZR, turns = (KSTEPS - sl + ZR - 1) / ZR;   // steps of a tile that take this place
+                // the products that read the place before (commit k turns + kk / ZR - 1)
+                if (kk >= ZR) gave_up |= !tc5_wait(bar_k + 8 * sl, (uint32_t)(k * turns + kk / ZR - 1) & 1, state);
+                tc5::fence_after_sync();
+                uint32_t w[kPlanes][2];
+                const long long *zr = zc + slot(kk * 16 + wq * 4);
+#pragma unroll
+                for (int p = 0; p < 2; p++) {
+                    const longlong2 z2 = *(const longlong2 *)(zr + 2 * p);
                     uint32_t d[kPlanes];
                     cut_pair(z2.x, z2.y, d);
 #pragma unroll
                     for (int s = 0; s < kPlanes; s++) w[s][p] = d[s];
                 }
 #pragma unroll
-                for (int s = 0; s < kPlanes; s++)
-                    tc5::st_x4(tmem + lane_off + Gm::T_ZD + ((u >> 1) - kk0) * 64 + s * 8 + (u & 1) * 4, w[s]);
-            }
-            tc5::wait_st();
-            if (r == 0) tc5_wait(bar_v, (uint32_t)(k & 1), state, sh);   // this tile's V planes
-            tc5::fence_before_sync();
-            __syncthreads();
-            if (sh.abort) break;
-            if (tid == 0) {
-                // one MMA per Z digit plane s and K step: B spans V planes
-                // 0 .. 8-s along N, so plane t lands in level s+t (D columns
-                // T_WACC + NB (s+t)); in the first K step level 8 is first
-                // written by its own MMA (s = 1, t = 7), every other level by s = 0
-                tc5::fence_after_sync();
-                const uint64_t vdesc = tc5::smem_desc(tc5::smem_addr(smem + Gm::S_V), 128, Gm::SBO_V);
-                for (int kk = kk0; kk < kk1; kk++)
-#pragma unroll
-                    for (int s = 0; s < kPlanes; s++) {
-                        const uint32_t a_t = tmem + Gm::T_ZD + (kk - kk0) * 64 + s * 8;
-                        const uint64_t b0 = vdesc + (uint64_t)((kk * 256) >> 4);
-                        const int nt = s == 0 ? kPlanes : kLevels5 - s;          // planes t = 0 .. nt-1
-                        if (kk == 0 && s == 1) {
-                            tc5::mma_tmem_a(tmem + Gm::T_WACC + NBC * 8, a_t, b0 + (uint64_t)((7 * Gm::VPLANE) >> 4),
-                                            tc5::idesc_f16_f32(128, NBC), 0u);
-                            tc5::mma_tmem_a(tmem + Gm::T_WACC + NBC, a_t, b0, tc5::idesc_f16_f32(128, NBC * 7), 1u);
-                        } else {
-                            tc5::mma_tmem_a(tmem + Gm::T_WACC + NBC * s, a_t, b0, tc5::idesc_f16_f32(128, NBC * nt),
-                                            (kk > 0 || s > 0) ? 1u : 0u);
-                        }
-                    }
-                tc5::commit(bar_mma);
-                // publish the previous tile while the products run: its stores
-                // happened before the barriers since, and the fence and release
-                // here make them visible at GPU scope before the flag
-                if (r == 0 && k > 0 && g + 1 != hold_group) {
-                    __threadfence();
-                    st_release(progress + (long long)g * C + c, k);
-                }
-            }
-        }
-        if (sh.abort) break;
-        mma_pending = true;
-        if (tc5_wait(bar_mma, mma_phase & 1, state, sh)) mma_pending = false;
-        mma_phase++;
-        tc5::fence_after_sync();
-        // the V buffer is free: request the next tile's V planes
-        if (tid == 0 && k + 1 < K) {
-            tc5::bulk_load(tc5::smem_addr(smem + Gm::S_V), rec_g + (size_t)(k + 1) * Gm::REC, Gm::VBYTES, bar_v);
-            v_issued = k + 2;
-        }
-        // ---- fold W's levels (reflectors q0 .. q0+NB/4-1 of this column), cut
-        // W into digit planes (TMEM: K step q/16, columns s*8 + (q%16)/2)
-        tc5_wait(bar_u, (uint32_t)(k & 1), state, sh);   // this tile's U part (row exponents)
-        {
-            constexpr int QW = NBC / 4;
-            const int q0 = wq * QW;
-            uint32_t a[kLevels5][QW];
-#pragma unroll
-            for (int l = 0; l < kLevels5; l++) {
-                if constexpr (QW == 8) {
-                    tc5::ld_x8(tmem + lane_off + Gm::T_WACC + NBC * l + q0, a[l]);
-                } else {
-                    tc5::ld_x4(tmem + lane_off + Gm::T_WACC + NBC * l + q0, a[l]);
-                }
-            }
-            tc5::wait_ld();
-            uint32_t wd[kPlanes][QW / 2];
-#pragma unroll
-            for (int p = 0; p < QW / 2; p++) {
-                long long wi[2];
-#pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    const int i = 2 * p + u;
-                    int Lv[kLevels5];
-                    // levels 0..2 stay below 2^22 (at most 3 pairs, the top
-                    // digits bounded by 32 and 64): one addition converts them
-#pragma unroll
-                    for (int l = 0; l < 3; l++) Lv[l] = (int)(magic_bits(a[l][i]) - kMagicBits);
-#pragma unroll
-                    for (int l = 3; l < kLevels5; l++) Lv[l] = __float2int_rn(__uint_as_float(a[l][i]));
-                    wi[u] = fold9(Lv, eV[q0 + i]);
-                }
-                uint32_t d[kPlanes];
-                cut_pair(wi[0], wi[1], d);
-#pragma unroll
-                for (int s = 0; s < kPlanes; s++) wd[s][p] = d[s];
-            }
-            // (the W digits go to the Z-digit columns, dead since the W
-            // products completed; the W levels stay untouched until the dZ
-            // products, issued after the barrier below)
-            const uint32_t wcol = Gm::T_WD + (q0 >> 4) * 64 + (q0 & 15) / 2;
-#pragma unroll
-            for (int s = 0; s < kPlanes; s++) {
-                if constexpr (QW == 8) {
-                    tc5::st_x4(tmem + lane_off + wcol + s * 8, wd[s]);
-                } else {
-                    tc5::st_x2(tmem + lane_off + wcol + s * 8, wd[s]);
-                }
-            }
-            tc5::wait_st();
-        }
-        tc5::fence_before_sync();
-        __syncthreads();
-        if (sh.abort) break;
-        // ---- dZ^T = W^T U^T by row chunks (M 128, N = rows x planes, K NB),
-        // folded into the window: Zs -= dZ
-#pragma unroll
-        for (int ch = 0; ch < Gm::CHUNKS; ch++) {
-            const int j0 = ch * Gm::NCH;
-            const int N = (LP - j0) < Gm::NCH ? (LP - j0) : Gm::NCH;
-            if (ch) {
+                for (int s = 0; s < kPlanes; s++) tc5::st_x2(tmem + lane_off + Gm::T_ZD + sl * 64 + s * 8 + wq * 2, w[s]);
+                tc5::wait_st();
                 tc5::fence_before_sync();
-                __syncthreads();  // the previous chunk's levels are read before they are overwritten
-                if (sh.abort) break;
+                workers_arrive(1 + kk);
             }
-            if (tid == 0) {
-                // per W digit plane s and K step one MMA whose B spans the
-                // chunk's U planes 0 .. 8-s along N (level l = s+t at D
-                // columns T_DZ + l N); level 8 first written alone (s = 1, t = 7)
-                tc5::fence_after_sync();
-                const uint64_t udesc =
-                    tc5::smem_desc(tc5::smem_addr(smem + Gm::S_U) + (uint32_t)j0 * Gm::SBO_U, 128, Gm::SBO_U);
-                const uint32_t pstride = (uint32_t)(N / 8) * Gm::SBO_U;   // bytes between the chunk's planes
-#pragma unroll
-                for (int kd = 0; kd < KD; kd++)
-#pragma unroll
-                    for (int s = 0; s < kPlanes; s++) {
-                        const uint32_t a_t = tmem + Gm::T_WD + kd * 64 + s * 8;
-                        const uint64_t b0 = udesc + (uint64_t)((kd * 256) >> 4);
-                        const int nt = s == 0 ? kPlanes : kLevels5 - s;
-                        if (kd == 0 && s == 1) {
-                            tc5::mma_tmem_a(tmem + Gm::T_DZ + 8 * N, a_t, b0 + (uint64_t)((7 * pstride) >> 4),
-                                            tc5::idesc_f16_f32(128, N), 0u);
-                            tc5::mma_tmem_a(tmem + Gm::T_DZ + N, a_t, b0, tc5::idesc_f16_f32(128, 7 * N), 1u);
-                        } else {
-                            tc5::mma_tmem_a(tmem + Gm::T_DZ + s * N, a_t, b0, tc5::idesc_f16_f32(128, nt * N),
-                                            (kd > 0 || s > 0) ? 1u : 0u);
-                        }
-                    }
-                tc5::commit(bar_mma);
+            {
+                constexpr int sl = (KSTEPS - 1) % ZR, turns = (KSTEPS - sl + ZR - 1) / ZR;
+                gave_up |= !tc5_wait(bar_k + 8 * sl, (uint32_t)(k * turns + (KSTEPS - 1) / ZR) & 1, state);
             }
-            mma_pending = true;
-            if (tc5_wait(bar_mma, mma_phase & 1, state, sh)) mma_pending = false;
-            mma_phase++;
             tc5::fence_after_sync();
-            // this thread: rows j0 + wq*N/4 .. +N/4 of its column (8 or 4),
-            // all levels fetched in one round of TMEM loads
-            long long *zw = Zs + col * ZROW;
-            const int jb = wq * (N / 4);
-            uint32_t a8[kLevels5][8];
-            if (N == 32) {
-#pragma unroll
-                for (int l = 0; l < kLevels5; l++) tc5::ld_x8(tmem + lane_off + Gm::T_DZ + l * N + jb, a8[l]);
-            } else {
+            // ---- fold W's levels (reflectors q0 .. q0+NB/4-1 of this column), cut
+            // W into digit planes (TMEM: K step q/16, columns s*8 + (q%16)/2)
+            gave_up |= !tc5_wait(bar_u, (uint32_t)(k & 1), state);   // this tile's U part (row exponents)
+            {
+                constexpr int QW = NBC / 4;
+                const int q0 = wq * QW;
+                uint32_t a[kLevels5][QW];
 #pragma unroll
                 for (int l = 0; l < kLevels5; l++) {
-                    uint32_t a4[4];
-                    tc5::ld_x4(tmem + lane_off + Gm::T_DZ + l * N + jb, a4);
-#pragma unroll
-                    for (int i = 0; i < 4; i++) a8[l][i] = a4[i];
+                    if constexpr (QW == 8) {
+                        tc5::ld_x8(tmem + lane_off + Gm::T_WACC + NBC * l + q0, a[l]);
+                    } else {
+                        tc5::ld_x4(tmem + lane_off + Gm::T_WACC + NBC * l + q0, a[l]);
+                    }
                 }
-            }
-            tc5::wait_ld();
+                tc5::wait_ld();
+                uint32_t wd[kPlanes][QW / 2];
 #pragma unroll
-            for (int p = 0; p < 4; p++) {
-                if (2 * p >= N / 4) break;
-                const int j = j0 + jb + 2 * p;
-                if (j >= L) continue;
-                long long dz[2];
+                for (int p = 0; p < QW / 2; p++) {
+                    long long wi[2];
 #pragma unroll
-                for (int u = 0; u < 2; u++) {
-                    uint32_t bits[kLevels5];
+                    for (int u = 0; u < 2; u++) {
+                        uint32_t f[kLevels5];
 #pragma unroll
-                    for (int l = 0; l < kLevels5; l++) bits[l] = magic_bits(a8[l][2 * p + u]);
-                    dz[u] = fold9_bits(bits, eU[j + u]);
+                        for (int l = 0; l < kLevels5; l++) f[l] = Gm::WMAGIC == 9 ? magic_bits(a[l][2 * p + u]) : a[l][2 * p + u];
+                        if constexpr (Gm::WMAGIC == 9) wi[u] = fold9_bits<false>(f, eV[q0 + 2 * p + u]);
+                        else wi[u] = fold9_big<Gm::WMAGIC>(f, eV[q0 + 2 * p + u]);
+                    }
+                    uint32_t d[kPlanes];
+                    cut_pair(wi[0], wi[1], d);
+#pragma unroll
+                    for (int s = 0; s < kPlanes; s++) wd[s][p] = d[s];
                 }
-                longlong2 *zp = (longlong2 *)(zw + j);
-                longlong2 z2 = *zp;
-                z2.x -= dz[0];
-                if (j + 1 < L) z2.y -= dz[1];
-                *zp = z2;
+                // (the W digits go to the Z-digit columns, dead since the W
+                // products completed; the W levels stay untouched until the dZ
+                // products, issued after the barrier below)
+                const uint32_t wcol = Gm::T_WD + (q0 >> 4) * 64 + (q0 & 15) / 2;
+#pragma unroll
+                for (int s = 0; s < kPlanes; s++) {
+                    if constexpr (QW == 8) {
+                        tc5::st_x4(tmem + lane_off + wcol + s * 8, wd[s]);
+                    } else {
+                        tc5::st_x2(tmem + lane_off + wcol + s * 8, wd[s]);
+                    }
+                }
+                tc5::wait_st();
             }
-        }
-        tc5::fence_before_sync();   // this tile's TMEM reads precede the next tile's TMEM writes
-        __syncthreads();
-        tc5::fence_after_sync();
-        if (sh.abort) break;
-        // the U part is consumed (planes by the MMAs, exponents by the folds
-        // above): request the next tile's (a thread other than the one that
-        // polls the dependency flags and issues the MMAs)
-        if (tid == 32 && k + 1 < K) {
-            tc5::fence_proxy_async_smem();
-            tc5::bulk_load(tc5::smem_addr(smem + Gm::S_U), rec_g + (size_t)(k + 1) * Gm::REC + Gm::VBYTES, Gm::UPART,
-                           bar_u);
-            sh.u_issued = k + 2;
-        }
-        // ---- store the rows final for this group (all rows after the last
-        // tile): all of a warp's shared-memory reads first, then the stores
-        {
-            constexpr int CW = kCols5 / (kThreads5 / 32);
-            constexpr int H = (L + 31) / 32;
+            tc5::fence_before_sync();
+            if (in_step(gave_up)) break;
+            // ---- dZ by chunks, folded into the window: Zs -= dZ
+            const bool far = *(const int *)(smem + Gm::S_U + Gm::U_FAR) != 0;
+#pragma unroll 1
+            for (int ch = 0; ch < Gm::CHUNKS; ch++) {
+                const int jb = ch * Gm::NCH + wq * (Gm::NCH / 4);
+                gave_up |= !tc5_wait(bar_dz + 8 * (ch & 1), (dz_phase >> (ch & 1)) & 1, state);
+                dz_phase ^= 1u << (ch & 1);
+                tc5::fence_after_sync();
+                // this thread: four rows of its column, all levels fetched in one
+                // round of TMEM loads
+                uint32_t a4[kLevels5][4];
+#pragma unroll
+                for (int l = 0; l < kLevels5; l++)
+                    tc5::ld_x4(tmem + lane_off + Gm::T_DZ + (ch & 1) * Gm::DZBUF + l * Gm::NCH + wq * (Gm::NCH / 4), a4[l]);
+                tc5::wait_ld();
+                tc5::fence_before_sync();
+                if (ch + 2 < Gm::CHUNKS) workers_arrive(1 + ch);
+                long long *zw = Zs + col * ZROW + slot(jb);
+                auto fold_rows = [&](auto FAR) {
+#pragma unroll
+                    for (int p = 0; p < 2; p++) {
+                        const int j = jb + 2 * p;
+                        if (j >= L) continue;
+                        long long dz[2];
+#pragma unroll
+                        for (int u = 0; u < 2; u++) {
+                            uint32_t bits[kLevels5];
+#pragma unroll
+                            for (int l = 0; l < kLevels5; l++) bits[l] = magic_bits(a4[l][2 * p + u]);
+                            dz[u] = fold9_bits<FAR.value>(bits, eU[j + u]);
+                        }
+                        longlong2 *zp = (longlong2 *)(zw + 2 * p);
+                        longlong2 z2 = *zp;
+                        z2.x -= dz[0];
+                        if (j + 1 < L) z2.y -= dz[1];
+                        *zp = z2;
+                    }
+                };
+                if (!far) fold_rows(Bool<false>{});
+                else fold_rows(Bool<true>{});
+            }
+            tc5::fence_before_sync();   // this tile's TMEM reads precede the next tile's TMEM writes
+            if (in_step(gave_up)) break;
+            tc5::fence_after_sync();
+            // ---- store the rows final for this group (all rows after the last
+            // tile), and bring in the next tile's new rows if they are there: per
+            // batch of the warp's columns the loads set out first, then the final
+            // rows leave, then the new rows take their slots (the same warp's, so
+            // no block barrier between the two).  HN > 2: two batches, to stay
+            // within 128 registers
+            constexpr int H = (L + 31) / 32, HN = (ADV + 31) / 32;
+            constexpr int CS = HN > 2 ? CW / 2 : CW;
+            loaded = sh.ready != 0;
             const int jhi = (k == K - 1) ? L : ADV;
-            long long v[CW][H];
-#pragma unroll
-            for (int i = 0; i < CW; i++)
-#pragma unroll
-                for (int h = 0; h < H; h++) {
-                    const int j = lane + 32 * h;
-                    v[i][h] = (j < jhi) ? Zs[(warp * CW + i) * ZROW + j] : 0ll;
-                }
+            const int base_n = base + ADV % LP < LP ? base + ADV % LP : base + ADV % LP - LP;
+            const int ncol = min(nev - col0 - warp * CW, CW);   // columns of this warp that there are
+            long long *zg0 = Zi + (long long)(col0 + warp * CW) * ldz + row0 + lane;
             bool bad = false;
+#pragma unroll 1
+            for (int i0 = 0; i0 < CW; i0 += CS) {
+                long long *zg = zg0 + i0 * ldz;
+                long long vn[CS][HN];
+                if (loaded) {
 #pragma unroll
-            for (int i = 0; i < CW; i++) {
-                const int cc = warp * CW + i;
-                if (col0 + cc >= nev) continue;
-                long long *zg = Zi + (long long)(col0 + cc) * ldz;
+                    for (int h = 0; h < HN; h++) {
+                        const bool ok = CARRY + lane + 32 * h < L && row0 + ADV + CARRY + lane + 32 * h < nrows;
+#pragma unroll
+                        for (int i = 0; i < CS; i++) {
+                            vn[i][h] = 0;
+                            if (ok && i0 + i < ncol) vn[i][h] = __ldcg(zg + i * ldz + ADV + CARRY + 32 * h);
+                        }
+                    }
+                }
+                // rows 32 h of several columns: shared-memory reads, then stores
 #pragma unroll
                 for (int h = 0; h < H; h++) {
-                    const int j = lane + 32 * h;
-                    if (j < jhi && row0 + j < nrows) {
-                        bad |= tc_out_of_range(v[i][h]);
-                        zg[row0 + j] = v[i][h];
+                    if (32 * h >= jhi) break;
+                    const bool ok = lane + 32 * h < jhi && row0 + lane + 32 * h < nrows;
+                    const long long *zs = Zs + (warp * CW + i0) * ZROW + slot(min(lane + 32 * h, LP - 1));
+                    long long v[CS];
+#pragma unroll
+                    for (int i = 0; i < CS; i++) v[i] = zs[i * ZROW];
+                    if (ok) {
+                        bool any = false;   // a high word at or beyond the limit: a cheap superset
+#pragma unroll
+                        for (int i = 0; i < CS; i++)
+                            if (i0 + i < ncol) {
+                                any |= (uint32_t)((int)(v[i] >> 32) + 0x1fffffff) >= 0x3fffffffu;
+                                zg[i * ldz + 32 * h] = v[i];
+                            }
+                        if (any)
+                            for (int i = 0; i < CS; i++) bad |= i0 + i < ncol && tc_out_of_range(v[i]);
+                    }
+                }
+                if (loaded) {
+                    __syncwarp();
+#pragma unroll
+                    for (int h = 0; h < HN; h++) {
+                        const int j = CARRY + lane + 32 * h;   // its slot in the next tile's window
+                        long long *zs = Zs + (warp * CW + i0) * ZROW + (j + base_n < LP ? j + base_n : j + base_n - LP);
+                        if (j < L) {
+#pragma unroll
+                            for (int i = 0; i < CS; i++) zs[i * ZROW] = vn[i][h];
+                        }
                     }
                 }
             }
             if (bad) tc_set_error(state, GB_ERR_RANGE);
-        }
-        // every thread's stores happen before thread 0's fence and release
-        // (barrier, then a cumulative release at GPU scope); the release of
-        // tile k is issued during tile k+1 (after its products are issued),
-        // that of the item's last tile right here
-        __syncthreads();
-        if (tid == 0 && k == K - 1 && g + 1 != hold_group) {
-            __threadfence();
-            st_release(progress + (long long)g * C + c, k + 1);
+            base = base_n;
+            in_step(false);
         }
     }
     // ---- leave: no copy or MMA of this CTA may still be in flight when its
     // TMEM is released (bounded waits; a timeout was already recorded)
     __syncthreads();
-    if (tid == 0) {
+    if (warp == kWork5 / 32) {
         if (v_issued > 0) tc5::mbar_wait(bar_v, (uint32_t)((v_issued - 1) & 1), kMbarTimeoutNs);
-        if (sh.u_issued > 0) tc5::mbar_wait(bar_u, (uint32_t)((sh.u_issued - 1) & 1), kMbarTimeoutNs);
+        if (u_issued > 0) tc5::mbar_wait(bar_u, (uint32_t)((u_issued - 1) & 1), kMbarTimeoutNs);
+        __syncwarp();
+        if (tc5::elect_one()) tc5::commit(bar_end);   // after every MMA of this block (the same lane issued them all)
+        tc5::mbar_wait(bar_end, 0, kMbarTimeoutNs);
     }
-    if (mma_pending) tc5::mbar_wait(bar_mma, (mma_phase - 1) & 1, kMbarTimeoutNs);
     tc5::fence_before_sync();
     __syncthreads();
     if (warp == 0) {
         tc5::fence_after_sync();
-        tc5::tmem_dealloc(tmem, kTmemCols);
+        tc5::tmem_dealloc(*(volatile uint32_t *)tmem_slot, kTmemCols);
     }
 }
 
@@ -1043,7 +1222,23 @@ cudaError_t run_tc5(int n, int nev, const double *hh_v, const double *hh_tau, do
     if ((e = cudaFuncSetAttribute(pipeline_tc5<B, RF>, cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::SMEM)) !=
         cudaSuccess)
         return e;
-    const int want = column_batch > 0 ? column_batch : kColumnBatch5;
+    // Column blocks per ticket batch: at least kColumnBatch5, and as many as make a
+    // batch's work (CB groups x tiles over the SMs) twice the chain of its
+    // groups (a tile each, then the longest group's tiles), in equal batches:
+    // n = 4096, 20 blocks: 10.0 ms in one batch, 11.5 in batches of 8; complex, 10
+    // blocks: 25.1 against 36.2; n = 16384: 8 (218 ms; 32 blocks at once, which
+    // re-read Z more, 220)
+    int want = column_batch;
+    if (want <= 0) {
+        int dev = 0, sms = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+        const long long Kmax = group_tiles(n, B, Gm::NB, 0);
+        const long long chain = (4LL * sms * (G + Kmax) + (long long)G * Kmax - 1) / ((long long)G * Kmax);
+        const long long least = chain > kColumnBatch5 ? chain : kColumnBatch5;
+        const int batches = (int)(C / least > 1 ? C / least : 1);
+        want = (C + batches - 1) / batches;
+    }
     const int CB = C < want ? C : want;
     if ((e = mark_kernel_begin(st)) != cudaSuccess) return e;
     pipeline_tc5<B, RF><<<(unsigned)G * (unsigned)C, kThreads5, Gm::SMEM, st>>>(
