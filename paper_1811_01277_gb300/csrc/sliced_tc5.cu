@@ -32,11 +32,11 @@
 // What bounds it: 36 x 2 m n k FP16 flops at the tensor rate for long k; HBM
 // traffic of C and of the digit planes (16 bytes per entry) for k <= 128.
 // Measured on a GB300 (whole calls, slicing included; before: the same scheme
-// on bf16 mma.sync, 43 pairs of 7-bit digits): 8192^3 139.8 -> 23.1 ms (47.7
-// TFLOP/s of FP64, 0.89 of the tensor rate over 36), 4096^3 17.9 -> 3.2 ms,
-// 3001 x 1777 x 4099 6.14 -> 1.28 ms; the n = 16320 panel products of a
+// on bf16 mma.sync, 43 pairs of 7-bit digits): 8192^3 139.8 -> 22.8 ms (48.2
+// TFLOP/s of FP64, 0.90 of the tensor rate over 36), 4096^3 17.9 -> 3.2 ms,
+// 3001 x 1777 x 4099 6.14 -> 1.26 ms; the n = 16320 panel products of a
 // solver: symmetric x 64 columns 9.0 -> 2.3 ms (1.4 of it slicing, HBM-bound),
-// rank-128 update 7.9 -> 1.9 ms; 64 x 4096, k = 16384 2.3 -> 0.78 ms.  Error
+// rank-128 update 7.9 -> 1.8 ms; 64 x 4096, k = 16384 2.3 -> 0.78 ms.  Error
 // against 64-bit references 1.2e-15 to 3.0e-15, as before.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -408,11 +408,13 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                     tc5::mbar_wait(tc5::smem_addr(&sy.full[i & 1]), (i >> 1) & 1, kWaitNs);
             }
         } else if (warp == kFoldWarps + 1) {
-            // ---- MMAs
-            if (lane == 0) {
+            // ---- MMAs (the warp together, an elected lane issuing: see tcgen05.cuh)
+            {
                 uint32_t q = 0, grp = 0;
                 bool ok = true;
+                auto wait_all = [&](auto *bar, uint32_t n) { return __all_sync(0xffffffffu, wait5(bar, n, sy)) != 0; };
                 auto mmas = [&](uint32_t st, bool high, bool first) {
+                    if (!tc5::elect_one()) return;
                     const uint32_t sa = tc5::smem_addr(smem + st * kStageBytes);
                     const uint64_t da = tc5::smem_desc(sa, 128, kSbo), db = tc5::smem_desc(sa + kBlockBytes, 128, kSbo);
 #pragma unroll
@@ -434,31 +436,35 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                     const Tile x = tile_of(p, t);
                     for (int kc = x.kc0; ok && kc < x.kc1; kc += kGroup, grp++) {
                         const int ns = min(kGroup, x.kc1 - kc), first = min(ns, 2);
-                        if (grp > 0 && !wait5(&sy.freed[0], grp - 1, sy)) { ok = false; break; }
+                        if (grp > 0 && !wait_all(&sy.freed[0], grp - 1)) { ok = false; break; }
                         tc5::fence_after_sync();
                         for (int c = 0; c < first && ok; c++) {
-                            if (!wait5(&sy.full[(q + c) & 1], (q + c) >> 1, sy)) { ok = false; break; }
+                            if (!wait_all(&sy.full[(q + c) & 1], (q + c) >> 1)) { ok = false; break; }
                             tc5::fence_after_sync();
                             mmas((q + c) & 1, false, c == 0);
-                            if (c == ns - 1) tc5::commit(tc5::smem_addr(&sy.ready[0]));
+                            __syncwarp();
+                            if (c == ns - 1 && tc5::elect_one()) tc5::commit(tc5::smem_addr(&sy.ready[0]));
                         }
                         if (!ok) break;
-                        if (grp > 0 && !wait5(&sy.freed[1], grp - 1, sy)) { ok = false; break; }
+                        if (grp > 0 && !wait_all(&sy.freed[1], grp - 1)) { ok = false; break; }
                         tc5::fence_after_sync();
                         for (int c = 0; c < first; c++) {
                             mmas((q + c) & 1, true, c == 0);
-                            tc5::commit(tc5::smem_addr(&sy.empty[(q + c) & 1]));
+                            __syncwarp();
+                            if (tc5::elect_one()) tc5::commit(tc5::smem_addr(&sy.empty[(q + c) & 1]));
                         }
                         for (int c = first; c < ns; c++) {
-                            if (!wait5(&sy.full[(q + c) & 1], (q + c) >> 1, sy)) { ok = false; break; }
+                            if (!wait_all(&sy.full[(q + c) & 1], (q + c) >> 1)) { ok = false; break; }
                             tc5::fence_after_sync();
                             mmas((q + c) & 1, false, false);
-                            if (c == ns - 1) tc5::commit(tc5::smem_addr(&sy.ready[0]));
+                            __syncwarp();
+                            if (c == ns - 1 && tc5::elect_one()) tc5::commit(tc5::smem_addr(&sy.ready[0]));
                             mmas((q + c) & 1, true, false);
-                            tc5::commit(tc5::smem_addr(&sy.empty[(q + c) & 1]));
+                            __syncwarp();
+                            if (tc5::elect_one()) tc5::commit(tc5::smem_addr(&sy.empty[(q + c) & 1]));
                         }
                         if (!ok) break;
-                        tc5::commit(tc5::smem_addr(&sy.ready[1]));
+                        if (tc5::elect_one()) tc5::commit(tc5::smem_addr(&sy.ready[1]));
                         q += ns;
                     }
                 }
@@ -466,7 +472,7 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                 // fold warps have waited for the last group; after a failure,
                 // wait here (bounded)
                 if (!ok) {
-                    tc5::commit(tc5::smem_addr(&sy.empty[q & 1]));
+                    if (tc5::elect_one()) tc5::commit(tc5::smem_addr(&sy.empty[q & 1]));
                     for (long long i = 0; i < 100000; i++) __nanosleep(100);
                 }
             }
