@@ -67,8 +67,8 @@
 // 4096 takes 25.8 thousand clocks (34.3 with everything in the same 16 warps and
 // K steps and chunks in series): cuts and the first product 6.1, folding
 // and cutting W 3.2, the second product and its folds 10.1, loads and
-// stores 5.0.  Whole calls: n = 16384, nev = 4096 261 -> 193 ms; complex n = 4096,
-// nev = 1228 37.1 -> 20.5; n = nev = 1024, nbw = 32 (a chain of 64 groups) 1.24 -> 0.92.
+// stores 5.0.  Whole calls: n = 16384, nev = 4096 261 -> 184 ms; complex n = 4096,
+// nev = 1228 37.1 -> 20.5; n = nev = 1024, nbw = 32 (a chain of 64 groups) 1.24 -> 0.91.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -301,12 +301,22 @@ __device__ __forceinline__ long long fixed_row(double x, int e)
 
 // ---- per-tile records ------------------------------------------------------
 
+// The digit planes of eight values that are neighbours along K: 16 bytes a plane
+__device__ __forceinline__ void put_octet(unsigned char *dst, int plane_stride, const long long (&x)[8])
+{
+    uint32_t w[4][kPlanes];
+#pragma unroll
+    for (int i = 0; i < 4; i++) cut_pair(x[2 * i], x[2 * i + 1], w[i]);
+#pragma unroll
+    for (int t = 0; t < kPlanes; t++)
+        *(uint4 *)(dst + t * plane_stride) = make_uint4(w[0][t], w[1][t], w[2][t], w[3][t]);
+}
+
 template <int B>
 constexpr size_t prep_smem_bytes()
 {
     using Gm = Geo<B, 1>;
-    return (size_t)(2 * Gm::LP * (Gm::NB + 1) + 2 * Gm::NB * (Gm::NB + 1) + 2 * Gm::NB) * 8 +
-           (size_t)(Gm::NB + Gm::LP) * 4;
+    return (size_t)(2 * Gm::LP * (Gm::NB + 1) + Gm::NB * (Gm::NB + 1) + 3 * Gm::NB) * 8 + (size_t)(Gm::NB + Gm::LP) * 4;
 }
 
 template <int B>
@@ -317,8 +327,12 @@ constexpr size_t prep_smem_bytes_z()
            (size_t)(Gm::NB + Gm::LC) * 4;
 }
 
+// The records of a real band (65 thousand tiles at n = 16384).  Bounded by the FP64
+// pipe, two multiply-adds per clock and SM: 40 thousand clocks a tile for b = 64
+// (Gram 13, substitution 24), 22.7 -> 14 ms at n = 16384 against a Gram matrix and
+// a product V T with half of the lanes idle and T by a chain of 32 steps.
 template <int B>
-__global__ void __launch_bounds__(256) tc5_tile_prep(int n, const double *__restrict__ hh_v,
+__global__ void __launch_bounds__(256, 2) tc5_tile_prep(int n, const double *__restrict__ hh_v,
                                                      const double *__restrict__ hh_tau,
                                                      const long long *__restrict__ off,
                                                      unsigned char *__restrict__ rec)
@@ -331,11 +345,11 @@ __global__ void __launch_bounds__(256) tc5_tile_prep(int n, const double *__rest
     extern __shared__ double psm[];
     double *V = psm;                      // [LP][NB1]
     double *U = V + LP * NB1;             // [LP][NB1]
-    double *T = U + LP * NB1;             // [NB][NB1]
-    double *Gr = T + NB * NB1;            // [NB][NB1]
+    double *Gr = U + LP * NB1;            // [NB][NB1]
     double *tau = Gr + NB * NB1;          // [NB]
-    double *nv = tau + NB;                // [NB]
-    int *seV = (int *)(nv + NB);          // [NB]
+    double *nv = tau + NB;                // [NB] column norms of V, and their inverses
+    double *rn = nv + NB;                 // [NB]
+    int *seV = (int *)(rn + NB);          // [NB]
     int *seU = seV + NB;                  // [LP]
     const int s0 = 1 + g * NB;
     // reflector q of the tile occupies window rows q .. q+len-1 of column q
@@ -357,58 +371,52 @@ __global__ void __launch_bounds__(256) tc5_tile_prep(int n, const double *__rest
         tau[threadIdx.x] = (s <= n - 1 && s + k * b < n) ? hh_tau[sweep_first(n, b, s) + k] : 0.0;
     }
     __syncthreads();
-    // Gram matrix (upper triangle), T by the forward recurrence
-    // T(q,q) = tau_q, T(0:q,q) = -tau_q T(0:q,0:q) V(:,0:q)^T v_q
-    for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
-        const int p = e / NB, q = e % NB;
+    // Gram matrix (upper triangle): diagonals d and NB - d together make rows of
+    // NB products of like length, so that no lane idles on the FP64 pipe
+    for (int e = threadIdx.x; e < NB * (NB / 2 + 1); e += blockDim.x) {
+        const int d = e / NB, i = e % NB;                    // d = 0: the squares
+        const int p = i < NB - d ? i : i - (NB - d), q = i < NB - d ? i + d : p + NB - d;
+        if (2 * d == NB && i >= NB / 2) continue;
         double a = 0.0;
-        if (p < q)
-            for (int j = q; j < min(p + b, LP); j++) a = fma(V[j * NB1 + p], V[j * NB1 + q], a);
+        for (int j = q; j < min(p + b, LP); j++) a = fma(V[j * NB1 + p], V[j * NB1 + q], a);
         Gr[p * NB1 + q] = a;
     }
     __syncthreads();
-    for (int q = 0; q < NB; q++) {
-        if (threadIdx.x < NB) {
-            const int i = threadIdx.x;
-            double t = 0.0;
-            if (i < q) {
-                for (int p = i; p < q; p++) t = fma(T[i * NB1 + p], Gr[p * NB1 + q], t);
-                t = -tau[q] * t;
-            } else if (i == q) {
-                t = tau[q];
-            }
-            T[i * NB1 + q] = t;
-        }
-        __syncthreads();
-    }
-    // U = V T; V(j, p) vanishes outside p <= j < p + b
-    for (int e = threadIdx.x; e < LP * NB; e += blockDim.x) {
-        const int j = e / NB, q = e % NB;
-        double a = 0.0;
-        for (int p = max(0, j - b + 1); p <= min(q, j); p++) a = fma(V[j * NB1 + p], T[p * NB1 + q], a);
-        U[j * NB1 + q] = a;
-    }
-    // unit columns of V (U rescaled to keep U V^T): |v_q^T z| <= ||z||, so W
-    // stays inside the column's fixed-point range whatever tau is
     if (threadIdx.x < NB) {
-        const int q = threadIdx.x;
-        double a = 0.0;
-        for (int j = q; j < min(q + b, LP); j++) a = fma(V[j * NB1 + q], V[j * NB1 + q], a);
-        nv[q] = sqrt(a);
-        Gr[q] = a > 0.0 ? 1.0 / nv[q] : 0.0;  // the Gram matrix is no longer needed
+        const double a = Gr[threadIdx.x * NB1 + threadIdx.x];
+        nv[threadIdx.x] = a > 0.0 ? sqrt(a) : 1.0;
+        rn[threadIdx.x] = a > 0.0 ? 1.0 / nv[threadIdx.x] : 1.0;
     }
     __syncthreads();
-    // one division per column, not per entry (the FP64 pipe bounds this kernel)
-    for (int e = threadIdx.x; e < LP * NB; e += blockDim.x) {
-        const int j = e / NB, q = e % NB;
-        if (nv[q] > 0.0) {
-            V[j * NB1 + q] = V[j * NB1 + q] * Gr[q];
-            U[j * NB1 + q] = U[j * NB1 + q] * nv[q];
+    // U T^{-1} = V with T^{-1} = D^{-1} + the strict upper part of V^T V (D the
+    // taus), row by row: u_p = tau_p (v_p - sum_{q<p} u_q G_qp).  A thread keeps its
+    // row's sums in registers; the rows take three warps, a different three from tile to
+    // tile (each scheduler has a quarter of the FP64 pipe).  Then unit columns of V
+    // (U rescaled to keep U V^T): |v_q^T z| <= ||z||, so W stays inside the
+    // column's fixed-point range whatever tau is.
+    bool far = false;
+    unsigned char *ru = rec + ((size_t)off[g] + k) * Gm::REC + Gm::VBYTES;
+    const int row = (int)((threadIdx.x + 32u * (blockIdx.x + blockIdx.y)) % blockDim.x);
+    if (row < LP) {
+        double a[NB] = {};   // sum_{q<p} u_q G_qp of the columns p to come
+        unsigned long long m = 0;
+#pragma unroll
+        for (int p = 0; p < NB; p++) {
+            const double v = V[row * NB1 + p], u = tau[p] * (v - a[p]);
+#pragma unroll
+            for (int q = p + 1; q < NB; q++) a[q] = fma(u, Gr[p * NB1 + q], a[q]);
+            const double us = u * nv[p];
+            const unsigned long long w = (unsigned long long)__double_as_longlong(us) & ~(1ull << 63);
+            m = w > m ? w : m;
+            U[row * NB1 + p] = us;
+            V[row * NB1 + p] = v * rn[p];
         }
+        seU[row] = max(exponent_above(m), kMinExp);
+        far = seU[row] > 13;
+        ((FoldConst *)(ru + Gm::U_EU))[row] = fold_const(seU[row], kLoBias);
     }
     __syncthreads();
     unsigned char *r = rec + ((size_t)off[g] + k) * Gm::REC;
-    unsigned char *ru = r + Gm::VBYTES;
     if (threadIdx.x < NB) {
         unsigned long long m = 0;
         for (int j = 0; j < LP; j++) {
@@ -417,17 +425,6 @@ __global__ void __launch_bounds__(256) tc5_tile_prep(int n, const double *__rest
         }
         seV[threadIdx.x] = max(exponent_above(m), kMinExp);
         ((FoldConst *)(ru + Gm::U_EV))[threadIdx.x] = fold_const(seV[threadIdx.x], Gm::WMAGIC == 9 ? kLoBias : kLoBias4);
-    }
-    bool far = false;
-    for (int j = threadIdx.x; j < LP; j += blockDim.x) {
-        unsigned long long m = 0;
-        for (int q = 0; q < NB; q++) {
-            const unsigned long long u = (unsigned long long)__double_as_longlong(U[j * NB1 + q]) & ~(1ull << 63);
-            m = u > m ? u : m;
-        }
-        seU[j] = max(exponent_above(m), kMinExp);
-        far |= seU[j] > 13;
-        ((FoldConst *)(ru + Gm::U_EU))[j] = fold_const(seU[j], kLoBias);
     }
     const int any_far = __syncthreads_or(far);
     if (threadIdx.x == 0) *(int *)(ru + Gm::U_FAR) = any_far;
@@ -439,24 +436,21 @@ __global__ void __launch_bounds__(256) tc5_tile_prep(int n, const double *__rest
     // within it plane t at t (rows of the chunk / 8) SBO_U, then
     // (j%16/8) SBO_U + (q/8) 128 + (j%8) 16 + (q%8) 2 (again the planes of a
     // chunk contiguous along N)
-    for (int e = threadIdx.x; e < NB * LP; e += blockDim.x) {
-        const int q = e / LP, j = e % LP;
-        const unsigned long long y = (unsigned long long)fixed_row(V[j * NB1 + q], seV[q]) + kDigitBias;
-        const int o = (q >> 3) * Gm::SBO_V + (j >> 3) * 128 + (q & 7) * 16 + (j & 7) * 2;
+    for (int e = threadIdx.x; e < NB * (LP / 8); e += blockDim.x) {
+        const int q = e % NB, jo = e / NB;
+        long long x[8];
 #pragma unroll
-        for (int t = 0; t < kPlanes; t++)
-            *(__half *)(r + t * Gm::VPLANE + o) = __float2half_rn((float)((int)((y >> (56 - 8 * t)) & 0xff) - 128));
+        for (int i = 0; i < 8; i++) x[i] = fixed_row(V[(jo * 8 + i) * NB1 + q], seV[q]);
+        put_octet(r + (q >> 3) * Gm::SBO_V + jo * 128 + (q & 7) * 16, Gm::VPLANE, x);
     }
-    for (int e = threadIdx.x; e < LP * NB; e += blockDim.x) {
-        const int j = e / NB, q = e % NB;
-        const unsigned long long y = (unsigned long long)fixed_row(U[j * NB1 + q], seU[j]) + kDigitBias;
-        const int ch = j / Gm::NCH, rows = min(Gm::NCH, LP - ch * Gm::NCH);
-        const int o = ch * Gm::NCH * Gm::SBO_U + ((j % Gm::NCH) >> 3) * Gm::SBO_U + (q >> 3) * 128 + (j & 7) * 16 +
-                      (q & 7) * 2;
+    for (int e = threadIdx.x; e < LP * (NB / 8); e += blockDim.x) {
+        const int j = e % LP, qo = e / LP;
+        long long x[8];
 #pragma unroll
-        for (int t = 0; t < kPlanes; t++)
-            *(__half *)(ru + t * (rows / 8) * Gm::SBO_U + o) =
-                __float2half_rn((float)((int)((y >> (56 - 8 * t)) & 0xff) - 128));
+        for (int i = 0; i < 8; i++) x[i] = fixed_row(U[j * NB1 + qo * 8 + i], seU[j]);
+        put_octet(ru + j / Gm::NCH * Gm::NCH * Gm::SBO_U + ((j % Gm::NCH) >> 3) * Gm::SBO_U + qo * 128 +
+                      (j & 7) * 16,
+                  Gm::NCH / 8 * Gm::SBO_U, x);
     }
 }
 
@@ -603,38 +597,30 @@ __global__ void __launch_bounds__(256) tc5_tile_prep_z(int n, const double2 *__r
     if (threadIdx.x == 0) *(int *)(ru + Gm::U_FAR) = any_far;
     // V' (N = q' = 2q+p', K = j' = 2j+p) and the second product's B
     // (N = j', K = q'), in the layouts of the real record
-    for (int e = threadIdx.x; e < NBC * LP; e += blockDim.x) {
-        const int qq = e / LP, jj = e % LP;
-        const int q = qq >> 1, pq = qq & 1, j = jj >> 1, pj = jj & 1;
-        double x = 0.0;
-        if (j < LC) {
-            const double2 v = V[j * NB1 + q];
-            x = (pj == pq) ? v.x : (pj ? v.y : -v.y);
-        }
-        const unsigned long long y = (unsigned long long)fixed_row(x, seV[q]) + kDigitBias;
-        const int o = (qq >> 3) * Gm::SBO_V + (jj >> 3) * 128 + (qq & 7) * 16 + (jj & 7) * 2;
+    for (int e = threadIdx.x; e < NBC * (LP / 8); e += blockDim.x) {
+        const int qq = e % NBC, jo = e / NBC, q = qq >> 1;
+        long long x[8];
 #pragma unroll
-        for (int t = 0; t < kPlanes; t++)
-            *(__half *)(r + t * Gm::VPLANE + o) = __float2half_rn((float)((int)((y >> (56 - 8 * t)) & 0xff) - 128));
+        for (int i = 0; i < 8; i += 2) {      // the two real rows of complex row j
+            const int j = jo * 4 + i / 2;
+            const double2 v = j < LC ? V[j * NB1 + q] : zero;
+            x[i] = fixed_row((qq & 1) ? -v.y : v.x, seV[q]);
+            x[i + 1] = fixed_row((qq & 1) ? v.x : v.y, seV[q]);
+        }
+        put_octet(r + (qq >> 3) * Gm::SBO_V + jo * 128 + (qq & 7) * 16, Gm::VPLANE, x);
     }
-    for (int e = threadIdx.x; e < LP * NBC; e += blockDim.x) {
-        const int jj = e / NBC, qq = e % NBC;
-        const int q = qq >> 1, pq = qq & 1, j = jj >> 1, pj = jj & 1;
-        double x = 0.0;
-        int ev = kMinExp;
-        if (j < LC) {
-            const double2 u = U[j * NB1 + q];
-            x = (pj == pq) ? u.x : (pq ? -u.y : u.y);
-            ev = seU[j];
-        }
-        const unsigned long long y = (unsigned long long)fixed_row(x, ev) + kDigitBias;
-        const int ch = jj / Gm::NCH, rows = min(Gm::NCH, LP - ch * Gm::NCH);
-        const int o = ch * Gm::NCH * Gm::SBO_U + ((jj % Gm::NCH) >> 3) * Gm::SBO_U + (qq >> 3) * 128 + (jj & 7) * 16 +
-                      (qq & 7) * 2;
+    for (int e = threadIdx.x; e < LP * (NBC / 8); e += blockDim.x) {
+        const int jj = e % LP, qo = e / LP, j = jj >> 1;
+        const int ev = j < LC ? seU[j] : kMinExp;
+        long long x[8];
 #pragma unroll
-        for (int t = 0; t < kPlanes; t++)
-            *(__half *)(ru + t * (rows / 8) * Gm::SBO_U + o) =
-                __float2half_rn((float)((int)((y >> (56 - 8 * t)) & 0xff) - 128));
+        for (int i = 0; i < 8; i += 2) {
+            const double2 u = j < LC ? U[j * NB1 + qo * 4 + i / 2] : zero;
+            x[i] = fixed_row((jj & 1) ? u.y : u.x, ev);
+            x[i + 1] = fixed_row((jj & 1) ? u.x : -u.y, ev);
+        }
+        put_octet(ru + jj / Gm::NCH * Gm::NCH * Gm::SBO_U + ((jj % Gm::NCH) >> 3) * Gm::SBO_U + qo * 128 + (jj & 7) * 16,
+                  Gm::NCH / 8 * Gm::SBO_U, x);
     }
 }
 
