@@ -64,7 +64,9 @@ extern "C" {
                                   {16,32,64} and n >= 512, else PIPELINE for real
                                   data with nbw in {8,16,32,64}, else WAVEFRONT */
 #define GB_VARIANT_WAVEFRONT 1 /* one launch per anti-diagonal of the tile DAG */
-#define GB_VARIANT_PIPELINE 2  /* one persistent launch, tiles ordered by flags */
+#define GB_VARIANT_PIPELINE 2  /* one persistent launch, tiles ordered by flags; with the
+                                  default blocking, few columns take 32-column blocks
+                                  with four lanes a column */
 #define GB_VARIANT_PIPELINE_TC 3 /* the pipeline's schedule with every tile applied in
                                     compact WY form on the bf16 tensor cores (exact
                                     digit slicing, Z in per-column 64-bit fixed point
@@ -260,7 +262,7 @@ int gb_band_to_tridi_z(int n, int nbw, const double *AB, int ldab, double *d, do
  * FP32; the low-precision half of gb_solve_mixed_d) and GB_SOLVE_FP64_EMULATED_GEMM (accepted and ignored:
  * no product of either solver goes through a vendor BLAS).  By
  * default the large products (the full->band SYMM and SYR2K, the band->full
- * GEMMs, the Newton-Schulz SYRK and SYMM) run on the bf16 tensor cores by
+ * GEMMs, the Newton-Schulz SYRK and SYMM) run on the tcgen05 tensor cores by
  * exact digit slicing (gb_dgemm_sliced below); GB_SOLVE_DFMA_PRODUCTS runs
  * them on the FP64 FMA pipe instead.  Asynchronous; device-side status of
  * the dependency waits through gb_solve_query. */
@@ -280,7 +282,7 @@ int gb_solve_query(const void *workspace, int n, int nev, int nbw, void *stream)
  * same arguments, workspace rule (gb_solve_workspace_bytes_z) and flags as
  * gb_solve_d (GB_SOLVE_RECORD_STAGES is ignored; GB_SOLVE_FP32_PRODUCTS is
  * refused with -12: the mixed-precision solve is real only).  The large complex
- * products run sliced on the bf16 tensor cores (GB_SOLVE_DFMA_PRODUCTS:
+ * products run sliced on the tcgen05 tensor cores (GB_SOLVE_DFMA_PRODUCTS:
  * on the FP64 FMA pipe), the b x b panel products in this library's complex
  * DFMA kernel, and the back-transformation on the tcgen05 tensor cores
  * (nbw in {16, 32, 64}, n >= 512).  Device-side status of the waits of the
@@ -348,7 +350,7 @@ size_t gb_solve_batched_workspace_bytes(int count, const int *n, const int *nev,
  * get a Rayleigh-Ritz rotation X_J <- X_J G_JJ^(-1/2) Y_J (Y_J the
  * eigenvectors of G_JJ^(-1/2) S_JJ G_JJ^(-1/2)), and E is taken in the
  * rotated basis (r / 2 inside a cluster).  The products are sliced on the
- * bf16 tensor cores (FP64-accurate; 6 n^3 flops a step: X^T X and
+ * tcgen05 tensor cores (FP64-accurate; 6 n^3 flops a step: X^T X and
  * X^T (A X) on their lower triangles); ||A||_2 is taken as max |lambda_i|,
  * the other norms bounded by Frobenius norms.
  * Arguments (device pointers): 1 n >= 1; 2 A (n x n symmetric, lower
@@ -551,7 +553,7 @@ gb_autotune *gb_autotune_load(const char *path);
 
 /* FP64 matrix products (column-major, device pointers, asynchronous on
  * `stream`).  The paper's solver hands these steps to BLAS (Sec. 3.2: the
- * GPU version calls cuBLAS for the matrix products of the reduction and the
+ * GPU version calls a vendor BLAS for the matrix products of the reduction and the
  * back-transformations); here they run in this library's DFMA-tiled kernels,
  * which the solver uses internally.  `workspace` (8-byte aligned, or NULL
  * with ws_bytes 0) holds split-K partial products: a call splits the
@@ -578,13 +580,13 @@ int gb_dsyr2k(int n, int k, double alpha, const double *A, int lda, const double
 int gb_dsyrk(int n, int k, double alpha, const double *A, int lda, double beta, double *C, int ldc,
              void *stream);
 
-/* The same products computed on the bf16 tensor cores: every row of op(A)
+/* The same products computed on the tcgen05 tensor cores: every row of op(A)
  * and every column of op(B) is scaled by a power of two and cut exactly into
- * eight 7-bit digits (error-free splitting, Ozaki, Ogita, Oishi and Rump,
- * Numer. Algorithms 59, 2012); digit-plane products are formed with
- * mma.sync bf16, accumulated exactly (one FP32 accumulator per digit level,
- * exact over 128 values of k, folded into 64-bit integers), and the result
- * is rounded to FP64 once.  Accuracy is that of an FP64 product measured
+ * eight balanced base-256 digits in FP16 (error-free splitting, Ozaki, Ogita,
+ * Oishi and Rump, Numer. Algorithms 59, 2012); digit-plane products are formed
+ * with tcgen05.mma, accumulated exactly (one FP32 accumulator per digit level
+ * in tensor memory, exact over 128 values of k, folded into 96-bit integers),
+ * and the result is rounded to FP64 once.  Accuracy is that of an FP64 product measured
  * against the scaled maxima: |C - alpha op(A) op(B)| <~ 2^-53 k |alpha|
  * max_j |op(A)_ij| max_i |op(B)_ij| per entry.  Inputs must be finite;
  * subnormal inputs are read as zero.  The paper's products are BLAS calls

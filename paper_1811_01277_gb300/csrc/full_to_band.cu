@@ -1,7 +1,7 @@
 // Device kernels of the full -> band reduction (the first step of the
 // two-stage reduction, Sec. 2) and of the band -> full back-transformation:
 // Householder QR of a tall panel, the block-reflector T matrix, and the
-// small conversions around the GEMMs (which run in cuBLAS, see solve.cu).
+// small conversions around the products (solve.cu).
 //
 // Panel QR (m x nb, column-major, leading dimension lda): panel_qr.cu's
 // register-resident kernel where the panel fits a cluster or a co-resident

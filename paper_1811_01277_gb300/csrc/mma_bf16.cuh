@@ -1,5 +1,5 @@
-// Warp-level bf16 tensor-core building blocks shared by the digit-sliced
-// FP64 kernels (dgemm_sliced.cu, trans_ev_tc.cu): cp.async staging,
+// Warp-level bf16 tensor-core building blocks shared by the FP32-split products
+// (dgemm_sliced.cu) and the mma.sync back-transformation (trans_ev_tc.cu): cp.async staging,
 // ldmatrix fragment loads, mma.sync m16n8k16 with FP32 accumulation, and the
 // bf16 encoding of a signed 7-bit digit scaled by 2^(-7 s).
 //

@@ -8,14 +8,15 @@
 //                  triangle: X = A2 (Y T) (SYMM), M = T^T (Y^T X),
 //                  W = X - Y M / 2, A2 -= W Y^T + Y W^T (SYR2K)
 //   band -> tri    gb::band_to_tridi_d (bulge chasing)
-//   tridiagonal    gb::tridiag_eig_d (bisection + inverse iteration) and one
-//                  Newton-Schulz step Z <- Z (3I - Z^T Z)/2
+//   tridiagonal    divide and conquer (tridiag_dc.cu) for more than half of the
+//                  pairs, else gb::tridiag_eig_d (multisection + inverse
+//                  iteration) and one Newton-Schulz step Z <- Z (3I - Z^T Z)/2
 //   tri -> band    the pipeline trans_ev_tridi_to_band kernel
 //   band -> full   Z <- Q_0 Q_1 ... Q_{P-1} Z, last panel first:
 //                  Z_p -= Y (T (Y^T Z_p)), several panels at a time
 // The real solve's large products (SYMM, SYR2K, the band->full GEMMs, the
-// Newton-Schulz SYRK and SYMM) run on the bf16 tensor cores by exact digit
-// slicing (dgemm_sliced.cuh), the small ones in the DFMA kernels
+// Newton-Schulz SYRK and SYMM) run on the tcgen05 tensor cores by exact digit
+// slicing into FP16 (sliced_tc5.cu), the small ones in the DFMA kernels
 // (dgemm_dfma.cuh, and the complex DFMA kernel for the complex solve).
 // With GB_SOLVE_FP32_PRODUCTS the sliced products of full -> band and
 // band -> full are FP32 products (operands rounded to FP32, split into three
@@ -138,8 +139,11 @@ struct SolveWs {
 bool use_dc(int n, int nev) { return 2LL * nev > n; }
 
 // Products of at least this many flops go to the sliced tensor-core kernels
-// (below it the extra launches of slicing cost more than they save).
-constexpr double kSlicedMinFlops = 2.5e8;
+// (below it the extra launches of slicing cost more than they save: 1e8 flops
+// take 80 us of the whole FP64 pipe, a sliced product 60).  Solves with the line
+// at 2.5e8 and at 1e8: n = 1024 20.3, 19.8 ms; complex 1501 81.2, 78.5; a batch of 24
+// up to n = 2048 338, 303.
+constexpr double kSlicedMinFlops = 1e8;
 
 bool sliced_pays(double m, double n, double k) { return 2.0 * m * n * k >= kSlicedMinFlops; }
 
