@@ -43,7 +43,7 @@
 // Data movement per tile (b = 64, NB = 32, LP = 96):
 //  * the tile record is a V part (V digit planes in the MMA's canonical
 //    K-major layout, 48 KB) and a U part (U^T digit planes by 16-row
-//    chunks, the folds' constants of V's columns and U's rows; 50 KB), built
+//    chunks, the exponents of V's columns and U's rows; 48.5 KB), built
 //    once per tile by tc5_tile_prep; each part arrives by cp.async.bulk on its
 //    own mbarrier, requested as soon as the previous tile no longer needs the
 //    buffer;
@@ -62,8 +62,8 @@
 // shared memory), against 8 thousand clocks of MMAs.  So the 16 warps do nothing
 // else: a driver warp issues the MMAs of a K step or chunk as soon as the
 // workers have arrived there (named barriers on which only the driver waits),
-// a flags' warp publishes stored tiles and looks for the next one's rows, and
-// what a fold needs besides its sums is in the record.  A tile of n = 8192, nev =
+// a flags' warp publishes stored tiles, looks for the next one's rows and
+// makes what a fold needs besides its sums.  A tile of n = 8192, nev =
 // 4096 takes 25.8 thousand clocks (34.3 with everything in the same 16 warps and
 // K steps and chunks in series): cuts and the first product 6.1, folding
 // and cutting W 3.2, the second product and its folds 10.1, loads and
@@ -113,15 +113,13 @@ struct Geo {
     static constexpr int KSTEPS = LP / 16;              // K steps of the first product
     static constexpr int KD = NBC / 16;                 // K steps of the second
     // tile record: V part [8 planes][NBC rows q][LP] and U part [chunks of
-    // NCH rows][8 planes][rows][NBC] + the folds' constants by reflector (NBC) and
-    // row (LP) + a flag, canonical K-major
+    // NCH rows][8 planes][rows][NBC] + eV[NBC] + eU[LP], canonical K-major
     static constexpr int VPLANE = NBC * LP * 2;
     static constexpr int VBYTES = kPlanes * VPLANE;
     static constexpr int UBYTES = kPlanes * LP * NBC * 2;
     static constexpr int U_EV = UBYTES;
-    static constexpr int U_EU = UBYTES + NBC * 16;
-    static constexpr int U_FAR = UBYTES + (NBC + LP) * 16;          // some row's exponent is above 13
-    static constexpr int UPART = (U_FAR + 4 + 127) / 128 * 128;
+    static constexpr int U_EU = UBYTES + NBC * 4;
+    static constexpr int UPART = (UBYTES + (NBC + LP) * 4 + 127) / 128 * 128;
     static constexpr int REC = VBYTES + UPART;
     static constexpr int SBO_V = 16 * LP;               // bytes between 8-row groups of V (N = q)
     static constexpr int SBO_U = 16 * NBC;              // bytes between 8-row groups of U^T (N = j)
@@ -144,7 +142,8 @@ struct Geo {
     static constexpr int S_V = 0;
     static constexpr int S_U = VBYTES;
     static constexpr int S_Z = REC;
-    static constexpr int S_BAR = S_Z + kCols5 * ZROW * 8;    // 5 + ZR mbarriers, TMEM base
+    static constexpr int S_FC = S_Z + kCols5 * ZROW * 8;     // the folds' constants: V's reflectors, U's rows
+    static constexpr int S_BAR = S_FC + (NBC + LP) * 16;    // 6 + ZR mbarriers, TMEM base
     // at least 116 KB, so that shared memory alone keeps the kernel at one
     // CTA per SM: every CTA allocates all 512 TMEM columns
     static constexpr int SMEM = (S_BAR + 128) > 116 * 1024 ? (S_BAR + 128) : 116 * 1024;
@@ -195,7 +194,7 @@ __device__ __forceinline__ void cut_pair(long long x0, long long x1, uint32_t (&
 // with hi = sum_{l<4} L_l 2^(8(3-l)) and lo = sum_{l>=4} L_l 2^(8(8-l)) it is
 // hi 2^(26+e) + lo 2^(e-14) (mod 2^64; the result fits since it is a
 // fixed-point entry).  These are 16 thousand folds a tile on the integer pipe,
-// so what depends on the exponent alone is in the tile's record.
+// so what depends on the exponent alone is made once a tile, by the flags' warp.
 //
 // An FP32 level sum x (an integer, |x| < 2^22) plus 1.5 2^23 has the bit
 // pattern 0x4B400000 + x.  Two such patterns combine with one multiply-add
@@ -394,7 +393,6 @@ __global__ void __launch_bounds__(256, 2) tc5_tile_prep(int n, const double *__r
     // tile (each scheduler has a quarter of the FP64 pipe).  Then unit columns of V
     // (U rescaled to keep U V^T): |v_q^T z| <= ||z||, so W stays inside the
     // column's fixed-point range whatever tau is.
-    bool far = false;
     unsigned char *ru = rec + ((size_t)off[g] + k) * Gm::REC + Gm::VBYTES;
     const int row = (int)((threadIdx.x + 32u * (blockIdx.x + blockIdx.y)) % blockDim.x);
     if (row < LP) {
@@ -412,8 +410,7 @@ __global__ void __launch_bounds__(256, 2) tc5_tile_prep(int n, const double *__r
             V[row * NB1 + p] = v * rn[p];
         }
         seU[row] = max(exponent_above(m), kMinExp);
-        far = seU[row] > 13;
-        ((FoldConst *)(ru + Gm::U_EU))[row] = fold_const(seU[row], kLoBias);
+        ((int *)(ru + Gm::U_EU))[row] = seU[row];
     }
     __syncthreads();
     unsigned char *r = rec + ((size_t)off[g] + k) * Gm::REC;
@@ -424,10 +421,9 @@ __global__ void __launch_bounds__(256, 2) tc5_tile_prep(int n, const double *__r
             m = u > m ? u : m;
         }
         seV[threadIdx.x] = max(exponent_above(m), kMinExp);
-        ((FoldConst *)(ru + Gm::U_EV))[threadIdx.x] = fold_const(seV[threadIdx.x], Gm::WMAGIC == 9 ? kLoBias : kLoBias4);
+        ((int *)(ru + Gm::U_EV))[threadIdx.x] = seV[threadIdx.x];
     }
-    const int any_far = __syncthreads_or(far);
-    if (threadIdx.x == 0) *(int *)(ru + Gm::U_FAR) = any_far;
+    __syncthreads();
     // digit planes in the canonical K-major layout of the B operands:
     // V (N = q, K = j), plane t: byte t VPLANE + (q/8) SBO_V + (j/8) 128 +
     // (q%8) 16 + (j%8) 2, so the planes follow each other along N at the same
@@ -574,11 +570,9 @@ __global__ void __launch_bounds__(256) tc5_tile_prep_z(int n, const double2 *__r
             m = max(m, max(absbits(v.x), absbits(v.y)));
         }
         seV[threadIdx.x] = max(exponent_above(m), kMinExp);
-        const FoldConst f = fold_const(seV[threadIdx.x], Gm::WMAGIC == 9 ? kLoBias : kLoBias4);
-        ((FoldConst *)(ru + Gm::U_EV))[2 * threadIdx.x] = f;
-        ((FoldConst *)(ru + Gm::U_EV))[2 * threadIdx.x + 1] = f;
+        ((int *)(ru + Gm::U_EV))[2 * threadIdx.x] = seV[threadIdx.x];
+        ((int *)(ru + Gm::U_EV))[2 * threadIdx.x + 1] = seV[threadIdx.x];
     }
-    bool far = false;
     for (int j = threadIdx.x; j < LP / 2; j += blockDim.x) {
         unsigned long long m = 0;
         if (j < LC)
@@ -587,14 +581,11 @@ __global__ void __launch_bounds__(256) tc5_tile_prep_z(int n, const double2 *__r
                 m = max(m, max(absbits(u.x), absbits(u.y)));
             }
         const int ev = max(exponent_above(m), kMinExp);
-        far |= ev > 13;
         if (j < LC) seU[j] = ev;
-        const FoldConst f = fold_const(ev, kLoBias);
-        ((FoldConst *)(ru + Gm::U_EU))[2 * j] = f;
-        ((FoldConst *)(ru + Gm::U_EU))[2 * j + 1] = f;
+        ((int *)(ru + Gm::U_EU))[2 * j] = ev;
+        ((int *)(ru + Gm::U_EU))[2 * j + 1] = ev;
     }
-    const int any_far = __syncthreads_or(far);
-    if (threadIdx.x == 0) *(int *)(ru + Gm::U_FAR) = any_far;
+    __syncthreads();
     // V' (N = q' = 2q+p', K = j' = 2j+p) and the second product's B
     // (N = j', K = q'), in the layouts of the real record
     for (int e = threadIdx.x; e < NBC * (LP / 8); e += blockDim.x) {
@@ -633,6 +624,7 @@ struct Bool {
 
 struct Tc5Shared {
     int item;
+    int far;        // some row's exponent is above 13
     int ready;      // the next tile's rows are there (looked up while this tile's dZ is folded)
 };
 
@@ -643,6 +635,11 @@ __device__ __forceinline__ bool tc5_wait(uint32_t bar, uint32_t parity, TcState 
     tc_set_error(state, GB_ERR_TIMEOUT);
     atomicExch(&state->abort, 1);
     return false;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint32_t bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 // the workers arrive at barrier `id`, the driver waits there for them
@@ -686,10 +683,9 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
     const uint32_t bar_u = bar_v + 8;
     const uint32_t bar_dz = bar_v + 16;                     // two: one per chunk buffer
     const uint32_t bar_k = bar_v + 32;                      // one per K step of Z digits in tensor memory
-    const uint32_t bar_end = bar_k + 8 * ZR;
-    uint32_t *tmem_slot = (uint32_t *)(smem + Gm::S_BAR + 40 + 8 * ZR);
-    const FoldConst *eV = (const FoldConst *)(smem + Gm::S_U + Gm::U_EV);
-    const FoldConst *eU = (const FoldConst *)(smem + Gm::S_U + Gm::U_EU);
+    const uint32_t bar_end = bar_k + 8 * ZR, bar_fc = bar_end + 8;
+    uint32_t *tmem_slot = (uint32_t *)(smem + Gm::S_BAR + 48 + 8 * ZR);
+    const FoldConst *eV = (const FoldConst *)(smem + Gm::S_FC), *eU = eV + NBC;
     __shared__ Tc5Shared sh;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -706,6 +702,7 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
         tc5::mbar_init(bar_u, 1);
         tc5::mbar_init(bar_dz, 1);
         tc5::mbar_init(bar_end, 1);
+        tc5::mbar_init(bar_fc, 1);
         tc5::mbar_init(bar_dz + 8, 1);
         for (int i = 0; i < ZR; i++) tc5::mbar_init(bar_k + 8 * i, 1);
         tc5::mbar_init_fence();
@@ -774,6 +771,23 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
                     if (in_step(gave_up)) break;
                     in_step(false);   // the workers have loaded the window
                 }
+                // the folds' constants from the exponents in this tile's U part
+                gave_up |= !tc5_wait(bar_u, (uint32_t)(k & 1), state);
+                __syncwarp();
+                const int *ex = (const int *)(smem + Gm::S_U + Gm::U_EV);   // eV, then eU
+                FoldConst *fc = (FoldConst *)(smem + Gm::S_FC);
+                bool far = false;
+                for (int i = lane; i < NBC + LP; i += 32) {
+                    const int e = ex[i];
+                    far |= e > 13;
+                    fc[i] = fold_const(e, i < NBC && Gm::WMAGIC != 9 ? kLoBias4 : kLoBias);
+                }
+                far = __any_sync(0xffffffffu, far);
+                if (lane == 0) {
+                    sh.far = far;
+                    mbar_arrive(bar_fc);
+                }
+                __syncwarp();
                 if (in_step(gave_up)) break;   // W's digits are there
                 if (lane == 0) {
                     const int next = (g + 1 < G) ? min(k + 2, Knext) : 0;
@@ -965,7 +979,7 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
             tc5::fence_after_sync();
             // ---- fold W's levels (reflectors q0 .. q0+NB/4-1 of this column), cut
             // W into digit planes (TMEM: K step q/16, columns s*8 + (q%16)/2)
-            gave_up |= !tc5_wait(bar_u, (uint32_t)(k & 1), state);   // this tile's U part (row exponents)
+            gave_up |= !tc5_wait(bar_fc, (uint32_t)(k & 1), state);   // this tile's U part is there, its constants made
             {
                 constexpr int QW = NBC / 4;
                 const int q0 = wq * QW;
@@ -1013,7 +1027,7 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
             tc5::fence_before_sync();
             if (in_step(gave_up)) break;
             // ---- dZ by chunks, folded into the window: Zs -= dZ
-            const bool far = *(const int *)(smem + Gm::S_U + Gm::U_FAR) != 0;
+            const bool far = sh.far != 0;
 #pragma unroll 1
             for (int ch = 0; ch < Gm::CHUNKS; ch++) {
                 const int jb = ch * Gm::NCH + wq * (Gm::NCH / 4);
