@@ -703,7 +703,7 @@ def measure_solve(n, nev, nbw, cplx=False, spectrum="clustered", steps=1, warmup
                      "frac": F / (ms / 1e3) / 1e12 / FP64_PEAK_TFLOPS, "algorithmic_tflop": F / 1e12,
                      "by_stage_tflop": {k_: v_ / 1e12 for k_, v_ in Fst.items()},
                      "note": "algorithmic FP64 flops of the whole solve against the FP64 DFMA peak; "
-                             "large products on the bf16 tensor cores by exact digit slicing (FP64 "
+                             "large products on the tcgen05 tensor cores by exact digit slicing (FP64 "
                              "accuracy; the DFMA kernels with --dfma-products), the rest in DFMA kernels"},
         "accuracy": {"max_dlambda_over_norm": dlam, "residual_rel_fro": resid, "orth_max": orth,
                      "bound_50nu": 50 * n * u,
