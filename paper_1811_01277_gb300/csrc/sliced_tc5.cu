@@ -346,10 +346,12 @@ __device__ __forceinline__ double assemble(long long hi, uint32_t lo, int e, boo
     return __longlong_as_double((long long)(bits | ((unsigned long long)(neg & 0x80000000u) << 32)));
 }
 
-// The same by scalings, for results outside the normal range.
+// The same by scalings, for results outside the normal range.  The integer is
+// below 2^96 and e = ea + eb - 68 may go down to -2112, past the two factors of
+// scale_by_pow2: from e = -1300 on every result is a zero (of its sign).
 __device__ __noinline__ double scaled_odd(long long hi, uint32_t lo, int e)
 {
-    return scale_by_pow2((double)hi * 4294967296.0 + (double)lo, e);
+    return scale_by_pow2((double)hi * 4294967296.0 + (double)lo, max(e, -1300));
 }
 
 __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
@@ -583,8 +585,12 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                 }
                 if (any) {
 #pragma unroll
-                    for (int j = 0; j < 8; j++)
-                        v[j] = scaled_odd(hi[8 * h + j], lo[8 * h + j], er + __ldg(p.eb + min(cb + 8 * h + j, p.n - 1)));
+                    for (int j = 0; j < 8; j++) {
+                        bool odd;
+                        const int e = er + __ldg(p.eb + min(cb + 8 * h + j, p.n - 1));
+                        assemble(hi[8 * h + j], lo[8 * h + j], e, &odd);
+                        if (odd) v[j] = scaled_odd(hi[8 * h + j], lo[8 * h + j], e);
+                    }
                 }
                 if (bad) {   // a wait gave up
 #pragma unroll

@@ -96,3 +96,45 @@ def test_scales_at_the_ends_of_the_range(gb, e):
     ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
     gb.gb_dgemm_sliced("N", "N", m, n, k, 1.0, As, m, B, k, 0.0, C, m, ws, wsb, torch.cuda.current_stream())
     assert torch.equal(C.T, want)
+
+
+@pytest.mark.parametrize("e", [-1018, -1010, -1000, -990, -700, -560, -530, -500, 300, 500, 600])
+@pytest.mark.parametrize("form", ["gemm", "syrk", "zgemm"])
+def test_both_operands_scaled(gb, form, e):
+    """A and B of integers times 2^e: the product is the integers' times 2^(2 e),
+    from zero (below the subnormal range, of the sum's sign or none) over exact
+    subnormal and normal results to infinities; zero sums stay zeros."""
+    m, n, k = (70, 70, 40) if form == "syrk" else (130, 70, 40)
+    g = torch.Generator(device="cuda").manual_seed(11)
+    f = 2.0 ** e
+    st = torch.cuda.current_stream()
+    if form == "zgemm":
+        A = torch.complex(ints(g, k, m), ints(g, k, m))
+        B = torch.complex(ints(g, n, k), ints(g, n, k))
+        want = torch.view_as_real((A.T @ B.T).contiguous())
+        As, Bs = (torch.view_as_complex(torch.view_as_real(x) * f) for x in (A, B))
+        C = torch.zeros(n, m, dtype=torch.complex128, device="cuda")
+        wsb = gb.gb_zgemm_sliced_workspace_bytes(m, n, k)
+        ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+        gb.gb_zgemm_sliced("N", m, n, k, 1.0, As, m, Bs, k, 0.0, C, m, ws, wsb, st)
+        got = torch.view_as_real(C.T.contiguous())
+    elif form == "syrk":
+        A = ints(g, n, k)
+        A[:, 3] = 0.0                                     # a zero column of products among odd ones
+        A[5] = 0.0
+        want = (A @ A.T).tril()
+        C = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+        wsb = gb.gb_dsyrk_sliced_workspace_bytes(n, k)
+        ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+        gb.gb_dsyrk_sliced(n, k, 1.0, A * f, k, 0.0, C, n, ws, wsb, st)
+        got = C.T.tril()
+    else:
+        A, B = ints(g, k, m), ints(g, n, k)
+        B[5] = 0.0
+        want = A.T @ B.T
+        C = torch.zeros(n, m, dtype=torch.float64, device="cuda")
+        wsb = gb.gb_dgemm_sliced_workspace_bytes(m, n, k)
+        ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+        gb.gb_dgemm_sliced("N", "N", m, n, k, 1.0, A * f, m, B * f, k, 0.0, C, m, ws, wsb, st)
+        got = C.T
+    assert torch.equal(got, want * f * f)   # (each factor alone stays in the range)
