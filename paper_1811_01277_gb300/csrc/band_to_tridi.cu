@@ -14,10 +14,13 @@
 // to 2b-1 below the diagonal, where the bulges live), in a workspace.
 //
 // What bounds it: the chain of sweeps.  O(s,k) shares all but its last column
-// with O(s-1,k); the last column is the first of D(s-1,k), and its last entry
-// the beta of H(s-1,k+1).  D(s,k) shares all but its last row with D(s-1,k); that
-// row is the first of O(s-1,k+1) and, on the diagonal, the first entry of
-// D(s-1,k+1).  So sweep s trails sweep s-1 by one O step and one hop of those few
+// and row with O(s-1,k); the last column is the first of D(s-1,k), and its last
+// entry the beta of H(s-1,k+1).  The last row is zero but for that entry: its
+// columns were annihilated by H(s-m,k+1), m >= 2, so it is not loaded, the zeros
+// are never stored, and nothing has to wait for those blocks, one step ahead of
+// the ones whose flags O(s,k) looks at.  D(s,k) shares all but its last row with
+// D(s-1,k); that row is the first of O(s-1,k+1) and, on the diagonal, the first
+// entry of D(s-1,k+1).  So sweep s trails sweep s-1 by one O step and one hop of those few
 // entries, and the stage takes n times that.  One SM issues two FP64
 // multiply-adds per clock, so a step's arithmetic (4 b^2 multiply-adds in O, 2 b^2
 // and more in D) costs several microseconds on one SM; a sweep therefore runs
@@ -505,13 +508,9 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                         const int i = cp + G::TPC * u, gi = i0 + i;
                         if (gi < len) {
                             const T e = B[i * LD + col];
-                            if (col > 0) {
-                                *A.at(r + gi, c + col) = act ? nmad(sm.v[par][gi], wj, e) : e;
-                            } else if (gi > 0) {     // the annihilated column (its beta went its own way)
-                                T z;
-                                zero_of(z);
-                                *A.at(r + gi, c) = act ? z : e;
-                            }
+                            // (the annihilated column stays unstored: its beta went its own
+                            // way, and later sweeps know the zeros)
+                            if (col > 0) *A.at(r + gi, c + col) = act ? nmad(sm.v[par][gi], wj, e) : e;
                         }
                     }
                 }
@@ -632,6 +631,9 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                     const int i0 = rank * RW;
                     const int c = (k == 0) ? s - 1 : r - b;
                     const int ncols = (k == 0) ? 1 : b;
+                    // from the band: all but the last column, which follows below,
+                    // and the last row (zero up to there); the first sweep loads both
+                    const int lcols = s > 1 ? ncols - 1 : ncols, lrows = s > 1 ? min(len, b - 1) : len;
                     // rows run along the band's contiguous index
                     constexpr int NU = RW * BM / kLoaders, CH = NU < 8 ? NU : 8;
 #pragma unroll 1
@@ -641,8 +643,7 @@ chase_kernel(ChaseWork work, ChaseState *state, long long timeout_ns)
                         for (int u = 0; u < CH; u++) {
                             const int e = lt + kLoaders * (u0 + u), col = e / RW, i = e % RW;
                             zero_of(x[u]);
-                            // (the last column follows below)
-                            if (col < ncols - (s > 1 ? 1 : 0) && i0 + i < len) x[u] = ld_cg(A.at(r + i0 + i, c + col));
+                            if (col < lcols && i0 + i < lrows) x[u] = ld_cg(A.at(r + i0 + i, c + col));
                         }
 #pragma unroll
                         for (int u = 0; u < CH; u++) {
