@@ -783,6 +783,7 @@ pipeline_tc5(int n, int nev, long long *__restrict__ Zi, long long ldz, const un
                     fc[i] = fold_const(e, i < NBC && Gm::WMAGIC != 9 ? kLoBias4 : kLoBias);
                 }
                 far = __any_sync(0xffffffffu, far);
+                __syncwarp();   // every lane's constants before lane 0's arrival (a vote orders no memory)
                 if (lane == 0) {
                     sh.far = far;
                     mbar_arrive(bar_fc);
