@@ -33,7 +33,10 @@ namespace {
 
 __device__ __forceinline__ double dabs(double x) { return x < 0 ? -x : x; }
 
-// Gershgorin interval and the norm bound ||T||_inf (single block).
+__device__ __forceinline__ double nan_max(double a, double b) { return a > b || a != a ? a : b; }   // NaN if either is
+
+// Gershgorin interval and the norm bound ||T||_inf (single block); the norm is
+// infinite or NaN if an entry is.
 __global__ void __launch_bounds__(256) tridiag_bounds(int n, const double *__restrict__ d,
                                                       const double *__restrict__ e, double *out)
 {
@@ -43,7 +46,7 @@ __global__ void __launch_bounds__(256) tridiag_bounds(int n, const double *__res
         double r = (i > 0 ? dabs(e[i - 1]) : 0.0) + (i < n - 1 ? dabs(e[i]) : 0.0);
         lo = fmin(lo, d[i] - r);
         hi = fmax(hi, d[i] + r);
-        nr = fmax(nr, dabs(d[i]) + r);
+        nr = nan_max(nr, dabs(d[i]) + r);
     }
     slo[threadIdx.x] = lo;
     shi[threadIdx.x] = hi;
@@ -53,14 +56,14 @@ __global__ void __launch_bounds__(256) tridiag_bounds(int n, const double *__res
         if (threadIdx.x < o) {
             slo[threadIdx.x] = fmin(slo[threadIdx.x], slo[threadIdx.x + o]);
             shi[threadIdx.x] = fmax(shi[threadIdx.x], shi[threadIdx.x + o]);
-            snr[threadIdx.x] = fmax(snr[threadIdx.x], snr[threadIdx.x + o]);
+            snr[threadIdx.x] = nan_max(snr[threadIdx.x], snr[threadIdx.x + o]);
         }
         __syncthreads();
     }
     if (threadIdx.x == 0) {
         out[0] = slo[0] - 2.0 * 0x1p-52 * snr[0];   // both zero for a zero matrix
         out[1] = shi[0] + 2.0 * 0x1p-52 * snr[0];
-        out[2] = snr[0] > 0 ? snr[0] : 1.0;
+        out[2] = snr[0] == 0.0 ? 1.0 : snr[0];
     }
 }
 
@@ -185,7 +188,8 @@ __global__ void __launch_bounds__(128) tridiag_bisect(int n, int nev, const doub
     const unsigned long long pivkey = abs_key(pivmin);
     const double nrm = bounds[2];
     const double abstol = 0x1p-53 * nrm;
-    bool done = k >= nev;
+    const bool finite = isfinite(nrm);   // else every eigenvalue is NaN
+    bool done = k >= nev || !finite;
     // first point whose count exceeds k (P: none)
     auto first_above = [&](int c) {
         int first = P;
@@ -238,11 +242,12 @@ __global__ void __launch_bounds__(128) tridiag_bisect(int n, int nev, const doub
             hi = nhi;
         }
     }
-    if (j == 0 && k < nev) lam[k] = 0.5 * (lo + hi);
+    if (j == 0 && k < nev) lam[k] = finite ? 0.5 * (lo + hi) : __longlong_as_double(0x7ff8000000000000ll);
 }
 
 // lam[k] = max(lam[0..k]): eigenvalues equal to working accuracy, found from
 // intervals of their own, may differ from ascending order in the last place.
+// A NaN stays where it is.
 __global__ void __launch_bounds__(1024) tridiag_ascending(int nev, double *__restrict__ lam)
 {
     __shared__ double top[1024];
@@ -259,8 +264,9 @@ __global__ void __launch_bounds__(1024) tridiag_ascending(int nev, double *__res
     }
     m = threadIdx.x > 0 ? top[threadIdx.x - 1] : -1.7976931348623157e308;
     for (int k = a; k < b; k++) {
-        m = fmax(m, lam[k]);
-        lam[k] = m;
+        const double x = lam[k];
+        m = fmax(m, x);
+        lam[k] = x != x ? x : m;
     }
 }
 
@@ -549,7 +555,7 @@ __global__ void __launch_bounds__(256) cluster_orthonormalise(int n, int nev, co
     const int k0 = blockIdx.x;
     const double gap = gap_rel * bounds[2];
     if (k0 > 0 && lam[k0] - lam[k0 - 1] <= gap) return;   // not the first member
-    if (k0 + 1 >= nev || lam[k0 + 1] - lam[k0] > gap) return;  // a single eigenvalue
+    if (k0 + 1 >= nev || !(lam[k0 + 1] - lam[k0] <= gap)) return;  // a single eigenvalue (or NaN)
     int k1 = k0 + 1;
     while (k1 + 1 < nev && lam[k1 + 1] - lam[k1] <= gap) k1++;
     for (int k = k0 + 1; k <= k1; k++) {

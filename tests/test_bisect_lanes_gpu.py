@@ -70,3 +70,14 @@ def test_spectra(gb, kind):
     ev = solve(gb, A, nev)
     assert (ev.diff() >= 0).all()
     assert (ev - want[:nev]).abs().max() <= 1e-11 * max(float(want.abs().max()), 1e-300)
+
+
+@pytest.mark.parametrize("n,nev", [(40, 40), (300, 1), (600, 250)])
+@pytest.mark.parametrize("x", [float("nan"), float("inf"), float("-inf")])
+def test_nonfinite_matrix_gives_nan(gb, n, nev, x):
+    """No finite number may stand for an eigenvalue of a matrix that has none."""
+    g = torch.Generator(device="cuda").manual_seed(n)
+    R = torch.randn(n, n, generator=g, device="cuda", dtype=torch.float64)
+    A = 0.5 * (R + R.T)
+    A[n // 2, n // 2] = x
+    assert torch.isnan(solve(gb, A, nev)).all()
