@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kDcSetupThreads) dc_setup(int n, int t, const 
     const double r2 = 0.7071067811865476;
     // stable merge of the ascending halves: rank of each entry
     double dmax = 0.0, zmax = 0.0;
+    bool nan = rho != rho;
     for (int j = threadIdx.x; j < s; j += blockDim.x) {
         const double v = lam[off + j];
         int lo, hi, rank;
@@ -251,6 +252,26 @@ __global__ void __launch_bounds__(kDcSetupThreads) dc_setup(int n, int t, const 
         }
         dmax = fmax(dmax, fabs(v));
         zmax = fmax(zmax, fabs(z));
+        nan |= v != v || z != z;
+    }
+    // Ranks exist among numbers only: with a NaN, positions would be taken twice
+    // and others left as they were in the workspace, which later kernels index
+    // with.  Such a merge keeps its columns where they are, and every eigenvalue
+    // of it is NaN.
+    if (__syncthreads_or(nan)) {
+        for (int j = threadIdx.x; j < s; j += blockDim.x) {
+            a.perm[off + j] = j;
+            a.ndpos[off + j] = -1;
+            a.defl_idx[off + j] = j;
+            a.defl_d[off + j] = __longlong_as_double(0x7ff8000000000000ll);
+        }
+        if (threadIdx.x == 0) {
+            a.cnt[3 * off] = 0;
+            a.cnt[3 * off + 1] = s;
+            a.cnt[3 * off + 2] = 0;
+            a.rho[off] = rho;
+        }
+        return;
     }
     dmax = block_max(dmax, red);
     zmax = block_max(zmax, red);

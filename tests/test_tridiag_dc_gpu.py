@@ -136,3 +136,43 @@ def test_solver_all_pairs_dc_against_bisection(gb):
         assert np.abs(w - np.sort(lam0)).max() / nrm <= 1e-11
         assert np.linalg.norm(A @ Zh - Zh * w) / np.linalg.norm(A) <= 50 * n * U
         assert np.abs(Zh.T @ Zh - np.eye(nev)).max() <= 50 * n * U
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 17, 300, 1100])
+@pytest.mark.parametrize("where", ["d", "e", "all"])
+def test_dc_nan_entries(gb, n, where):
+    """A NaN anywhere in T: every eigenvalue is NaN and nothing else in memory
+    is touched (positions come from the merges, not from comparisons with NaN)."""
+    g = np.random.default_rng(n)
+    d, e = g.standard_normal(n), g.standard_normal(max(n - 1, 0))
+    if where == "all":
+        d[:], e[:] = np.nan, np.nan
+    elif where == "d" or n == 1:
+        d[n // 3] = np.nan
+    else:
+        e[(n - 1) // 2] = np.nan
+    dev = torch.device("cuda")
+    wsb = gb.gb_tridiag_dc_workspace_bytes(n)
+    ws = torch.full((wsb + 4096,), 255, dtype=torch.uint8, device=dev)
+    Q = torch.full((n + 4, n), 7.0, dtype=torch.float64, device=dev)
+    lam = torch.zeros(n, dtype=torch.float64, device=dev)
+    gb.gb_tridiag_dc_d(n, torch.from_numpy(d).to(dev), torch.from_numpy(e if n > 1 else np.zeros(1)).to(dev), lam, Q, n,
+                       ws, wsb, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert torch.isnan(lam).all()
+    assert (Q[n:] == 7.0).all() and (ws[wsb:] == 255).all()
+
+
+def test_solve_of_a_nan_matrix(gb):
+    """All pairs of a matrix with one NaN (the solver's divide-and-conquer
+    path): NaN eigenvalues."""
+    n = 300
+    A = torch.eye(n, dtype=torch.float64, device="cuda")
+    A[7, 3] = A[3, 7] = float("nan")
+    wsb = gb.gb_solve_workspace_bytes(n, n, 32)
+    ws = torch.full((wsb,), 255, dtype=torch.uint8, device="cuda")
+    ev = torch.zeros(n, dtype=torch.float64, device="cuda")
+    Z = torch.zeros(n, n, dtype=torch.float64, device="cuda")
+    gb.gb_solve_d(n, n, 32, A, n, ev, Z, n, ws, wsb, torch.cuda.current_stream())
+    torch.cuda.synchronize()
+    assert torch.isnan(ev).all()
