@@ -588,8 +588,9 @@ int gb_dsyrk(int n, int k, double alpha, const double *A, int lda, double beta, 
  * in tensor memory, exact over 128 values of k, folded into 96-bit integers),
  * and the result is rounded to FP64 once.  Accuracy is that of an FP64 product measured
  * against the scaled maxima: |C - alpha op(A) op(B)| <~ 2^-53 k |alpha|
- * max_j |op(A)_ij| max_i |op(B)_ij| per entry.  Inputs must be finite;
- * subnormal inputs are read as zero.  The paper's products are BLAS calls
+ * max_j |op(A)_ij| max_i |op(B)_ij| per entry.  A NaN or
+ * infinite entry makes every result of its row or column NaN; subnormal
+ * inputs are read as zero.  The paper's products are BLAS calls
  * (Sec. 3.2); this is how they run fastest on a part whose FP64 pipe is
  * narrow.  `workspace` (256-byte aligned) must hold the *_workspace_bytes
  * figure: the digit planes of both operands and split-K partials.  Same

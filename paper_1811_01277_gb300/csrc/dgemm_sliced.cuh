@@ -14,8 +14,8 @@
 // to FP64 once, at the end (sliced_tc5.cu).
 //
 // Accuracy is that of an FP64 product measured against the scaled maxima:
-// |C - AB| <~ 2^-53 k max_j|a_ij| max_i|b_ij| per entry.  Inputs must be
-// finite; subnormal inputs are read as zero.
+// |C - AB| <~ 2^-53 k max_j|a_ij| max_i|b_ij| per entry.  A row with
+// a NaN or an infinity gives NaN results; subnormal inputs are read as zero.
 //
 // FP32 products (digits = kSplitPlanes): every entry is rounded to FP32 and
 // split exactly into three bf16 parts h0 + h1 + h2 with their own

@@ -94,8 +94,14 @@ __device__ __forceinline__ uint32_t digits_of(uint32_t a, uint32_t b, int bi)
 }
 
 // Row exponent from the high word of the row's largest magnitude (0 for rows
-// of zeros and subnormals, which read as zero).
-__device__ __forceinline__ int exponent_of(uint32_t hi) { return (hi >> 20) ? (int)(hi >> 20) - 1022 : 0; }
+// of zeros and subnormals, which read as zero).  A row with a NaN or an infinity
+// gets an exponent far beyond the others: its digits are zeros, and the epilogue
+// knows its results for NaN.
+constexpr int kNonFinite = 1 << 20;
+__device__ __forceinline__ int exponent_of(uint32_t hi)
+{
+    return hi >= 0x7ff00000u ? kNonFinite : (hi >> 20) ? (int)(hi >> 20) - 1022 : 0;
+}
 
 __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
@@ -580,8 +586,9 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                 for (int j = 0; j < 8; j++) {
                     bool odd;
                     const int c = cb + 8 * h + j;
-                    v[j] = assemble(hi[8 * h + j], lo[8 * h + j], er + __ldg(p.eb + min(c, p.n - 1)), &odd);
-                    any |= odd;
+                    const int e = er + __ldg(p.eb + min(c, p.n - 1));
+                    v[j] = assemble(hi[8 * h + j], lo[8 * h + j], e, &odd);
+                    any |= odd || e > kNonFinite / 2;
                 }
                 if (any) {
 #pragma unroll
@@ -590,6 +597,8 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                         const int e = er + __ldg(p.eb + min(cb + 8 * h + j, p.n - 1));
                         assemble(hi[8 * h + j], lo[8 * h + j], e, &odd);
                         if (odd) v[j] = scaled_odd(hi[8 * h + j], lo[8 * h + j], e);
+                        // (alpha = 0 asks for no product)
+                        if (e > kNonFinite / 2) v[j] = p.alpha == 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
                     }
                 }
                 if (bad) {   // a wait gave up

@@ -138,3 +138,70 @@ def test_both_operands_scaled(gb, form, e):
         gb.gb_dgemm_sliced("N", "N", m, n, k, 1.0, A * f, m, B * f, k, 0.0, C, m, ws, wsb, st)
         got = C.T
     assert torch.equal(got, want * f * f)   # (each factor alone stays in the range)
+
+
+@pytest.mark.parametrize("x", [float("nan"), float("inf"), float("-inf")])
+@pytest.mark.parametrize("k", [40, 300, 4100])
+def test_nonfinite_entries_give_nan(gb, k, x):
+    """A NaN or infinity in a row of op(A) or a column of op(B) makes that row or
+    column of the product NaN; every other entry is exact.  (Entries below 1/2
+    beside it: nothing overflows by itself.)"""
+    m, n = 140, 75
+    g = torch.Generator(device="cuda").manual_seed(k)
+    A, B, C = ints(g, k, m) / 32, ints(g, n, k) / 32, ints(g, n, m)
+    want = C.T - A.T @ B.T
+    A[k // 2, 7] = x
+    B[3, k - 1] = x
+    want[7] = float("nan")
+    want[:, 3] = float("nan")
+    wsb = gb.gb_dgemm_sliced_workspace_bytes(m, n, k)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream()
+    got = C.clone()
+    gb.gb_dgemm_sliced("N", "N", m, n, k, -1.0, A, m, B, k, 1.0, got, m, ws, wsb, st)
+    assert torch.equal(torch.nan_to_num(got.T, nan=1e9), torch.nan_to_num(want, nan=1e9))
+    got = C.clone()
+    gb.gb_dgemm_sliced("N", "N", m, n, k, 0.0, A, m, B, k, 2.0, got, m, ws, wsb, st)   # alpha = 0: no product
+    assert torch.equal(got, 2.0 * C)
+
+
+@pytest.mark.parametrize("x", [float("nan"), float("inf")])
+def test_nonfinite_entries_of_the_other_forms(gb, x):
+    """The symmetric, rank-2k and complex forms: a stored entry (i, j) reaches
+    rows and columns i and j, a complex one both parts."""
+    n, k = 200, 50
+    g = torch.Generator(device="cuda").manual_seed(9)
+    st = torch.cuda.current_stream()
+    S = ints(g, n, n)
+    S = S.tril() + S.tril(-1).T
+    X, Y, C = ints(g, k, n), ints(g, k, n), ints(g, n, n)
+    want = S @ X.T
+    want[[150, 20]] = float("nan")
+    Sx = S.clone()
+    Sx[150, 20] = x
+    wsb = gb.gb_dsymm_sliced_workspace_bytes("L", n, k)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    out = torch.zeros(k, n, dtype=torch.float64, device="cuda")
+    gb.gb_dsymm_sliced("L", n, k, 1.0, Sx.T.contiguous(), n, X, n, 0.0, out, n, ws, wsb, st)
+    assert torch.equal(torch.nan_to_num(out.T, nan=1e9), torch.nan_to_num(want, nan=1e9))
+    low = torch.ones(n, n, dtype=torch.bool, device="cuda").tril()
+    want = C.T - (X.T @ Y + Y.T @ X)
+    want[33] = float("nan")
+    want[:, 33] = float("nan")
+    want = torch.where(low, want, C.T)
+    X[4, 33] = x
+    wsb = gb.gb_dsyr2k_sliced_workspace_bytes(n, k)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    out = C.clone()
+    gb.gb_dsyr2k_sliced(n, k, -1.0, X, n, Y, n, 1.0, out, n, ws, wsb, st)
+    assert torch.equal(torch.nan_to_num(out.T, nan=1e9), torch.nan_to_num(want, nan=1e9))
+    A, B = torch.complex(ints(g, k, n), ints(g, k, n)), torch.complex(ints(g, n, k), ints(g, n, k))
+    want = torch.view_as_real((A.T @ B.T).contiguous())
+    want[61] = float("nan")
+    A[2, 61] = complex(1.0, x)
+    wsb = gb.gb_zgemm_sliced_workspace_bytes(n, n, k)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    out = torch.zeros(n, n, dtype=torch.complex128, device="cuda")
+    gb.gb_zgemm_sliced("N", n, n, k, 1.0, A, n, B, k, 0.0, out, n, ws, wsb, st)
+    got = torch.view_as_real(out.T.contiguous())
+    assert torch.equal(torch.nan_to_num(got, nan=1e9), torch.nan_to_num(want, nan=1e9))
