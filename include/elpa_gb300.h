@@ -265,7 +265,8 @@ int gb_band_to_tridi_z(int n, int nbw, const double *AB, int ldab, double *d, do
  * GEMMs, the Newton-Schulz SYRK and SYMM) run on the tcgen05 tensor cores by
  * exact digit slicing (gb_dgemm_sliced below); GB_SOLVE_DFMA_PRODUCTS runs
  * them on the FP64 FMA pipe instead.  Asynchronous; device-side status of
- * the dependency waits through gb_solve_query. */
+ * the waits of the panels, the bulge chase, the products and the
+ * back-transformation through gb_solve_query. */
 #define GB_SOLVE_FP64_EMULATED_GEMM 1
 #define GB_SOLVE_RECORD_STAGES 2 /* record CUDA events at the stage boundaries */
 #define GB_SOLVE_DFMA_PRODUCTS 4 /* products on the FP64 FMA pipe, not sliced */
@@ -286,7 +287,8 @@ int gb_solve_query(const void *workspace, int n, int nev, int nbw, void *stream)
  * on the FP64 FMA pipe), the b x b panel products in this library's complex
  * DFMA kernel, and the back-transformation on the tcgen05 tensor cores
  * (nbw in {16, 32, 64}, n >= 512).  Device-side status of the waits of the
- * bulge chase and of the back-transformation through gb_solve_query_z. */
+ * panels, the bulge chase, the products and the back-transformation through
+ * gb_solve_query_z. */
 size_t gb_solve_workspace_bytes_z(int n, int nev, int nbw);
 int gb_solve_z(int n, int nev, int nbw, const double *A, int lda, double *ev, double *Z, int ldz,
                void *workspace, size_t ws_bytes, void *stream, int flags);
@@ -589,8 +591,9 @@ int gb_dsyrk(int n, int k, double alpha, const double *A, int lda, double beta, 
  * and the result is rounded to FP64 once.  Accuracy is that of an FP64 product measured
  * against the scaled maxima: |C - alpha op(A) op(B)| <~ 2^-53 k |alpha|
  * max_j |op(A)_ij| max_i |op(B)_ij| per entry.  A NaN or
- * infinite entry makes every result of its row or column NaN; subnormal
- * inputs are read as zero.  The paper's products are BLAS calls
+ * infinite entry makes every result of its row or column NaN, and so does a
+ * wait of the kernel that exceeds its bound in the tiles not finished by then;
+ * subnormal inputs are read as zero.  The paper's products are BLAS calls
  * (Sec. 3.2); this is how they run fastest on a part whose FP64 pipe is
  * narrow.  `workspace` (256-byte aligned) must hold the *_workspace_bytes
  * figure: the digit planes of both operands and split-K partials.  Same

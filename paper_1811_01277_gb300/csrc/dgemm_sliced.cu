@@ -255,12 +255,12 @@ cudaError_t sliced_reduce_launch(int m, int n, int splits, const double *part, d
 }
 
 cudaError_t sliced_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double alpha, double beta, double *C,
-                        long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st)
+                        long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st, int *status)
 {
     if (m <= 0 || n <= 0) return cudaSuccess;
     if (A.K != B.K || A.Kp != B.Kp || m > A.R || n > B.R) return cudaErrorInvalidValue;
     if (A.digits != B.digits) return cudaErrorInvalidValue;
-    if (A.digits == kSlices) return tc5_gemm(A, B, m, n, alpha, beta, C, ldc, fill, work, work_elems, st);
+    if (A.digits == kSlices) return tc5_gemm(A, B, m, n, alpha, beta, C, ldc, fill, work, work_elems, st, status);
     if (A.digits != kSplitPlanes || fill == kFillZLower) return cudaErrorInvalidValue;
     const int tiles_m = (m + kBM - 1) / kBM, tiles_n = (n + kBN - 1) / kBN;
     long long tiles = (long long)tiles_m * tiles_n;
@@ -345,7 +345,7 @@ size_t sliced_syrk_ws_bytes(int n, int k) { return sliced_ws(n, 0, k, 0, 0, null
 
 cudaError_t sliced_dgemm(char transa, char transb, int m, int n, int k, double alpha, const double *A, long long lda,
                          const double *B, long long ldb, double beta, double *C, long long ldc, void *ws,
-                         cudaStream_t st, int digits)
+                         cudaStream_t st, int digits, int *status)
 {
     SlicedWs w = sliced_ws(m, n, k, 0, 0, ws);
     SlicedOp a, b;
@@ -353,11 +353,12 @@ cudaError_t sliced_dgemm(char transa, char transb, int m, int n, int k, double a
     if (e != cudaSuccess) return e;
     if ((e = slice_matrix(transb == 'N' ? kViewCol : kViewRow, n, k, B, ldb, w.b, &b, st, digits)) != cudaSuccess)
         return e;
-    return sliced_gemm(a, b, m, n, alpha, beta, C, ldc, kFillAll, w.part, kPartialElems, st);
+    return sliced_gemm(a, b, m, n, alpha, beta, C, ldc, kFillAll, w.part, kPartialElems, st, status);
 }
 
 cudaError_t sliced_dsymm(char side, int m, int n, double alpha, const double *S, long long lds, const double *B,
-                         long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st, int digits)
+                         long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st, int digits,
+                          int *status)
 {
     const int K = side == 'L' ? m : n;
     SlicedWs w = sliced_ws(m, n, K, 0, 0, ws);
@@ -370,12 +371,12 @@ cudaError_t sliced_dsymm(char side, int m, int n, double alpha, const double *S,
         if ((e = slice_matrix(kViewRow, m, n, B, ldb, w.a, &a, st, digits)) != cudaSuccess) return e;
         if ((e = slice_matrix(kViewSym, n, n, S, lds, w.b, &b, st, digits)) != cudaSuccess) return e;
     }
-    return sliced_gemm(a, b, m, n, alpha, beta, C, ldc, kFillAll, w.part, kPartialElems, st);
+    return sliced_gemm(a, b, m, n, alpha, beta, C, ldc, kFillAll, w.part, kPartialElems, st, status);
 }
 
 cudaError_t sliced_dsyr2k_lower(int n, int k, double alpha, const double *A, long long lda, const double *B,
                                 long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st,
-                                int digits)
+                                int digits, int *status)
 {
     // A B^T + B A^T = [A B] [B A]^T
     SlicedWs w = sliced_ws(n, n, 2 * k, n, 2 * k, ws);
@@ -394,18 +395,18 @@ cudaError_t sliced_dsyr2k_lower(int n, int k, double alpha, const double *A, lon
     SlicedOp a, b;
     if ((e = slice_matrix(kViewRow, n, 2 * k, AB, n, w.a, &a, st, digits)) != cudaSuccess) return e;
     if ((e = slice_matrix(kViewRow, n, 2 * k, BA, n, w.b, &b, st, digits)) != cudaSuccess) return e;
-    return sliced_gemm(a, b, n, n, alpha, beta, C, ldc, kFillLower, w.part, kPartialElems, st);
+    return sliced_gemm(a, b, n, n, alpha, beta, C, ldc, kFillLower, w.part, kPartialElems, st, status);
 }
 
 cudaError_t sliced_dsyrk_lower_t(int n, int k, double alpha, const double *A, long long lda, double beta, double *C,
-                                 long long ldc, void *ws, cudaStream_t st, int digits)
+                                 long long ldc, void *ws, cudaStream_t st, int digits, int *status)
 {
     // A^T A: both operands are the columns of A
     SlicedWs w = sliced_ws(n, 0, k, 0, 0, ws);
     SlicedOp a;
     cudaError_t e = slice_matrix(kViewCol, n, k, A, lda, w.a, &a, st, digits);
     if (e != cudaSuccess) return e;
-    return sliced_gemm(a, a, n, n, alpha, beta, C, ldc, kFillLower, w.part, kPartialElems, st);
+    return sliced_gemm(a, a, n, n, alpha, beta, C, ldc, kFillLower, w.part, kPartialElems, st, status);
 }
 
 // ---- complex products (interleaved storage; real alpha, beta) ----
@@ -420,29 +421,31 @@ size_t sliced_zher2k_ws_bytes(int n, int k)
 
 cudaError_t sliced_zgemm(char transa, int m, int n, int k, double alpha, const double *A, long long lda,
                          const double *B, long long ldb, double beta, double *C, long long ldc, void *ws,
-                         cudaStream_t st)
+                         cudaStream_t st, int *status)
 {
     SlicedWs w = sliced_ws(2 * m, n, 2 * k, 0, 0, ws);
     SlicedOp a, b;
     cudaError_t e = slice_matrix(transa == 'N' ? kViewZExpandN : kViewZExpandC, 2 * m, 2 * k, A, lda, w.a, &a, st);
     if (e != cudaSuccess) return e;
     if ((e = slice_matrix(kViewCol, n, 2 * k, B, 2 * ldb, w.b, &b, st)) != cudaSuccess) return e;
-    return sliced_gemm(a, b, 2 * m, n, alpha, beta, C, 2 * ldc, kFillAll, w.part, kPartialElems, st);
+    return sliced_gemm(a, b, 2 * m, n, alpha, beta, C, 2 * ldc, kFillAll, w.part, kPartialElems, st, status);
 }
 
 cudaError_t sliced_zhemm_left(int m, int n, double alpha, const double *S, long long lds, const double *B,
-                              long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st)
+                              long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st,
+                              int *status)
 {
     SlicedWs w = sliced_ws(2 * m, n, 2 * m, 0, 0, ws);
     SlicedOp a, b;
     cudaError_t e = slice_matrix(kViewZHermExpand, 2 * m, 2 * m, S, lds, w.a, &a, st);
     if (e != cudaSuccess) return e;
     if ((e = slice_matrix(kViewCol, n, 2 * m, B, 2 * ldb, w.b, &b, st)) != cudaSuccess) return e;
-    return sliced_gemm(a, b, 2 * m, n, alpha, beta, C, 2 * ldc, kFillAll, w.part, kPartialElems, st);
+    return sliced_gemm(a, b, 2 * m, n, alpha, beta, C, 2 * ldc, kFillAll, w.part, kPartialElems, st, status);
 }
 
 cudaError_t sliced_zher2k_lower(int n, int k, double alpha, const double *X, long long ldx, const double *Y,
-                                long long ldy, double beta, double *C, long long ldc, void *ws, cudaStream_t st)
+                                long long ldy, double beta, double *C, long long ldc, void *ws, cudaStream_t st,
+                                int *status)
 {
     // X Y^H + Y X^H = [X Y] [Y X]^H
     SlicedWs w = sliced_ws(2 * n, n, 4 * k, n, 4 * k, ws);
@@ -461,7 +464,7 @@ cudaError_t sliced_zher2k_lower(int n, int k, double alpha, const double *X, lon
     SlicedOp a, b;
     if ((e = slice_matrix(kViewZExpandN, 2 * n, 4 * k, XY, n, w.a, &a, st)) != cudaSuccess) return e;
     if ((e = slice_matrix(kViewZRowConj, n, 4 * k, YX, n, w.b, &b, st)) != cudaSuccess) return e;
-    return sliced_gemm(a, b, 2 * n, n, alpha, beta, C, 2 * ldc, kFillZLower, w.part, kPartialElems, st);
+    return sliced_gemm(a, b, 2 * n, n, alpha, beta, C, 2 * ldc, kFillZLower, w.part, kPartialElems, st, status);
 }
 
 }  // namespace gb
@@ -670,6 +673,23 @@ int gb_zher2k_sliced(int n, int k, double alpha, const double *X, int ldx, const
     if (ws_bytes < gb::sliced_zher2k_ws_bytes(n, k)) return -12;
     cudaError_t e = gb::sliced_zher2k_lower(n, k, alpha, X, ldx, Y, ldy, beta, C, ldc, workspace, (cudaStream_t)stream);
     return e == cudaSuccess ? GB_OK : GB_ERR_CUDA;
+}
+
+// Fault-injection hook of the tests (not in the header): C = A B, N N, whose
+// blocks stop copying operands after `hold` stages, with waits of wait_ns.
+int gb_test_sliced_hold(int m, int n, int k, const double *A, const double *B, double *C, void *workspace,
+                        long long wait_ns, int hold, int *status, void *stream)
+{
+    const cudaStream_t st = (cudaStream_t)stream;
+    gb::SlicedWs w = gb::sliced_ws(m, n, k, 0, 0, workspace);
+    gb::SlicedOp a, b;
+    if (gb::slice_matrix(gb::kViewRow, m, k, A, m, w.a, &a, st) != cudaSuccess ||
+        gb::slice_matrix(gb::kViewCol, n, k, B, k, w.b, &b, st) != cudaSuccess)
+        return GB_ERR_CUDA;
+    return gb::tc5_gemm(a, b, m, n, 1.0, 0.0, C, m, gb::kFillAll, w.part, gb::kPartialElems, st, status, wait_ns, hold) ==
+                   cudaSuccess
+               ? GB_OK
+               : GB_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -95,17 +95,24 @@ enum SlicedFill {
 // (A.R >= m, B.R >= n, A.K == B.K): row r of A times row c of B; `fill`
 // selects the entries written.  Both operands split: the FP32 product.  `work` (doubles) holds split-K partials; the
 // reduction splits while splits * m * n <= work_elems.
+// `status` (here and below): null, or a device word that receives
+// GB_ERR_TIMEOUT when one of the product's waits gives up; C then holds NaN in
+// every tile that was not finished.
 cudaError_t sliced_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double alpha, double beta, double *C,
-                        long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st);
+                        long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st,
+                        int *status = nullptr);
 
 // The digit form's parts (sliced_tc5.cu): plane bytes of an R x K operand, its
 // padded rows, cutting it (rmax: one word per row, scratch), and the product.
+// wait_ns: limit of the product's waits (0: the default); hold: for tests, a
+// block's copies end after that many stages (-1: never).
 size_t tc5_planes_bytes(int R, int K);
 int tc5_rows_padded(int R);
 cudaError_t tc5_slice_matrix(SliceView view, int R, int K, const double *src, long long ld, uint32_t *rmax,
                              uint16_t *planes, int *e, cudaStream_t st);
 cudaError_t tc5_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double alpha, double beta, double *C,
-                     long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st);
+                     long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st, int *status = nullptr,
+                     long long wait_ns = 0, int hold = -1);
 // C = alpha (sum of `splits` partials of m x n) + beta C
 cudaError_t sliced_reduce_launch(int m, int n, int splits, const double *part, double alpha, double beta, double *C,
                                  long long ldc, int fill, cudaStream_t st);
@@ -119,30 +126,32 @@ size_t sliced_syr2k_ws_bytes(int n, int k);
 size_t sliced_syrk_ws_bytes(int n, int k);
 cudaError_t sliced_dgemm(char transa, char transb, int m, int n, int k, double alpha, const double *A, long long lda,
                          const double *B, long long ldb, double beta, double *C, long long ldc, void *ws,
-                         cudaStream_t st, int digits = kSlices);
+                         cudaStream_t st, int digits = kSlices, int *status = nullptr);
 cudaError_t sliced_dsymm(char side, int m, int n, double alpha, const double *S, long long lds, const double *B,
                          long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st,
-                         int digits = kSlices);
+                         int digits = kSlices, int *status = nullptr);
 cudaError_t sliced_dsyr2k_lower(int n, int k, double alpha, const double *A, long long lda, const double *B,
                                 long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st,
-                                int digits = kSlices);
+                                int digits = kSlices, int *status = nullptr);
 cudaError_t sliced_dsyrk_lower_t(int n, int k, double alpha, const double *A, long long lda, double beta, double *C,
-                                 long long ldc, void *ws, cudaStream_t st, int digits = kSlices);
+                                 long long ldc, void *ws, cudaStream_t st, int digits = kSlices, int *status = nullptr);
 
 // Complex (interleaved) products with real alpha, beta; lda etc. in complex
 // elements.  C (m x n) = alpha op(A) B + beta C, op = 'N' or 'C'.
 size_t sliced_zgemm_ws_bytes(int m, int n, int k);
 cudaError_t sliced_zgemm(char transa, int m, int n, int k, double alpha, const double *A, long long lda,
                          const double *B, long long ldb, double beta, double *C, long long ldc, void *ws,
-                         cudaStream_t st);
+                         cudaStream_t st, int *status = nullptr);
 // C (m x n) = alpha S B + beta C, S Hermitian (lower triangle stored).
 size_t sliced_zhemm_ws_bytes(int m, int n);
 cudaError_t sliced_zhemm_left(int m, int n, double alpha, const double *S, long long lds, const double *B,
-                              long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st);
+                              long long ldb, double beta, double *C, long long ldc, void *ws, cudaStream_t st,
+                              int *status = nullptr);
 // Lower triangle of C (n x n) = alpha (X Y^H + Y X^H) + beta C, X, Y n x k;
 // the diagonal's imaginary parts are set to zero.
 size_t sliced_zher2k_ws_bytes(int n, int k);
 cudaError_t sliced_zher2k_lower(int n, int k, double alpha, const double *X, long long ldx, const double *Y,
-                                long long ldy, double beta, double *C, long long ldc, void *ws, cudaStream_t st);
+                                long long ldy, double beta, double *C, long long ldc, void *ws, cudaStream_t st,
+                                int *status = nullptr);
 
 }  // namespace gb

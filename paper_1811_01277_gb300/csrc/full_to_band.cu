@@ -256,7 +256,7 @@ int panel_chunks(int m) { return (m + kChunk - 1) / kChunk; }
 
 size_t panel_part_bytes(int m, int is_complex);
 cudaError_t panel_qr_resident(int is_complex, int m, int nb, double *P, long long lda, double *tau, double *Y,
-                              long long ldy, void *part, cudaStream_t st, bool *done);
+                              long long ldy, void *part, int *status, cudaStream_t st, bool *done);
 cudaError_t panel_y_and_t_prep(int m, int nb, const double *P, long long lda, double *Y, long long ldy,
                                cudaStream_t st);
 
@@ -270,12 +270,13 @@ size_t panel_qr_part_bytes(int m, int is_complex)
 }
 
 // Householder QR of the m x nb panel P (lda) and its explicit reflectors Y
-// (ldy); part holds panel_qr_part_bytes(m, 0) bytes, 256-byte aligned.
+// (ldy); part holds panel_qr_part_bytes(m, 0) bytes, 256-byte aligned; status as
+// for panel_qr_resident.
 cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
-                     cudaStream_t st)
+                     int *status, cudaStream_t st)
 {
     bool done = false;
-    cudaError_t er = panel_qr_resident(0, m, nb, P, lda, tau, Y, ldy, part, st, &done);
+    cudaError_t er = panel_qr_resident(0, m, nb, P, lda, tau, Y, ldy, part, status, st, &done);
     if (er != cudaSuccess || done) return er;
     const int nch = panel_chunks(m);
     double *norm_a = part, *norm_b = part + nch, *dots = part + 2 * nch;

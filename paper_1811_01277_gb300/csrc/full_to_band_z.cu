@@ -198,17 +198,18 @@ __global__ void __launch_bounds__(256) real_to_complex(long long rows, long long
 int panel_chunks(int m);
 
 cudaError_t panel_qr_resident(int is_complex, int m, int nb, double *P, long long lda, double *tau, double *Y,
-                              long long ldy, void *part, cudaStream_t st, bool *done);
+                              long long ldy, void *part, int *status, cudaStream_t st, bool *done);
 cudaError_t zpanel_y(int m, int nb, const double *P, long long lda, double *Y, long long ldy, cudaStream_t st);
 
 // Householder QR of the complex m x nb panel P and its explicit reflectors Y:
 // panel_qr.cu's kernel where the panel fits it, else the form above; part
-// holds panel_qr_part_bytes(m, 1) bytes, 256-byte aligned.
+// holds panel_qr_part_bytes(m, 1) bytes, 256-byte aligned; status as for
+// panel_qr_resident.
 cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
-                      cudaStream_t st)
+                      int *status, cudaStream_t st)
 {
     bool done = false;
-    cudaError_t er = panel_qr_resident(1, m, nb, P, lda, tau, Y, ldy, part, st, &done);
+    cudaError_t er = panel_qr_resident(1, m, nb, P, lda, tau, Y, ldy, part, status, st, &done);
     if (er != cudaSuccess || done) return er;
     const int nch = panel_chunks(m);
     double *norm_a = part, *norm_b = part + nch;

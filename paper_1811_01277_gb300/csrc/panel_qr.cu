@@ -33,6 +33,7 @@
 
 #include <algorithm>
 
+#include "elpa_gb300.h"
 #include "reduction.cuh"
 
 namespace gb {
@@ -64,10 +65,19 @@ struct PanelGrid {
     T ms[1];                    // [2][blocks][NB]
 };
 
+// How a panel's waits end: their limit, the status word that receives
+// GB_ERR_TIMEOUT (or null) and, for tests, the column at which block 0 does not
+// arrive (-1: none).
+struct PanelWait {
+    long long ns = kPanelWaitNs;
+    int *status = nullptr;
+    int hold = -1;
+};
+
 template <class T, int NB, int LPC, int RPT, bool GRID>
 __global__ void __launch_bounds__(NB *LPC, 1)
 panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__ tau_out, T *__restrict__ Y,
-                long long ldy, PanelGrid<T, NB> *gx)
+                long long ldy, PanelGrid<T, NB> *gx, PanelWait pw)
 {
     constexpr int CH = LPC * RPT;
     __shared__ PanelShared<T, NB, CH> sm;
@@ -140,10 +150,14 @@ panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__
             }
         }
         __syncthreads();
+        // a block that gave up neither waits nor arrives any more, so that no
+        // other block takes a late arrival for the one it waits for
+        const bool arrive = !sm.gave_up && (i != pw.hold || rank != 0);
         if (GRID) {
             if (tid == 0) {
                 __threadfence();
-                asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gx->arrivals) : "memory");
+                if (arrive)
+                    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&gx->arrivals) : "memory");
                 const unsigned int need = (unsigned int)(i + 1) * (unsigned int)blocks;
                 unsigned long long t0 = 0;
                 for (long long it = 0; !sm.gave_up; it++) {
@@ -151,21 +165,21 @@ panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__
                     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(got) : "l"(&gx->arrivals) : "memory");
                     if (got >= need) break;
                     if (it == 0) t0 = now_ns();
-                    if ((it & 63) == 63 && (long long)(now_ns() - t0) > kPanelWaitNs) sm.gave_up = 1;
+                    if ((it & 63) == 63 && (long long)(now_ns() - t0) > pw.ns) sm.gave_up = 1;
                 }
             }
             __syncthreads();
         } else {
-            if (tid < blocks) {
+            if (tid < blocks && arrive) {
                 asm volatile("fence.acq_rel.cluster;" ::: "memory");
                 mbar_arrive_remote(&sm.bar[par], tid);
             }
             const uint32_t bar = tc5::smem_addr(&sm.bar[par]);
             const uint32_t phase = (uint32_t)(i >> 1) & 1;
-            if (!mbar_try_cluster(bar, phase)) {
+            if (!*(volatile int *)&sm.gave_up && !mbar_try_cluster(bar, phase)) {
                 const unsigned long long t0 = now_ns();
                 for (long long it = 1; !mbar_try_cluster(bar, phase); it++)
-                    if ((it & 63) == 0 && (long long)(now_ns() - t0) > kPanelWaitNs) {
+                    if ((it & 63) == 0 && (long long)(now_ns() - t0) > pw.ns) {
                         sm.gave_up = 1;
                         break;
                     }
@@ -231,7 +245,14 @@ panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__
     T nan;
     zero_of(nan);
     *(double *)&nan = __longlong_as_double(0x7ff8000000000000ll);
-    if (sm.gave_up && tid < nb) tau_out[tid] = nan;   // a wait gave up: the result is void and says so
+    // a wait gave up: the result is void and says so, in this block's rows
+    // (which no other block writes), in tau and in the status word
+    if (sm.gave_up) {
+        if (tid < nb) tau_out[tid] = nan;
+        if (tid == 0 && pw.status) atomicExch(pw.status, GB_ERR_TIMEOUT);
+#pragma unroll
+        for (int t = 0; t < RPT; t++) a[t] = nan;
+    }
     if (rank == 0 && tid >= steps && tid < nb) zero_of(tau_out[tid]);
 #pragma unroll
     for (int t = 0; t < RPT; t++) {
@@ -242,6 +263,7 @@ panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__
                 T y = a[t];
                 if (r < col) zero_of(y);
                 else if (r == col) one_of(y);
+                if (sm.gave_up) y = nan;
                 Y[(long long)col * ldy + r] = y;
             }
         }
@@ -253,7 +275,8 @@ panel_qr_kernel(int m, int nb, T *__restrict__ P, long long lda, T *__restrict__
 }
 
 template <class T, int NB, int LPC, int RPT>
-cudaError_t launch_cluster(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, cudaStream_t st)
+cudaError_t launch_cluster(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, const PanelWait &pw,
+                           cudaStream_t st)
 {
     constexpr int CH = LPC * RPT;
     auto kernel = panel_qr_kernel<T, NB, LPC, RPT, false>;
@@ -273,14 +296,14 @@ cudaError_t launch_cluster(int m, int nb, T *P, long long lda, T *tau, T *Y, lon
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, m, nb, P, lda, tau, Y, ldy, (PanelGrid<T, NB> *)nullptr);
+    return cudaLaunchKernelEx(&cfg, kernel, m, nb, P, lda, tau, Y, ldy, (PanelGrid<T, NB> *)nullptr, pw);
 }
 
 // *done = false (and nothing launched) where the grid does not fit in
 // 1 / `share` of the device's co-resident capacity
 template <class T, int NB, int LPC, int RPT>
 cudaError_t launch_grid(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, void *part, int sms,
-                        int share, cudaStream_t st, bool *done)
+                        int share, PanelWait pw, cudaStream_t st, bool *done)
 {
     constexpr int CH = LPC * RPT;
     auto kernel = panel_qr_kernel<T, NB, LPC, RPT, true>;
@@ -291,25 +314,25 @@ cudaError_t launch_grid(int m, int nb, T *P, long long lda, T *tau, T *Y, long l
     if ((long long)blocks * share > (long long)per_sm * sms) return cudaSuccess;
     if ((e = cudaMemsetAsync(part, 0, 256, st)) != cudaSuccess) return e;
     PanelGrid<T, NB> *gx = (PanelGrid<T, NB> *)part;
-    void *args[] = {&m, &nb, &P, &lda, &tau, &Y, &ldy, &gx};
+    void *args[] = {&m, &nb, &P, &lda, &tau, &Y, &ldy, &gx, &pw};
     *done = true;
     return cudaLaunchCooperativeKernel((const void *)kernel, dim3(blocks), dim3(NB * LPC), args, 0, st);
 }
 
 template <class T>
-cudaError_t panel_qr_t(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, void *part, cudaStream_t st,
-                       bool *done)
+cudaError_t panel_qr_t(int m, int nb, T *P, long long lda, T *tau, T *Y, long long ldy, void *part, const PanelWait &pw,
+                       cudaStream_t st, bool *done)
 {
     constexpr bool Z = sizeof(T) == 16;
     *done = true;
     if (nb <= 32) {
-        if (m <= 32 * kClusterMax) return launch_cluster<T, 32, 8, 4>(m, nb, P, lda, tau, Y, ldy, st);
-        if (m <= 64 * kClusterMax) return launch_cluster<T, 32, 8, 8>(m, nb, P, lda, tau, Y, ldy, st);
-        if (m <= 128 * kClusterMax) return launch_cluster<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, st);
+        if (m <= 32 * kClusterMax) return launch_cluster<T, 32, 8, 4>(m, nb, P, lda, tau, Y, ldy, pw, st);
+        if (m <= 64 * kClusterMax) return launch_cluster<T, 32, 8, 8>(m, nb, P, lda, tau, Y, ldy, pw, st);
+        if (m <= 128 * kClusterMax) return launch_cluster<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, pw, st);
     } else {
-        if (m <= 32 * kClusterMax) return launch_cluster<T, 64, 4, 8>(m, nb, P, lda, tau, Y, ldy, st);
-        if (m <= 64 * kClusterMax) return launch_cluster<T, 64, 4, 16>(m, nb, P, lda, tau, Y, ldy, st);
-        if (!Z && m <= 128 * kClusterMax) return launch_cluster<T, 64, Z ? 4 : 8, 16>(m, nb, P, lda, tau, Y, ldy, st);
+        if (m <= 32 * kClusterMax) return launch_cluster<T, 64, 4, 8>(m, nb, P, lda, tau, Y, ldy, pw, st);
+        if (m <= 64 * kClusterMax) return launch_cluster<T, 64, 4, 16>(m, nb, P, lda, tau, Y, ldy, pw, st);
+        if (!Z && m <= 128 * kClusterMax) return launch_cluster<T, 64, Z ? 4 : 8, 16>(m, nb, P, lda, tau, Y, ldy, pw, st);
     }
     *done = false;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -324,13 +347,13 @@ cudaError_t panel_qr_t(int m, int nb, T *P, long long lda, T *tau, T *Y, long lo
     // room beside it; the tallest panels (over 9728 rows real, 4864 complex)
     // may take all of it
     if (nb <= 32) {
-        e = launch_grid<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 2, st, done);
+        e = launch_grid<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 2, pw, st, done);
         if (e != cudaSuccess || *done) return e;
-        return launch_grid<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 1, st, done);
+        return launch_grid<T, 32, 8, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 1, pw, st, done);
     }
-    e = launch_grid<T, 64, 4, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 2, st, done);
+    e = launch_grid<T, 64, 4, 16>(m, nb, P, lda, tau, Y, ldy, part, sms, 2, pw, st, done);
     if (e != cudaSuccess || *done) return e;
-    return launch_grid<T, 64, 4, Z ? 16 : 32>(m, nb, P, lda, tau, Y, ldy, part, sms, 1, st, done);
+    return launch_grid<T, 64, 4, Z ? 16 : 32>(m, nb, P, lda, tau, Y, ldy, part, sms, 1, pw, st, done);
 }
 
 // T (nb x nb upper triangular) of the block reflector I - Y T Y^H is the
@@ -494,11 +517,36 @@ size_t panel_part_bytes(int m, int is_complex)
 // QR of the m x nb panel P (lda, nb <= 64) and, where Y is not null, its
 // explicit reflectors (ldy).  *done = false: nothing was done, the panel is
 // too tall for one co-resident grid (or for a cluster, under capture).
+// `status`: a device word that receives GB_ERR_TIMEOUT when a wait gives up, or
+// null.
 cudaError_t panel_qr_resident(int is_complex, int m, int nb, double *P, long long lda, double *tau, double *Y,
-                              long long ldy, void *part, cudaStream_t st, bool *done)
+                              long long ldy, void *part, int *status, cudaStream_t st, bool *done)
 {
-    if (is_complex) return panel_qr_t<Zc>(m, nb, (Zc *)P, lda, (Zc *)tau, (Zc *)Y, ldy, part, st, done);
-    return panel_qr_t<double>(m, nb, P, lda, tau, Y, ldy, part, st, done);
+    PanelWait pw;
+    pw.status = status;
+    if (is_complex) return panel_qr_t<Zc>(m, nb, (Zc *)P, lda, (Zc *)tau, (Zc *)Y, ldy, part, pw, st, done);
+    return panel_qr_t<double>(m, nb, P, lda, tau, Y, ldy, part, pw, st, done);
 }
 
 }  // namespace gb
+
+extern "C" {
+
+// Fault-injection hook of the tests (not in the header): a panel of which
+// block 0 does not arrive at column `hold`, with waits of wait_ns.
+int gb_test_panel_hold(int is_complex, int m, int nb, double *P, double *tau, double *Y, void *part, long long wait_ns,
+                       int hold, int *status, void *stream)
+{
+    gb::PanelWait pw;
+    pw.ns = wait_ns;
+    pw.status = status;
+    pw.hold = hold;
+    bool done = false;
+    const cudaStream_t st = (cudaStream_t)stream;
+    const cudaError_t e =
+        is_complex ? gb::panel_qr_t<gb::Zc>(m, nb, (gb::Zc *)P, m, (gb::Zc *)tau, (gb::Zc *)Y, m, part, pw, st, &done)
+                   : gb::panel_qr_t<double>(m, nb, P, m, tau, Y, m, part, pw, st, &done);
+    return e == cudaSuccess && done ? GB_OK : GB_ERR_CUDA;
+}
+
+}  // extern "C"

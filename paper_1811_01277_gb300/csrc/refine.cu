@@ -561,7 +561,7 @@ namespace gb {
 
 namespace {
 
-// status slots (2 x 256 bytes) | X (n x n) | lambda (n) | one region that
+// status slots (3 x 256 bytes) | X (n x n) | lambda (n) | one region that
 // the low-precision solve and then the refinement steps use
 struct MixedWs {
     char *status;
@@ -579,7 +579,7 @@ MixedWs mixed_carve(int n, int nbw, char *base)
         off += a256(bytes);
         return p;
     };
-    w.status = take(512);
+    w.status = take(768);
     w.X = (double *)take((size_t)n * n * 8);
     w.lam = (double *)take((size_t)n * 8);
     w.region_bytes = std::max(gb_solve_workspace_bytes(n, n, nbw), gb_refine_syev_workspace_bytes(n));
@@ -637,7 +637,7 @@ int gb_solve_mixed_query(const void *workspace, int n, int nev, int nbw, void *s
     if (!workspace) return -1;
     if (cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess) return GB_ERR_CUDA;
     const gb::MixedWs w = gb::mixed_carve(n, nbw, (char *)workspace);
-    for (int i = 0; i < 2; i++) {
+    for (int i = 0; i < 3; i++) {
         int head[3] = {0, 0, 0};  // ticket, abort, error
         if (cudaMemcpy(head, w.status + 256 * i, sizeof(head), cudaMemcpyDeviceToHost) != cudaSuccess)
             return GB_ERR_CUDA;

@@ -45,6 +45,7 @@
 #include <algorithm>
 
 #include "dgemm_sliced.cuh"
+#include "elpa_gb300.h"
 #include "mma_bf16.cuh"
 #include "slice_views.cuh"
 #include "tcgen05.cuh"
@@ -268,6 +269,9 @@ struct ProductArgs {
     long long ldc;
     int fill, swapped;            // swapped: entry (row of A, row of B) is C(row of B, row of A)
     double *part;                 // split-K partials (C's orientation, leading dimension rows of C)
+    int *status;                  // null, or receives GB_ERR_TIMEOUT when a wait gives up
+    long long wait_ns;            // limit of the waits
+    uint32_t hold;                // for tests: a block's copies end after this many stages
 };
 
 struct Tile {
@@ -308,9 +312,9 @@ struct Tc5Sync {
     int abort;
 };
 
-__device__ __forceinline__ bool wait5(const unsigned long long *bar, uint32_t parity, Tc5Sync &sy)
+__device__ __forceinline__ bool wait5(const unsigned long long *bar, uint32_t parity, Tc5Sync &sy, long long wait_ns)
 {
-    if (tc5::mbar_wait(tc5::smem_addr(bar), parity & 1, kWaitNs)) return true;
+    if (tc5::mbar_wait(tc5::smem_addr(bar), parity & 1, wait_ns)) return true;
     *(volatile int *)&sy.abort = 1;
     return false;
 }
@@ -396,7 +400,7 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                     const unsigned char *gb_ = p.B + ((size_t)(x.tn >> 1) * p.KC) * kBlockBytes + (x.tn & 1) * kBPlane;
                     for (int kc = x.kc0; kc < x.kc1; kc++, q++) {
                         const int st = q & 1;
-                        if (q >= 2 && !wait5(&sy.empty[st], (q >> 1) - 1, sy)) {
+                        if (q == p.hold || (q >= 2 && !wait5(&sy.empty[st], (q >> 1) - 1, sy, p.wait_ns))) {
                             ok = false;
                             break;
                         }
@@ -420,7 +424,7 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
             {
                 uint32_t q = 0, grp = 0;
                 bool ok = true;
-                auto wait_all = [&](auto *bar, uint32_t n) { return __all_sync(0xffffffffu, wait5(bar, n, sy)) != 0; };
+                auto wait_all = [&](auto *bar, uint32_t n) { return __all_sync(0xffffffffu, wait5(bar, n, sy, p.wait_ns)) != 0; };
                 auto mmas = [&](uint32_t st, bool high, bool first) {
                     if (!tc5::elect_one()) return;
                     const uint32_t sa = tc5::smem_addr(smem + st * kStageBytes);
@@ -491,6 +495,7 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
         const int quarter = warp & 3, c0 = (warp >> 2) * kCols;
         const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16) + c0;
         uint32_t grp = 0;
+        bool bad = false;   // a wait gave up: this tile and the block's later ones are NaN
         for (long long t = blockIdx.x; t < p.tiles; t += gridDim.x) {
             const Tile x = tile_of(p, t);
             long long hi[kCols];
@@ -525,8 +530,8 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                         if (wanted(cb + j)) old[j] = src[j * cs];
                 }
             }
-            for (int kc = x.kc0; kc < x.kc1; kc += kGroup, grp++) {
-                wait5(&sy.ready[0], grp, sy);
+            for (int kc = x.kc0; kc < x.kc1 && !bad; kc += kGroup, grp++) {
+                wait5(&sy.ready[0], grp, sy, p.wait_ns);
                 tc5::fence_after_sync();
 #pragma unroll
                 for (int h = 0; h < kCols / 8; h++) {
@@ -545,7 +550,7 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                 __syncwarp();
                 if (lane == 0)
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc5::smem_addr(&sy.freed[0])) : "memory");
-                wait5(&sy.ready[1], grp, sy);
+                wait5(&sy.ready[1], grp, sy, p.wait_ns);
                 tc5::fence_after_sync();
 #pragma unroll
                 for (int h = 0; h < kCols / 8; h++) {
@@ -566,9 +571,8 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                 __syncwarp();
                 if (lane == 0)
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc5::smem_addr(&sy.freed[1])) : "memory");
-                if (*(volatile int *)&sy.abort) break;
+                bad = *(volatile int *)&sy.abort != 0;
             }
-            const bool bad = *(volatile int *)&sy.abort != 0;
             // entry (r, c) of A B^T times 2^(ea + eb - 68)
             const int er = r < p.m ? p.ea[r] - 68 : 0;
             double *out = p.C + r * rs;
@@ -601,7 +605,7 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                         if (e > kNonFinite / 2) v[j] = p.alpha == 0.0 ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
                     }
                 }
-                if (bad) {   // a wait gave up
+                if (bad) {
 #pragma unroll
                     for (int j = 0; j < 8; j++) v[j] = __longlong_as_double(0x7ff8000000000000ll);
                 }
@@ -633,11 +637,11 @@ __global__ void __launch_bounds__(kThreads5, 1) tc5_product(const ProductArgs p)
                     }
                 }
             }
-            if (bad) break;
         }
     }
     tc5::fence_before_sync();
     __syncthreads();
+    if (tid == 0 && sy.abort && p.status) atomicExch(p.status, GB_ERR_TIMEOUT);
     if (warp == 0) {
         tc5::fence_after_sync();
         tc5::tmem_dealloc(tmem, 512);
@@ -679,7 +683,8 @@ cudaError_t tc5_slice_matrix(SliceView view, int R, int K, const double *src, lo
 // C = alpha A B^T + beta C for two digit-plane operands; arguments checked by
 // sliced_gemm.
 cudaError_t tc5_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double alpha, double beta, double *C,
-                     long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st)
+                     long long ldc, int fill, double *work, size_t work_elems, cudaStream_t st, int *status,
+                     long long wait_ns, int hold)
 {
     int dev = 0, sms = 148;
     cudaError_t e;
@@ -726,6 +731,9 @@ cudaError_t tc5_gemm(const SlicedOp &A, const SlicedOp &B, int m, int n, double 
     p.fill = fill;
     p.swapped = sw;
     p.part = splits > 1 ? work : nullptr;
+    p.status = status;
+    p.wait_ns = wait_ns > 0 ? wait_ns : kWaitNs;
+    p.hold = hold >= 0 ? (uint32_t)hold : 0xffffffffu;
     // opt in to the large dynamic shared memory (cheap; per device, so every call)
     if ((e = cudaFuncSetAttribute(tc5_product, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem5)) != cudaSuccess)
         return e;

@@ -42,11 +42,11 @@ namespace gb {
 
 size_t tridiag_dc_workspace_bytes(int n);
 cudaError_t tridiag_dc_d(int n, int nev, const double *d, const double *e, double *lam, double *Z, long long ldz,
-                         void *ws, cudaStream_t st);
+                         void *ws, cudaStream_t st, int *status = nullptr);
 
 size_t panel_qr_part_bytes(int m, int is_complex);
 cudaError_t panel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
-                     cudaStream_t st);
+                     int *status, cudaStream_t st);
 cudaError_t panels_y(int is_complex, int m, int nb, int np, const double *P, long long lda, double *Y, long long ldy,
                      cudaStream_t st);
 cudaError_t panel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt,
@@ -55,7 +55,7 @@ cudaError_t newton_schulz_matrix(int k, double *G, long long ldg, cudaStream_t s
 cudaError_t band_from_full(int n, int b, const double *A, long long lda, double *AB, long long ldab, cudaStream_t st);
 
 cudaError_t zpanel_qr(int m, int nb, double *P, long long lda, double *tau, double *Y, long long ldy, double *part,
-                      cudaStream_t st);
+                      int *status, cudaStream_t st);
 cudaError_t zpanel_t(int nb, const double *G, long long ldg, const double *tau, double *T, long long ldt,
                      cudaStream_t st);
 cudaError_t zband_from_full(int n, int b, const double *A, long long lda, double *AB, long long ldab,
@@ -129,6 +129,7 @@ cudaEvent_t *stage_events(cudaStream_t st)
 struct SolveWs {
     double *Aw, *tauP, *Tall, *Y, *Y2, *YT, *X, *Pm, *M, *G, *part, *AB, *d, *e, *hv, *ht, *Ztri, *Gns, *S, *S2, *gw,
         *gw2, *Yg, *Gg, *Tg;
+    int *status;   // 256 bytes, the error in the third word: panels and products whose waits gave up
     void *chase, *eig, *tev, *sl, *dc;
     size_t chase_bytes, tev_bytes, gw_elems, gw2_elems, sl_bytes, total, ptotal;
 };
@@ -226,6 +227,7 @@ SolveWs carve(int n, int nev, int b, char *base, char *pbase = nullptr, bool spl
     w.gw2 = (double *)take(w.gw2_elems * 8);
     w.chase_bytes = gb::band_to_tridi_workspace_bytes(n, b);
     w.chase = ptake(w.chase_bytes);
+    w.status = (int *)ptake(256);
     w.eig = take(gb::tridiag_eig_workspace_bytes(n, nev));
     w.tev_bytes = gb_trans_ev_workspace_bytes(n, b, nev, 0, nullptr);
     w.tev = take(w.tev_bytes ? w.tev_bytes : 256);
@@ -241,6 +243,7 @@ SolveWs carve(int n, int nev, int b, char *base, char *pbase = nullptr, bool spl
 struct SolveWsZ {
     double *Aw, *tauP, *Tall, *Y, *YT, *X, *Pm, *M, *G, *part, *AB, *d, *e, *hv, *ht, *Zre, *Gns, *Zns, *S, *S2, *gw,
         *Yg, *Gg, *Tg;
+    int *status;
     void *chase, *eig, *sl, *tev, *dc;
     size_t chase_bytes, gw_elems, sl_bytes, tev_bytes, total;
 };
@@ -301,6 +304,7 @@ SolveWsZ carve_z(int n, int nev, int b, char *base)
     w.gw = (double *)take(w.gw_elems * 8);
     w.chase_bytes = gb::band_to_tridi_workspace_bytes_z(n, b);
     w.chase = take(w.chase_bytes);
+    w.status = (int *)take(256);
     w.eig = take(gb::tridiag_eig_workspace_bytes(n, nev));
     w.sl_bytes = zsliced_region_bytes(n, nev, b);
     w.sl = w.sl_bytes ? take(w.sl_bytes) : nullptr;
@@ -379,6 +383,7 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     // the caller's stream applies the rest of that update (the rank-2b update
     // of the trailing lower triangle, the bulk of the flops)
     GB_STAGE(0);
+    GB_CU(cudaMemsetAsync(w.status, 0, 256, st));
     GB_CU(cudaMemcpy2DAsync(w.Aw, (size_t)n * 8, A, (size_t)lda * 8, (size_t)n * 8, n, cudaMemcpyDeviceToDevice, st));
     // small problems factor their panels in line: the helper stream would
     // gain little there and would double the streams concurrent solves use
@@ -393,7 +398,8 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         double *panel = w.Aw + (long long)j * ldw + (j + b);
         double *Yp = Ybuf[p & 1];
         cudaError_t e;
-        if ((e = gb::panel_qr(m, b, panel, ldw, w.tauP + (long long)p * b, Yp, m, w.part, fst)) != cudaSuccess)
+        if ((e = gb::panel_qr(m, b, panel, ldw, w.tauP + (long long)p * b, Yp, m, w.part, w.status + 2, fst)) !=
+            cudaSuccess)
             return e;
         if ((e = gb::dfma_gemm('T', 'N', b, b, m, 1.0, Yp, m, Yp, m, 0.0, w.G, b, w.gw2, w.gw2_elems, fst)) !=
             cudaSuccess)
@@ -406,7 +412,7 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     // lower triangle of C -= X Y^T + Y X^T
     auto update = [&](int m, const double *X, const double *Yp, long long ldy, double *C) -> cudaError_t {
         if (use_sliced(m, m, b))
-            return gb::sliced_dsyr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, w.sl, st, pd);
+            return gb::sliced_dsyr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, w.sl, st, pd, w.status + 2);
         return gb::dfma_syr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, st);
     };
     int pp = 0;
@@ -427,7 +433,7 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         // only the lower triangle of A2 is kept: X = A2 (Y T) (symmetric
         // product), W = X - Y M / 2, then A2 -= W Y^T + Y W^T on the lower triangle
         if (use_sliced(m, b, m))
-            GB_CU(gb::sliced_dsymm('L', m, b, 1.0, A2, ldw, w.YT, m, 0.0, w.X, m, w.sl, st, pd));
+            GB_CU(gb::sliced_dsymm('L', m, b, 1.0, A2, ldw, w.YT, m, 0.0, w.X, m, w.sl, st, pd, w.status + 2));
         else
             GB_CU(gb::dfma_symm('L', m, b, 1.0, A2, ldw, w.YT, m, 0.0, w.X, m, w.gw, w.gw_elems, st));
         GB_CU(gb::dfma_gemm('T', 'N', b, b, m, 1.0, Yp, m, w.X, m, 0.0, w.Pm, b, w.gw, w.gw_elems, st));
@@ -464,7 +470,7 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     // inverse iteration and one Newton-Schulz orthogonalisation step
     GB_STAGE(2);
     if (w.dc && !(flags & GB_SOLVE_TRIDIAG_BISECT)) {
-        GB_CU(gb::tridiag_dc_d(n, nev, w.d, w.e, ev, Z, ldz, w.dc, st));
+        GB_CU(gb::tridiag_dc_d(n, nev, w.d, w.e, ev, Z, ldz, w.dc, st, w.status + 2));
         GB_STAGE(3);
         GB_STAGE(4);
     } else {
@@ -474,12 +480,13 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         GB_STAGE(4);
         // G = Z^T Z (lower triangle), M = (3I - G)/2, Z <- Z M
         if (use_sliced(nev, nev, n))
-            GB_CU(gb::sliced_dsyrk_lower_t(nev, n, 1.0, w.Ztri, n, 0.0, w.Gns, nev, w.sl, st));
+            GB_CU(gb::sliced_dsyrk_lower_t(nev, n, 1.0, w.Ztri, n, 0.0, w.Gns, nev, w.sl, st, gb::kSlices, w.status + 2));
         else
             GB_CU(gb::dfma_syrk_lower_t(nev, n, 1.0, w.Ztri, n, 0.0, w.Gns, nev, st));
         GB_CU(gb::newton_schulz_matrix(nev, w.Gns, nev, st));
         if (use_sliced(n, nev, nev))
-            GB_CU(gb::sliced_dsymm('R', n, nev, 1.0, w.Gns, nev, w.Ztri, n, 0.0, Z, ldz, w.sl, st));
+            GB_CU(gb::sliced_dsymm('R', n, nev, 1.0, w.Gns, nev, w.Ztri, n, 0.0, Z, ldz, w.sl, st, gb::kSlices,
+                                    w.status + 2));
         else
             GB_CU(gb::dfma_symm('R', n, nev, 1.0, w.Gns, nev, w.Ztri, n, 0.0, Z, ldz, w.gw, w.gw_elems, st));
     }
@@ -494,7 +501,8 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     auto gemm = [&](char ta, int m_, int n_, int k_, double alpha, const double *A_, long long la, const double *B_,
                     long long lb, double beta, double *C_, long long lc, int digits) -> cudaError_t {
         if (use_sliced(m_, n_, k_))
-            return gb::sliced_dgemm(ta, 'N', m_, n_, k_, alpha, A_, la, B_, lb, beta, C_, lc, w.sl, st, digits);
+            return gb::sliced_dgemm(ta, 'N', m_, n_, k_, alpha, A_, la, B_, lb, beta, C_, lc, w.sl, st, digits,
+                                    w.status + 2);
         return gb::dfma_gemm(ta, 'N', m_, n_, k_, alpha, A_, la, B_, lb, beta, C_, lc, w.gw, w.gw_elems, st);
     };
     const int per = group_panels(n, b);
@@ -581,6 +589,7 @@ int solve_z_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     const int P = b < n ? (n - 1) / b : 0;  // panels of full -> band
     if (parts & kPartFront) {
     // ---- full -> band: A2 <- Q^H A2 Q, Q = I - Y T Y^H
+    GB_CU(cudaMemsetAsync(w.status, 0, 256, st));
     GB_CU(cudaMemcpy2DAsync(Aw, (size_t)n * 16, A, (size_t)lda * 16, (size_t)n * 16, n, cudaMemcpyDeviceToDevice, st));
     int pp = 0;
     for (int j = 0; j + b < n; j += b, pp++) {
@@ -589,13 +598,13 @@ int solve_z_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         C *A2 = Aw + (long long)(j + b) * ldw + (j + b);
         double *tau = w.tauP + (long long)pp * b * 2;
         C *T = (C *)(w.Tall + (long long)pp * b * b * 2);
-        GB_CU(gb::zpanel_qr(m, b, (double *)panel, ldw, tau, (double *)Y, m, w.part, st));
+        GB_CU(gb::zpanel_qr(m, b, (double *)panel, ldw, tau, (double *)Y, m, w.part, w.status + 2, st));
         GB_CU(zg('C', 'N', b, b, m, one, Y, m, Y, m, zero, G, b, 0));
         GB_CU(gb::zpanel_t(b, (const double *)G, b, tau, (double *)T, b, st));
         GB_CU(zg('N', 'N', m, b, b, one, Y, m, T, b, zero, YT, m, 0));
         if (use_zsliced(m, b, m))
             GB_CU(gb::sliced_zhemm_left(m, b, 1.0, (const double *)A2, ldw, (const double *)YT, m, 0.0, (double *)X, m,
-                                        w.sl, st));
+                                        w.sl, st, w.status + 2));
         else
             GB_CU(zg('H', 'N', m, b, m, one, A2, ldw, YT, m, zero, X, m, 0));
         GB_CU(zg('C', 'N', b, b, m, one, Y, m, X, m, zero, Pm, b, 0));
@@ -604,7 +613,7 @@ int solve_z_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         // lower triangle of A2 -= X Y^H + Y X^H (Hermitian rank-2b update)
         if (use_zsliced(m, m, b)) {
             GB_CU(gb::sliced_zher2k_lower(m, b, -1.0, (const double *)X, m, (const double *)Y, m, 1.0, (double *)A2,
-                                          ldw, w.sl, st));
+                                          ldw, w.sl, st, w.status + 2));
         } else {
             GB_CU(zg('N', 'C', m, m, b, mone, X, m, Y, m, one, A2, ldw, 1));
             GB_CU(zg('N', 'C', m, m, b, mone, Y, m, X, m, one, A2, ldw, 1));
@@ -621,16 +630,17 @@ int solve_z_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     // ---- real tridiagonal eigenpairs (divide and conquer, or bisection,
     // inverse iteration and Newton-Schulz), promoted to complex Z
     if (w.dc && !(flags & GB_SOLVE_TRIDIAG_BISECT)) {
-        GB_CU(gb::tridiag_dc_d(n, nev, w.d, w.e, ev, w.Zns, n, w.dc, st));
+        GB_CU(gb::tridiag_dc_d(n, nev, w.d, w.e, ev, w.Zns, n, w.dc, st, w.status + 2));
     } else {
         GB_CU(gb::tridiag_eig_d(n, nev, w.d, w.e, ev, w.Zre, n, w.eig, st));
         if (zslice_ok && sliced_pays(nev, nev, n))
-            GB_CU(gb::sliced_dsyrk_lower_t(nev, n, 1.0, w.Zre, n, 0.0, w.Gns, nev, w.sl, st));
+            GB_CU(gb::sliced_dsyrk_lower_t(nev, n, 1.0, w.Zre, n, 0.0, w.Gns, nev, w.sl, st, gb::kSlices, w.status + 2));
         else
             GB_CU(gb::dfma_syrk_lower_t(nev, n, 1.0, w.Zre, n, 0.0, w.Gns, nev, st));
         GB_CU(gb::newton_schulz_matrix(nev, w.Gns, nev, st));
         if (zslice_ok && sliced_pays(n, nev, nev))
-            GB_CU(gb::sliced_dsymm('R', n, nev, 1.0, w.Gns, nev, w.Zre, n, 0.0, w.Zns, n, w.sl, st));
+            GB_CU(gb::sliced_dsymm('R', n, nev, 1.0, w.Gns, nev, w.Zre, n, 0.0, w.Zns, n, w.sl, st, gb::kSlices,
+                                    w.status + 2));
         else
             GB_CU(gb::dfma_symm('R', n, nev, 1.0, w.Gns, nev, w.Zre, n, 0.0, w.Zns, n, w.gw, w.gw_elems, st));
     }
@@ -645,7 +655,7 @@ int solve_z_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
                     C *C_, long long lc) -> cudaError_t {
         if (use_zsliced(m_, n_, k_))
             return gb::sliced_zgemm(oa, m_, n_, k_, subtract ? -1.0 : 1.0, (const double *)A_, la, (const double *)B_, lb,
-                                    subtract ? 1.0 : 0.0, (double *)C_, lc, w.sl, st);
+                                    subtract ? 1.0 : 0.0, (double *)C_, lc, w.sl, st, w.status + 2);
         return zg(oa, 'N', m_, n_, k_, subtract ? mone : one, A_, la, B_, lb, subtract ? one : zero, C_, lc, 0);
     };
     C *Yg = (C *)w.Yg, *Gg = (C *)w.Gg, *Tg = (C *)w.Tg;
@@ -765,6 +775,7 @@ int gb_solve_query_z(const void *workspace, int n, int nev, int nbw, void *strea
     SolveWsZ w = carve_z(n, nev, nbw, (char *)workspace);
     int rc = gb_trans_ev_query(w.chase, w.chase_bytes, stream);
     if (rc != GB_OK) return rc;
+    if ((rc = gb_trans_ev_query(w.status, 256, stream)) != GB_OK) return rc;
     return gb_trans_ev_query(w.tev, w.tev_bytes, stream);
 }
 
@@ -828,9 +839,9 @@ namespace gb {
 cudaError_t solve_status_copy(const void *ws, int n, int nev, int nbw, void *dst, cudaStream_t st)
 {
     SolveWs w = carve(n, nev, nbw, (char *)ws);
-    const void *src[2] = {w.chase, w.tev};
-    const size_t bytes[2] = {w.chase_bytes, w.tev_bytes};
-    for (int i = 0; i < 2; i++) {
+    const void *src[3] = {w.chase, w.tev, w.status};
+    const size_t bytes[3] = {w.chase_bytes, w.tev_bytes, 256};
+    for (int i = 0; i < 3; i++) {
         char *d = (char *)dst + 256 * i;
         const cudaError_t e = bytes[i] >= 256 ? cudaMemcpyAsync(d, src[i], 16, cudaMemcpyDeviceToDevice, st)
                                               : cudaMemsetAsync(d, 0, 16, st);
@@ -849,6 +860,7 @@ int gb_solve_query(const void *workspace, int n, int nev, int nbw, void *stream)
     SolveWs w = carve(n, nev, nbw, (char *)workspace);
     int rc = gb_trans_ev_query(w.chase, w.chase_bytes, stream);
     if (rc != GB_OK) return rc;
+    if ((rc = gb_trans_ev_query(w.status, 256, stream)) != GB_OK) return rc;
     return gb_trans_ev_query(w.tev, w.tev_bytes, stream);
 }
 
@@ -1220,6 +1232,7 @@ int gb_solve_batched_staged_query(const void *workspace, int count, const int *n
         const int s = i % nslots;
         char *scr = (char *)base + (L.total - L.scratch_slot * (size_t)nslots) + L.scratch_slot * (size_t)s;
         const SolveWs w = carve(n[i], nev[i], b, scr, (char *)base + L.persist_off[i], true);
+        if ((rc = gb_trans_ev_query(w.status, 256, stream)) != GB_OK) return rc;
         // each slot's last problem left its back-transformation's status in the slot
         if (i + nslots >= count && (rc = gb_trans_ev_query(w.tev, w.tev_bytes, stream)) != GB_OK) return rc;
     }

@@ -767,9 +767,9 @@ DcWs dc_carve(int n, char *base)
 size_t tridiag_dc_workspace_bytes(int n) { return n >= 1 ? dc_carve(n, nullptr).total : 0; }
 
 // lam[0..nev) ascending and Z[:, 0..nev) (ldz) the matching eigenvectors of
-// the tridiagonal (d, e); asynchronous on st.
+// the tridiagonal (d, e); asynchronous on st.  status: as for sliced_gemm.
 cudaError_t tridiag_dc_d(int n, int nev, const double *d, const double *e, double *lam, double *Z, long long ldz,
-                         void *ws, cudaStream_t st)
+                         void *ws, cudaStream_t st, int *status)
 {
     if (n < 1 || nev < 1) return cudaSuccess;
     DcWs w = dc_carve(n, (char *)ws);
@@ -819,10 +819,10 @@ cudaError_t tridiag_dc_d(int n, int nev, const double *d, const double *e, doubl
                 const double *Um = w.U + (size_t)off * n;
                 const size_t ld = (size_t)n;
                 if ((err = sliced_dgemm('N', 'N', n1, s, n1, 1.0, Q + off + off * ld, n, Um, s, 0.0, Qn + off + off * ld,
-                                        n, w.sl, st)) != cudaSuccess)
+                                        n, w.sl, st, kSlices, status)) != cudaSuccess)
                     return err;
                 if ((err = sliced_dgemm('N', 'N', n2, s, n2, 1.0, Q + (off + n1) + (off + n1) * ld, n, Um + n1, s, 0.0,
-                                        Qn + (off + n1) + off * ld, n, w.sl, st)) != cudaSuccess)
+                                        Qn + (off + n1) + off * ld, n, w.sl, st, kSlices, status)) != cudaSuccess)
                     return err;
             }
         }
@@ -852,7 +852,7 @@ int gb_tridiag_dc_d(int n, const double *d, const double *e, double *lam, double
     if (ldq < n) return -6;
     if (!workspace || ((uintptr_t)workspace % 256) != 0) return -7;
     if (ws_bytes < gb::tridiag_dc_workspace_bytes(n)) return -8;
-    const cudaError_t err = gb::tridiag_dc_d(n, n, d, e, lam, Q, ldq, workspace, (cudaStream_t)stream);
+    const cudaError_t err = gb::tridiag_dc_d(n, n, d, e, lam, Q, ldq, workspace, (cudaStream_t)stream, nullptr);
     return err == cudaSuccess ? GB_OK : GB_ERR_CUDA;
 }
 
