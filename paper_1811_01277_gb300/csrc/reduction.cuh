@@ -168,8 +168,12 @@ __device__ __forceinline__ ReflZ reflector(Zc alpha, double ss)
         // sg (a + nrm) + i im, |alpha - beta|^2 = (a + nrm)^2 + im^2
         tau = Zc{fma(a, inv, 1.0), sg * alpha.im * inv};
         const double dr = a + nrm, dd = fma(dr, dr, alpha.im * alpha.im);
-        const double f = mid_range(dd) ? newton_recip(dd) : 1.0 / dd;
-        scal = Zc{sg * dr * f, -alpha.im * f};
+        if (mid_range(dd)) {
+            const double f = newton_recip(dd);
+            scal = Zc{sg * dr * f, -alpha.im * f};
+        } else {   // 1 / dd overflows from dd = 2^-1024 down, the quotients do not
+            scal = Zc{sg * dr / dd, -alpha.im / dd};
+        }
     }
     return {tau, scal, beta};
 }

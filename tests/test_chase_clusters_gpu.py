@@ -94,3 +94,47 @@ def test_chase_concurrent(gb, cplx, n, b):
             assert gb.gb_trans_ev_query(w[4], wsb, st) == 0
             for x, y in zip(w[:4], alone[:4]):
                 assert torch.equal(x, y)
+
+
+def tiny_column(m, size, cplx):
+    """A column of m entries of about `size`, its reflector (tau, v) computed on
+    the column times 2^500, and the bound on either's error: the sum of squares
+    s is taken unscaled, each of its 2 m roundings up to 2^-1075, so tau and v
+    are off by up to 4 (2 m 2^-1075 / s) and a few units of 2^-53."""
+    g = np.random.default_rng(m)
+    x = g.uniform(0.5, 1.0, m) * (np.exp(2j * np.pi * g.random(m)) if cplx else 1.0) * size
+    y = x * 2.0 ** 500
+    nrm = np.linalg.norm(y)
+    beta = -nrm if y[0].real >= 0 else nrm
+    s = (nrm * 2.0 ** -500) ** 2
+    bound = 8 * m * 2.0 ** -1074 / s + 16 * U
+    return x, (beta - y[0]) / beta, y[1:] / (y[0] - beta), bound
+
+
+SIZES = [1e-140, 1e-150, 1e-154, 1e-155, 2e-156]
+
+
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("cplx", [False, True], ids=["real", "complex"])
+def test_reflector_of_a_tiny_column(gb, cplx, size):
+    """H(1,0) of a band matrix whose first column below the diagonal has a
+    norm around the square root of the smallest numbers."""
+    n, b = 40, 16
+    x, tau, v, bound = tiny_column(b, size, cplx)
+    B = inputs.band_symmetric(n, b, seed=3, cplx=cplx)
+    AB = np.zeros((n, b + 1), dtype=B.dtype)
+    for k in range(b + 1):
+        AB[:n - k, k] = np.diag(B, -k)
+    AB[0, 1:] = x
+    dev, st = torch.device("cuda"), torch.cuda.current_stream()
+    dt = torch.complex128 if cplx else torch.float64
+    cnt = gb.gb_hh_count(n, b)
+    d, e = torch.zeros(n, dtype=torch.float64, device=dev), torch.zeros(n, dtype=torch.float64, device=dev)
+    hv, ht = torch.zeros(cnt * b, dtype=dt, device=dev), torch.zeros(cnt, dtype=dt, device=dev)
+    wsb = (gb.gb_band_to_tridi_workspace_bytes_z if cplx else gb.gb_band_to_tridi_workspace_bytes)(n, b)
+    ws = torch.empty(wsb, dtype=torch.uint8, device=dev)
+    run = gb.gb_band_to_tridi_z if cplx else gb.gb_band_to_tridi_d
+    run(n, b, torch.from_numpy(AB).to(dev), b + 1, d, e, hv, ht, ws, wsb, st)
+    assert gb.gb_trans_ev_query(ws, wsb, st) == 0
+    assert abs(ht[0].item() - tau) <= bound
+    assert np.abs(hv[1:b].cpu().numpy() - v).max() <= bound

@@ -5,7 +5,12 @@ leave threads idle.  The eigenvalues come out right, with residual and
 orthogonality at rounding level, only if every panel's reflectors and T do.
 Bounds: max |dlambda| / ||A|| <= 1e-11, residual and orthogonality 50 n u.
 """
+import ctypes
+
+import numpy as np
 import pytest
+
+from test_chase_clusters_gpu import SIZES, tiny_column
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -50,3 +55,26 @@ def test_solve_through_panel_forms(gb, n, nbw, cplx):
     V = Z.mT
     assert torch.linalg.norm(A @ V - V * ev) / torch.linalg.norm(A) <= 50 * n * U
     assert (V.mH @ V - torch.eye(nev, dtype=dt, device="cuda")).abs().max() <= 50 * n * U
+
+
+@pytest.mark.parametrize("size", SIZES)
+@pytest.mark.parametrize("m", [40, 600])
+@pytest.mark.parametrize("cplx", [False, True], ids=["real", "complex"])
+def test_reflector_of_a_tiny_column(gb, cplx, m, size):
+    """A panel's first column with a norm around the square root of the smallest
+    numbers (the panel alone: one block, and a cluster)."""
+    x, tau, v, bound = tiny_column(m, size, cplx)
+    nb = 32
+    g = np.random.default_rng(m)
+    P = g.standard_normal((nb, m)) + (1j * g.standard_normal((nb, m)) if cplx else 0.0)
+    P[0] = x
+    Pd = torch.from_numpy(P).cuda()
+    Y, t = torch.zeros_like(Pd), torch.zeros(nb, dtype=Pd.dtype, device="cuda")
+    part = torch.empty(1 << 16, dtype=torch.uint8, device="cuda")
+    ptr = [ctypes.c_void_p(a.data_ptr()) for a in (Pd, t, Y, part)]
+    rc = gb.load().gb_test_panel_hold(ctypes.c_int(cplx), ctypes.c_int(m), ctypes.c_int(nb), *ptr,
+                                      ctypes.c_longlong(10 ** 9), ctypes.c_int(-1), None,
+                                      ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == 0
+    assert abs(t[0].item() - tau) <= bound
+    assert np.abs(Y[0, 1:].cpu().numpy() - v).max() <= bound
