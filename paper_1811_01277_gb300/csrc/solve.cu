@@ -148,6 +148,14 @@ constexpr double kSlicedMinFlops = 1e8;
 
 bool sliced_pays(double m, double n, double k) { return 2.0 * m * n * k >= kSlicedMinFlops; }
 
+// GB_SOLVE_FP32_PRODUCTS takes FP32 products from here on (of one panel, where
+// several go together).  The line is one of accuracy: smaller problems keep
+// FP64 throughout (n <= 1400 or so with nbw = 64), so it does not follow the
+// speed of the sliced products.
+constexpr double kFp32MinFlops = 2.5e8;
+
+bool fp32_product(double m, double n, double k) { return 2.0 * m * n * k >= kFp32MinFlops; }
+
 // Panels whose block reflectors band -> full applies as one, I - Y T Y^H with Y
 // up to 256 columns wide: T's off-diagonal blocks follow from Y^H Y, and the
 // eigenvectors are read and written once per group instead of once per panel.
@@ -361,9 +369,11 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     // large products on the tensor cores unless the caller asks for DFMA
     const bool slice_ok = w.sl && !(flags & GB_SOLVE_DFMA_PRODUCTS);
     auto use_sliced = [&](double m_, double n_, double k_) { return slice_ok && sliced_pays(m_, n_, k_); };
-    // the sliced products of full -> band and band -> full: FP32 products
+    // the large sliced products of full -> band and band -> full: FP32 products
     // (the FP32 split) for the low-precision half of the mixed-precision solve
-    const int pd = (flags & GB_SOLVE_FP32_PRODUCTS) ? gb::kSplitPlanes : gb::kSlices;
+    auto digits = [&](double m_, double n_, double k_) {
+        return (flags & GB_SOLVE_FP32_PRODUCTS) && fp32_product(m_, n_, k_) ? gb::kSplitPlanes : gb::kSlices;
+    };
     cudaStream_t st = (cudaStream_t)stream;
     cudaEvent_t *sev = nullptr;
     if (flags & GB_SOLVE_RECORD_STAGES) {
@@ -412,7 +422,7 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     // lower triangle of C -= X Y^T + Y X^T
     auto update = [&](int m, const double *X, const double *Yp, long long ldy, double *C) -> cudaError_t {
         if (use_sliced(m, m, b))
-            return gb::sliced_dsyr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, w.sl, st, pd, w.status + 2);
+            return gb::sliced_dsyr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, w.sl, st, digits(m, m, b), w.status + 2);
         return gb::dfma_syr2k_lower(m, b, -1.0, X, ldy, Yp, ldy, 1.0, C, ldw, st);
     };
     int pp = 0;
@@ -433,7 +443,8 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
         // only the lower triangle of A2 is kept: X = A2 (Y T) (symmetric
         // product), W = X - Y M / 2, then A2 -= W Y^T + Y W^T on the lower triangle
         if (use_sliced(m, b, m))
-            GB_CU(gb::sliced_dsymm('L', m, b, 1.0, A2, ldw, w.YT, m, 0.0, w.X, m, w.sl, st, pd, w.status + 2));
+            GB_CU(gb::sliced_dsymm('L', m, b, 1.0, A2, ldw, w.YT, m, 0.0, w.X, m, w.sl, st, digits(m, b, m),
+                                    w.status + 2));
         else
             GB_CU(gb::dfma_symm('L', m, b, 1.0, A2, ldw, w.YT, m, 0.0, w.X, m, w.gw, w.gw_elems, st));
         GB_CU(gb::dfma_gemm('T', 'N', b, b, m, 1.0, Yp, m, w.X, m, 0.0, w.Pm, b, w.gw, w.gw_elems, st));
@@ -499,9 +510,9 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
     // ---- band -> full, last group of panels first
     GB_STAGE(6);
     auto gemm = [&](char ta, int m_, int n_, int k_, double alpha, const double *A_, long long la, const double *B_,
-                    long long lb, double beta, double *C_, long long lc, int digits) -> cudaError_t {
+                    long long lb, double beta, double *C_, long long lc, int planes) -> cudaError_t {
         if (use_sliced(m_, n_, k_))
-            return gb::sliced_dgemm(ta, 'N', m_, n_, k_, alpha, A_, la, B_, lb, beta, C_, lc, w.sl, st, digits,
+            return gb::sliced_dgemm(ta, 'N', m_, n_, k_, alpha, A_, la, B_, lb, beta, C_, lc, w.sl, st, planes,
                                     w.status + 2);
         return gb::dfma_gemm(ta, 'N', m_, n_, k_, alpha, A_, la, B_, lb, beta, C_, lc, w.gw, w.gw_elems, st);
     };
@@ -518,6 +529,7 @@ int solve_d_parts(int n, int nev, int nbw, const double *A, int lda, double *ev,
             GB_CU(gb::panel_t(wide, w.Gg, wide, w.tauP + (long long)p0 * b, w.Tg, wide, st));
             T = w.Tg;
         }
+        const int pd = digits(b, nev, m);
         GB_CU(gemm('T', wide, nev, m, 1.0, w.Yg, m, Zr, ldz, 0.0, w.S, wide, pd));
         GB_CU(gemm('N', wide, nev, wide, 1.0, T, wide, w.S, wide, 0.0, w.S2, wide, gb::kSlices));
         GB_CU(gemm('N', m, nev, wide, -1.0, w.Yg, m, w.S2, wide, 1.0, Zr, ldz, pd));

@@ -111,6 +111,16 @@ def test_mixed_solve_small_problem_takes_fp64_products(gb):
     assert d <= 1e-11 and r <= 50 * n * U and o <= 50 * n * U
 
 
+@pytest.mark.parametrize("n,nev,nbw", [(512, 512, 32), (700, 350, 64), (1000, 1000, 64), (1300, 400, 64)])
+def test_mixed_solve_medium_problem_takes_fp64_products(gb, n, nev, nbw):
+    """FP32 products begin where one panel's product has 2.5e8 flops: below
+    that, zero refinement steps give FP64 results."""
+    lam = np.sort(np.random.default_rng(n).uniform(-1.0, 1.0, n))
+    A = inputs.symmetric_with_spectrum(lam, seed=47)
+    d, r, o = errs(A, *mixed(gb, A, nev, nbw, 0), lam)
+    assert d <= 1e-11 and r <= 50 * n * U and o <= 50 * n * U
+
+
 def test_mixed_argument_errors(gb):
     f = gb.gb_solve_mixed_d
     x = torch.zeros(8, dtype=torch.float64, device="cuda")
