@@ -88,7 +88,8 @@ typedef struct gb_trans_ev_opts {
     int sweeps_per_tile; /* nb: consecutive sweeps per tile, 1..32 (rounded up to
                             4, 8 or 16 for WAVEFRONT and 8 or 16 for PIPELINE) */
     int cols_per_block;  /* eigenvector columns per thread block: 32, 64 or 128
-                            (PIPELINE: 64 or 128) */
+                            (PIPELINE: 64 or 128; by default 64, or 32 with
+                            four lanes a column where the columns are few) */
     int spin_limit;      /* PIPELINE only: polls before a dependency wait gives up
                             (0 = default; every wait also gives up after 10 s) */
     int test_hold_group; /* fault-injection hook for tests: when g+1 > 0, sweep
@@ -96,8 +97,9 @@ typedef struct gb_trans_ev_opts {
                             next group's wait must give up; 0 = off */
     int column_batch;    /* PIPELINE, PIPELINE_TC and PIPELINE_TC5: column blocks
                             per ticket batch, 1..1024 (0 = default: 16, 8 for
-                            PIPELINE_TC (64-column blocks), 8 for PIPELINE_TC5
-                            (128-column blocks)).  Items of one batch run
+                            PIPELINE_TC (64-column blocks), for PIPELINE_TC5
+                            (128-column blocks) at least 8 and as many as keep
+                            the device busy along a batch's chain of groups).  Items of one batch run
                             group after group; smaller batches keep fewer
                             eigenvector rows live in L2, larger ones read the
                             reflectors fewer times. */
@@ -125,8 +127,8 @@ long long gb_hh_index(int n, int nbw, int s, int k);
 /* Largest band width the kernels of this build accept. */
 int gb_max_nbw(void);
 
-/* Bytes of device workspace a call needs (0 is possible); the workspace must
- * be 256-byte aligned.  Returns 0 for invalid arguments as well. */
+/* Bytes of device workspace a call needs (0 is possible; more columns never
+ * need less); the workspace must be 256-byte aligned.  Returns 0 for invalid arguments as well. */
 size_t gb_trans_ev_workspace_bytes(int n, int nbw, int nev, int is_complex,
                                    const gb_trans_ev_opts *opts);
 

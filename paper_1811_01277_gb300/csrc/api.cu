@@ -17,6 +17,7 @@ constexpr size_t kMaxSmem = 227 * 1024;
 struct Opts {
     int variant, nb, threads, hold, column_batch, lead_tiles;
     bool lanes;   // PIPELINE with several lanes per column (its default blocking, few columns)
+    int ws_cols;  // columns per block that PIPELINE's workspace is sized for
     long long spin;
 };
 
@@ -27,7 +28,8 @@ constexpr long long kTimeoutNs = 10LL * 1000 * 1000 * 1000;
 // Returns 0 or -11 (opts is the 11th argument of the device entry points).
 // AUTO picks PIPELINE_TC5 (tcgen05) for real or complex data with nbw in
 // {16,32,64} and n >= 512, PIPELINE for the other real cases with nbw in
-// {8,16,32,64} (nb = 16, 64 columns per block) and WAVEFRONT otherwise;
+// {8,16,32,64} (nb = 16, 64 columns per block, or 32 with four lanes a column
+// where the columns are few) and WAVEFRONT otherwise;
 // PIPELINE requested for other cases runs as WAVEFRONT, either tensor-core
 // variant requested for unsupported real cases runs as PIPELINE, and for
 // complex data PIPELINE_TC (real only) and an unsupported PIPELINE_TC5 run as
@@ -67,11 +69,14 @@ int resolve(const gb_trans_ev_opts *o, int n, int nbw, int nev, int is_complex, 
     }
     if (variant == GB_VARIANT_PIPELINE && !pipe_ok) variant = GB_VARIANT_WAVEFRONT;
     r->variant = variant;
-    r->lanes = variant == GB_VARIANT_PIPELINE && !nb && !threads && !r->lead_tiles && n > 1 && nev > 0 &&
-               gb::pipeline_takes_lanes(n, nbw, nev);
+    const bool plain = variant == GB_VARIANT_PIPELINE && !nb && !threads && !r->lead_tiles;   // the default blocking
+    r->lanes = plain && n > 1 && nev > 0 && gb::pipeline_takes_lanes(n, nbw, nev);
     const bool smem = is_complex || nbw > kMaxRegNbw;
     r->nb = nb ? nb : (smem ? 8 : 16);
     r->threads = r->lanes ? 32 : threads ? threads : (variant == GB_VARIANT_PIPELINE || smem ? 64 : 128);
+    // 32-column blocks whichever kernel runs: a workspace for many columns then
+    // serves fewer as well
+    r->ws_cols = plain ? 32 : r->threads;
     // the shared-memory kernels take 32 or 64 columns per block and shrink
     // them or the tile depth until the window fits
     if (smem) {
@@ -145,7 +150,7 @@ size_t gb_trans_ev_workspace_bytes(int n, int nbw, int nev, int is_complex, cons
     if (o.variant == GB_VARIANT_PIPELINE_TC5 && n > 1 && nev > 0)
         return gb::pipeline_tc5_workspace_bytes(n, nbw, nev, is_complex);
     if (o.variant == GB_VARIANT_PIPELINE && !is_complex && n > 1 && nev > 0)
-        return gb::pipeline_workspace_bytes(n, nev, o.nb, o.threads);
+        return gb::pipeline_workspace_bytes(n, nev, o.nb, o.ws_cols);
     return 0;  // the wavefront variant needs no workspace
 }
 

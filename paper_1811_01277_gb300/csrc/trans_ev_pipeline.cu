@@ -338,8 +338,11 @@ pipeline_lanes_d(int n, int nev, const double *__restrict__ hh_v, const double *
 // that one thread per column issues fewer FP64 instructions in all.
 bool pipeline_takes_lanes(int n, int b, int nev)
 {
+    int dev = 0, sms = 152;   // (as without a device, where sizes can still be asked for)
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        sms = 152;
     const long long warps = (nev + 31) / 32, flight = std::min<long long>(group_count(n, 16), (n - 1 + b - 1) / b);
-    return pipeline_supported(b) && warps * flight <= 456;
+    return pipeline_supported(b) && warps * flight <= 3LL * sms;
 }
 
 template <int B, int NB, int THREADS>

@@ -207,3 +207,20 @@ def test_newer_entry_points_check_arguments_host_only(lib):
         gb.gb_solve_batched_graph_create(*args, None, 1 << 30, 2)
     assert e.value.status == -10
     assert gb.gb_solve_batched_graph_nodes(None) == -1
+
+
+@pytest.mark.parametrize("n,b", [(2, 1), (40, 8), (130, 16), (333, 32), (500, 16), (500, 64), (600, 8), (600, 64),
+                                 (2000, 8), (2000, 32)])
+@pytest.mark.parametrize("variant", [0, 1, 2, 3, 4])
+def test_workspace_grows_with_the_columns(lib, n, b, variant):
+    """A workspace sized for many columns serves fewer: no size falls as the
+    number of columns rises, for the back-transformation and for the solves."""
+    nevs = sorted({1, 2, 31, 32, 33, 64, 65, 96, 97, 128, 129, 224, 256, 257, 448, 449, 500, 1000, 1001, 2000})
+    nevs = [k for k in nevs if k <= n]
+    for cplx in (False, True):
+        sizes = [gb.gb_trans_ev_workspace_bytes(n, b, k, cplx, {"variant": variant}) for k in nevs]
+        assert sizes == sorted(sizes)
+    if variant == 0:
+        for f in (gb.gb_solve_workspace_bytes, gb.gb_solve_workspace_bytes_z):
+            sizes = [f(n, k, b) for k in nevs]
+            assert sizes == sorted(sizes) and sizes[0] > 0

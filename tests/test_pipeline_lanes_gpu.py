@@ -61,3 +61,23 @@ def test_nonfinite_entries_reach_the_same_rows(gb):
     one = {"variant": 2, "sweeps_per_tile": 16, "cols_per_block": 64}
     a, c = run(gb, n, b, hv, ht, Z), run(gb, n, b, hv, ht, Z, one)
     assert np.array_equal(np.isfinite(a), np.isfinite(c))
+
+
+def test_workspace_of_more_columns_serves_fewer(gb):
+    """Columns taken in chunks of 256 with a last one of 224, the workspace sized
+    once for 256: n = 1000, nbw = 8, where 224 columns take 32-column blocks."""
+    n, b = 1000, 8
+    hv, ht = inputs.synthetic_reflectors(n, b, seed=2)
+    Z = inputs.z_gaussian(n, 480, seed=4)
+    want = oracle.trans_ev(n, b, hv, ht, Z)
+    Zt = torch.from_numpy(np.ascontiguousarray(Z.T)).cuda()
+    hvd, htd = torch.from_numpy(hv).cuda(), torch.from_numpy(ht).cuda()
+    wsb = gb.gb_trans_ev_workspace_bytes(n, b, 256, 0)
+    ws = torch.empty(wsb, dtype=torch.uint8, device="cuda")
+    st = torch.cuda.current_stream()
+    for c in (0, 256):
+        k = min(256, 480 - c)
+        gb.gb_trans_ev_tridi_to_band_d(n, b, k, hvd, htd, Zt[c:c + k], n, ws, wsb, st)
+        assert gb.gb_trans_ev_query(ws, wsb, st) == 0
+    got = Zt.cpu().numpy().T
+    assert np.max(np.linalg.norm(got - want, axis=0) / np.linalg.norm(Z, axis=0)) <= 1e-12
