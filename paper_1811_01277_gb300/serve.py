@@ -13,7 +13,8 @@ With stage_batching the server also batches one stage across requests: each
 admitted request runs its first stage (full -> band) on its slot, and the
 bulge chases of every request whose first stage has finished run together
 in one persistent launch on one of a few chase lanes (streams); each request
-then runs its remaining stages on its slot again.  The results are
+then runs its remaining stages on its slot again.  A request waits for the
+first stages of others of like size only.  The results are
 bit-identical to the one-call solve.  Merging pays little when the requests'
 chases already overlap on their own streams; it pays when more problems are
 ready at once than there are streams.
@@ -28,6 +29,14 @@ from dataclasses import dataclass, field
 import torch
 
 from . import _lib as gb
+
+
+# Stage batching: a request whose front is done waits for the fronts of others
+# up to this many times its size, to share their chase launch; a small one does
+# not wait for a large one's.  Sizes 512 to 2048 served in 12 slots on a GB300:
+# 88.9 - 92.8 solves/s; waiting for every front 92.2 - 94.0, for none (after 2 ms)
+# 77.5 - 83.2.
+LIKE_SIZE = 2.0
 
 
 @dataclass
@@ -167,10 +176,13 @@ class EigenServer:
             if lane["end"] is not None:
                 continue
             ready = [r for r in self.active if r._phase == "chase_wait"]
-            # fronts finish within a few milliseconds of one another: a launch
-            # waits until at least as many requests are ready as are still in
-            # their fronts, or it would take them one by one
-            if not ready or len(ready) < sum(r._phase == "front" for r in self.active):
+            # fronts of like sizes finish close together: a launch waits until at
+            # least as many requests are ready as such fronts are under way, or
+            # it would take them one by one (see LIKE_SIZE)
+            if not ready:
+                break
+            limit = LIKE_SIZE * min(r.n for r in ready)
+            if len(ready) < sum(r._phase == "front" and r.n <= limit for r in self.active):
                 break
             kind = ready[0].complex
             batch = [r for r in ready if r.complex == kind]

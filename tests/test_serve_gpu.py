@@ -154,6 +154,25 @@ def test_stage_batching_equals_one_call_solves(serve):
         check(mats[r.rid], r.ev.cpu().numpy(), r.Z.cpu().numpy().T, spectra[r.rid])
 
 
+def test_small_request_does_not_wait_for_large_fronts(serve):
+    """With stage batching a small request beside two large ones starts its
+    chase when it is ready: alone, long before their first stages end."""
+    dev = torch.device("cuda")
+    g = torch.Generator(device=dev).manual_seed(1)
+
+    def request(rid, n):
+        R = torch.randn(n, n, generator=g, dtype=torch.float64, device=dev)
+        return serve.Request(rid=rid, A=0.5 * (R + R.T), nev=n // 4, arrival=0.0)
+
+    # (sizes whose first stage fits a stream's launch queue: issuing it does not
+    # block; the first run loads the kernels)
+    for _ in range(2):
+        srv = serve.EigenServer(slots=3, stage_batching=True)
+        done = srv.run([request(0, 2400), request(1, 2400), request(2, 200)])
+    assert all(r.status == 0 for r in done)
+    assert done[0].rid == 2 and srv.chase_sizes[0] == 1
+
+
 def test_stage_api_real_equals_one_call(serve):
     """gb_solve_stage_front / _chase_batched / _back on three real problems
     (their chases in one launch) give the same bits as gb_solve_d."""
