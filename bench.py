@@ -38,8 +38,8 @@ WORKLOADS = {
 # FP64 DFMA: 2 lanes per clock per SM on GB300 (1.25 TFLOP/s nominal at the
 # 2070 MHz maximum SM clock over 152 SMs: 152 * 2 * 2 flop * 2.07e9).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
-# measured constants of this part (one GB300, SM clock 2070 MHz throughout;
-# profiles/fp64_peak_and_variant_sweep.md): the DFMA pipe and the legacy
+# measured constants of this part (one GB300, SM clock 2070 MHz throughout, a
+# standalone microbenchmark): the DFMA pipe and the legacy
 # warp-level bf16 mma.sync m16n8k16 path
 FP64_DFMA_MEASURED_TFLOPS = 1.256
 MMA_SYNC_BF16_TFLOPS = 606.0

@@ -1,4 +1,4 @@
-// FP64 matrix products on the bf16 tensor cores by exact digit slicing (the
+// FP64 matrix products on the tensor cores by exact digit slicing (the
 // error-free splitting idea of Ozaki, Ogita, Oishi and Rump, "Error-free
 // transformations of matrix multiplication by using fast routines of matrix
 // multiplication", Numer. Algorithms 59 (2012), in its fixed-point form).
@@ -7,8 +7,8 @@
 // so that its largest entry is below one, rounded to 62 fraction bits and cut
 // into kSlices balanced base-256 digits in [-128, 127], each exact in FP16.
 // The product of digit planes i (of A) and j (of B) lands in "level" i + j.
-// Pairs with i + j <= 7 are formed; the rest lie 2^-62 sqrt(k) below the scaled
-// row / column maxima.  Every level has its own FP32 tensor-core accumulator;
+// Pairs with i + j <= 7 are formed; the rest are below 7.1 k 2^-62 of the scaled
+// row / column maxima (about 2^-62 sqrt(k) with random signs).  Every level has its own FP32 tensor-core accumulator;
 // over 128 consecutive k its sum is an integer of at most 2^24, so it is exact,
 // and it is folded into one 96-bit integer per output.  The result is rounded
 // to FP64 once, at the end (sliced_tc5.cu).
@@ -77,7 +77,8 @@ struct SlicedOp {
 size_t sliced_bytes(int R, int K);
 
 // Slices an R x K view of src into buf (sliced_bytes(R, K) bytes, 256-byte
-// aligned); fills *out.  Two launches and a memset on st.  `digits`:
+// aligned); fills *out.  One launch on st (the FP32 split, and digits of at most
+// 160 values of k), else two and a memset.  `digits`:
 // kSlices (the FP64-accurate digits) or kSplitPlanes (the FP32 split; both
 // operands of a product must then be split).
 cudaError_t slice_matrix(SliceView view, int R, int K, const double *src, long long ld, void *buf, SlicedOp *out,

@@ -6,8 +6,9 @@
 // two (|x| <= 2^62), cut into eight digits d_s in [-128, 127], exact in FP16.
 // The 36 digit pairs s + t <= 7 accumulate in FP32, one accumulator per level
 // l = s + t, over at most 128 values of k: (l + 1) 128 2^14 <= 2^24, so every
-// sum is exact.  The dropped levels lie below 2^-62 sqrt(k) of the row maxima's
-// product, under the 2^-57 sqrt(k) that 56-bit digits leave.
+// sum is exact.  The dropped levels, the first of them seven pairs of up to
+// 2^14 a value of k, lie below 7.1 k 2^-62 of the row maxima's product; with digits
+// of random signs about 2^-62 sqrt(k), where 56-bit digits left 2^-57 sqrt(k).
 //
 // One CTA owns a 128 x 64 tile of C: 8 levels x 64 columns of FP32 fill the
 // 512 columns of tensor memory.  One MMA per A plane s and half of the levels:
@@ -34,7 +35,7 @@
 // Measured on a GB300 (whole calls, slicing included; before: the same scheme
 // on bf16 mma.sync, 43 pairs of 7-bit digits): 8192^3 139.8 -> 22.8 ms (48.2
 // TFLOP/s of FP64, 0.90 of the tensor rate over 36), 4096^3 17.9 -> 3.2 ms,
-// 3001 x 1777 x 4099 6.14 -> 1.26 ms; the n = 16320 panel products of a
+// 3001 x 1777 x 4099 6.14 -> 1.29 ms; the n = 16320 panel products of a
 // solver: symmetric x 64 columns 9.0 -> 2.3 ms (1.4 of it slicing, HBM-bound),
 // rank-128 update 7.9 -> 1.8 ms; 64 x 4096, k = 16384 2.3 -> 0.78 ms.  Error
 // against 64-bit references 1.2e-15 to 3.0e-15, as before.

@@ -142,8 +142,7 @@ bool use_dc(int n, int nev) { return 2LL * nev > n; }
 // Products of at least this many flops go to the sliced tensor-core kernels
 // (below it the extra launches of slicing cost more than they save: 1e8 flops
 // take 80 us of the whole FP64 pipe, a sliced product 60).  Solves with the line
-// at 2.5e8 and at 1e8: n = 1024 20.3, 19.8 ms; complex 1501 81.2, 78.5; a batch of 24
-// up to n = 2048 338, 303.
+// at 2.5e8 and at 1e8: n = 1024 20.3, 19.8 ms; complex 1501 81.2, 78.5.
 constexpr double kSlicedMinFlops = 1e8;
 
 bool sliced_pays(double m, double n, double k) { return 2.0 * m * n * k >= kSlicedMinFlops; }
