@@ -135,15 +135,13 @@ __device__ __forceinline__ void cut_tile(int tid, const double *t, int sr, int s
 
 __device__ __forceinline__ int cut_row(int tid) { return ((tid >> 5) << 3) | (tid & 7); }
 
-constexpr int kMaxK = 256;   // k a block of the row maxima covers
-
-// High words of the row maxima, 32 rows x kMaxK values of k a block.
+// High words of the row maxima, 32 rows x `span` values of k a block.
 __global__ void __launch_bounds__(256) tc5_rowmax(int view, const double *__restrict__ src, long long ld, int R, int K,
-                                                  uint32_t *__restrict__ rmax)
+                                                  int span, uint32_t *__restrict__ rmax)
 {
     __shared__ uint32_t red[8][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
-    const int r0 = blockIdx.y * 32, kb = blockIdx.x * kMaxK, ke = min(K, kb + kMaxK);
+    const int r0 = blockIdx.y * 32, kb = blockIdx.x * span, ke = min(K, kb + span);
     if (view == kViewRow || view == kViewZExpandN || view == kViewZRowConj) {   // r runs along memory
         uint32_t m = 0;
         if (r0 + tx < R)
@@ -183,18 +181,18 @@ __global__ void __launch_bounds__(256) tc5_rowmax(int view, const double *__rest
     }
 }
 
-// Digits of 32 rows x 128 k a block, the row maxima known.  A symmetric view
-// reads each stored tile once and writes it and its mirror image.
+// Digits of 32 rows x `chunks` chunks of 32 k a block, the row maxima known.  A
+// symmetric view reads each stored tile once and writes it and its mirror image.
 __global__ void __launch_bounds__(256) tc5_slice(int view, const double *__restrict__ src, long long ld, int R, int K,
-                                                 int rows, int KC, const uint32_t *__restrict__ rmax,
+                                                 int rows, int KC, int chunks, const uint32_t *__restrict__ rmax,
                                                  unsigned char *__restrict__ planes, int *__restrict__ e_out)
 {
     __shared__ double t[32][33];
     const int tid = threadIdx.y * 32 + threadIdx.x;
     const int r0 = blockIdx.y * 32;
     if (blockIdx.x == 0 && tid < 32) e_out[r0 + tid] = r0 + tid < R ? exponent_of(rmax[r0 + tid]) : 0;
-    for (int c = 0; c < 4; c++) {
-        const int k0 = (blockIdx.x * 4 + c) * 32;
+    for (int c = 0; c < chunks; c++) {
+        const int k0 = (blockIdx.x * chunks + c) * 32;
         if (k0 >= KC * 32 || (view == kViewSym && k0 > r0)) break;
         load_tile(view, src, ld, R, K, r0, k0, t);
         __syncthreads();
@@ -215,7 +213,10 @@ __global__ void __launch_bounds__(256) tc5_slice(int view, const double *__restr
 
 // Short rows (K <= 160): a block takes all k of its 32 rows, maxima first,
 // then digits (the second read comes from L2): one launch instead of three.
-__global__ void __launch_bounds__(256) tc5_slice_rows(int view, const double *__restrict__ src, long long ld, int R, int K,
+// The view is a template argument: a short kernel's time is latency, and a
+// switch per load adds to it (A^T B of 100 x 100 x 100 51.7 -> 43.6 us a call).
+template <int view>
+__global__ void __launch_bounds__(256) tc5_slice_rows(const double *__restrict__ src, long long ld, int R, int K,
                                                       int rows, int KC, unsigned char *__restrict__ planes,
                                                       int *__restrict__ e_out)
 {
@@ -235,12 +236,15 @@ __global__ void __launch_bounds__(256) tc5_slice_rows(int view, const double *__
             ex[tx] = exponent_of(m);
         }
     } else {
-        for (int i = ty; i < 32; i += 8) {
-            m = 0;
-            if (r0 + i < R)
-                for (int k = tx; k < K; k += 32) m = max(m, abs_hi(view_at(view, src, ld, r0 + i, k)));
-            m = __reduce_max_sync(0xffffffffu, m);
-            if (tx == 0) ex[i] = exponent_of(m);
+        uint32_t row[4] = {0, 0, 0, 0};   // (all rows' loads before the first reduction)
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            if (r0 + ty + 8 * q < R)
+                for (int k = tx; k < K; k += 32) row[q] = max(row[q], abs_hi(view_at(view, src, ld, r0 + ty + 8 * q, k)));
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            m = __reduce_max_sync(0xffffffffu, row[q]);
+            if (tx == 0) ex[ty + 8 * q] = exponent_of(m);
         }
     }
     __syncthreads();
@@ -669,15 +673,37 @@ cudaError_t tc5_slice_matrix(SliceView view, int R, int K, const double *src, lo
     // one launch where a block's rows are short (10 us for 512 blocks at K = 64;
     // 33 us at K = 512, where the three launches of the tiled form are faster)
     if (K <= 160 && view != kViewSym) {
-        tc5_slice_rows<<<rows / 32, block, 0, st>>>((int)view, src, ld, R, K, rows, KC, (unsigned char *)planes, e);
+        auto run = [&](auto kernel) {
+            kernel<<<rows / 32, block, 0, st>>>(src, ld, R, K, rows, KC, (unsigned char *)planes, e);
+        };
+        switch (view) {
+        case kViewRow: run(tc5_slice_rows<kViewRow>); break;
+        case kViewCol: run(tc5_slice_rows<kViewCol>); break;
+        case kViewZExpandN: run(tc5_slice_rows<kViewZExpandN>); break;
+        case kViewZExpandC: run(tc5_slice_rows<kViewZExpandC>); break;
+        case kViewZHermExpand: run(tc5_slice_rows<kViewZHermExpand>); break;
+        default: run(tc5_slice_rows<kViewZRowConj>); break;
+        }
         return cudaGetLastError();
     }
     cudaError_t err = cudaMemsetAsync(rmax, 0, (size_t)rows * sizeof(uint32_t), st);
     if (err != cudaSuccess) return err;
-    tc5_rowmax<<<dim3((K + kMaxK - 1) / kMaxK, rows / 32), block, 0, st>>>((int)view, src, ld, R, K, rmax);
+    // A block's chunks of k are a chain of loads, so they go to blocks of their
+    // own until other blocks hide the chain, at about 32 blocks an SM.  Symmetric
+    // n x n times 64 columns, one chunk a block against eight (maxima) and four
+    // (digits): n = 200 52.8 and 69.2 us, 1000 73.9 and 90.4, 2000 107 and 141; transposed
+    // operands 200 52.9 and 65.1, 2500 151 and 152, 4000 282 and 237.
+    int dev = 0, sms = 0;
+    if ((err = cudaGetDevice(&dev)) != cudaSuccess) return err;
+    if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return err;
+    const long long tiles = (long long)KC * (rows / 32);
+    const int chunks = tiles <= 32LL * sms ? 1 : 4;
+    // (maxima of long rows: blocks of more k, two an SM, for fewer atomics)
+    const int span = view == kViewSym && chunks == 1 ? 32 : 32 * (int)std::min(8LL, std::max(1LL, tiles / (2 * sms)));
+    tc5_rowmax<<<dim3((K + span - 1) / span, rows / 32), block, 0, st>>>((int)view, src, ld, R, K, span, rmax);
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
-    tc5_slice<<<dim3((KC + 3) / 4, rows / 32), block, 0, st>>>((int)view, src, ld, R, K, rows, KC, rmax,
-                                                               (unsigned char *)planes, e);
+    tc5_slice<<<dim3((KC + chunks - 1) / chunks, rows / 32), block, 0, st>>>((int)view, src, ld, R, K, rows, KC, chunks, rmax,
+                                                                             (unsigned char *)planes, e);
     return cudaGetLastError();
 }
 

@@ -205,3 +205,24 @@ def test_nonfinite_entries_of_the_other_forms(gb, x):
     gb.gb_zgemm_sliced("N", n, n, k, 1.0, A, n, B, k, 0.0, out, n, ws, wsb, st)
     got = torch.view_as_real(out.T.contiguous())
     assert torch.equal(torch.nan_to_num(got, nan=1e9), torch.nan_to_num(want, nan=1e9))
+
+
+@pytest.mark.parametrize("n", [161, 300, 2200, 2600])
+def test_long_operands_exact(gb, n):
+    """Operands of one chunk of k a block and (n = 2600) of several: symmetric,
+    and general ones along rows and columns."""
+    c = 5
+    g = torch.Generator(device="cuda").manual_seed(n)
+    st = torch.cuda.current_stream()
+    S, B = ints(g, n, n), ints(g, c, n)
+    Y = S.tril() + S.tril(-1).T
+    out = torch.zeros(c, n, dtype=torch.float64, device="cuda")
+    wsb = gb.gb_dsymm_sliced_workspace_bytes("L", n, c)
+    ws = torch.full((wsb,), 255, dtype=torch.uint8, device="cuda")
+    gb.gb_dsymm_sliced("L", n, c, 1.0, S.T.contiguous(), n, B, n, 0.0, out, n, ws, wsb, st)
+    assert torch.equal(out.T, Y @ B.T)
+    for ta in "NT":
+        wsb = gb.gb_dgemm_sliced_workspace_bytes(n, c, n)
+        ws = torch.full((wsb,), 255, dtype=torch.uint8, device="cuda")
+        gb.gb_dgemm_sliced(ta, "N", n, c, n, 1.0, S, n, B, n, 0.0, out, n, ws, wsb, st)
+        assert torch.equal(out.T, (S.T if ta == "N" else S) @ B.T)
