@@ -248,29 +248,51 @@ int sm_count()
     return sms;
 }
 
-// Tile and splits.  64 x 64 tiles where they alone give each SM two CTAs (99 %
-// of the FP64 pipe in long products), else 32 x 32 ones; then the reduction is
-// split until every SM has two CTAs, keeping 16 values of k per split and the
-// partials within the workspace.
+// Tile and splits: the cheapest of 64 x 64 and 32 x 32 tiles, the reduction in
+// one piece or split so that the CTAs fill one to eight per SM (16 values of k
+// a split at least, the partials within the workspace).  The cost of a shape
+// is its fullest SM's FP64 issue, two FMAs a clock, with kEdge values of k for a
+// CTA's start and end, and for splits the partials' way through memory; 32 x 32
+// tiles issue 4 % slower, a CTA alone on its SM 6 %.  (Splitting to two CTAs an SM
+// left its last wave half empty: 64 x 4096, k = 16384 8.24 ms in 512 CTAs, 7.2 in 1024.)
 struct Shape {
     int ts, splits;
 };
 
 Shape choose_shape(const Gemm &g, size_t work_elems)
 {
-    const long long target = 2LL * sm_count();
-    auto tiles = [&](int ts) {
-        const long long tm = (g.m + ts - 1) / ts, tn = (g.n + ts - 1) / ts;
-        return g.lower ? tm * (tm + 1) / 2 : tm * tn;
-    };
-    Shape s{64, 1};
-    if (tiles(64) < target) s.ts = 32;
-    const long long t = tiles(s.ts), k = (long long)g.k + g.k2;
-    if (g.partial && !g.lower && t < target) {
-        long long sp = std::min({(target + t - 1) / t, k / 16, 64LL, (long long)(work_elems / ((size_t)g.m * g.n))});
-        s.splits = (int)std::max(1LL, sp);
+    constexpr int kEdge = 8;
+    const long long sms = sm_count(), k = (long long)g.k + g.k2, out = (long long)g.m * g.n;
+    const long long most = g.partial && !g.lower ? std::min({k / 16, 64LL, (long long)(work_elems / (size_t)out)}) : 1;
+    Shape best{32, 1};
+    double least = 0.0;
+    for (int ts : {64, 32}) {
+        if (ts == 64 && std::min(g.m, g.n) <= 32) continue;
+        const long long tm = (g.m + ts - 1) / ts, tn = (g.n + ts - 1) / ts, bk = 512 / ts;
+        const long long t = g.lower ? tm * (tm + 1) / 2 : tm * tn;
+        long long sp = 1;
+        for (int per = 0; per <= 8; per++) {   // CTAs per SM (0: no split)
+            if (per) {
+                const long long next = std::min(per * sms / t, most);
+                if (next <= sp) {
+                    if (sp >= most) break;
+                    continue;
+                }
+                sp = next;
+            }
+            const long long kc = ((k + sp - 1) / sp + bk - 1) / bk * bk;
+            const long long fullest = (t * sp + sms - 1) / sms;
+            double clocks = (double)fullest * (ts * ts / 2) * (double)(kc + kEdge);
+            if (ts == 32) clocks *= 1.04;
+            if (fullest == 1) clocks *= 1.06;
+            if (sp > 1) clocks += 3000.0 + (double)(sp * out) * 16.0 / 3300.0;   // a launch; 6.8 TB/s at 2.07 GHz
+            if (least == 0.0 || clocks < least) {
+                least = clocks;
+                best = Shape{ts, (int)sp};
+            }
+        }
     }
-    return s;
+    return best;
 }
 
 template <int MA, int MB, int TS>
